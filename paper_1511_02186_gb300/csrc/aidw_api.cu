@@ -113,7 +113,6 @@ struct aidw_ctx {
     aidw_kernel_times last{};
     bool last_valid = false;
     int slots_cache[3][4][2] = {};  // [precision][kp bucket][with_idx] knn slots
-    int wslots_cache[3][3][2] = {};  // [precision][queries per thread 2/4/8][tile 256/512]
     aidw_tune_config tune = aidw::tune_default();
     ServingRuntime *serving = nullptr;
     int64_t serving_queue_limit = 4096;  // requests waiting for admission at most
@@ -123,7 +122,7 @@ namespace aidw {
 
 // ---- memory accounting --------------------------------------------------------------------
 
-int ctx_alloc(aidw_ctx *ctx, size_t bytes, cudaStream_t st, void **p)
+int ctx_alloc(aidw_ctx *ctx, size_t bytes, cudaStream_t st, void **p, bool *injected)
 {
     *p = nullptr;
     if (bytes == 0)
@@ -133,6 +132,8 @@ int ctx_alloc(aidw_ctx *ctx, size_t bytes, cudaStream_t st, void **p)
         if (ctx->fail_after >= 0) {
             if (ctx->fail_after == 0) {
                 ctx->fail_after = -1;
+                if (injected)
+                    *injected = true;
                 return AIDW_ERR_OOM;
             }
             --ctx->fail_after;
@@ -250,10 +251,87 @@ static PassPlan plan_pass(int64_t m, int64_t n_pad, int qpb, int slots_total, in
     return pp;
 }
 
+// Phase 2 cut into (query blocks) x (data splits of whole granules).
+static PassPlan weights_split(int64_t m, int64_t n_sum, int qpb, int64_t S)
+{
+    PassPlan pp{};
+    const int64_t G = n_sum / kSplitGranule;
+    S = std::max<int64_t>(1, std::min<int64_t>(S, std::min<int64_t>(G, kMaxSplitsW)));
+    const int64_t per = (G + S - 1) / S;
+    pp.q_per_block = qpb;
+    pp.qblocks = static_cast<int>((m + qpb - 1) / qpb);
+    pp.splits = static_cast<int>((G + per - 1) / per);
+    pp.split_len = per * kSplitGranule;
+    return pp;
+}
+
+// What phase 2 costs in a precision, measured on GB300 (ns).
+struct WeightsCost {
+    double pair;  // one SM, full of CTAs, per pair
+    double cta;   // one SM, per CTA (start, tables, first tile, sums out)
+    double part;  // whole GPU, per query and split (partial sums written and merged)
+    bool shares;  // several CTAs share an SM; one alone leaves it partly idle
+};
+
+// The split count with the least estimated time among those that give every SM about 1, 2, ...
+// 48 CTAs (at least up to 8 splits): an SM's share of the CTAs (rounded up) times their cost, over the rate a few
+// co-resident CTAs reach, plus a part of one CTA for the uneven end and the cost of the partial
+// sums. Measured (FP32, us with the finalisation; the split count the estimate takes, and
+// 2,048-point granules with at most 64 splits before): 1,024 x 1,024: 14 against 29; 257 x
+// 300,007: 57 against 143; 8,192 x 1M: 2,800 against 2,959 (37 splits of 1,216 slots).
+static PassPlan plan_weights(int64_t m, int64_t n_sum, int qpb, int sm_count,
+                             const WeightsCost &wc)
+{
+    const int64_t qblocks = (m + qpb - 1) / qpb;
+    PassPlan best{};
+    double best_t = 1e300;
+    int64_t last = 0;
+    for (int per_sm = 1; per_sm <= 48; ++per_sm) {
+        const int64_t S = std::max<int64_t>(static_cast<int64_t>(per_sm) * sm_count / qblocks,
+                                            std::min(per_sm, 8));
+        const PassPlan pp = weights_split(m, n_sum, qpb, S);
+        if (pp.splits == last)
+            continue;
+        last = pp.splits;
+        const int64_t items = qblocks * pp.splits;
+        const double k = static_cast<double>((items + sm_count - 1) / sm_count);
+        const double one = static_cast<double>(pp.split_len) * qpb * wc.pair;
+        const double idle = wc.shares ? 1.0 + 0.35 / (k * std::sqrt(k)) : 1.0;
+        const double t = k * (one + wc.cta) * idle + 0.3 * one +
+                         wc.part * static_cast<double>(m) * pp.splits;
+        if (t < best_t * (1.0 - 1e-9)) {
+            best_t = t;
+            best = pp;
+        }
+    }
+    return best;
+}
+
 // AIDW_F64 and AIDW_F64X share the FP64 arrays, phase 1, selection and finalisation.
 static bool f64_arrays(int precision)
 {
     return precision == AIDW_F64 || precision == AIDW_F64X;
+}
+
+// Point groups per phase-2 CTA. Without them a CTA serves 256 queries (FP64: 1,024), with them
+// a quarter of that, which wastes fewer lanes beyond the last query but shares a tile among
+// fewer queries. Measured (us, 1 group / 4 groups): FP32 257 x 300,007: 78 / 57, 1,024 x 1M:
+// 389 / 383, 4,096 x 1M: 1,413 / 1,427; FP64 257 x 16,384: 274 / 145, 4,100 x 16,384: 1,122 /
+// 1,000, 8,191 x 131,072: 13,010 / 13,279; F64X 4,100 x 65,536: 2,190 / 2,109, 16,384 x 262,144:
+// 31,813 / 32,170. A function of the precision and m alone: the groups regroup the partial sums.
+static int weights_point_groups(int precision, int64_t m)
+{
+    const int64_t q1 = precision == AIDW_F64 ? 1024 : 256, q4 = q1 / kPointGroups;
+    const double lanes1 = static_cast<double>((m + q1 - 1) / q1 * q1);
+    const double lanes4 = static_cast<double>((m + q4 - 1) / q4 * q4);
+    return m <= 2048 || lanes4 * 1.02 < lanes1 ? kPointGroups : 1;
+}
+
+static WeightsCost weights_cost(int precision)
+{
+    return precision == AIDW_F32C ? WeightsCost{0.048, 150.0, 0.006, true}
+           : precision == AIDW_F64 ? WeightsCost{1.75, 6000.0, 0.05, false}
+                                   : WeightsCost{1.1, 500.0, 0.05, true};
 }
 
 static int kp_bucket(int kp)
@@ -261,8 +339,9 @@ static int kp_bucket(int kp)
     return kp <= 8 ? 0 : (kp <= 12 ? 1 : (kp <= 16 ? 2 : 3));
 }
 
-Plan make_plan(aidw_ctx *ctx, int precision, int64_t n_pad, int64_t m, int k, bool with_idx,
-               int force_knn_splits, int force_w_splits, const aidw_tune_config *cfg)
+Plan make_plan(aidw_ctx *ctx, int precision, int64_t n, int64_t n_pad, int64_t m, int k,
+               bool with_idx, int force_knn_splits, int force_w_splits,
+               const aidw_tune_config *cfg)
 {
     const aidw_tune_config &tc = cfg ? *cfg : ctx->tune;
     const bool f64 = f64_arrays(precision);
@@ -277,14 +356,11 @@ Plan make_plan(aidw_ctx *ctx, int precision, int64_t n_pad, int64_t m, int k, bo
     int &ks = ctx->slots_cache[precision][kp_bucket(f64 ? k : pl.kp)][with_idx ? 1 : 0];
     if (!ks)
         ks = f64 ? f64_knn_slots_per_sm(k, with_idx) : f32_knn_slots_per_sm(pl.kp, with_idx);
-    int &ws = ctx->wslots_cache[precision][pl.qw == 2 ? 0 : (pl.qw == 4 ? 1 : 2)]
-                               [pl.tw == 256 ? 0 : 1];
-    if (!ws)
-        ws = x ? f64x_w_slots_per_sm()
-               : (f64 ? f64_w_slots_per_sm() : f32_w_slots_per_sm(pl.qw, pl.tw));
+    pl.pg = weights_point_groups(precision, m);
     const int qk = f64 ? f64_knn_queries_per_block(k) : f32_knn_queries_per_block(pl.kp);
-    const int qw = x ? f64x_w_queries_per_block()
-                     : (f64 ? f64_w_queries_per_block() : f32_w_queries_per_block(pl.qw));
+    const int qw = x ? f64x_w_queries_per_block(pl.pg)
+                     : (f64 ? f64_w_queries_per_block(pl.pg)
+                            : f32_w_queries_per_block(pl.qw, pl.pg));
     // A split restarts its neighbour lists: about k (1 + ln(n_split / k)) insertions per query,
     // each a rescan of a chunk by a partly idle warp. Measured on GB300 at n = m = 2^20,
     // k = 10, every extra split costs about as much as scanning 100,000 more points.
@@ -293,19 +369,16 @@ Plan make_plan(aidw_ctx *ctx, int precision, int64_t n_pad, int64_t m, int k, bo
     // which co-resident CTAs share: it is planned as one CTA per SM (measured at n = 1M,
     // 4,096 queries: 8 splits 24 ms, 37 splits 39 ms).
     pl.knn = plan_pass(m, n_pad, qk, (f64 ? 1 : ks) * ctx->sm_count, 10000 * k);
-    pl.w = plan_pass(m, n_pad, qw, ws * ctx->sm_count, 1024);
-    const int64_t G = n_pad / kPadPoints;
-    auto force = [&](PassPlan &pp, int S) {
-        if (S <= 0)
-            return;
-        S = static_cast<int>(S > G ? G : S);
-        S = S > kMaxSplits ? kMaxSplits : S;
+    const int64_t n_sum = (n + kSplitGranule - 1) / kSplitGranule * kSplitGranule;
+    pl.w = force_w_splits > 0 ? weights_split(m, n_sum, qw, force_w_splits)
+                              : plan_weights(m, n_sum, qw, ctx->sm_count, weights_cost(precision));
+    if (force_knn_splits > 0) {
+        const int64_t G = n_pad / kPadPoints;
+        const int64_t S = std::min<int64_t>(std::min<int64_t>(force_knn_splits, G), kMaxSplits);
         const int64_t per = (G + S - 1) / S;
-        pp.splits = static_cast<int>((G + per - 1) / per);
-        pp.split_len = per * kPadPoints;
-    };
-    force(pl.knn, force_knn_splits);
-    force(pl.w, force_w_splits);
+        pl.knn.splits = static_cast<int>((G + per - 1) / per);
+        pl.knn.split_len = per * kPadPoints;
+    }
     return pl;
 }
 
@@ -716,27 +789,38 @@ int interpolate_impl(aidw_ctx *ctx, aidw_dataset dsid, const void *qx, const voi
         force_knn_splits == -2 && ds.n_pad / kTileF32Knn <= kMaxCullTiles;
     const bool warp = force_knn_splits == -1 ||
                       (force_knn_splits == 0 && use_warp_knn(p->precision, ds, m, ctx->sm_count));
-    Plan pl = make_plan(ctx, p->precision, ds.n_pad, m, p->k, out_knn != nullptr,
-                        force_knn_splits > 0 ? force_knn_splits : 0, force_w_splits, cfg);
-    const bool cull = force_cull || (!warp && force_knn_splits == 0 &&
-                                     use_culled_knn(p->precision, ds, m, out_knn != nullptr, pl));
-    if (cull)
-        plan_culled_knn(&pl, ds.n_pad);
-    if (warp) {
-        // One list per query, [k][m], for the selection kernel.
-        pl.knn.splits = 1;
-        pl.knn.split_len = ds.n_pad;
-    }
-    const size_t sb = scratch_bytes(p->precision, pl, p->k) +
-                      (cull ? culled_extra_bytes(m, p->precision) : 0);
     // Staging for host arrays.
     const size_t b_q = (kq == 0 ? align256(m * es) : 0) + (kqy == 0 ? align256(m * es) : 0);
     const size_t b_o = ko == 0 ? align256(m * es) : 0;
     const size_t b_a = (out_alpha && ka == 0) ? align256(m * sizeof(float)) : 0;
     const size_t b_n = (out_knn && kn == 0) ? align256(m * p->k * sizeof(int32_t)) : 0;
-    const size_t total = sb + b_q + b_o + b_a + b_n;
+    Plan pl;
+    bool cull;
+    size_t sb, total;
     void *blk = nullptr;
-    rc = ctx_alloc(ctx, total, st, &blk);
+    for (int w_splits = force_w_splits;;) {
+        pl = make_plan(ctx, p->precision, ds.n, ds.n_pad, m, p->k, out_knn != nullptr,
+                       force_knn_splits > 0 ? force_knn_splits : 0, w_splits, cfg);
+        cull = force_cull || (!warp && force_knn_splits == 0 &&
+                              use_culled_knn(p->precision, ds, m, out_knn != nullptr, pl));
+        if (cull)
+            plan_culled_knn(&pl, ds.n_pad);
+        if (warp) {
+            // One list per query, [k][m], for the selection kernel.
+            pl.knn.splits = 1;
+            pl.knn.split_len = ds.n_pad;
+        }
+        sb = scratch_bytes(p->precision, pl, p->k) +
+             (cull ? culled_extra_bytes(m, p->precision) : 0);
+        total = sb + b_q + b_o + b_a + b_n;
+        bool injected = false;
+        rc = ctx_alloc(ctx, total, st, &blk, &injected);
+        // Where the planned partial sums do not fit, fewer phase-2 splits (slower, the same
+        // result within the split regrouping) may.
+        if (rc != AIDW_ERR_OOM || injected || force_w_splits > 0 || pl.w.splits <= 1)
+            break;
+        w_splits = pl.w.splits / 2;
+    }
     if (rc)
         return rc;
     Scratch sc;

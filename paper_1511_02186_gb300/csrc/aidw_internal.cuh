@@ -40,7 +40,20 @@ constexpr int kErrTimeout = 1;
 
 // Kernel shape shared by every scan kernel.
 constexpr int kThreads = 128;   // threads per CTA
-constexpr int kMaxSplits = 64;  // data-range splits per pass
+constexpr int kMaxSplits = 64;  // data-range splits of a phase-1 scan
+// Phase 2 cuts the data at any multiple of kSplitGranule points (whole chunks of every precision's
+// summation loop) into at most kMaxSplitsW splits.
+constexpr int kSplitGranule = 32;
+constexpr int kMaxSplitsW = 512;
+// Threads that share the merge of one query's splits (1, 8 or 32): a thread's loads are a chain
+// a few deep, and few queries with many splits would leave most SMs idle. 32 threads read 8
+// neighbouring queries at a time, which many queries pay for (8,191 queries x 342 splits in FP64:
+// 200 us against 110).
+inline int finalize_threads(int splits, int64_t m)
+{
+    return splits >= 64 && m <= 2048 ? 32 : (splits >= 16 ? 8 : 1);
+}
+constexpr int kPointGroups = 4;  // phase 2 with point groups (Plan::pg)
 
 // Levels and bounds of Eq. 5 and Eq. 6, passed to kernels by value.
 struct AlphaMap {
@@ -68,12 +81,12 @@ struct DatasetDev {
 };
 
 // How one scan pass is cut into work: query blocks (one CTA each) times data-range splits,
-// each split a whole number of kPadPoints-point granules.
+// each split a whole number of granules (kPadPoints points in phase 1, kSplitGranule in phase 2).
 struct PassPlan {
     int q_per_block;   // queries handled by one CTA
     int qblocks;       // ceil(m / q_per_block)
     int splits;        // S: data-range splits, each scanned by its own CTA
-    int64_t split_len; // points per split (multiple of kPadPoints)
+    int64_t split_len; // points per split (whole granules)
 };
 
 struct Plan {
@@ -86,6 +99,7 @@ struct Plan {
     int tw;        // FP32 phase 2: data points per shared-memory tile (256 or 512)
     int knn_slots; // phase-1 CTAs resident on the whole GPU (occupancy x SMs)
     int kq;        // pruned phase 1: queries per thread (2 or 4)
+    int pg;        // phase 2: point groups per CTA (1: every thread sees every point)
 };
 
 // Per-query parameters of phase 2 produced by the selection kernel.
@@ -198,9 +212,8 @@ cudaError_t launch_f64x_weights(const DatasetDev &ds, const Plan &pl, const doub
 // allows (used to cut splits into whole waves). FP32 shapes follow the tuning fields of
 // aidw_tune_config (kp: k-list length, qw: phase-2 queries per thread, tw: tile points).
 int f32_knn_queries_per_block(int kp);
-int f32_w_queries_per_block(int qw);
+int f32_w_queries_per_block(int qw, int pg);
 int f32_knn_slots_per_sm(int kp, bool with_idx);
-int f32_w_slots_per_sm(int qw, int tw);
 // k-list length for k under a minimum (aidw_tune_config.knn_list).
 int f32_list_length(int k, int kp_min);
 // Queries per thread of the pruned phase 1 for list length kp under the shape's request
@@ -213,11 +226,9 @@ inline int cull_queries_per_thread(int kp, int requested)
 aidw_tune_config tune_default();
 bool tune_valid(const aidw_tune_config &c);
 int f64_knn_queries_per_block(int k);
-int f64_w_queries_per_block();
+int f64_w_queries_per_block(int pg);
 int f64_knn_slots_per_sm(int k, bool with_idx);
-int f64_w_slots_per_sm();
-int f64x_w_queries_per_block();
-int f64x_w_slots_per_sm();
+int f64x_w_queries_per_block(int pg);
 
 // Pipe-rate microbenchmarks (probe.cu).
 cudaError_t run_pipe_probe(int sm_count, aidw_pipe_rates *out);

@@ -33,7 +33,8 @@ class NvtxScope {
 struct ServingRuntime;
 
 // Device memory from the context's pool, charged to its HBM budget (stream-ordered).
-int ctx_alloc(aidw_ctx *ctx, size_t bytes, cudaStream_t st, void **p);
+// *injected (nullable) is set when the failure is an injected one (aidw_debug_fail_alloc_after).
+int ctx_alloc(aidw_ctx *ctx, size_t bytes, cudaStream_t st, void **p, bool *injected = nullptr);
 void ctx_free(aidw_ctx *ctx, void *p, size_t bytes, cudaStream_t st);
 size_t ctx_budget_left(aidw_ctx *ctx);
 int *ctx_err_word(aidw_ctx *ctx);
@@ -49,8 +50,9 @@ int pointer_kind(const void *p, int device);
 int validate_params(const aidw_params *p, int64_t n);
 AlphaMap alpha_map(const aidw_params &p);
 // Shape from `cfg`, or from the context's shape when cfg is null.
-Plan make_plan(aidw_ctx *ctx, int precision, int64_t n_pad, int64_t m, int k, bool with_idx,
-               int force_knn_splits, int force_w_splits, const aidw_tune_config *cfg = nullptr);
+Plan make_plan(aidw_ctx *ctx, int precision, int64_t n, int64_t n_pad, int64_t m, int k,
+               bool with_idx, int force_knn_splits, int force_w_splits,
+               const aidw_tune_config *cfg = nullptr);
 aidw_tune_config ctx_tune(aidw_ctx *ctx);
 void ctx_set_tune(aidw_ctx *ctx, const aidw_tune_config &c);
 int interpolate_impl(aidw_ctx *ctx, int64_t dsid, const void *qx, const void *qy, int64_t m,

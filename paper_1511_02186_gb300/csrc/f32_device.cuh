@@ -798,7 +798,7 @@ __device__ __forceinline__ int64_t weights_end(const DatasetDev &ds, int64_t p_e
     return min(p_end, (ds.n + kChunkW - 1) / kChunkW * kChunkW);
 }
 
-// Tiles of TW points a phase-2 unit over [p_begin, p_end) loads.
+// Tiles of TW points a phase-2 unit over [p_begin, p_end) loads (the last one possibly partly).
 template <int TW>
 __device__ __forceinline__ int weights_tiles(const DatasetDev &ds, int64_t p_begin,
                                              int64_t p_end)
@@ -807,7 +807,11 @@ __device__ __forceinline__ int weights_tiles(const DatasetDev &ds, int64_t p_beg
     return e > p_begin ? static_cast<int>((e - p_begin + TW - 1) / TW) : 0;
 }
 
-template <int Q, int TW>
+// PG > 1 cuts the CTA's threads into PG groups of kThreads / PG, each thread still holding Q
+// queries: the CTA serves Q kThreads / PG queries, and each group sums its own PG-th part of
+// every chunk (kChunkW points of PG chunks to a Kahan merge); the groups' sums are merged at the
+// end. A call with few queries then wastes fewer lanes on queries it does not have.
+template <int Q, int TW, int PG = 1>
 __device__ __forceinline__ bool weights_unit(const DatasetDev &ds, int64_t m, int64_t qbase,
                                              int64_t p_begin, int64_t p_end,
                                              const float *__restrict__ qx,
@@ -820,8 +824,11 @@ __device__ __forceinline__ bool weights_unit(const DatasetDev &ds, int64_t m, in
 {
     static_assert(Q % 2 == 0, "queries are processed in packed pairs");
     static_assert(TW % kChunkW == 0 && kPadPoints % TW == 0, "whole chunks, whole tiles");
+    static_assert(kThreads % (32 * PG) == 0, "whole warps per group");
     constexpr int H = Q / 2;
+    constexpr int QT = kThreads / PG;  // threads (and query columns) of one point group
     const int tid = threadIdx.x;
+    const int tq = PG == 1 ? tid : tid % QT, pg = PG == 1 ? 0 : tid / QT;
     const int ntiles = weights_tiles<TW>(ds, p_begin, p_end);
     const int64_t p_sum = weights_end(ds, p_end);
 
@@ -829,7 +836,7 @@ __device__ __forceinline__ bool weights_unit(const DatasetDev &ds, int64_t m, in
     float hw[Q], cw[Q], hz[Q], cz[Q];
 #pragma unroll
     for (int j = 0; j < Q; ++j) {
-        const int64_t q = min(qbase + j * kThreads + tid, m - 1);
+        const int64_t q = min(qbase + j * QT + tq, m - 1);
         const float2 o = __ldcg(reinterpret_cast<const float2 *>(qp + q));
         const float a = qx[q], b = qy[q];
         if (j & 1) {
@@ -847,16 +854,19 @@ __device__ __forceinline__ bool weights_unit(const DatasetDev &ds, int64_t m, in
     }
     const float2 eps2 = make_float2(kEpsF32, kEpsF32);
 
-    constexpr uint32_t kBxy = TW * sizeof(float4);
-    constexpr uint32_t kBz = TW * sizeof(float2);
+    // Tile t of the unit: whole chunks only, so a split may start and end at any multiple of
+    // kChunkW (its last tile is loaded up to the split's end and no further).
+    auto load_tile = [&](int t) {
+        const uint32_t b = (ts.seq + t) & 1;
+        const int64_t o = p_begin + static_cast<int64_t>(t) * TW;
+        const uint32_t len = static_cast<uint32_t>(min(static_cast<int64_t>(TW), p_sum - o));
+        mbar_arrive_expect_tx(&ts.bar[b], len * (sizeof(float4) + sizeof(float2)));
+        tma_load_1d(txy[b], ds.nxy2 + o, len * sizeof(float4), &ts.bar[b]);
+        tma_load_1d(tz[b], ds.zz + o, len * sizeof(float2), &ts.bar[b]);
+    };
     if (tid == 0) {
-        for (int t = 0; t < 2 && t < ntiles; ++t) {
-            const uint32_t b = (ts.seq + t) & 1;
-            const int64_t o = p_begin + static_cast<int64_t>(t) * TW;
-            mbar_arrive_expect_tx(&ts.bar[b], kBxy + kBz);
-            tma_load_1d(txy[b], ds.nxy2 + o, kBxy, &ts.bar[b]);
-            tma_load_1d(tz[b], ds.zz + o, kBz, &ts.bar[b]);
-        }
+        for (int t = 0; t < 2 && t < ntiles; ++t)
+            load_tile(t);
     }
 
     for (int t = 0; t < ntiles; ++t) {
@@ -873,27 +883,32 @@ __device__ __forceinline__ bool weights_unit(const DatasetDev &ds, int64_t m, in
         }
         const int64_t t0 = p_begin + static_cast<int64_t>(t) * TW;
         const int cend = static_cast<int>(min(static_cast<int64_t>(TW), p_sum - t0));
-        for (int c = 0; c < cend; c += kChunkW) {
+        for (int c = 0; c < cend; c += PG * kChunkW) {
             float2 sw[H], sz[H];
 #pragma unroll
             for (int h = 0; h < H; ++h)
                 sw[h] = sz[h] = make_float2(0.0f, 0.0f);
-            // The whole chunk unrolled (measured: 355 ms at 1M x 1M against 357-359 ms for
-            // steps of 4, 8 or 16 points, with 70 registers instead of 80).
+            for (int i = 0; i < PG; ++i) {
+                const int cg = c + i * kChunkW + pg * (kChunkW / PG);
+                if (PG > 1 && cg >= cend)
+                    break;
+                // The whole chunk unrolled (measured: 355 ms at 1M x 1M against 357-359 ms for
+                // steps of 4, 8 or 16 points, with 70 registers instead of 80).
 #pragma unroll
-            for (int u = 0; u < kChunkW; ++u) {
-                const float4 p = txy[b][c + u];
-                const float2 zz = tz[b][c + u];
+                for (int u = 0; u < kChunkW / PG; ++u) {
+                    const float4 p = txy[b][cg + u];
+                    const float2 zz = tz[b][cg + u];
 #pragma unroll
-                for (int h = 0; h < H; ++h) {
-                    const float2 dx = __fadd2_rn(qxp[h], make_float2(p.x, p.y));
-                    const float2 dy = __fadd2_rn(qyp[h], make_float2(p.z, p.w));
-                    const float2 d2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, eps2));
-                    const float2 lg = make_float2(lg2_approx(d2.x), lg2_approx(d2.y));
-                    const float2 e = __ffma2_rn(lg, nsp[h], ccp[h]);
-                    const float2 w = make_float2(ex2_approx(e.x), ex2_approx(e.y));
-                    sw[h] = __fadd2_rn(sw[h], w);
-                    sz[h] = __ffma2_rn(w, zz, sz[h]);
+                    for (int h = 0; h < H; ++h) {
+                        const float2 dx = __fadd2_rn(qxp[h], make_float2(p.x, p.y));
+                        const float2 dy = __fadd2_rn(qyp[h], make_float2(p.z, p.w));
+                        const float2 d2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, eps2));
+                        const float2 lg = make_float2(lg2_approx(d2.x), lg2_approx(d2.y));
+                        const float2 e = __ffma2_rn(lg, nsp[h], ccp[h]);
+                        const float2 w = make_float2(ex2_approx(e.x), ex2_approx(e.y));
+                        sw[h] = __fadd2_rn(sw[h], w);
+                        sz[h] = __ffma2_rn(w, zz, sz[h]);
+                    }
                 }
             }
 #pragma unroll
@@ -907,16 +922,37 @@ __device__ __forceinline__ bool weights_unit(const DatasetDev &ds, int64_t m, in
         __syncthreads();
         if (tid == 0 && t + 2 < ntiles) {
             fence_proxy_async_smem();
-            const int64_t o = p_begin + static_cast<int64_t>(t + 2) * TW;
-            mbar_arrive_expect_tx(&ts.bar[b], kBxy + kBz);
-            tma_load_1d(txy[b], ds.nxy2 + o, kBxy, &ts.bar[b]);
-            tma_load_1d(tz[b], ds.zz + o, kBz, &ts.bar[b]);
+            load_tile(t + 2);
         }
     }
     ts.seq += ntiles;
+    if constexpr (PG > 1) {
+        // Group g's sums, in group order, onto group 0's (the tile buffers are free: every
+        // thread has passed the last tile's closing barrier, or loaded none).
+        float4 *g = &txy[0][0];
+        static_assert(sizeof(float4) * Q * kThreads <= sizeof(float4) * 2 * TW, "fits the tiles");
+        if (pg > 0) {
+#pragma unroll
+            for (int j = 0; j < Q; ++j)
+                g[j * kThreads + tid] = make_float4(hw[j], cw[j], hz[j], cz[j]);
+        }
+        __syncthreads();
+        if (pg > 0)
+            return true;
+        for (int i = 1; i < PG; ++i) {
+#pragma unroll
+            for (int j = 0; j < Q; ++j) {
+                const float4 v = g[j * kThreads + i * QT + tq];
+                kahan_add(hw[j], cw[j], v.x);
+                kahan_add(hw[j], cw[j], -v.y);
+                kahan_add(hz[j], cz[j], v.z);
+                kahan_add(hz[j], cz[j], -v.w);
+            }
+        }
+    }
 #pragma unroll
     for (int j = 0; j < Q; ++j) {
-        const int64_t q = qbase + j * kThreads + tid;
+        const int64_t q = qbase + j * QT + tq;
         if (q >= m)
             continue;
         float *o = part_sum + static_cast<int64_t>(s) * 4 * m + q;
@@ -928,16 +964,24 @@ __device__ __forceinline__ bool weights_unit(const DatasetDev &ds, int64_t m, in
     return true;
 }
 
+// The compensated sums of splits s0, s0 + step, ... of one query, added up in FP64.
+__device__ __forceinline__ void merge_splits(int64_t q, int64_t m, int s0, int step, int S,
+                                             const float *part_sum, double &W, double &WZ)
+{
+#pragma unroll 4
+    for (int s = s0; s < S; s += step) {
+        const float *o = part_sum + static_cast<int64_t>(s) * 4 * m + q;
+        W += static_cast<double>(__ldcg(o)) + static_cast<double>(__ldcg(o + m));
+        WZ += static_cast<double>(__ldcg(o + 2 * m)) + static_cast<double>(__ldcg(o + 3 * m));
+    }
+}
+
 // Eq. 1 for one query: merge the S splits' compensated sums in FP64 and divide.
 __device__ __forceinline__ float finalize_query(int64_t q, int64_t m, int S,
                                                 const float *part_sum)
 {
     double W = 0.0, WZ = 0.0;
-    for (int s = 0; s < S; ++s) {
-        const float *o = part_sum + static_cast<int64_t>(s) * 4 * m + q;
-        W += static_cast<double>(__ldcg(o)) + static_cast<double>(__ldcg(o + m));
-        WZ += static_cast<double>(__ldcg(o + 2 * m)) + static_cast<double>(__ldcg(o + 3 * m));
-    }
+    merge_splits(q, m, 0, 1, S, part_sum, W, WZ);
     return static_cast<float>(WZ / W);
 }
 

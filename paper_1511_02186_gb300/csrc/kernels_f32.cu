@@ -14,6 +14,10 @@ namespace {
 
 using namespace f32dev;
 
+// Phase 2 with point groups: the CTA's four warps each take a quarter of every tile's chunks for
+// the same 64 queries (2 per lane, whatever the shape's queries per thread).
+constexpr int kQueriesPG = 2;
+
 template <int KP, int Q, bool IDX>
 __global__ void __launch_bounds__(kThreads)
 f32_knn_kernel(DatasetDev ds, int64_t m, PassPlan pp, const float *__restrict__ qx,
@@ -86,7 +90,7 @@ f32_knn_cull_kernel(DatasetDev ds, int64_t m, int qpb, int ntiles, int ntiles_p2
                               reinterpret_cast<int32_t *>(order + ntiles_p2), cs);
 }
 
-template <int Q, int TW>
+template <int Q, int TW, int PG>
 __global__ void __launch_bounds__(kThreads)
 f32_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const float *__restrict__ qx,
                    const float *__restrict__ qy, const QParamF32 *__restrict__ qp,
@@ -100,17 +104,38 @@ f32_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const float *__restric
     const int s = blockIdx.y;
     const int64_t p_begin = static_cast<int64_t>(s) * pp.split_len;
     const int64_t p_end = min(p_begin + pp.split_len, ds.n_pad);
-    weights_unit<Q, TW>(ds, m, static_cast<int64_t>(blockIdx.x) * pp.q_per_block, p_begin,
-                        p_end, qx, qy, qp, s, part_sum, err, txy, tz, ts);
+    weights_unit<Q, TW, PG>(ds, m, static_cast<int64_t>(blockIdx.x) * pp.q_per_block, p_begin,
+                            p_end, qx, qy, qp, s, part_sum, err, txy, tz, ts);
 }
 
+// R threads per query (a block serves 256 / R queries): each sums every R-th split's partial
+// sums, the block adds the R sums up. One thread per query leaves a call with few queries and
+// many splits waiting on a chain of loads.
+template <int R>
 __global__ void __launch_bounds__(256)
 f32_finalize_kernel(int64_t m, int S, const float *__restrict__ part_sum,
                     float *__restrict__ out, const uint32_t *__restrict__ perm)
 {
-    const int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    constexpr int C = 256 / R;
+    const int col = threadIdx.x % C, r = threadIdx.x / C;
+    const int64_t q = static_cast<int64_t>(blockIdx.x) * C + col;
+    double W = 0.0, WZ = 0.0;
     if (q < m)
-        out[perm ? perm[q] : q] = finalize_query(q, m, S, part_sum);
+        merge_splits(q, m, r, R, S, part_sum, W, WZ);
+    if constexpr (R > 1) {
+        __shared__ double2 sum[R][C];
+        sum[r][col] = make_double2(W, WZ);
+        __syncthreads();
+        if (r > 0)
+            return;
+#pragma unroll
+        for (int i = 1; i < R; ++i) {
+            W += sum[i][col].x;
+            WZ += sum[i][col].y;
+        }
+    }
+    if (q < m)
+        out[perm ? perm[q] : q] = static_cast<float>(WZ / W);
 }
 
 template <int KP, int Q, bool IDX>
@@ -183,9 +208,9 @@ int f32_knn_queries_per_block(int kp)
     return kThreads * (kp <= 16 ? 4 : 2);
 }
 
-int f32_w_queries_per_block(int qw)
+int f32_w_queries_per_block(int qw, int pg)
 {
-    return kThreads * qw;
+    return pg > 1 ? kThreads * kQueriesPG / pg : kThreads * qw;
 }
 
 int f32_knn_slots_per_sm(int kp, bool with_idx)
@@ -198,21 +223,23 @@ int f32_knn_slots_per_sm(int kp, bool with_idx)
     }
 }
 
-template <int Q, int TW>
-int w_slots_t()
+namespace {
+
+using WeightsKernel = void (*)(DatasetDev, int64_t, PassPlan, const float *, const float *,
+                               const QParamF32 *, float *, int *);
+
+WeightsKernel weights_kernel_for(int qw, int tw, int pg)
 {
-    int n = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f32_weights_kernel<Q, TW>, kThreads, 0);
-    return n > 0 ? n : 1;
+    if (pg > 1)
+        return f32_weights_kernel<kQueriesPG, 512, kPointGroups>;
+    if (tw == 256)
+        return qw == 2 ? f32_weights_kernel<2, 256, 1>
+                       : (qw == 8 ? f32_weights_kernel<8, 256, 1> : f32_weights_kernel<4, 256, 1>);
+    return qw == 2 ? f32_weights_kernel<2, 512, 1>
+                   : (qw == 8 ? f32_weights_kernel<8, 512, 1> : f32_weights_kernel<4, 512, 1>);
 }
 
-int f32_w_slots_per_sm(int qw, int tw)
-{
-    if (tw == 256)
-        return qw == 2 ? w_slots_t<2, 256>()
-                       : (qw == 8 ? w_slots_t<8, 256>() : w_slots_t<4, 256>());
-    return qw == 2 ? w_slots_t<2, 512>() : (qw == 8 ? w_slots_t<8, 512>() : w_slots_t<4, 512>());
-}
+}  // namespace
 
 cudaError_t launch_f32_knn(const DatasetDev &ds, const Plan &pl, const float *qx,
                            const float *qy, int k, const Scratch &sc, int *err,
@@ -291,13 +318,7 @@ cudaError_t launch_f32_weights(const DatasetDev &ds, const Plan &pl, const float
                                const float *qy, const Scratch &sc, int *err, cudaStream_t st)
 {
     dim3 grid(pl.w.qblocks, pl.w.splits);
-    auto fn = f32_weights_kernel<4, 512>;
-    if (pl.tw == 256)
-        fn = pl.qw == 2 ? f32_weights_kernel<2, 256>
-                        : (pl.qw == 8 ? f32_weights_kernel<8, 256> : f32_weights_kernel<4, 256>);
-    else
-        fn = pl.qw == 2 ? f32_weights_kernel<2, 512>
-                        : (pl.qw == 8 ? f32_weights_kernel<8, 512> : f32_weights_kernel<4, 512>);
+    const WeightsKernel fn = weights_kernel_for(pl.qw, pl.tw, pl.pg);
     fn<<<grid, kThreads, 0, st>>>(ds, pl.m, pl.w, qx, qy,
                                   static_cast<const QParamF32 *>(sc.qparam),
                                   static_cast<float *>(sc.part_sum), err);
@@ -307,9 +328,12 @@ cudaError_t launch_f32_weights(const DatasetDev &ds, const Plan &pl, const float
 cudaError_t launch_f32_finalize(const Plan &pl, const Scratch &sc, float *out, cudaStream_t st,
                                 const uint32_t *perm)
 {
-    const int64_t blocks = (pl.m + 255) / 256;
-    f32_finalize_kernel<<<static_cast<unsigned>(blocks), 256, 0, st>>>(
-        pl.m, pl.w.splits, static_cast<const float *>(sc.part_sum), out, perm);
+    const int R = finalize_threads(pl.w.splits, pl.m);
+    const unsigned blocks = static_cast<unsigned>((pl.m * R + 255) / 256);
+    auto fn = R == 32 ? f32_finalize_kernel<32>
+                      : (R == 8 ? f32_finalize_kernel<8> : f32_finalize_kernel<1>);
+    fn<<<blocks, 256, 0, st>>>(pl.m, pl.w.splits, static_cast<const float *>(sc.part_sum), out,
+                               perm);
     return cudaGetLastError();
 }
 

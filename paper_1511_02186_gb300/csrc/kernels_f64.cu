@@ -706,7 +706,10 @@ __device__ __forceinline__ void fixed_to_doubles(unsigned __int128 v, double &hi
 }
 
 // One CTA of 512 threads per SM (12 KB of 256-point tiles plus 72 KB of tables).
-template <int Q>
+// With PG point groups the CTA serves Q kThreadsW64 / PG queries: each group sums its own part of
+// every chunk and the groups' sums are merged at the end (a call with few queries fills its CTAs
+// that way). Only the chunks up to the last real point are summed.
+template <int Q, int PG>
 __global__ void __launch_bounds__(kThreadsW64, 1)
 f64_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restrict__ qx,
                    const double *__restrict__ qy, const QParamF64 *__restrict__ qp,
@@ -724,13 +727,17 @@ f64_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restri
     const int64_t qbase = static_cast<int64_t>(blockIdx.x) * pp.q_per_block;
     const int64_t p_begin = static_cast<int64_t>(s) * pp.split_len;
     const int64_t p_end = min(p_begin + pp.split_len, ds.n_pad);
-    const int ntiles = static_cast<int>((p_end - p_begin) / kTileW64);
+    const int64_t p_sum = min(p_end, (ds.n + kChunkW - 1) / kChunkW * kChunkW);
+    const int ntiles =
+        p_sum > p_begin ? static_cast<int>((p_sum - p_begin + kTileW64 - 1) / kTileW64) : 0;
+    constexpr int QT = kThreadsW64 / PG;
+    const int tq = tid % QT, pg = tid / QT;
 
     double qxr[Q], qyr[Q], ns[Q], cc[Q], hz[Q], cz[Q];
     unsigned __int128 aw[Q];
 #pragma unroll
     for (int j = 0; j < Q; ++j) {
-        const int64_t q = min(qbase + j * kThreadsW64 + tid, m - 1);
+        const int64_t q = min(qbase + j * QT + tq, m - 1);
         qxr[j] = qx[q];
         qyr[j] = qy[q];
         const QParamF64 o = qp[q];
@@ -745,15 +752,18 @@ f64_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restri
         fence_mbar_init();
     }
     __syncthreads();
-    constexpr uint32_t kBxy = kTileW64 * sizeof(double2);
-    constexpr uint32_t kBz = kTileW64 * sizeof(double);
+    auto load_tile = [&](int t) {
+        const int b = t & 1;
+        const int64_t o = p_begin + static_cast<int64_t>(t) * kTileW64;
+        const uint32_t len =
+            static_cast<uint32_t>(min(static_cast<int64_t>(kTileW64), p_sum - o));
+        mbar_arrive_expect_tx(&bar[b], len * (sizeof(double2) + sizeof(double)));
+        tma_load_1d(txy[b], ds.xy64 + o, len * sizeof(double2), &bar[b]);
+        tma_load_1d(tz[b], ds.z64 + o, len * sizeof(double), &bar[b]);
+    };
     if (tid == 0) {
-        for (int t = 0; t < 2 && t < ntiles; ++t) {
-            const int64_t o = p_begin + static_cast<int64_t>(t) * kTileW64;
-            mbar_arrive_expect_tx(&bar[t], kBxy + kBz);
-            tma_load_1d(txy[t], ds.xy64 + o, kBxy, &bar[t]);
-            tma_load_1d(tz[t], ds.z64 + o, kBz, &bar[t]);
-        }
+        for (int t = 0; t < 2 && t < ntiles; ++t)
+            load_tile(t);
     }
     bool ok = true;
     for (int t = 0; t < ntiles; ++t) {
@@ -767,25 +777,32 @@ f64_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restri
             }
             break;
         }
-        for (int c = 0; c < kTileW64; c += kChunkW) {
+        const int cend = static_cast<int>(min(
+            static_cast<int64_t>(kTileW64), p_sum - p_begin - static_cast<int64_t>(t) * kTileW64));
+        for (int c = 0; c < cend; c += PG * kChunkW) {
             double sz[Q];
 #pragma unroll
             for (int j = 0; j < Q; ++j)
                 sz[j] = 0.0;
-            // One point at a time (the Q queries' chains interleave): 109.1 ms on 8,192 x 1M
-            // against 124.5 ms unrolled by 4 and 109.6 ms by 2.
+            for (int i = 0; i < PG; ++i) {
+                const int cg = c + i * kChunkW + pg * (kChunkW / PG);
+                if (PG > 1 && cg >= cend)
+                    break;
+                // One point at a time (the Q queries' chains interleave): 109.1 ms on 8,192 x
+                // 1M against 124.5 ms unrolled by 4 and 109.6 ms by 2.
 #pragma unroll 1
-            for (int u = 0; u < kChunkW; ++u) {
-                const double2 p = txy[b][c + u];
-                const double pz = tz[b][c + u];
+                for (int u = 0; u < kChunkW / PG; ++u) {
+                    const double2 p = txy[b][cg + u];
+                    const double pz = tz[b][cg + u];
 #pragma unroll
-                for (int j = 0; j < Q; ++j) {
-                    const double d2 = dist2_eps(qxr[j], qyr[j], p.x, p.y);
-                    unsigned __int128 w96;
-                    const double w = f64math::exp2_t<true>(
-                        __fma_rn(f64math::log2_t(d2, tabs), ns[j], cc[j]), tabs, &w96);
-                    aw[j] += w96;
-                    sz[j] = __fma_rn(w, pz, sz[j]);
+                    for (int j = 0; j < Q; ++j) {
+                        const double d2 = dist2_eps(qxr[j], qyr[j], p.x, p.y);
+                        unsigned __int128 w96;
+                        const double w = f64math::exp2_t<true>(
+                            __fma_rn(f64math::log2_t(d2, tabs), ns[j], cc[j]), tabs, &w96);
+                        aw[j] += w96;
+                        sz[j] = __fma_rn(w, pz, sz[j]);
+                    }
                 }
             }
 #pragma unroll
@@ -795,17 +812,42 @@ f64_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restri
         __syncthreads();
         if (tid == 0 && t + 2 < ntiles) {
             fence_proxy_async_smem();
-            const int64_t o = p_begin + static_cast<int64_t>(t + 2) * kTileW64;
-            mbar_arrive_expect_tx(&bar[b], kBxy + kBz);
-            tma_load_1d(txy[b], ds.xy64 + o, kBxy, &bar[b]);
-            tma_load_1d(tz[b], ds.z64 + o, kBz, &bar[b]);
+            load_tile(t + 2);
         }
     }
     if (!ok)
         return;
+    if constexpr (PG > 1) {
+        // The groups' sums, in group order, onto group 0's, through the tables' memory (no
+        // thread reads a table after the last tile's closing barrier).
+        __syncthreads();
+        unsigned __int128 *gw = reinterpret_cast<unsigned __int128 *>(f64_dyn);
+        double2 *gz = reinterpret_cast<double2 *>(gw + Q * kThreadsW64);
+        static_assert((sizeof(unsigned __int128) + sizeof(double2)) * Q * kThreadsW64 <=
+                          f64math::kTablesBytes, "fits the tables' memory");
+        if (pg > 0) {
+#pragma unroll
+            for (int j = 0; j < Q; ++j) {
+                gw[j * kThreadsW64 + tid] = aw[j];
+                gz[j * kThreadsW64 + tid] = make_double2(hz[j], cz[j]);
+            }
+        }
+        __syncthreads();
+        if (pg > 0)
+            return;
+        for (int i = 1; i < PG; ++i) {
+#pragma unroll
+            for (int j = 0; j < Q; ++j) {
+                aw[j] += gw[j * kThreadsW64 + i * QT + tq];
+                const double2 v = gz[j * kThreadsW64 + i * QT + tq];
+                kahan_add(hz[j], cz[j], v.x);
+                kahan_add(hz[j], cz[j], -v.y);
+            }
+        }
+    }
 #pragma unroll
     for (int j = 0; j < Q; ++j) {
-        const int64_t q = qbase + j * kThreadsW64 + tid;
+        const int64_t q = qbase + j * QT + tq;
         if (q >= m)
             continue;
         double *o = part_sum + static_cast<int64_t>(s) * 4 * m + q;
@@ -815,22 +857,43 @@ f64_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restri
     }
 }
 
+// R threads per query, as f32_finalize_kernel's.
+template <int R>
 __global__ void __launch_bounds__(256)
 f64_finalize_kernel(int64_t m, int S, const double *__restrict__ part_sum,
                     double *__restrict__ out, const uint32_t *__restrict__ perm)
 {
-    const int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (q >= m)
-        return;
+    constexpr int C = 256 / R;
+    const int col = threadIdx.x % C, r = threadIdx.x / C;
+    const int64_t q = static_cast<int64_t>(blockIdx.x) * C + col;
     double W = 0.0, Wc = 0.0, WZ = 0.0, WZc = 0.0;
-    for (int s = 0; s < S; ++s) {
-        const double *o = part_sum + static_cast<int64_t>(s) * 4 * m + q;
-        kahan_add(W, Wc, o[0]);
-        kahan_add(W, Wc, o[m]);
-        kahan_add(WZ, WZc, o[2 * m]);
-        kahan_add(WZ, WZc, o[3 * m]);
+    if (q < m) {
+#pragma unroll 4
+        for (int s = r; s < S; s += R) {
+            const double *o = part_sum + static_cast<int64_t>(s) * 4 * m + q;
+            kahan_add(W, Wc, o[0]);
+            kahan_add(WZ, WZc, o[2 * m]);
+            Wc -= o[m];  // the parts below an ulp of the sums join the compensation
+            WZc -= o[3 * m];
+        }
     }
-    out[perm ? perm[q] : q] = (WZ - WZc) / (W - Wc);  // Eq. 1
+    if constexpr (R > 1) {
+        __shared__ double2 w[R][C], z[R][C];
+        w[r][col] = make_double2(W, Wc);
+        z[r][col] = make_double2(WZ, WZc);
+        __syncthreads();
+        if (r > 0)
+            return;
+#pragma unroll
+        for (int i = 1; i < R; ++i) {
+            kahan_add(W, Wc, w[i][col].x);
+            kahan_add(WZ, WZc, z[i][col].x);
+            Wc += w[i][col].y;
+            WZc += z[i][col].y;
+        }
+    }
+    if (q < m)
+        out[perm ? perm[q] : q] = (WZ - WZc) / (W - Wc);  // Eq. 1
 }
 
 template <int KP>
@@ -883,9 +946,9 @@ int f64_knn_queries_per_block(int k)
     return kThreads * (k <= 16 ? 2 : 1);
 }
 
-int f64_w_queries_per_block()
+int f64_w_queries_per_block(int pg)
 {
-    return kThreadsW64 * kQW64;
+    return kThreadsW64 * kQW64 / pg;
 }
 
 int f64_knn_slots_per_sm(int k, bool with_idx)
@@ -897,25 +960,20 @@ int f64_knn_slots_per_sm(int k, bool with_idx)
     return knn_slots_t<32>(with_idx);
 }
 
-// The FP64 phase-2 kernel takes its log2 / exp2 tables in dynamic shared memory.
-cudaError_t prepare_f64_weights()
+namespace {
+
+using WeightsKernel64 = void (*)(DatasetDev, int64_t, PassPlan, const double *, const double *,
+                                 const QParamF64 *, double *, int *);
+
+// The FP64 phase-2 kernel, which takes its log2 / exp2 tables in dynamic shared memory.
+cudaError_t weights64_kernel_for(int pg, WeightsKernel64 *fn)
 {
-    return cudaFuncSetAttribute(f64_weights_kernel<kQW64>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize,
+    *fn = pg > 1 ? f64_weights_kernel<kQW64, kPointGroups> : f64_weights_kernel<kQW64, 1>;
+    return cudaFuncSetAttribute(*fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 static_cast<int>(f64math::kTablesBytes));
 }
 
-int f64_w_slots_per_sm()
-{
-    int n = 0;
-    if (prepare_f64_weights() != cudaSuccess) {
-        cudaGetLastError();
-        return 1;
-    }
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f64_weights_kernel<kQW64>, kThreadsW64,
-                                                  f64math::kTablesBytes);
-    return n > 0 ? n : 1;
-}
+}  // namespace
 
 cudaError_t launch_f64_knn(const DatasetDev &ds, const Plan &pl, const double *qx,
                            const double *qy, int k, const Scratch &sc, int *err,
@@ -998,10 +1056,11 @@ cudaError_t launch_f64_weights(const DatasetDev &ds, const Plan &pl, const doubl
                                const double *qy, const Scratch &sc, int *err, cudaStream_t st)
 {
     dim3 grid(pl.w.qblocks, pl.w.splits);
-    const cudaError_t e = prepare_f64_weights();
+    WeightsKernel64 fn;
+    const cudaError_t e = weights64_kernel_for(pl.pg, &fn);
     if (e != cudaSuccess)
         return e;
-    f64_weights_kernel<kQW64><<<grid, kThreadsW64, f64math::kTablesBytes, st>>>(
+    fn<<<grid, kThreadsW64, f64math::kTablesBytes, st>>>(
         ds, pl.m, pl.w, qx, qy, static_cast<const QParamF64 *>(sc.qparam),
         static_cast<double *>(sc.part_sum), err);
     return cudaGetLastError();
@@ -1010,9 +1069,12 @@ cudaError_t launch_f64_weights(const DatasetDev &ds, const Plan &pl, const doubl
 cudaError_t launch_f64_finalize(const Plan &pl, const Scratch &sc, double *out,
                                 cudaStream_t st, const uint32_t *perm)
 {
-    const int64_t blocks = (pl.m + 255) / 256;
-    f64_finalize_kernel<<<static_cast<unsigned>(blocks), 256, 0, st>>>(
-        pl.m, pl.w.splits, static_cast<const double *>(sc.part_sum), out, perm);
+    const int R = finalize_threads(pl.w.splits, pl.m);
+    const unsigned blocks = static_cast<unsigned>((pl.m * R + 255) / 256);
+    auto fn = R == 32 ? f64_finalize_kernel<32>
+                      : (R == 8 ? f64_finalize_kernel<8> : f64_finalize_kernel<1>);
+    fn<<<blocks, 256, 0, st>>>(pl.m, pl.w.splits, static_cast<const double *>(sc.part_sum), out,
+                               perm);
     return cudaGetLastError();
 }
 

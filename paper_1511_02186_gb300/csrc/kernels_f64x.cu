@@ -32,7 +32,7 @@ __device__ __forceinline__ void drain_x(uint64_t *bar, int t, int ntiles)
 // One block of kThreads * Q queries against one data split; per query the two double-float
 // sums (w, w z) go to part_sum as four doubles (sum of w hi, lo, sum of w z hi, lo), which the
 // FP64 finalisation adds up.
-template <int Q>
+template <int Q, int PG>
 __global__ void __launch_bounds__(kThreads)
 f64x_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restrict__ qx,
                     const double *__restrict__ qy, const QParamF64X *__restrict__ qp,
@@ -50,7 +50,12 @@ f64x_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restr
     const int64_t qbase = static_cast<int64_t>(blockIdx.x) * pp.q_per_block;
     const int64_t p_begin = static_cast<int64_t>(s) * pp.split_len;
     const int64_t p_end = min(p_begin + pp.split_len, ds.n_pad);
-    const int ntiles = static_cast<int>((p_end - p_begin) / kTileF64W);
+    // Chunks of padding only are not summed (their weights are exactly 0).
+    const int64_t p_sum = min(p_end, (ds.n + kSplitGranule - 1) / kSplitGranule * kSplitGranule);
+    const int ntiles =
+        p_sum > p_begin ? static_cast<int>((p_sum - p_begin + kTileF64W - 1) / kTileF64W) : 0;
+    constexpr int QT = kThreads / PG;
+    const int tq = PG == 1 ? tid : tid % QT, pg = PG == 1 ? 0 : tid / QT;
 
     if (tid == 0) {
         mbar_init(&bar[0], 1);
@@ -58,15 +63,18 @@ f64x_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restr
         fence_mbar_init();
     }
     __syncthreads();
-    constexpr uint32_t kBxy = kTileF64W * sizeof(double2);
-    constexpr uint32_t kBz = kTileF64W * sizeof(double);
+    auto load_tile = [&](int t) {
+        const int b = t & 1;
+        const int64_t o = p_begin + static_cast<int64_t>(t) * kTileF64W;
+        const uint32_t len =
+            static_cast<uint32_t>(min(static_cast<int64_t>(kTileF64W), p_sum - o));
+        mbar_arrive_expect_tx(&bar[b], len * (sizeof(double2) + sizeof(double)));
+        tma_load_1d(txy[b], ds.xy64 + o, len * sizeof(double2), &bar[b]);
+        tma_load_1d(tz[b], ds.z64 + o, len * sizeof(double), &bar[b]);
+    };
     if (tid == 0) {
-        for (int t = 0; t < 2 && t < ntiles; ++t) {
-            const int64_t o = p_begin + static_cast<int64_t>(t) * kTileF64W;
-            mbar_arrive_expect_tx(&bar[t], kBxy + kBz);
-            tma_load_1d(txy[t], ds.xy64 + o, kBxy, &bar[t]);
-            tma_load_1d(tz[t], ds.z64 + o, kBz, &bar[t]);
-        }
+        for (int t = 0; t < 2 && t < ntiles; ++t)
+            load_tile(t);
     }
 
     double qxr[Q], qyr[Q];
@@ -74,7 +82,7 @@ f64x_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restr
     dfm::RefLog ref[Q];
 #pragma unroll
     for (int j = 0; j < Q; ++j) {
-        const int64_t q = min(qbase + j * kThreads + tid, m - 1);
+        const int64_t q = min(qbase + j * QT + tq, m - 1);
         qxr[j] = qx[q];
         qyr[j] = qy[q];
         const QParamF64X o = qp[q];
@@ -96,33 +104,40 @@ f64x_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restr
             }
             break;
         }
-        for (int i = tid; i < kTileF64W; i += kThreads) {
+        const int cend = static_cast<int>(min(
+            static_cast<int64_t>(kTileF64W), p_sum - p_begin - static_cast<int64_t>(t) * kTileF64W));
+        for (int i = tid; i < cend; i += kThreads) {
             const double z = tz[b][i];
             const float h = __double2float_rn(z);
             tzf[i] = make_float2(h, __double2float_rn(z - static_cast<double>(h)));
         }
         __syncthreads();
-        for (int c = 0; c < kTileF64W; c += kChunkX) {
+        for (int c = 0; c < cend; c += PG * kChunkX) {
             float aw[Q], cw[Q], az[Q], cz[Q];
 #pragma unroll
             for (int j = 0; j < Q; ++j)
                 aw[j] = cw[j] = az[j] = cz[j] = 0.0f;
+            for (int i = 0; i < PG; ++i) {
+                const int cg = c + i * kChunkX + pg * (kChunkX / PG);
+                if (PG > 1 && cg >= cend)
+                    break;
 #pragma unroll 2
-            for (int u = 0; u < kChunkX; ++u) {
-                const double2 p = txy[b][c + u];
-                const float2 pz = tzf[c + u];
+                for (int u = 0; u < kChunkX / PG; ++u) {
+                    const double2 p = txy[b][cg + u];
+                    const float2 pz = tzf[cg + u];
 #pragma unroll
-                for (int j = 0; j < Q; ++j) {
-                    const double d2 = dist2_eps_x(qxr[j], qyr[j], p.x, p.y);
-                    float vh, vl, yh, yl, wh, wl, e, zh, zl;
-                    dfm::log2_ratio(d2, ref[j], tabs, vh, vl);
-                    dfm::mul(kh[j], kl[j], vh, vl, yh, yl);  // -y = kappa log2(d^2 / d1^2)
-                    dfm::exp2_df(-yh, -yl, tabs, wh, wl);
-                    dfm::two_sum(aw[j], wh, aw[j], e);
-                    cw[j] = __fadd_rn(cw[j], __fadd_rn(e, wl));
-                    dfm::mul(wh, wl, pz.x, pz.y, zh, zl);
-                    dfm::two_sum(az[j], zh, az[j], e);
-                    cz[j] = __fadd_rn(cz[j], __fadd_rn(e, zl));
+                    for (int j = 0; j < Q; ++j) {
+                        const double d2 = dist2_eps_x(qxr[j], qyr[j], p.x, p.y);
+                        float vh, vl, yh, yl, wh, wl, e, zh, zl;
+                        dfm::log2_ratio(d2, ref[j], tabs, vh, vl);
+                        dfm::mul(kh[j], kl[j], vh, vl, yh, yl);  // -y = kappa log2(d^2 / d1^2)
+                        dfm::exp2_df(-yh, -yl, tabs, wh, wl);
+                        dfm::two_sum(aw[j], wh, aw[j], e);
+                        cw[j] = __fadd_rn(cw[j], __fadd_rn(e, wl));
+                        dfm::mul(wh, wl, pz.x, pz.y, zh, zl);
+                        dfm::two_sum(az[j], zh, az[j], e);
+                        cz[j] = __fadd_rn(cz[j], __fadd_rn(e, zl));
+                    }
                 }
             }
 #pragma unroll
@@ -134,17 +149,36 @@ f64x_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restr
         __syncthreads();
         if (tid == 0 && t + 2 < ntiles) {
             fence_proxy_async_smem();
-            const int64_t o = p_begin + static_cast<int64_t>(t + 2) * kTileF64W;
-            mbar_arrive_expect_tx(&bar[b], kBxy + kBz);
-            tma_load_1d(txy[b], ds.xy64 + o, kBxy, &bar[b]);
-            tma_load_1d(tz[b], ds.z64 + o, kBz, &bar[b]);
+            load_tile(t + 2);
         }
     }
     if (!ok)
         return;
+    if constexpr (PG > 1) {
+        // The point groups' sums, in group order, onto group 0's (through the tile memory, free
+        // after the last tile's closing barrier).
+        float4 *g = reinterpret_cast<float4 *>(&txy[0][0]);
+        static_assert(sizeof(float4) * Q * kThreads <= sizeof(double2) * kTileF64W, "fits");
+        if (pg > 0) {
+#pragma unroll
+            for (int j = 0; j < Q; ++j)
+                g[j * kThreads + tid] = make_float4(Wh[j], Wl[j], Zh[j], Zl[j]);
+        }
+        __syncthreads();
+        if (pg > 0)
+            return;
+        for (int i = 1; i < PG; ++i) {
+#pragma unroll
+            for (int j = 0; j < Q; ++j) {
+                const float4 v = g[j * kThreads + i * QT + tq];
+                dfm::add(Wh[j], Wl[j], v.x, v.y);
+                dfm::add(Zh[j], Zl[j], v.z, v.w);
+            }
+        }
+    }
 #pragma unroll
     for (int j = 0; j < Q; ++j) {
-        const int64_t q = qbase + j * kThreads + tid;
+        const int64_t q = qbase + j * QT + tq;
         if (q >= m)
             continue;
         double *o = part_sum + static_cast<int64_t>(s) * 4 * m + q;
@@ -179,23 +213,28 @@ __global__ void df_weight_probe_kernel(const double *__restrict__ d2,
 
 }  // namespace
 
-int f64x_w_queries_per_block()
+namespace {
+
+using WeightsKernelX = void (*)(DatasetDev, int64_t, PassPlan, const double *, const double *,
+                                const QParamF64X *, double *, int *);
+
+WeightsKernelX weightsx_kernel_for(int pg)
 {
-    return kThreads * kQX;
+    return pg > 1 ? f64x_weights_kernel<kQX, kPointGroups> : f64x_weights_kernel<kQX, 1>;
 }
 
-int f64x_w_slots_per_sm()
+}  // namespace
+
+int f64x_w_queries_per_block(int pg)
 {
-    int n = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f64x_weights_kernel<kQX>, kThreads, 0);
-    return n > 0 ? n : 1;
+    return kThreads * kQX / pg;
 }
 
 cudaError_t launch_f64x_weights(const DatasetDev &ds, const Plan &pl, const double *qx,
                                 const double *qy, const Scratch &sc, int *err, cudaStream_t st)
 {
     dim3 grid(pl.w.qblocks, pl.w.splits);
-    f64x_weights_kernel<kQX><<<grid, kThreads, 0, st>>>(
+    weightsx_kernel_for(pl.pg)<<<grid, kThreads, 0, st>>>(
         ds, pl.m, pl.w, qx, qy, static_cast<const QParamF64X *>(sc.qparam),
         static_cast<double *>(sc.part_sum), err);
     return cudaGetLastError();

@@ -90,7 +90,7 @@ extern "C" int aidw_interpolate_noalloc(aidw_ctx *ctx, aidw_dataset ds, const fl
     if (!base)
         return AIDW_ERR_CUDA;
     const cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const Plan planned = make_plan(ctx, AIDW_F32C, dev.n_pad, m, p->k, false, 0, 0);
+    const Plan planned = make_plan(ctx, AIDW_F32C, dev.n, dev.n_pad, m, p->k, false, 0, 0);
 
     // Per-query phase 1 where aidw_interpolate would take it (one list per query, no ordering).
     if (use_warp_knn(AIDW_F32C, dev, m, 0)) {
@@ -98,7 +98,7 @@ extern "C" int aidw_interpolate_noalloc(aidw_ctx *ctx, aidw_dataset ds, const fl
         pl.knn.splits = 1;
         pl.knn.split_len = dev.n_pad;
         while (scratch_bytes(AIDW_F32C, pl, p->k) > kNoAllocScratchBytes && pl.w.splits > 1) {
-            pl = make_plan(ctx, AIDW_F32C, dev.n_pad, m, p->k, false, 0, pl.w.splits - 1);
+            pl = make_plan(ctx, AIDW_F32C, dev.n, dev.n_pad, m, p->k, false, 0, pl.w.splits - 1);
             pl.knn.splits = 1;
             pl.knn.split_len = dev.n_pad;
         }
@@ -118,7 +118,7 @@ extern "C" int aidw_interpolate_noalloc(aidw_ctx *ctx, aidw_dataset ds, const fl
         const size_t extra = culled_extra_bytes(m, AIDW_F32C);
         while (scratch_bytes(AIDW_F32C, pl, p->k) + extra > kNoAllocScratchBytes &&
                pl.w.splits > 1) {
-            pl = make_plan(ctx, AIDW_F32C, dev.n_pad, m, p->k, false, 0, pl.w.splits - 1);
+            pl = make_plan(ctx, AIDW_F32C, dev.n, dev.n_pad, m, p->k, false, 0, pl.w.splits - 1);
             plan_culled_knn(&pl, dev.n_pad);
         }
         const size_t sb = scratch_bytes(AIDW_F32C, pl, p->k);
@@ -139,7 +139,7 @@ extern "C" int aidw_interpolate_noalloc(aidw_ctx *ctx, aidw_dataset ds, const fl
            (pl.knn.splits > 1 || pl.w.splits > 1)) {
         const int s1 = pl.knn.splits > 1 ? pl.knn.splits - 1 : 1;
         const int s2 = pl.w.splits > 1 ? pl.w.splits - 1 : 1;
-        pl = make_plan(ctx, AIDW_F32C, dev.n_pad, m, p->k, false, s1, s2);
+        pl = make_plan(ctx, AIDW_F32C, dev.n, dev.n_pad, m, p->k, false, s1, s2);
     }
     if (scratch_bytes(AIDW_F32C, pl, p->k) > kNoAllocScratchBytes)
         return AIDW_ERR_INVALID_ARG;  // m * (4k + 24) bytes exceed the 16 MiB area
