@@ -563,30 +563,29 @@ bool use_culled_knn(int precision, const DatasetDev &ds, int64_t m, bool with_id
            static_cast<double>(m) >= need;
 }
 
-// Whether a call takes the per-query phase 1 (one warp per query). In FP32 its cost grows with
-// the query count alone (about 25 ns of the GPU per query against 1M points, 13 ns against
-// 65,536), while the block scans share their tiles among a block's queries and gain as the
-// queries get denser. Measured phase 1 (ms, against 1M uniform points / 65,536 clustered
-// points; block scans = the split scan below 12,600 queries, the pruned scan above):
-//   queries        1,024   4,096   8,192   32,768   131,072
-//   block scans    2.63    3.41    4.46    1.93     1.09     /  0.61  0.64  0.73  0.54  0.46
-//   warp per query 0.24    0.25    0.34    0.99     3.24     /  0.13  0.14  0.19  0.49  1.67
-// so FP32 calls of up to kWarpKnnMaxQueries take it. In FP64 and FP64X (exact FP64 distances
-// per lane, read through the Z-order map) the block scans cost far more, measured phase 1 (ms):
-//   queries        512    2,048  8,192  16,384  32,768  65,536  131,072  262,144
-//   1M uniform:  split scan 10.9 17.5 32.4 45.2 60.8 114 198; pruned scan 141 92.0 58.0 39.3
-//                24.3 15.4 13.1; warp per query 0.19 0.26 0.66 1.20 2.26 4.49 8.73
-//   65,536 clustered: split 3.74 5.45 10.4 13.9 20.1 39.4 77.4 145; pruned 24.9 17.5 9.24
-//                6.78 5.30 5.22 6.20 8.07; warp 0.11 0.14 0.35 0.62 1.20 2.32 4.58 9.06
-// so FP64 calls of up to kWarpKnnMaxQueriesF64 take it.
+// Whether a call takes the per-query phase 1 (one warp per query). Its cost grows with the query
+// count alone, while the block scans share their tiles among a block's queries and gain as the
+// queries get denser. Measured phase 1 in FP32 (us; pruned scan with the query ordering / warp
+// per query):
+//   queries              16,384       65,536      131,072     262,144      1,048,576
+//   1M uniform        3,276 / 102  1,976 / 303  1,544 / 580  1,415 / 1,124  1,902 / 4,345
+//   262,147 clustered 1,784 / 88   1,259 / 290  1,250 / 554  1,088 / 1,051  1,175 / 3,986
+//   65,536 clustered    660 / 68     498 / 212    474 / 409    558 / 777      609 / 3,011
+//   16,384 uniform      290 / 60     288 / 196    270 / 368    305 / 708      519 / 2,721
+// so the crossing lies near 3,500 n^(1/3) queries, and a call of many more queries than points
+// orders them. The FP64 pruned scan is slower than the warp scan at every count measured
+// (65,536 clustered, 262,144 queries: 8,184 / 1,375; 1M uniform, 16,384: 43,274 / 170).
 constexpr int64_t kWarpKnnMaxQueries = 32768;
-constexpr int64_t kWarpKnnMaxQueriesF64 = 131072;
+constexpr double kWarpKnnPerCbrt = 3500.0;
+constexpr double kWarpKnnPerPoint = 1.9;
 
-bool use_warp_knn(int precision, const DatasetDev &ds, int64_t m, int sm_count)
+bool use_warp_knn(int precision, const DatasetDev &ds, int64_t m)
 {
-    (void)ds;
-    (void)sm_count;
-    return m <= (precision == AIDW_F32C ? kWarpKnnMaxQueries : kWarpKnnMaxQueriesF64);
+    if (precision != AIDW_F32C)
+        return true;
+    const double n = static_cast<double>(ds.n_pad);
+    const double most = std::min(kWarpKnnPerPoint * n, kWarpKnnPerCbrt * std::cbrt(n));
+    return m <= kWarpKnnMaxQueries || static_cast<double>(m) <= most;
 }
 
 void plan_culled_knn(Plan *pl, int64_t n_pad)
@@ -788,7 +787,7 @@ int interpolate_impl(aidw_ctx *ctx, aidw_dataset dsid, const void *qx, const voi
     const bool force_cull =
         force_knn_splits == -2 && ds.n_pad / kTileF32Knn <= kMaxCullTiles;
     const bool warp = force_knn_splits == -1 ||
-                      (force_knn_splits == 0 && use_warp_knn(p->precision, ds, m, ctx->sm_count));
+                      (force_knn_splits == 0 && use_warp_knn(p->precision, ds, m));
     // Staging for host arrays.
     const size_t b_q = (kq == 0 ? align256(m * es) : 0) + (kqy == 0 ? align256(m * es) : 0);
     const size_t b_o = ko == 0 ? align256(m * es) : 0;

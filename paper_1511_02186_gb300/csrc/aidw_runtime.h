@@ -78,7 +78,7 @@ int enqueue_culled(aidw_ctx *ctx, const DatasetDev &ds, double r_exp, const Plan
 // The per-query phase 1 (one warp per query, caller order): whether a call of `precision`
 // takes it, and the enqueue (phase 1, selection, phase 2, finalisation; the plan keeps one list
 // split). Query and output arrays are float for AIDW_F32C, double otherwise.
-bool use_warp_knn(int precision, const DatasetDev &ds, int64_t m, int sm_count);
+bool use_warp_knn(int precision, const DatasetDev &ds, int64_t m);
 int enqueue_warp(aidw_ctx *ctx, const DatasetDev &ds, double r_exp, const Plan &pl,
                  const aidw_params &p, const void *qx, const void *qy, const Scratch &sc,
                  void *out, float *out_alpha, int32_t *out_knn, cudaStream_t st, bool profile);

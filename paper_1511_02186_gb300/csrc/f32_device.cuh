@@ -20,7 +20,6 @@ namespace f32dev {
 constexpr int kChunkKnn = 8;  // points between neighbour-list threshold checks
 constexpr int kChunkW = 32;   // points summed in plain FP32 before a Kahan merge
 constexpr float kFilterMargin = 1.0f + 9.5367431640625e-07f;  // 1 + 2^-20
-constexpr float kBoundShrink = 1.0f - 9.5367431640625e-07f;   // 1 - 2^-20, box bounds
 
 // Squared distance from negated data coordinates: q + (-p) is exactly q - p.
 __device__ __forceinline__ float dist2_neg(float qx, float qy, float npx, float npy)
@@ -352,138 +351,139 @@ static __device__ __noinline__ void fused_select_query(const float *d, int k,
 // queries together (knn_cull_unit); when the queries lie far apart compared with the data points
 // (few queries, or many fewer queries than points) the block shares little, its warps scan the
 // union of what each query needs, and a call with few queries leaves most SMs idle. Here a warp
-// serves one query at a time: its 32 lanes hold the 32 smallest squared distances seen so far
-// as a list sorted across the lanes (lane j the j-th smallest, with the point's stored
-// position), scan 32 points per step with one point per lane, and take the points closer than
-// the k-th entry: a few by shifting the larger entries up one lane each, more by a bitonic sort
-// of the step's candidates and a bitonic merge with the list.
-// The points are visited through the dataset's box hierarchy (warp_visit_boxes: 32-tile
-// super-tiles, 512-point tiles, 64-point sub-tiles), nearest box first at every level, skipping
-// every box whose bound exceeds the current k-th distance. The bounds are shrunk by 2^-20 for
-// rounding as in knn_cull_unit, so no skipped point could enter the list: the k smallest values
-// are those of a full scan. k <= 32.
+// serves one query at a time: warp_walk visits the sub-tiles that may hold a neighbour, 64 points
+// at a time, two per lane, and WarpNearest keeps the points within the current bound thr on the
+// k-th distance. The box bounds are shrunk by 2^-20 for rounding as in knn_cull_unit, so no
+// skipped point could enter the list: the k smallest values are those of a full scan. k <= 32.
 // ---------------------------------------------------------------------------------------------
-// Up to this many candidates in a step are inserted one at a time; more are sorted and merged.
-constexpr int kWarpInsertMax = 6;
 
-// Squared-distance lower bound from (qx, qy) to a box (xmin, ymin, xmax, ymax), shrunk for
-// rounding; +inf for an empty box.
-__device__ __forceinline__ float box_bound(float qx, float qy, float4 b)
-{
-    const float dx = fmaxf(0.0f, fmaxf(b.x - qx, qx - b.z));
-    const float dy = fmaxf(0.0f, fmaxf(b.y - qy, qy - b.w));
-    return __fmul_rn(__fmaf_rn(dx, dx, __fmul_rn(dy, dy)), kBoundShrink);
-}
+struct WarpEntry {
+    float d;
+    int32_t i;
+};
 
-// Compare-exchange of a bitonic network across lanes: in an ascending run (up) the lower lane
-// of each pair keeps the smaller entry. Equal entries stay where they are.
-__device__ __forceinline__ void warp_cx(float &v, int32_t &i, int stride, bool up)
-{
-    const float ov = __shfl_xor_sync(kFullMask, v, stride);
-    const int32_t oi = __shfl_xor_sync(kFullMask, i, stride);
-    const bool lower = (threadIdx.x & stride) == 0;
-    const bool take = (lower == up) ? (ov < v) : (ov > v);
-    if (take) {
-        v = ov;
-        i = oi;
-    }
-}
-
-// Points [p, p + 32) of the Z-ordered copy, one per lane, against the warp's list (ld, li) and
-// its k-th entry thr (warp-uniform, updated).
-__device__ __forceinline__ void warp_scan32(const float4 *__restrict__ nxy2, int64_t p, float qx,
-                                            float qy, int k, float &ld, int32_t &li, float &thr)
+// Cuts a warp's buffer of cnt <= kWarpBuffer candidates to the k smallest, sorted in the buffer's
+// first entries; lane j returns the j-th smallest of them ((+inf, -1) beyond the last). Each lane
+// counts the entries smaller than its one or two (read four at a time as broadcasts), which is
+// where they go: about 5 instructions per entry and no chain across the lanes (a bitonic sort
+// took 2,080 clocks, and a query with a poor first bound cuts 20 times). Out of line: inlined
+// where a scan cuts, a launch with few queries waits for its instructions.
+template <bool IDX>
+__device__ __noinline__ WarpEntry warp_cut(float *bd, int32_t *bi, int cnt, int k)
 {
     const int lane = threadIdx.x & 31;
-    const float4 pt = nxy2[p + lane];
-    const float d = dist2_neg(qx, qy, pt.x, pt.z);
-    unsigned cand = __ballot_sync(kFullMask, d < thr);
-    if (!cand)
-        return;
-    if (__popc(cand) <= kWarpInsertMax) {
-        // Few candidates: each is inserted in turn by shifting the larger entries up one lane.
-        while (cand) {
-            const int src = __ffs(cand) - 1;
-            cand &= cand - 1;
-            const float c = __shfl_sync(kFullMask, d, src);
-            if (!(c < thr))
-                continue;
-            const int32_t ci = static_cast<int32_t>(p + src);
-            const float up = __shfl_up_sync(kFullMask, ld, 1);
-            const int32_t upi = __shfl_up_sync(kFullMask, li, 1);
-            if (!(ld <= c)) {
-                const bool here = lane == 0 || up <= c;
-                ld = here ? c : up;
-                li = here ? ci : upi;
-            }
-            thr = __shfl_sync(kFullMask, ld, k - 1);
+    if (lane < 4 && cnt + lane < kWarpBuffer)
+        bd[cnt + lane] = CUDART_INF_F;
+    __syncwarp();
+    const bool has0 = lane < cnt, has1 = lane + 32 < cnt;
+    const float v0 = bd[lane], v1 = bd[lane + 32];
+    const int32_t i0 = IDX ? bi[lane] : 0, i1 = IDX ? bi[lane + 32] : 0;
+    int r0 = 0, r1 = 0, q0 = 0, q1 = 0;  // entries below, entries equal (itself included)
+    const auto below = [](const float4 d, float v) {
+        return (d.x < v) + (d.y < v) + (d.z < v) + (d.w < v);
+    };
+    const auto equal = [](const float4 d, float v) {
+        return (d.x == v) + (d.y == v) + (d.z == v) + (d.w == v);
+    };
+    const float4 *b4 = reinterpret_cast<const float4 *>(bd);
+#pragma unroll 2
+    for (int j = 0; 4 * j < cnt; ++j) {
+        const float4 d = b4[j];
+        r0 += below(d, v0);
+        q0 += equal(d, v0);
+        if (cnt > 32) {
+            r1 += below(d, v1);
+            q1 += equal(d, v1);
         }
-        return;
     }
-    const bool is_cand = (cand >> lane) & 1u;
-    float v = is_cand ? d : CUDART_INF_F;
-    int32_t vi = is_cand ? static_cast<int32_t>(p + lane) : -1;
-#pragma unroll
-    for (int size = 2; size <= 32; size <<= 1) {
-#pragma unroll
-        for (int stride = size >> 1; stride > 0; stride >>= 1)
-            warp_cx(v, vi, stride, (lane & size) == 0);
+    if (__any_sync(kFullMask, (has0 && q0 > 1) || (has1 && q1 > 1))) {
+        // Equal distances keep their order of arrival.
+        for (int j = 0; j < cnt; ++j) {
+            r0 += bd[j] == v0 && j < lane;
+            r1 += bd[j] == v1 && j < lane + 32;
+        }
     }
-    // The 32 smallest of the two sorted lists, as a bitonic sequence, then sorted.
-    const float rv = __shfl_sync(kFullMask, v, 31 - lane);
-    const int32_t ri = __shfl_sync(kFullMask, vi, 31 - lane);
-    if (rv < ld) {
-        ld = rv;
-        li = ri;
+    __syncwarp();
+    if (has0 && r0 < k) {
+        bd[r0] = v0;
+        if (IDX)
+            bi[r0] = i0;
     }
-#pragma unroll
-    for (int stride = 16; stride > 0; stride >>= 1)
-        warp_cx(ld, li, stride, true);
-    thr = __shfl_sync(kFullMask, ld, k - 1);
+    if (has1 && r1 < k) {
+        bd[r1] = v1;
+        if (IDX)
+            bi[r1] = i1;
+    }
+    __syncwarp();
+    const bool has = lane < min(cnt, k);
+    return {has ? bd[lane] : CUDART_INF_F, IDX && has ? bi[lane] : -1};
 }
 
-// Visit key of a box for an FP32 query (make_visit_key); ~0 for an empty box.
-__device__ __forceinline__ unsigned long long box_key(float qx, float qy, float4 b)
-{
-    const float cx = 0.5f * (b.x + b.z) - qx, cy = 0.5f * (b.y + b.w) - qy;
-    return make_visit_key(box_bound(qx, qy, b), fmaf(cx, cx, cy * cy));
-}
-
-// The FP32 visitor of warp_visit_boxes: the warp's list (ld, li) and its k-th entry thr.
-struct WarpKnnF32 {
-    const float4 *nxy2;
+// The FP32 visitor of warp_walk. thr is the largest float while fewer than k points are known, so
+// that points at an infinite distance (padding, overflow) never enter.
+template <bool IDX>
+struct WarpNearest {
     float qx, qy;
     int k;
-    float ld;
-    int32_t li;
-    float thr;
+    float *bd;     // [kWarpBuffer] the warp's candidates in shared memory: squared distances
+    int32_t *bi;   // and stored positions
+    float thr = 3.402823466e38f;
+    int cnt = 0;
 
-    __device__ __forceinline__ unsigned long long key(float4 b) const
+    __device__ __forceinline__ bool usable(float bound, float4) const
     {
-        return box_key(qx, qy, b);
+        return bound < CUDART_INF_F;
     }
-    // A box may hold an entering point unless its bound exceeds the k-th distance.
-    __device__ __forceinline__ bool open(unsigned long long key) const
+    __device__ __forceinline__ WarpEntry cut()
     {
-        return key != ~0ull && !(visit_key_bound(key) > thr);
+        const WarpEntry e = warp_cut<IDX>(bd, bi, cnt, k);
+        thr = fminf(thr, __shfl_sync(kFullMask, e.d, k - 1));
+        cnt = min(cnt, k);
+        return e;
     }
-    __device__ __forceinline__ void scan(int64_t p)
+    __device__ __forceinline__ void settle()
     {
-#pragma unroll
-        for (int u = 0; u < kSubTile; u += 32)
-            warp_scan32(nxy2, p + u, qx, qy, k, ld, li, thr);
+        if (cnt >= k + kWarpSettle)
+            cut();
+    }
+    __device__ __forceinline__ void take(float d, int32_t pos)
+    {
+        unsigned c = __ballot_sync(kFullMask, d <= thr);
+        if (!c)
+            return;
+        if (cnt + __popc(c) > kWarpBuffer) {
+            cut();
+            c = __ballot_sync(kFullMask, d <= thr);
+        }
+        const int lane = threadIdx.x & 31;
+        if ((c >> lane) & 1u) {
+            const int o = cnt + __popc(c & ((1u << lane) - 1u));
+            bd[o] = d;
+            if (IDX)
+                bi[o] = pos;
+        }
+        cnt += __popc(c);
+    }
+    __device__ __forceinline__ void scan(int64_t p, float4 a, float4 b)
+    {
+        const int32_t pos = static_cast<int32_t>(p) + (threadIdx.x & 31);
+        const float da = dist2_neg(qx, qy, a.x, a.z), db = dist2_neg(qx, qy, b.x, b.z);
+        take(da, pos);
+        take(db, pos + 32);
     }
 };
 
-// The k nearest stored points of (qx, qy) by one warp: lanes 0..k-1 end holding the k smallest
-// squared distances in ascending order (ld) and the points' stored positions (li).
-__device__ __forceinline__ void warp_knn(const DatasetDev &ds, float qx, float qy, int k,
-                                         float &ld, int32_t &li)
+// The k nearest stored points of (qx, qy) by one warp: lanes 0..k-1 return the k smallest squared
+// distances in ascending order and, with IDX, the points' stored positions. A non-finite query
+// has none: (+inf, -1).
+template <bool IDX>
+__device__ __forceinline__ WarpEntry warp_knn(const DatasetDev &ds, float qx, float qy, int k,
+                                              float *bd, int32_t *bi)
 {
-    WarpKnnF32 v{ds.nxy2, qx, qy, k, CUDART_INF_F, -1, CUDART_INF_F};
-    warp_visit_boxes(ds, v);
-    ld = v.ld;
-    li = v.li;
+    WarpNearest<IDX> v{qx, qy, k, bd, bi};
+    if (isfinite(qx) && isfinite(qy))
+        warp_walk(ds, v);
+    return v.cut();
 }
 
 // Shared-memory scratch of a pruned phase-1 unit.

@@ -48,26 +48,25 @@ f32_select_kernel(int64_t m, int S, int k, double r_exp, AlphaMap am,
 }
 
 // Phase 1 with one warp per query (warp_knn), in the caller's order: each query's k nearest
-// squared distances (and stored positions mapped to caller indices when part_idx is non-null)
-// as one split's lists [k][m], for the selection kernel, which amortises its FP64 work over a
-// thread per query.
+// squared distances (and, with IDX, stored positions mapped to caller indices) as one split's
+// lists [k][m], for the selection kernel, which amortises its FP64 work over a thread per query.
+template <bool IDX>
 __global__ void __launch_bounds__(kThreads)
 f32_knn_warp_kernel(DatasetDev ds, int64_t m, const float *__restrict__ qx,
                     const float *__restrict__ qy, int k, float *__restrict__ part_d2,
                     int32_t *__restrict__ part_idx)
 {
     constexpr int W = kThreads / 32;
-    const int lane = threadIdx.x & 31;
+    __shared__ __align__(16) float bd[W][kWarpBuffer];
+    __shared__ int32_t bi[W][IDX ? kWarpBuffer : 1];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t nwarps = static_cast<int64_t>(gridDim.x) * W;
-    for (int64_t q = static_cast<int64_t>(blockIdx.x) * W + (threadIdx.x >> 5); q < m;
-         q += nwarps) {
-        float ld;
-        int32_t li;
-        warp_knn(ds, qx[q], qy[q], k, ld, li);
+    for (int64_t q = static_cast<int64_t>(blockIdx.x) * W + w; q < m; q += nwarps) {
+        const WarpEntry e = warp_knn<IDX>(ds, qx[q], qy[q], k, bd[w], bi[w]);
         if (lane < k) {
-            part_d2[static_cast<int64_t>(lane) * m + q] = ld;
-            if (part_idx)
-                part_idx[static_cast<int64_t>(lane) * m + q] = li >= 0 ? ds.orig[li] : -1;
+            part_d2[static_cast<int64_t>(lane) * m + q] = e.d;
+            if (IDX)
+                part_idx[static_cast<int64_t>(lane) * m + q] = e.i >= 0 ? ds.orig[e.i] : -1;
         }
     }
 }
@@ -281,9 +280,9 @@ cudaError_t launch_f32_knn_warp(const DatasetDev &ds, int64_t m, const float *qx
     const int64_t want = (m + W - 1) / W;
     const int64_t cap = static_cast<int64_t>(sm_count) * 16;
     const unsigned grid = static_cast<unsigned>(std::max<int64_t>(1, std::min(want, cap)));
-    f32_knn_warp_kernel<<<grid, kThreads, 0, st>>>(ds, m, qx, qy, k,
-                                                   static_cast<float *>(sc.part_d2),
-                                                   sc.part_idx);
+    auto fn = sc.part_idx ? f32_knn_warp_kernel<true> : f32_knn_warp_kernel<false>;
+    fn<<<grid, kThreads, 0, st>>>(ds, m, qx, qy, k, static_cast<float *>(sc.part_d2),
+                                  sc.part_idx);
     return cudaGetLastError();
 }
 

@@ -476,124 +476,162 @@ f64_knn_cull_kernel(DatasetDev ds, int64_t m, int qpb, int ntiles, int ntiles_p2
 }
 
 // ---------------------------------------------------------------------------------------------
-// FP64 phase 1 with one warp per query (the FP32 form is in f32_device.cuh): the warp's lanes
-// hold the k smallest (distance, caller index) pairs seen so far as a list sorted across the
-// lanes, 32 points are scanned per step (one per lane, read from the FP64 copy through the
-// Z-order map, exact distance as in the other FP64 scans), and the points that precede the k-th
-// entry are inserted one at a time when they are few, else sorted and merged. The pairs order by
-// distance, then caller index, so the lists are the k smallest pairs whatever the visit order:
-// those of the caller-order scan, ties going to the lower index. Boxes are walked by
-// warp_visit_boxes with FP64 bounds from the FP32 boxes widened for rounding (box_bound64).
+// FP64 phase 1 with one warp per query (the FP32 form is in f32_device.cuh). warp_walk runs on
+// the FP32 copy of the points (sequential in Z-order, unlike the FP64 copy it maps to) with the
+// query rounded to float, and a point whose FP32 distance is within thr goes into the buffer by
+// its stored position. Only when the buffer is cut are the new candidates read from the FP64 copy
+// and their exact distances formed, as in the other FP64 scans, two a lane at a time. The
+// candidates order by (distance, caller index), compared as integers (a non-negative double's
+// bits order like its value; GB300 compares doubles at 2 a clock per SM), so the lists are the k
+// smallest pairs whatever the visit order: those of the caller-order scan, ties going to the
+// lower index.
+//
+// thr for an exact k-th squared distance T: rounding to float moves the query by at most
+// 2^-24 |q|_1 and a point within r = sqrt(T) of it by at most 2^-24 (|q|_1 + r), and the FP32
+// distance of the rounded points carries a relative error below 2^-22, so that a point within r
+// has an FP32 distance of at most r (1 + 2^-21) + |q|_1 2^-22; the margins used are twice that. The
+// boxes hold the rounded points, so the same thr prunes them.
 // ---------------------------------------------------------------------------------------------
-constexpr int kWarpInsertMax64 = 6;
 
-// (a, ai) precedes (b, bi): smaller distance, or equal distance and lower caller index.
-__device__ __forceinline__ bool pair_lt(double a, int32_t ai, double b, int32_t bi)
-{
-    return a < b || (a == b && ai < bi);
-}
 
-// Compare-exchange of a bitonic network across lanes on (distance, index) pairs.
-__device__ __forceinline__ void warp_cx64(double &v, int32_t &i, int stride, bool up)
+// A candidate: the bits of its squared distance and its caller index. Missing entries and padding
+// points are (+inf, INT32_MAX), which no pair precedes.
+struct WarpEntry64 {
+    unsigned long long d;
+    int32_t i;
+};
+constexpr unsigned long long kInfBits = 0x7ff0000000000000ull;
+
+// Entry e of a warp's buffer: the first `sorted` hold (distance, caller index), the others a
+// stored position in bi.
+__device__ __forceinline__ WarpEntry64 warp_entry64(const unsigned long long *bd,
+                                                    const int32_t *bi, int e, int sorted,
+                                                    int cnt, const int32_t *orig,
+                                                    const double2 *xy64, double qx, double qy)
 {
-    const double ov = __shfl_xor_sync(kFullMask, v, stride);
-    const int32_t oi = __shfl_xor_sync(kFullMask, i, stride);
-    const bool lower = (threadIdx.x & stride) == 0;
-    const bool take = (lower == up) ? pair_lt(ov, oi, v, i) : pair_lt(v, i, ov, oi);
-    if (take) {
-        v = ov;
-        i = oi;
+    WarpEntry64 v{kInfBits, INT32_MAX};
+    if (e < sorted) {
+        v = {bd[e], bi[e]};
+    } else if (e < cnt) {
+        const int32_t o = orig[bi[e]];
+        if (o >= 0) {
+            const double2 p = xy64[o];
+            const double d = dist2_exact(qx, qy, p.x, p.y);
+            v = {static_cast<unsigned long long>(__double_as_longlong(d)), o};
+        }
     }
+    return v;
 }
 
-// The FP64 visitor of warp_visit_boxes. Empty list entries and padding points are
-// (+inf, INT32_MAX), which no pair precedes.
-struct WarpKnnF64 {
+// Cuts a warp's buffer to the k smallest pairs, as warp_cut does in FP32 (where every lane counts
+// the entries that precede its own).
+__device__ __noinline__ WarpEntry64 warp_cut64(unsigned long long *bd, int32_t *bi, int sorted,
+                                               int cnt, int k, const int32_t *orig,
+                                               const double2 *xy64, double qx, double qy)
+{
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    const WarpEntry64 a = warp_entry64(bd, bi, lane, sorted, cnt, orig, xy64, qx, qy);
+    const WarpEntry64 b = warp_entry64(bd, bi, lane + 32, sorted, cnt, orig, xy64, qx, qy);
+    __syncwarp();
+    bd[lane] = a.d;  // (+inf, INT32_MAX) beyond cnt
+    bi[lane] = a.i;
+    bd[lane + 32] = b.d;
+    bi[lane + 32] = b.i;
+    __syncwarp();
+    int r0 = 0, r1 = 0, q0 = 0, q1 = 0;  // entries below, entries equal (itself included)
+    const ulonglong2 *b2 = reinterpret_cast<const ulonglong2 *>(bd);
+#pragma unroll 2
+    for (int j = 0; 2 * j < cnt; ++j) {
+        const ulonglong2 d = b2[j];
+        r0 += (d.x < a.d) + (d.y < a.d);
+        q0 += (d.x == a.d) + (d.y == a.d);
+        if (cnt > 32) {
+            r1 += (d.x < b.d) + (d.y < b.d);
+            q1 += (d.x == b.d) + (d.y == b.d);
+        }
+    }
+    const bool has0 = lane < cnt, has1 = lane + 32 < cnt;
+    if (__any_sync(kFullMask, (has0 && q0 > 1) || (has1 && q1 > 1))) {
+        // Equal distances: the lower caller index first (equal pairs by position).
+        for (int j = 0; j < cnt; ++j) {
+            const unsigned long long d = bd[j];
+            const int32_t i = bi[j];
+            r0 += d == a.d && (i < a.i || (i == a.i && j < lane));
+            r1 += d == b.d && (i < b.i || (i == b.i && j < lane + 32));
+        }
+    }
+    __syncwarp();
+    if (has0 && r0 < k) {
+        bd[r0] = a.d;
+        bi[r0] = a.i;
+    }
+    if (has1 && r1 < k) {
+        bd[r1] = b.d;
+        bi[r1] = b.i;
+    }
+    __syncwarp();
+    if (lane < min(cnt, k))
+        return {bd[lane], bi[lane]};
+    return {kInfBits, INT32_MAX};
+}
+
+// The FP64 visitor of warp_walk.
+struct WarpNearest64 {
     const int32_t *orig;
     const double2 *xy64;
-    double qx, qy;
-    float qxf, qyf;
+    double qxd, qyd;
+    float qx, qy;
     int k;
-    double ld;     // this lane's list entry
-    int32_t li;
-    double thr;    // the k-th entry (warp-uniform)
-    int32_t thi;
+    unsigned long long *bd;  // [kWarpBuffer] the warp's candidates in shared memory
+    int32_t *bi;
+    float thr;   // +inf at first
+    int sorted;  // entries cut so far
+    int cnt;
 
-    __device__ __forceinline__ unsigned long long key(float4 b) const
+    __device__ __forceinline__ bool usable(float, float4 box) const
     {
-        if (!(b.x <= b.z))
-            return ~0ull;  // empty box
-        const float lb = __double2float_rd(box_bound64(b, qx, qy, qx, qy));
-        const float cx = 0.5f * (b.x + b.z) - qxf, cy = 0.5f * (b.y + b.w) - qyf;
-        return make_visit_key(lb, fmaf(cx, cx, cy * cy));
+        return box.x <= box.z;  // not empty
     }
-    // The bound is below every distance in the box, so a box whose bound exceeds the k-th
-    // distance holds no point that precedes the k-th pair, even at a tie.
-    __device__ __forceinline__ bool open(unsigned long long key) const
+    __device__ __forceinline__ WarpEntry64 cut()
     {
-        return key != ~0ull && !(static_cast<double>(visit_key_bound(key)) > thr);
+        const WarpEntry64 e = warp_cut64(bd, bi, sorted, cnt, k, orig, xy64, qxd, qyd);
+        cnt = min(cnt, k);
+        sorted = cnt;
+        const double T = __longlong_as_double(
+            static_cast<long long>(__shfl_sync(kFullMask, e.d, k - 1)));
+        const float mag = __fadd_ru(fabsf(qx), fabsf(qy));
+        const float r = __fsqrt_ru(__double2float_ru(T));
+        const float rt = __fadd_ru(__fmul_ru(r, 1.0f + 0x1p-20f), __fmul_ru(mag, 0x1p-21f));
+        thr = __fadd_ru(__fmul_ru(rt, rt), 0x1p-140f);  // the term covers subnormal rounding
+        return e;
     }
-    __device__ __forceinline__ void scan(int64_t p)
+    __device__ __forceinline__ void settle()
     {
-#pragma unroll
-        for (int u = 0; u < kSubTile; u += 32)
-            scan32(p + u);
+        if (cnt >= k + kWarpSettle)
+            cut();
     }
-    __device__ __forceinline__ void scan32(int64_t p)
+    __device__ __forceinline__ void take(float df, int32_t pos)
     {
+        unsigned c = __ballot_sync(kFullMask, !(df > thr));
+        if (!c)
+            return;
+        if (cnt + __popc(c) > kWarpBuffer) {
+            cut();
+            c = __ballot_sync(kFullMask, !(df > thr));
+        }
         const int lane = threadIdx.x & 31;
-        const int32_t o = orig[p + lane];
-        double d = CUDART_INF;
-        int32_t id = INT32_MAX;
-        if (o >= 0) {
-            const double2 pt = xy64[o];
-            d = dist2_exact(qx, qy, pt.x, pt.y);
-            id = o;
-        }
-        unsigned cand = __ballot_sync(kFullMask, pair_lt(d, id, thr, thi));
-        if (!cand)
-            return;
-        if (__popc(cand) <= kWarpInsertMax64) {
-            while (cand) {
-                const int src = __ffs(cand) - 1;
-                cand &= cand - 1;
-                const double c = __shfl_sync(kFullMask, d, src);
-                const int32_t ci = __shfl_sync(kFullMask, id, src);
-                if (!pair_lt(c, ci, thr, thi))
-                    continue;
-                const double up = __shfl_up_sync(kFullMask, ld, 1);
-                const int32_t upi = __shfl_up_sync(kFullMask, li, 1);
-                if (pair_lt(c, ci, ld, li)) {
-                    const bool here = lane == 0 || pair_lt(up, upi, c, ci);
-                    ld = here ? c : up;
-                    li = here ? ci : upi;
-                }
-                thr = __shfl_sync(kFullMask, ld, k - 1);
-                thi = __shfl_sync(kFullMask, li, k - 1);
-            }
-            return;
-        }
-        const bool is_cand = (cand >> lane) & 1u;
-        double v = is_cand ? d : CUDART_INF;
-        int32_t vi = is_cand ? id : INT32_MAX;
-#pragma unroll
-        for (int size = 2; size <= 32; size <<= 1) {
-#pragma unroll
-            for (int stride = size >> 1; stride > 0; stride >>= 1)
-                warp_cx64(v, vi, stride, (lane & size) == 0);
-        }
-        // The 32 smallest of the two sorted lists, as a bitonic sequence, then sorted.
-        const double rv = __shfl_sync(kFullMask, v, 31 - lane);
-        const int32_t ri = __shfl_sync(kFullMask, vi, 31 - lane);
-        if (pair_lt(rv, ri, ld, li)) {
-            ld = rv;
-            li = ri;
-        }
-#pragma unroll
-        for (int stride = 16; stride > 0; stride >>= 1)
-            warp_cx64(ld, li, stride, true);
-        thr = __shfl_sync(kFullMask, ld, k - 1);
-        thi = __shfl_sync(kFullMask, li, k - 1);
+        if ((c >> lane) & 1u)
+            bi[cnt + __popc(c & ((1u << lane) - 1u))] = pos;
+        cnt += __popc(c);
+    }
+    __device__ __forceinline__ void scan(int64_t p, float4 a, float4 b)
+    {
+        const int32_t pos = static_cast<int32_t>(p) + (threadIdx.x & 31);
+        const float ax = __fadd_rn(qx, a.x), ay = __fadd_rn(qy, a.z);
+        const float bx = __fadd_rn(qx, b.x), by = __fadd_rn(qy, b.z);
+        take(__fmaf_rn(ax, ax, __fmul_rn(ay, ay)), pos);
+        take(__fmaf_rn(bx, bx, __fmul_rn(by, by)), pos + 32);
     }
 };
 
@@ -605,18 +643,22 @@ f64_knn_warp_kernel(DatasetDev ds, int64_t m, const double *__restrict__ qx,
                     int32_t *__restrict__ part_idx)
 {
     constexpr int W = kThreads / 32;
-    const int lane = threadIdx.x & 31;
+    __shared__ __align__(16) unsigned long long bd[W][kWarpBuffer];
+    __shared__ int32_t bi[W][kWarpBuffer];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t nwarps = static_cast<int64_t>(gridDim.x) * W;
-    for (int64_t q = static_cast<int64_t>(blockIdx.x) * W + (threadIdx.x >> 5); q < m;
-         q += nwarps) {
+    for (int64_t q = static_cast<int64_t>(blockIdx.x) * W + w; q < m; q += nwarps) {
         const double x = qx[q], y = qy[q];
-        WarpKnnF64 v{ds.orig, ds.xy64, x, y, static_cast<float>(x), static_cast<float>(y), k,
-                     CUDART_INF, INT32_MAX, CUDART_INF, INT32_MAX};
-        warp_visit_boxes(ds, v);
+        WarpNearest64 v{ds.orig, ds.xy64, x, y, static_cast<float>(x), static_cast<float>(y), k,
+                        bd[w], bi[w], CUDART_INF_F, 0, 0};
+        if (!isnan(x) && !isnan(y))  // a NaN query has no neighbours
+            warp_walk(ds, v);
+        const WarpEntry64 e = v.cut();
         if (lane < k) {
-            part_d2[static_cast<int64_t>(lane) * m + q] = v.ld;
+            part_d2[static_cast<int64_t>(lane) * m + q] =
+                __longlong_as_double(static_cast<long long>(e.d));
             if (part_idx)
-                part_idx[static_cast<int64_t>(lane) * m + q] = v.li;
+                part_idx[static_cast<int64_t>(lane) * m + q] = e.i;
         }
     }
 }
