@@ -53,6 +53,8 @@ inline int finalize_threads(int splits, int64_t m)
 {
     return splits >= 64 && m <= 2048 ? 32 : (splits >= 16 ? 8 : 1);
 }
+// Largest |log2 of d1^power| of a query in an integer power class.
+constexpr float kClassMaxLog2 = 64.0f;
 constexpr int kPointGroups = 4;  // phase 2 with point groups (Plan::pg)
 
 // Levels and bounds of Eq. 5 and Eq. 6, passed to kernels by value.
@@ -78,6 +80,7 @@ struct DatasetDev {
     const double *z64;      // [n_pad] caller's order
     int64_t n;
     int64_t n_pad;
+    float z_max;            // largest |z| of the FP32 copy
 };
 
 // How one scan pass is cut into work: query blocks (one CTA each) times data-range splits,
@@ -100,6 +103,8 @@ struct Plan {
     int knn_slots; // phase-1 CTAs resident on the whole GPU (occupancy x SMs)
     int kq;        // pruned phase 1: queries per thread (2 or 4)
     int pg;        // phase 2: point groups per CTA (1: every thread sees every point)
+    int pow_a;     // FP32 phase 2 by power classes: the integer powers of the two saturated levels
+    int pow_b;     // of Eq. 6 (0: none); both 0: phase 2 runs in the queries' own order
 };
 
 // Per-query parameters of phase 2 produced by the selection kernel.
@@ -122,6 +127,18 @@ struct QParamF64X {
 };
 static_assert(sizeof(QParamF64X) == sizeof(QParamF64), "shares the FP64 scratch layout");
 
+// The order FP32 phase 2 runs in when the queries are sorted into power classes (Plan::pow_a and
+// pow_b): class kClassA (power pow_a), kClassG (any power) and kClassB (pow_b), each in a region
+// of m entries, its query count in cnt[class].
+enum PowerClass { kClassA = 0, kClassG = 1, kClassB = 2, kClasses = 3 };
+struct ClassOrder {
+    uint32_t *cnt;  // [kClasses], zeroed by the phase-1 kernel
+    float *qx, *qy; // [kClasses][m]
+    QParamF32 *qp;  // [kClasses][m]
+    uint32_t *id;   // [kClasses][m] caller's query index
+    int pow_a, pow_b;
+};
+
 // Scratch buffers of one interpolation (device memory owned by the library or by the
 // caller of the allocation-free entry point).
 struct Scratch {
@@ -129,6 +146,7 @@ struct Scratch {
     int32_t *part_idx; // [S_knn][k][m] or null when indices are not kept
     void *qparam;      // [m] QParamF32 / QParamF64
     void *part_sum;    // [S_w][4][m] float (w_hi, w_lo, wz_hi, wz_lo) or double
+    ClassOrder cls;    // cnt null: no power classes
 };
 
 size_t scratch_bytes(int precision, const Plan &pl, int k);
@@ -140,7 +158,8 @@ cudaError_t launch_f32_knn(const DatasetDev &ds, const Plan &pl, const float *qx
                            cudaStream_t st);
 cudaError_t launch_f32_select(const Plan &pl, int k, double r_exp, const AlphaMap &am,
                               const Scratch &sc, float *out_alpha, int32_t *out_knn,
-                              cudaStream_t st, const uint32_t *perm = nullptr);
+                              cudaStream_t st, const float *qx, const float *qy,
+                              const uint32_t *perm = nullptr);
 cudaError_t launch_f32_weights(const DatasetDev &ds, const Plan &pl, const float *qx,
                                const float *qy, const Scratch &sc, int *err, cudaStream_t st);
 cudaError_t launch_f32_finalize(const Plan &pl, const Scratch &sc, float *out,
@@ -337,6 +356,20 @@ __device__ __forceinline__ float ex2_approx(float x)
 {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+__device__ __forceinline__ float rsq_approx(float x)
+{
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
 

@@ -49,10 +49,12 @@ bool dataset_lookup(aidw_ctx *ctx, int64_t id, DatasetDev *dev, double *r_exp);
 int pointer_kind(const void *p, int device);
 int validate_params(const aidw_params *p, int64_t n);
 AlphaMap alpha_map(const aidw_params &p);
-// Shape from `cfg`, or from the context's shape when cfg is null.
+// Shape from `cfg`, or from the context's shape when cfg is null. With `classes` (the call's
+// parameters) FP32 phase 2 may run by power classes; z_max is the dataset's largest |z|.
 Plan make_plan(aidw_ctx *ctx, int precision, int64_t n, int64_t n_pad, int64_t m, int k,
                bool with_idx, int force_knn_splits, int force_w_splits,
-               const aidw_tune_config *cfg = nullptr);
+               const aidw_tune_config *cfg = nullptr, const aidw_params *classes = nullptr,
+               float z_max = 0.0f);
 aidw_tune_config ctx_tune(aidw_ctx *ctx);
 void ctx_set_tune(aidw_ctx *ctx, const aidw_tune_config &c);
 int interpolate_impl(aidw_ctx *ctx, int64_t dsid, const void *qx, const void *qy, int64_t m,

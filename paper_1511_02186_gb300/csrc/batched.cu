@@ -105,8 +105,10 @@ __device__ __noinline__ bool batch_weights_unit(const BatchItemDev *itp, int qbl
     const int64_t p0 = static_cast<int64_t>(split) * it.w.split_len;
     const int64_t p1 = min(p0 + it.w.split_len, it.ds.n_pad);
     TileSeq ts{g_bar, seq};
-    return weights_unit<QW, TW>(it.ds, it.m, qbase, p0, p1, it.sqx, it.sqy, it.qparam, split,
-                                it.part_sum, err,
+    return weights_unit<QW, TW>(it.ds,
+                                unit_queries(it.sqx, it.sqy, it.qparam, it.m, qbase,
+                                             it.w.q_per_block),
+                                p0, p1, split, it.part_sum, err,
                                 reinterpret_cast<float4(*)[TW]>(&g_txy[0][0]),
                                 reinterpret_cast<float2(*)[TW]>(&g_tz[0][0]), ts);
 }

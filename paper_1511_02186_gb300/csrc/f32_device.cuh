@@ -789,6 +789,12 @@ __device__ __forceinline__ void select_query(int64_t q, int64_t m, int S, int k,
 // hold whole chunks, so neither Q nor TW changes any query's sequence of operations. Chunks
 // that hold only padding (from the first multiple of kChunkW at or above n) are not summed:
 // they would add weights of exactly 0; tiles made of them are not loaded.
+//
+// What bounds the loop: an SM issues 128 lane-operations a clock (an FP32x2 instruction counts
+// as two: it reads twice the operands), and its MUFU 16 lg2 or rsq or 32 ex2. A pair costs 7 FP32
+// operations, two MUFU ones and about 1.3 of loads and merges, 10.3 slots or 0.081 clocks,
+// against 0.094 clocks of MUFU; measured 0.100. With an integer power (POW > 0) the weight needs
+// one rsq (or rcp) and up to three products instead of lg2 and ex2: 0.063 clocks of MUFU.
 // ---------------------------------------------------------------------------------------------
 
 // End of the summed chunks of a split [p_begin, p_end): the dataset's last real point rounded
@@ -807,16 +813,71 @@ __device__ __forceinline__ int weights_tiles(const DatasetDev &ds, int64_t p_beg
     return e > p_begin ? static_cast<int>((e - p_begin + TW - 1) / TW) : 0;
 }
 
+// The queries of a phase-2 unit, consecutive in the order phase 2 runs in: query i (below n) at
+// (x, y) with parameters p; its partial sums go to column col(i) of m.
+struct UnitQueries {
+    const float *qx, *qy;
+    const QParamF32 *qp;
+    int64_t base, n, col0, m;
+
+    __device__ __forceinline__ void load(int64_t i, float &x, float &y, float2 &p) const
+    {
+        const int64_t q = base + min(i, n - 1);
+        p = __ldcg(reinterpret_cast<const float2 *>(qp + q));
+        x = qx[q];
+        y = qy[q];
+    }
+    __device__ __forceinline__ int64_t col(int64_t i) const
+    {
+        return col0 + i;
+    }
+};
+
+// The block of queries [qbase, qbase + count) of m.
+__device__ __forceinline__ UnitQueries unit_queries(const float *qx, const float *qy,
+                                                    const QParamF32 *qp, int64_t m,
+                                                    int64_t qbase, int64_t count)
+{
+    return {qx, qy, qp, qbase, min(count, m - qbase), qbase, m};
+}
+
+// How many of 32 consecutive points take the rsq form of an integer power, spread evenly; the
+// rest take lg2 and ex2, whose MUFU time fills what the products leave. Measured on 262,144^2
+// pairs (ms; all lg2 / 20 of 32 / all rsq): alpha = 5 22.0 / 18.65 / 18.84; alpha = 3 and 4 all
+// rsq 17.3 and 17.4; alpha = 1 and 2 14.8, where rsq (rcp) alone is 1/16 clock and every other
+// operation fits beside it.
+template <int POW>
+__device__ __forceinline__ constexpr bool rsq_point(int u)
+{
+    constexpr int share = POW == 0 ? 0 : (POW >= 5 ? 20 : 32);
+    return (u * share) % 32 < share;
+}
+
+// d2^(-POW/2) for a query pair, by one MUFU rsq (rcp for even powers up to 2) each.
+template <int POW>
+__device__ __forceinline__ float2 integer_power(float2 d2)
+{
+    if constexpr (POW == 2)
+        return make_float2(rcp_approx(d2.x), rcp_approx(d2.y));
+    const float2 r = make_float2(rsq_approx(d2.x), rsq_approx(d2.y));
+    if constexpr (POW == 1)
+        return r;
+    const float2 r2 = __fmul2_rn(r, r);
+    if constexpr (POW == 3)
+        return __fmul2_rn(r2, r);
+    const float2 r4 = __fmul2_rn(r2, r2);
+    return POW == 4 ? r4 : __fmul2_rn(r4, r);
+}
+
 // PG > 1 cuts the CTA's threads into PG groups of kThreads / PG, each thread still holding Q
 // queries: the CTA serves Q kThreads / PG queries, and each group sums its own PG-th part of
 // every chunk (kChunkW points of PG chunks to a Kahan merge); the groups' sums are merged at the
 // end. A call with few queries then wastes fewer lanes on queries it does not have.
-template <int Q, int TW, int PG = 1>
-__device__ __forceinline__ bool weights_unit(const DatasetDev &ds, int64_t m, int64_t qbase,
-                                             int64_t p_begin, int64_t p_end,
-                                             const float *__restrict__ qx,
-                                             const float *__restrict__ qy,
-                                             const QParamF32 *qp, int s,
+// POW > 0: every query's power is POW. The weights of the rsq points are d^-POW, summed apart and
+// brought to the others' scale d1^POW = 2^c once per chunk.
+template <int Q, int TW, int PG = 1, int POW = 0>
+__device__ __forceinline__ bool weights_unit(const DatasetDev &ds, const UnitQueries &uq,
+                                             int64_t p_begin, int64_t p_end, int s,
                                              float *__restrict__ part_sum,
                                              int *__restrict__ err,
                                              float4 (*txy)[TW],
@@ -832,23 +893,26 @@ __device__ __forceinline__ bool weights_unit(const DatasetDev &ds, int64_t m, in
     const int ntiles = weights_tiles<TW>(ds, p_begin, p_end);
     const int64_t p_sum = weights_end(ds, p_end);
 
-    float2 qxp[H], qyp[H], nsp[H], ccp[H];
+    float2 qxp[H], qyp[H], nsp[H], ccp[H], kkp[H];
     float hw[Q], cw[Q], hz[Q], cz[Q];
 #pragma unroll
     for (int j = 0; j < Q; ++j) {
-        const int64_t q = min(qbase + j * QT + tq, m - 1);
-        const float2 o = __ldcg(reinterpret_cast<const float2 *>(qp + q));
-        const float a = qx[q], b = qy[q];
+        float a, b;
+        float2 o;
+        uq.load(j * QT + tq, a, b, o);
+        const float kk = POW > 0 ? ex2_approx(o.y) : 0.0f;
         if (j & 1) {
             qxp[j / 2].y = a;
             qyp[j / 2].y = b;
             nsp[j / 2].y = o.x;
             ccp[j / 2].y = o.y;
+            kkp[j / 2].y = kk;
         } else {
             qxp[j / 2].x = a;
             qyp[j / 2].x = b;
             nsp[j / 2].x = o.x;
             ccp[j / 2].x = o.y;
+            kkp[j / 2].x = kk;
         }
         hw[j] = cw[j] = hz[j] = cz[j] = 0.0f;
     }
@@ -884,10 +948,10 @@ __device__ __forceinline__ bool weights_unit(const DatasetDev &ds, int64_t m, in
         const int64_t t0 = p_begin + static_cast<int64_t>(t) * TW;
         const int cend = static_cast<int>(min(static_cast<int64_t>(TW), p_sum - t0));
         for (int c = 0; c < cend; c += PG * kChunkW) {
-            float2 sw[H], sz[H];
+            float2 sw[H], sz[H], rw[H], rz[H];
 #pragma unroll
             for (int h = 0; h < H; ++h)
-                sw[h] = sz[h] = make_float2(0.0f, 0.0f);
+                sw[h] = sz[h] = rw[h] = rz[h] = make_float2(0.0f, 0.0f);
             for (int i = 0; i < PG; ++i) {
                 const int cg = c + i * kChunkW + pg * (kChunkW / PG);
                 if (PG > 1 && cg >= cend)
@@ -903,16 +967,26 @@ __device__ __forceinline__ bool weights_unit(const DatasetDev &ds, int64_t m, in
                         const float2 dx = __fadd2_rn(qxp[h], make_float2(p.x, p.y));
                         const float2 dy = __fadd2_rn(qyp[h], make_float2(p.z, p.w));
                         const float2 d2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, eps2));
-                        const float2 lg = make_float2(lg2_approx(d2.x), lg2_approx(d2.y));
-                        const float2 e = __ffma2_rn(lg, nsp[h], ccp[h]);
-                        const float2 w = make_float2(ex2_approx(e.x), ex2_approx(e.y));
-                        sw[h] = __fadd2_rn(sw[h], w);
-                        sz[h] = __ffma2_rn(w, zz, sz[h]);
+                        if (rsq_point<POW>(u)) {
+                            const float2 w = integer_power<POW>(d2);
+                            rw[h] = __fadd2_rn(rw[h], w);
+                            rz[h] = __ffma2_rn(w, zz, rz[h]);
+                        } else {
+                            const float2 lg = make_float2(lg2_approx(d2.x), lg2_approx(d2.y));
+                            const float2 e = __ffma2_rn(lg, nsp[h], ccp[h]);
+                            const float2 w = make_float2(ex2_approx(e.x), ex2_approx(e.y));
+                            sw[h] = __fadd2_rn(sw[h], w);
+                            sz[h] = __ffma2_rn(w, zz, sz[h]);
+                        }
                     }
                 }
             }
 #pragma unroll
             for (int h = 0; h < H; ++h) {
+                if (POW > 0) {
+                    sw[h] = __ffma2_rn(rw[h], kkp[h], sw[h]);
+                    sz[h] = __ffma2_rn(rz[h], kkp[h], sz[h]);
+                }
                 kahan_add(hw[2 * h], cw[2 * h], sw[h].x);
                 kahan_add(hw[2 * h + 1], cw[2 * h + 1], sw[h].y);
                 kahan_add(hz[2 * h], cz[2 * h], sz[h].x);
@@ -952,14 +1026,14 @@ __device__ __forceinline__ bool weights_unit(const DatasetDev &ds, int64_t m, in
     }
 #pragma unroll
     for (int j = 0; j < Q; ++j) {
-        const int64_t q = qbase + j * QT + tq;
-        if (q >= m)
+        const int64_t i = j * QT + tq;
+        if (i >= uq.n)
             continue;
-        float *o = part_sum + static_cast<int64_t>(s) * 4 * m + q;
+        float *o = part_sum + static_cast<int64_t>(s) * 4 * uq.m + uq.col(i);
         o[0] = hw[j];
-        o[m] = -cw[j];
-        o[2 * m] = hz[j];
-        o[3 * m] = -cz[j];
+        o[uq.m] = -cw[j];
+        o[2 * uq.m] = hz[j];
+        o[3 * uq.m] = -cz[j];
     }
     return true;
 }

@@ -18,15 +18,23 @@ using namespace f32dev;
 // the same 64 queries (2 per lane, whatever the shape's queries per thread).
 constexpr int kQueriesPG = 2;
 
+// The phase-1 kernel zeroes the power classes' counters, which the selection after it counts in.
+__device__ __forceinline__ void zero_classes(uint32_t *cnt)
+{
+    if (cnt && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kClasses)
+        cnt[threadIdx.x] = 0;
+}
+
 template <int KP, int Q, bool IDX>
 __global__ void __launch_bounds__(kThreads)
 f32_knn_kernel(DatasetDev ds, int64_t m, PassPlan pp, const float *__restrict__ qx,
                const float *__restrict__ qy, int k, float *__restrict__ part_d2,
-               int32_t *__restrict__ part_idx, int *__restrict__ err)
+               int32_t *__restrict__ part_idx, int *__restrict__ err, uint32_t *cls_cnt)
 {
     __shared__ __align__(128) float4 tile[2][kTileF32Knn];
     __shared__ __align__(8) uint64_t bar[2];
     extern __shared__ int32_t idx_smem[];  // [Q][KP][kThreads] when IDX
+    zero_classes(cls_cnt);
     init_tile_barriers(bar);
     TileSeq ts{bar, 0u};
     const int s = blockIdx.y;
@@ -36,15 +44,51 @@ f32_knn_kernel(DatasetDev ds, int64_t m, PassPlan pp, const float *__restrict__ 
                          p_end, qx, qy, k, s, part_d2, part_idx, err, tile, ts, idx_smem);
 }
 
+// A query's power class. Integer powers take the class loop where 2^c = d1^power (and with it
+// every unscaled weight d^-power) stays within 2^+-kClassMaxLog2.
+__device__ __forceinline__ int power_class(const QParamF32 &p, int pow_a, int pow_b)
+{
+    if (!(fabsf(p.c) <= kClassMaxLog2))
+        return kClassG;  // also NaN, and a query on a data point
+    const float twice = -2.0f * p.neg_s;
+    return twice == static_cast<float>(pow_a)   ? kClassA
+           : twice == static_cast<float>(pow_b) ? kClassB
+                                                : kClassG;
+}
+
 __global__ void __launch_bounds__(256)
 f32_select_kernel(int64_t m, int S, int k, double r_exp, AlphaMap am,
                   const float *__restrict__ part_d2, const int32_t *__restrict__ part_idx,
                   QParamF32 *__restrict__ qp, float *__restrict__ out_alpha,
-                  int32_t *__restrict__ out_knn, const uint32_t *__restrict__ perm)
+                  int32_t *__restrict__ out_knn, const uint32_t *__restrict__ perm,
+                  const float *__restrict__ qx, const float *__restrict__ qy, ClassOrder co)
 {
     const int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (q < m)
         select_query(q, m, S, k, r_exp, am, part_d2, part_idx, qp, out_alpha, out_knn, perm);
+    if (!co.cnt)
+        return;
+    // Each query to the next place of its class (a warp's queries stay together).
+    const int lane = threadIdx.x & 31;
+    QParamF32 p{0.0f, 0.0f};
+    int cls = kClasses;
+    if (q < m) {
+        p = qp[q];
+        cls = power_class(p, co.pow_a, co.pow_b);
+    }
+    const unsigned same = __match_any_sync(0xffffffffu, cls);
+    const int leader = __ffs(same) - 1;
+    uint32_t at = 0;
+    if (lane == leader && cls < kClasses)
+        at = atomicAdd(&co.cnt[cls], static_cast<uint32_t>(__popc(same)));
+    at = __shfl_sync(0xffffffffu, at, leader) + __popc(same & ((1u << lane) - 1u));
+    if (q < m) {
+        const int64_t o = static_cast<int64_t>(cls) * m + at;
+        co.qx[o] = qx[q];
+        co.qy[o] = qy[q];
+        co.qp[o] = p;
+        co.id[o] = perm ? perm[q] : static_cast<uint32_t>(q);
+    }
 }
 
 // Phase 1 with one warp per query (warp_knn), in the caller's order: each query's k nearest
@@ -54,8 +98,9 @@ template <bool IDX>
 __global__ void __launch_bounds__(kThreads)
 f32_knn_warp_kernel(DatasetDev ds, int64_t m, const float *__restrict__ qx,
                     const float *__restrict__ qy, int k, float *__restrict__ part_d2,
-                    int32_t *__restrict__ part_idx)
+                    int32_t *__restrict__ part_idx, uint32_t *cls_cnt)
 {
+    zero_classes(cls_cnt);
     constexpr int W = kThreads / 32;
     __shared__ __align__(16) float bd[W][kWarpBuffer];
     __shared__ int32_t bi[W][IDX ? kWarpBuffer : 1];
@@ -76,8 +121,9 @@ __global__ void __launch_bounds__(kThreads)
 f32_knn_cull_kernel(DatasetDev ds, int64_t m, int qpb, int ntiles, int ntiles_p2,
                     const float *__restrict__ sqx, const float *__restrict__ sqy, int k,
                     float *__restrict__ part_d2, int32_t *__restrict__ part_idx,
-                    int *__restrict__ err)
+                    int *__restrict__ err, uint32_t *cls_cnt)
 {
+    zero_classes(cls_cnt);
     extern __shared__ unsigned long long order[];  // [ntiles_p2], then the index lists if IDX
     __shared__ __align__(128) float4 tile[2][kTileF32Knn];
     __shared__ __align__(8) uint64_t bar[2];
@@ -103,8 +149,81 @@ f32_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const float *__restric
     const int s = blockIdx.y;
     const int64_t p_begin = static_cast<int64_t>(s) * pp.split_len;
     const int64_t p_end = min(p_begin + pp.split_len, ds.n_pad);
-    weights_unit<Q, TW, PG>(ds, m, static_cast<int64_t>(blockIdx.x) * pp.q_per_block, p_begin,
-                            p_end, qx, qy, qp, s, part_sum, err, txy, tz, ts);
+    const int64_t qbase = static_cast<int64_t>(blockIdx.x) * pp.q_per_block;
+    weights_unit<Q, TW, PG>(ds, unit_queries(qx, qy, qp, m, qbase, pp.q_per_block), p_begin,
+                            p_end, s, part_sum, err, txy, tz, ts);
+}
+
+// Phase 2 over the power classes: a block serves 256 queries of one class, with the class's loop.
+// The grid has a block for every 256 queries and one more per further class; the general class,
+// the slowest, comes first. Which loop a query takes depends on its own power and nearest
+// distance only. The shape is fixed (2 queries per thread, 512-point tiles).
+template <int POW>
+__device__ __forceinline__ void weights_class_unit(const DatasetDev &ds, const UnitQueries &uq,
+                                                   int64_t p_begin, int64_t p_end, int s,
+                                                   float *part_sum, int *err,
+                                                   float4 (*txy)[512], float2 (*tz)[512],
+                                                   TileSeq &ts)
+{
+    weights_unit<2, 512, 1, POW>(ds, uq, p_begin, p_end, s, part_sum, err, txy, tz, ts);
+}
+
+__global__ void __launch_bounds__(kThreads, 8)
+f32_weights_class_kernel(DatasetDev ds, int64_t m, PassPlan pp, ClassOrder co,
+                         float *__restrict__ part_sum, int *__restrict__ err)
+{
+    __shared__ __align__(128) float4 txy[2][512];
+    __shared__ __align__(128) float2 tz[2][512];
+    __shared__ __align__(8) uint64_t bar[2];
+    constexpr int kB = 2 * kThreads;
+    const int order[kClasses] = {kClassG, kClassA, kClassB};
+    int64_t u = blockIdx.x, col = 0;
+    int cls = -1;
+    int64_t n = 0;
+#pragma unroll
+    for (int i = 0; i < kClasses; ++i) {
+        const int64_t c = __ldcg(co.cnt + order[i]);
+        if (cls < 0) {
+            const int64_t blocks = (c + kB - 1) / kB;
+            if (u < blocks) {
+                cls = order[i];
+                n = c;
+            } else {
+                u -= blocks;
+                col += c;
+            }
+        }
+    }
+    if (cls < 0)
+        return;
+    init_tile_barriers(bar);
+    TileSeq ts{bar, 0u};
+    const int s = blockIdx.y;
+    const int64_t p_begin = static_cast<int64_t>(s) * pp.split_len;
+    const int64_t p_end = min(p_begin + pp.split_len, ds.n_pad);
+    const UnitQueries uq{co.qx, co.qy, co.qp, cls * m + u * kB,
+                         min(static_cast<int64_t>(kB), n - u * kB), col + u * kB, m};
+    const int pow = cls == kClassA ? co.pow_a : (cls == kClassB ? co.pow_b : 0);
+    switch (pow) {
+    case 1:
+        weights_class_unit<1>(ds, uq, p_begin, p_end, s, part_sum, err, txy, tz, ts);
+        break;
+    case 2:
+        weights_class_unit<2>(ds, uq, p_begin, p_end, s, part_sum, err, txy, tz, ts);
+        break;
+    case 3:
+        weights_class_unit<3>(ds, uq, p_begin, p_end, s, part_sum, err, txy, tz, ts);
+        break;
+    case 4:
+        weights_class_unit<4>(ds, uq, p_begin, p_end, s, part_sum, err, txy, tz, ts);
+        break;
+    case 5:
+        weights_class_unit<5>(ds, uq, p_begin, p_end, s, part_sum, err, txy, tz, ts);
+        break;
+    default:
+        weights_class_unit<0>(ds, uq, p_begin, p_end, s, part_sum, err, txy, tz, ts);
+        break;
+    }
 }
 
 // R threads per query (a block serves 256 / R queries): each sums every R-th split's partial
@@ -113,7 +232,7 @@ f32_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const float *__restric
 template <int R>
 __global__ void __launch_bounds__(256)
 f32_finalize_kernel(int64_t m, int S, const float *__restrict__ part_sum,
-                    float *__restrict__ out, const uint32_t *__restrict__ perm)
+                    float *__restrict__ out, const uint32_t *__restrict__ perm, ClassOrder co)
 {
     constexpr int C = 256 / R;
     const int col = threadIdx.x % C, r = threadIdx.x / C;
@@ -133,8 +252,17 @@ f32_finalize_kernel(int64_t m, int S, const float *__restrict__ part_sum,
             WZ += sum[i][col].y;
         }
     }
-    if (q < m)
-        out[perm ? perm[q] : q] = static_cast<float>(WZ / W);
+    if (q >= m)
+        return;
+    int64_t o = perm ? static_cast<int64_t>(perm[q]) : q;
+    if (co.cnt) {
+        // Column q of the class order: the general class, class A, class B.
+        const int64_t ng = co.cnt[kClassG], na = co.cnt[kClassA];
+        o = co.id[q < ng        ? kClassG * m + q
+                  : q < ng + na ? kClassA * m + (q - ng)
+                                : kClassB * m + (q - ng - na)];
+    }
+    out[o] = static_cast<float>(WZ / W);
 }
 
 template <int KP, int Q, bool IDX>
@@ -154,7 +282,7 @@ cudaError_t launch_cull_t(const DatasetDev &ds, const Plan &pl, const float *sqx
         return e;
     fn<<<pl.knn.qblocks, kThreads, dyn, st>>>(ds, pl.m, pl.knn.q_per_block, ntiles, p2, sqx,
                                               sqy, k, static_cast<float *>(sc.part_d2),
-                                              sc.part_idx, err);
+                                              sc.part_idx, err, sc.cls.cnt);
     return cudaGetLastError();
 }
 
@@ -173,7 +301,8 @@ cudaError_t launch_knn_t(const DatasetDev &ds, const Plan &pl, const float *qx,
     }
     dim3 grid(pl.knn.qblocks, pl.knn.splits);
     fn<<<grid, kThreads, dyn, st>>>(ds, pl.m, pl.knn, qx, qy, k,
-                                    static_cast<float *>(sc.part_d2), sc.part_idx, err);
+                                    static_cast<float *>(sc.part_d2), sc.part_idx, err,
+                                    sc.cls.cnt);
     return cudaGetLastError();
 }
 
@@ -262,13 +391,14 @@ cudaError_t launch_f32_knn(const DatasetDev &ds, const Plan &pl, const float *qx
 
 cudaError_t launch_f32_select(const Plan &pl, int k, double r_exp, const AlphaMap &am,
                               const Scratch &sc, float *out_alpha, int32_t *out_knn,
-                              cudaStream_t st, const uint32_t *perm)
+                              cudaStream_t st, const float *qx, const float *qy,
+                              const uint32_t *perm)
 {
     const int64_t blocks = (pl.m + 255) / 256;
     f32_select_kernel<<<static_cast<unsigned>(blocks), 256, 0, st>>>(
         pl.m, pl.knn.splits, k, r_exp, am, static_cast<const float *>(sc.part_d2),
         pl.with_idx ? sc.part_idx : nullptr, static_cast<QParamF32 *>(sc.qparam), out_alpha,
-        out_knn, perm);
+        out_knn, perm, qx, qy, sc.cls);
     return cudaGetLastError();
 }
 
@@ -282,7 +412,7 @@ cudaError_t launch_f32_knn_warp(const DatasetDev &ds, int64_t m, const float *qx
     const unsigned grid = static_cast<unsigned>(std::max<int64_t>(1, std::min(want, cap)));
     auto fn = sc.part_idx ? f32_knn_warp_kernel<true> : f32_knn_warp_kernel<false>;
     fn<<<grid, kThreads, 0, st>>>(ds, m, qx, qy, k, static_cast<float *>(sc.part_d2),
-                                  sc.part_idx);
+                                  sc.part_idx, sc.cls.cnt);
     return cudaGetLastError();
 }
 
@@ -316,6 +446,12 @@ cudaError_t launch_f32_knn_cull(const DatasetDev &ds, const Plan &pl, const floa
 cudaError_t launch_f32_weights(const DatasetDev &ds, const Plan &pl, const float *qx,
                                const float *qy, const Scratch &sc, int *err, cudaStream_t st)
 {
+    if (sc.cls.cnt) {
+        const dim3 grid(pl.w.qblocks + kClasses - 1, pl.w.splits);
+        f32_weights_class_kernel<<<grid, kThreads, 0, st>>>(
+            ds, pl.m, pl.w, sc.cls, static_cast<float *>(sc.part_sum), err);
+        return cudaGetLastError();
+    }
     dim3 grid(pl.w.qblocks, pl.w.splits);
     const WeightsKernel fn = weights_kernel_for(pl.qw, pl.tw, pl.pg);
     fn<<<grid, kThreads, 0, st>>>(ds, pl.m, pl.w, qx, qy,
@@ -332,7 +468,7 @@ cudaError_t launch_f32_finalize(const Plan &pl, const Scratch &sc, float *out, c
     auto fn = R == 32 ? f32_finalize_kernel<32>
                       : (R == 8 ? f32_finalize_kernel<8> : f32_finalize_kernel<1>);
     fn<<<blocks, 256, 0, st>>>(pl.m, pl.w.splits, static_cast<const float *>(sc.part_sum), out,
-                               perm);
+                               perm, sc.cls);
     return cudaGetLastError();
 }
 
