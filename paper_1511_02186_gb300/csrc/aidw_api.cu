@@ -565,7 +565,7 @@ int enqueue_interpolation(aidw_ctx *ctx, const DatasetDev &ds, double r_exp, con
     if (e != cudaSuccess)
         return AIDW_ERR_CUDA;
     marks.at(1);
-    e = f64 ? launch_f64_select(pl, p.k, r_exp, am, sc, out_alpha, out_knn, st, nullptr, x)
+    e = f64 ? launch_f64_select(pl, p.k, r_exp, am, sc, out_alpha, out_knn, st)
             : launch_f32_select(pl, p.k, r_exp, am, sc, out_alpha, out_knn, st,
                                   static_cast<const float *>(qx), static_cast<const float *>(qy));
     if (e != cudaSuccess)
@@ -692,8 +692,7 @@ int enqueue_culled(aidw_ctx *ctx, const DatasetDev &ds, double r_exp, const Plan
         ok = ok && gather_queries_f64(x, y, perm, m, sx, sy, st) == cudaSuccess;
         ok = ok && launch_f64_knn_cull(ds, pl, sx, sy, p.k, sc, ctx->d_err, st) == cudaSuccess;
         marks.at(1);
-        ok = ok && launch_f64_select(pl, p.k, r_exp, am, sc, out_alpha, out_knn, st, perm,
-                                     xp) == cudaSuccess;
+        ok = ok && launch_f64_select(pl, p.k, r_exp, am, sc, out_alpha, out_knn, st, perm) == cudaSuccess;
         marks.at(2);
         ok = ok && (xp ? launch_f64x_weights(ds, pl, sx, sy, sc, ctx->d_err, st)
                        : launch_f64_weights(ds, pl, sx, sy, sc, ctx->d_err, st)) == cudaSuccess;
@@ -756,8 +755,7 @@ int enqueue_warp(aidw_ctx *ctx, const DatasetDev &ds, double r_exp, const Plan &
         marks.at(0);
         ok = launch_f64_knn_warp(ds, pl, dx, dy, p.k, sc, ctx->sm_count, st) == cudaSuccess;
         marks.at(1);
-        ok = ok && launch_f64_select(pl, p.k, r_exp, am, sc, out_alpha, out_knn, st, nullptr,
-                                     x) == cudaSuccess;
+        ok = ok && launch_f64_select(pl, p.k, r_exp, am, sc, out_alpha, out_knn, st) == cudaSuccess;
         marks.at(2);
         ok = ok && (x ? launch_f64x_weights(ds, pl, dx, dy, sc, ctx->d_err, st)
                       : launch_f64_weights(ds, pl, dx, dy, sc, ctx->d_err, st)) == cudaSuccess;

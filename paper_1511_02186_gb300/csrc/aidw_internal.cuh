@@ -28,8 +28,8 @@ constexpr double kEpsF64 = 2.2250738585072014e-308;
 // Power scale used for coincident queries: w = 2^(kCoincScale (L1 - log2 d2)) is exactly 1 on
 // a coincident point (d2 == eps) and underflows to 0 everywhere else.
 constexpr float kCoincScaleF32 = 1.2676506e30f;  // 2^100
-constexpr double kCoincScaleF64 = 8.452712498170644e270;  // 2^900
-constexpr double kCoincScaleDf = 1.2676506002282294e30;   // 2^100 (AIDW_F64X: float range)
+constexpr double kCoincScaleF64 = 8.452712498170644e270;  // 2^900 (the paper's designs)
+constexpr double kCoincScaleDf = 1.2676506002282294e30;   // 2^100 (AIDW_F64 and AIDW_F64X)
 
 // Bounded waits: an mbarrier wait gives up after this many polls and raises the error word;
 // a wait on another CTA's counter gives up after kMaxWaitPolls polls of at least 256 ns
@@ -109,23 +109,16 @@ struct Plan {
 
 // Per-query parameters of phase 2 produced by the selection kernel.
 //   F32: w = ex2(fma(log2(d2), neg_s, c)), neg_s = -alpha/2, c = alpha/2 * log2(d1^2)
-//   F64: same with doubles.
+//   F64, F64X: kappa = alpha / 2 (the coincidence scale for a query on a data point) and the
+//   nearest squared distance the weights are relative to.
 struct QParamF32 {
     float neg_s;
     float c;
 };
 struct QParamF64 {
-    double neg_s;
-    double c;
-};
-
-// Per-query constants of the AIDW_F64X phase 2: kappa = alpha / 2 (the coincidence scale for a
-// query on a data point) and the nearest squared distance the weights are relative to.
-struct QParamF64X {
     double kappa;
     double d1sq;
 };
-static_assert(sizeof(QParamF64X) == sizeof(QParamF64), "shares the FP64 scratch layout");
 
 // The order FP32 phase 2 runs in when the queries are sorted into power classes (Plan::pow_a and
 // pow_b): class kClassA (power pow_a), kClassG (any power) and kClassB (pow_b), each in a region
@@ -202,8 +195,7 @@ cudaError_t launch_f64_knn(const DatasetDev &ds, const Plan &pl, const double *q
                            cudaStream_t st);
 cudaError_t launch_f64_select(const Plan &pl, int k, double r_exp, const AlphaMap &am,
                               const Scratch &sc, float *out_alpha, int32_t *out_knn,
-                              cudaStream_t st, const uint32_t *perm = nullptr,
-                              bool x_params = false);
+                              cudaStream_t st, const uint32_t *perm = nullptr);
 // Phase 1 over Z-ordered FP64 queries, pruned like launch_f32_knn_cull; with pl.with_idx the
 // lists are the k smallest (distance, caller index) pairs, so ties go to the lower index as in
 // the caller-order scan; sqx / sqy are the queries in Z-order and the dataset's points are read
@@ -221,8 +213,7 @@ cudaError_t launch_f64_weights(const DatasetDev &ds, const Plan &pl, const doubl
                                cudaStream_t st);
 cudaError_t launch_f64_finalize(const Plan &pl, const Scratch &sc, double *out,
                                 cudaStream_t st, const uint32_t *perm = nullptr);
-// AIDW_F64X phase 2 (kernels_f64x.cu); reads QParamF64X written by launch_f64_select with
-// x_params and leaves part_sum in the layout launch_f64_finalize reads.
+// AIDW_F64X phase 2 (kernels_f64x.cu); leaves part_sum in the layout launch_f64_finalize reads.
 cudaError_t launch_f64x_weights(const DatasetDev &ds, const Plan &pl, const double *qx,
                                 const double *qy, const Scratch &sc, int *err,
                                 cudaStream_t st);

@@ -106,12 +106,12 @@ __device__ __forceinline__ double fx52_to_double(long long a)
     return m == 0 ? 0.0 : __longlong_as_double(static_cast<long long>(b | s));
 }
 
-// log2(x) from the table entries of j = log2_index(x): q_j's coefficient magnitudes and
-// log2 F_j, all at 2^62. Horner in magnitudes: q(u) = A1 - u (A2 - u (A3 - u A4)), every
+// log2(x) at 2^52 (+inf and NaN as about 1,024) from the table entries of j = log2_index(x): q_j's
+// coefficient magnitudes and log2 F_j, all at 2^62. Horner in magnitudes: q(u) = A1 - u (A2 - u (A3 - u A4)), every
 // bracket positive.
-__device__ __forceinline__ double log2_finish(double x, unsigned long long a4,
-                                              unsigned long long a3, unsigned long long a2,
-                                              unsigned long long a1, unsigned long long log2f)
+__device__ __forceinline__ long long log2_fixed(double x, unsigned long long a4,
+                                                unsigned long long a3, unsigned long long a2,
+                                                unsigned long long a1, unsigned long long log2f)
 {
     const long long b = __double_as_longlong(x);
     // u: the mantissa bits below the index, exactly, at 2^73 (u 2^73 < 2^63).
@@ -123,25 +123,117 @@ __device__ __forceinline__ double log2_finish(double x, unsigned long long a4,
     const unsigned long long f = log2f + fx_mul(p, u);  // log2 F + u q(u) in [0, 1), at 2^62
     const int eb = static_cast<int>(b >> 52);
     // e + f at 2^52 (|e| <= 1074: below 2^63), f rounded to 2^-53.
-    const long long v = static_cast<long long>(eb - 1023) * (1ll << 52) +
-                        static_cast<long long>((f + (1ull << 9)) >> 10);
-    return (eb & 0x7FF) == 0x7FF ? CUDART_INF : fx52_to_double(v);  // +inf, and NaN (as +inf)
+    return static_cast<long long>(eb - 1023) * (1ll << 52) +
+           static_cast<long long>((f + (1ull << 9)) >> 10);
+}
+
+__device__ __forceinline__ bool inf_or_nan(double x)
+{
+    return (static_cast<uint32_t>(__double2hiint(x)) & 0x7FF00000u) == 0x7FF00000u;
+}
+
+// log2(x) at 2^52, x > 0 finite.
+__device__ __forceinline__ long long log2_52(double x, const Tables &t)
+{
+    const int j = log2_index(x);
+    const ulonglong2 a = t.la[j], c = t.lb[j];
+    return log2_fixed(x, a.x, a.y, c.x, c.y, t.lc[j]);
 }
 
 __device__ __forceinline__ double log2_t(double x, const Tables &t)
 {
-    const int j = log2_index(x);
-    const ulonglong2 a = t.la[j], c = t.lb[j];
-    return log2_finish(x, a.x, a.y, c.x, c.y, t.lc[j]);
+    return inf_or_nan(x) ? CUDART_INF : fx52_to_double(log2_52(x, t));  // NaN as +inf
 }
 
-// log2 with the tables read from global memory (per-query use): the same arithmetic, so the same
-// double as log2_t for every x.
-__device__ __forceinline__ double log2_c(double x)
+// 2^(k/1024 + r) for |k| < 2^21 and r at 2^73, |r| <= 2^62: T_j 2^r at 2^62 with j = k mod 1,024,
+// in (2^61.99, 2^63), and the power of two kk = floor(k / 1,024).
+__device__ __forceinline__ unsigned long long exp2_fixed(int k, long long r, const Tables &t,
+                                                         int &kk)
 {
-    const int j = log2_index(x);
-    return log2_finish(x, tab(kFxL2A4[j]), tab(kFxL2A3[j]), tab(kFxL2A2[j]), tab(kFxL2A1[j]),
-                       tab(kFxLog2F[j]));
+    const int j = k & (kExpN - 1);
+    kk = k >> kExpBits;
+    const ulonglong2 a = t.ea[j], c = t.eb[j];
+    // T_j 2^r = T_j + r (E1 + r (E2 + r E3)), in magnitudes, each product added or subtracted by
+    // the sign of r.
+    const bool rn = r < 0;
+    const unsigned long long ra = static_cast<unsigned long long>(rn ? -r : r);
+    unsigned long long q = fx_mul32(a.x, ra);  // its error is scaled by r^2 below
+    unsigned long long p = rn ? a.y - q : a.y + q;
+    q = fx_mul(p, ra);
+    p = rn ? c.x - q : c.x + q;
+    q = fx_mul(p, ra);
+    return rn ? c.y - q : c.y + q;
+}
+
+// v 2^(kk - 62) as a double, rounded once (v in (2^61.99, 2^63)), and with W96 in fixed point
+// with 96 fraction bits (truncated).
+template <bool W96>
+__device__ __forceinline__ double exp2_round(unsigned long long v, int kk, unsigned __int128 *w96)
+{
+    if (W96) {
+        // v 2^(kk - 62) 2^96 = v 2^(34 + kk).
+        const int sft = 34 + kk;
+        const unsigned __int128 w = v;
+        *w96 = sft >= 0 ? (w << (sft < 127 ? sft : 127)) : (-sft < 127 ? (w >> -sft) : 0);
+    }
+    // v has its leading one at bit 62 (lz = 1) or 61 (lz = 2).
+    const int lz = __clzll(static_cast<long long>(v));
+    const unsigned long long sig = ((v << (lz - 1)) + (1ull << 9)) >> 10;  // 53 bits, rounded
+    const unsigned long long eb = static_cast<unsigned long long>(1024 - lz + kk);
+    return __longlong_as_double(static_cast<long long>((eb << 52) + sig - (1ull << 52)));
+}
+
+// The power of Eq. 1 for one query in fixed point: s = kappa as S 2^(62 - sh - 63), sh in [0, 63],
+// and the reference logarithm l1 = log2(d1^2) at 2^52. A kappa of 2^62 and above (also the
+// coincidence scale) becomes 2^62, which gives every weight but the nearest distance's 0; below
+// 1/2 S keeps the absolute precision that y needs.
+struct FixedPower {
+    unsigned long long S;
+    long long l1;
+    int sh;
+};
+
+__device__ __forceinline__ FixedPower fixed_power(double kappa, double d1sq, const Tables &t)
+{
+    FixedPower p;
+    const long long b = __double_as_longlong(kappa);
+    int es = static_cast<int>(b >> 52) - 1023;  // kappa > 0, normal
+    p.S = (1ull << 63) | (static_cast<unsigned long long>(b & kMant) << 11);
+    if (es > 62) {
+        es = 62;
+        p.S = 1ull << 63;
+    }
+    if (es < -1) {
+        p.S = -1 - es < 64 ? p.S >> (-1 - es) : 0;
+        es = -1;
+    }
+    p.sh = 62 - es;
+    p.l1 = log2_52(d1sq, t);
+    return p;
+}
+
+// (d^2 / d1^2)^(-s) as a double and in 96-bit fixed point: y = s (log2 d^2 - log2 d1^2) at 2^53 as
+// the shifted 128-bit product, exactly 0 at the nearest distance, and 2^-y. 0 from y = 1,021 on
+// and for an infinite (a padding point's) or NaN d^2. Between the logarithm and the exponential
+// nothing is rounded to a double, packed or unpacked, and the FP64 pipe does one operation per
+// pair less than with y = fma(log2 d^2, -s, c).
+__device__ __forceinline__ double power_weight(double d2, const FixedPower &fp, const Tables &t,
+                                               unsigned __int128 *w96)
+{
+    const long long d = log2_52(d2, t) - fp.l1;
+    const bool neg = d < 0;  // by rounding only
+    const unsigned long long m = static_cast<unsigned long long>(neg ? -d : d);
+    const unsigned long long hi = __umul64hi(m, fp.S), lo = m * fp.S;
+    const unsigned long long y = (lo >> fp.sh) | ((hi << 1) << (63 - fp.sh));
+    if ((hi >> fp.sh) != 0 || y >= (1021ull << 53) || inf_or_nan(d2)) {
+        *w96 = 0;
+        return 0.0;
+    }
+    const int k = static_cast<int>((y + (1ull << 42)) >> 43);  // round(1024 y)
+    const long long r = static_cast<long long>((y - (static_cast<unsigned long long>(k) << 43)) << 20);
+    int kk;
+    const unsigned long long v = exp2_fixed(neg ? k : -k, neg ? r : -r, t, kk);
+    return exp2_round<true>(v, kk, w96);
 }
 
 // 2^y as a double; with W96, *w96 = 2^y in fixed point with 96 fraction bits (truncated; 0 when
@@ -184,31 +276,9 @@ __device__ __forceinline__ double exp2_t(double y, const Tables &t, unsigned __i
         r = -r;
         k = -k;
     }
-    const int j = static_cast<int>(k & (kExpN - 1));
-    const long long kk = k >> kExpBits;  // the power of two, floor(k / 1024)
-    const ulonglong2 a = t.ea[j], c = t.eb[j];
-    // T_j 2^r = T_j + r (E1 + r (E2 + r E3)) at 2^62, in (2^61.99, 2^63): in magnitudes, each
-    // product added or subtracted by the sign of r.
-    const bool rn = r < 0;
-    const unsigned long long ra = static_cast<unsigned long long>(rn ? -r : r);
-    unsigned long long q = fx_mul32(a.x, ra);  // its error is scaled by r^2 below
-    unsigned long long p = rn ? a.y - q : a.y + q;
-    q = fx_mul(p, ra);
-    p = rn ? c.x - q : c.x + q;
-    q = fx_mul(p, ra);
-    const unsigned long long uv = rn ? c.y - q : c.y + q;
-    const long long v = static_cast<long long>(uv);
-    if (W96) {
-        // v 2^(kk - 62) 2^96 = v 2^(34 + kk).
-        const long long sft = 34 + kk;
-        const unsigned __int128 w = uv;
-        *w96 = sft >= 0 ? (w << (sft < 127 ? sft : 127)) : (-sft < 127 ? (w >> -sft) : 0);
-    }
-    // The double: v has its leading one at bit 62 (lz = 1) or 61 (lz = 2).
-    const int lz = __clzll(v);
-    const unsigned long long sig = ((uv << (lz - 1)) + (1ull << 9)) >> 10;  // 53 bits, rounded
-    const unsigned long long eb = static_cast<unsigned long long>(1024 - lz + kk);
-    return __longlong_as_double(static_cast<long long>((eb << 52) + sig - (1ull << 52)));
+    int kk;
+    const unsigned long long v = exp2_fixed(static_cast<int>(k), r, t, kk);
+    return exp2_round<W96>(v, kk, w96);
 }
 
 }  // namespace f64math

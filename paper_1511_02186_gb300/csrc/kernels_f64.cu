@@ -667,8 +667,7 @@ __global__ void __launch_bounds__(256)
 f64_select_kernel(int64_t m, int S, int k, double r_exp, AlphaMap am,
                   const double *__restrict__ part_d2, const int32_t *__restrict__ part_idx,
                   QParamF64 *__restrict__ qp, float *__restrict__ out_alpha,
-                  int32_t *__restrict__ out_knn, const uint32_t *__restrict__ perm,
-                  bool x_params)
+                  int32_t *__restrict__ out_knn, const uint32_t *__restrict__ perm)
 {
     const int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (q >= m)
@@ -708,26 +707,12 @@ f64_select_kernel(int64_t m, int S, int k, double r_exp, AlphaMap am,
     const double alpha = alpha_eq6(mu, am);   // Eq. 6
     if (out_alpha)
         out_alpha[perm ? perm[q] : q] = static_cast<float>(alpha);
-    if (x_params) {
-        // AIDW_F64X: kappa kept within [2^-100, 2^100] (beyond, the weights are those of the
-        // bounds to far below the tolerance: all equal, or only the nearest points') and the
-        // reference squared distance.
-        QParamF64X x;
-        x.kappa = d1 == 0.0 ? kCoincScaleDf
-                            : fmax(fmin(0.5 * alpha, kCoincScaleDf), 1.0 / kCoincScaleDf);
-        x.d1sq = __dadd_rn(d1, kEpsF64);
-        reinterpret_cast<QParamF64X *>(qp)[q] = x;
-        return;
-    }
+    // kappa kept within [2^-100, 2^100] (beyond, the weights are those of the bounds to far below
+    // the tolerance: all equal, or only the nearest points').
     QParamF64 o;
-    if (d1 == 0.0) {
-        o.neg_s = -kCoincScaleF64;
-        o.c = kCoincScaleF64 * f64math::log2_c(kEpsF64);
-    } else {
-        const double sh = 0.5 * alpha;
-        o.neg_s = -sh;
-        o.c = sh * f64math::log2_c(__dadd_rn(d1, kEpsF64));
-    }
+    o.kappa = d1 == 0.0 ? kCoincScaleDf
+                        : fmax(fmin(0.5 * alpha, kCoincScaleDf), 1.0 / kCoincScaleDf);
+    o.d1sq = __dadd_rn(d1, kEpsF64);
     qp[q] = o;
 }
 
@@ -775,7 +760,14 @@ f64_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restri
     constexpr int QT = kThreadsW64 / PG;
     const int tq = tid % QT, pg = tid / QT;
 
-    double qxr[Q], qyr[Q], ns[Q], cc[Q], hz[Q], cz[Q];
+    if (tid == 0) {
+        mbar_init(&bar[0], 1);
+        mbar_init(&bar[1], 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    double qxr[Q], qyr[Q], hz[Q], cz[Q];
+    f64math::FixedPower fp[Q];
     unsigned __int128 aw[Q];
 #pragma unroll
     for (int j = 0; j < Q; ++j) {
@@ -783,17 +775,10 @@ f64_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restri
         qxr[j] = qx[q];
         qyr[j] = qy[q];
         const QParamF64 o = qp[q];
-        ns[j] = o.neg_s;
-        cc[j] = o.c;
+        fp[j] = f64math::fixed_power(o.kappa, o.d1sq, tabs);
         hz[j] = cz[j] = 0.0;
         aw[j] = 0;
     }
-    if (tid == 0) {
-        mbar_init(&bar[0], 1);
-        mbar_init(&bar[1], 1);
-        fence_mbar_init();
-    }
-    __syncthreads();
     auto load_tile = [&](int t) {
         const int b = t & 1;
         const int64_t o = p_begin + static_cast<int64_t>(t) * kTileW64;
@@ -840,8 +825,7 @@ f64_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restri
                     for (int j = 0; j < Q; ++j) {
                         const double d2 = dist2_eps(qxr[j], qyr[j], p.x, p.y);
                         unsigned __int128 w96;
-                        const double w = f64math::exp2_t<true>(
-                            __fma_rn(f64math::log2_t(d2, tabs), ns[j], cc[j]), tabs, &w96);
+                        const double w = f64math::power_weight(d2, fp[j], tabs, &w96);
                         aw[j] += w96;
                         sz[j] = __fma_rn(w, pz, sz[j]);
                     }
@@ -1033,13 +1017,13 @@ cudaError_t launch_f64_knn(const DatasetDev &ds, const Plan &pl, const double *q
 
 cudaError_t launch_f64_select(const Plan &pl, int k, double r_exp, const AlphaMap &am,
                               const Scratch &sc, float *out_alpha, int32_t *out_knn,
-                              cudaStream_t st, const uint32_t *perm, bool x_params)
+                              cudaStream_t st, const uint32_t *perm)
 {
     const int64_t blocks = (pl.m + 255) / 256;
     f64_select_kernel<<<static_cast<unsigned>(blocks), 256, 0, st>>>(
         pl.m, pl.knn.splits, k, r_exp, am, static_cast<const double *>(sc.part_d2),
         pl.with_idx ? sc.part_idx : nullptr, static_cast<QParamF64 *>(sc.qparam), out_alpha,
-        out_knn, perm, x_params);
+        out_knn, perm);
     return cudaGetLastError();
 }
 

@@ -35,7 +35,7 @@ __device__ __forceinline__ void drain_x(uint64_t *bar, int t, int ntiles)
 template <int Q, int PG>
 __global__ void __launch_bounds__(kThreads)
 f64x_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restrict__ qx,
-                    const double *__restrict__ qy, const QParamF64X *__restrict__ qp,
+                    const double *__restrict__ qy, const QParamF64 *__restrict__ qp,
                     double *__restrict__ part_sum, int *__restrict__ err)
 {
     __shared__ __align__(128) double2 txy[2][kTileF64W];
@@ -85,7 +85,7 @@ f64x_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restr
         const int64_t q = min(qbase + j * QT + tq, m - 1);
         qxr[j] = qx[q];
         qyr[j] = qy[q];
-        const QParamF64X o = qp[q];
+        const QParamF64 o = qp[q];
         kh[j] = __double2float_rn(o.kappa);
         kl[j] = __double2float_rn(o.kappa - static_cast<double>(kh[j]));
         ref[j] = dfm::ref_log(o.d1sq, tabs);
@@ -216,7 +216,7 @@ __global__ void df_weight_probe_kernel(const double *__restrict__ d2,
 namespace {
 
 using WeightsKernelX = void (*)(DatasetDev, int64_t, PassPlan, const double *, const double *,
-                                const QParamF64X *, double *, int *);
+                                const QParamF64 *, double *, int *);
 
 WeightsKernelX weightsx_kernel_for(int pg)
 {
@@ -235,7 +235,7 @@ cudaError_t launch_f64x_weights(const DatasetDev &ds, const Plan &pl, const doub
 {
     dim3 grid(pl.w.qblocks, pl.w.splits);
     weightsx_kernel_for(pl.pg)<<<grid, kThreads, 0, st>>>(
-        ds, pl.m, pl.w, qx, qy, static_cast<const QParamF64X *>(sc.qparam),
+        ds, pl.m, pl.w, qx, qy, static_cast<const QParamF64 *>(sc.qparam),
         static_cast<double *>(sc.part_sum), err);
     return cudaGetLastError();
 }
