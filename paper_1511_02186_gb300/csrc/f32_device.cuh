@@ -290,21 +290,13 @@ __device__ __forceinline__ bool knn_unit(const DatasetDev &ds, int64_t m, int64_
 // k-th distance.
 // ---------------------------------------------------------------------------------------------
 
-// Eq. 3-6 and the phase-2 parameters of one query from its k nearest squared distances d[0..k)
-// (ascending, each offset by kEpsF32): r_obs as an FP32 pairwise sum of the distances, R, mu and
-// alpha in FP64. Writes alpha to *alpha.
-__device__ __forceinline__ QParamF32 select_params(const float *d, int k, double r_exp,
-                                                   const AlphaMap &am, double *alpha_out)
+// Eq. 4-6 and the phase-2 parameters of one query from the sum of its k nearest distances (Eq. 3)
+// and its nearest squared distance (offset by kEpsF32): R, mu and alpha in FP64. Writes alpha to
+// *alpha.
+__device__ __forceinline__ QParamF32 select_power(float sum, float d1, int k, double r_exp,
+                                                  const AlphaMap &am, double *alpha_out)
 {
-    const float d1 = d[0];
-    // Eq. 3: mean of the k distances; sqrt of (d2 - eps) undoes the coincidence offset.
-    float v[AIDW_MAX_K];
-    for (int r = 0; r < k; ++r)
-        v[r] = __fsqrt_rn(__fsub_rn(d[r], kEpsF32));
-    for (int stride = 1; stride < k; stride *= 2)
-        for (int i = 0; i + stride < k; i += 2 * stride)
-            v[i] = __fadd_rn(v[i], v[i + stride]);
-    const double r_obs = static_cast<double>(v[0]) / k;
+    const double r_obs = static_cast<double>(sum) / k;
     const double R = r_obs / r_exp;           // Eq. 4
     const double mu = membership_eq5(R, am);  // Eq. 5
     const double alpha = alpha_eq6(mu, am);   // Eq. 6
@@ -322,6 +314,21 @@ __device__ __forceinline__ QParamF32 select_params(const float *d, int k, double
     }
     *alpha_out = alpha;
     return o;
+}
+
+// The same from the k nearest squared distances d[0..k) (ascending, each offset by kEpsF32): r_obs
+// is an FP32 pairwise sum of the distances.
+__device__ __forceinline__ QParamF32 select_params(const float *d, int k, double r_exp,
+                                                   const AlphaMap &am, double *alpha_out)
+{
+    // Eq. 3: mean of the k distances; sqrt of (d2 - eps) undoes the coincidence offset.
+    float v[AIDW_MAX_K];
+    for (int r = 0; r < k; ++r)
+        v[r] = __fsqrt_rn(__fsub_rn(d[r], kEpsF32));
+    for (int stride = 1; stride < k; stride *= 2)
+        for (int i = 0; i + stride < k; i += 2 * stride)
+            v[i] = __fadd_rn(v[i], v[i + stride]);
+    return select_power(v[0], d[0], k, r_exp, am, alpha_out);
 }
 
 // Selection fused into a pruned phase-1 unit (one unit holds every list of its queries, so
@@ -775,6 +782,41 @@ __device__ __forceinline__ void select_query(int64_t q, int64_t m, int S, int k,
     }
     double alpha;
     qp[q] = select_params(d, k, r_exp, am, &alpha);
+    if (out_alpha)
+        out_alpha[qo] = static_cast<float>(alpha);
+}
+
+// select_query for one split's list of k <= KP entries: the list in registers, every load and
+// square root in flight at once (the merge above keeps its lists in local memory and loads entry
+// by entry). Entries beyond k add 0 to the same pairwise sum, which changes no bit.
+template <int KP>
+__device__ __forceinline__ void select_query_one(int64_t q, int64_t m, int k, double r_exp,
+                                                 const AlphaMap &am, const float *part_d2,
+                                                 const int32_t *part_idx, QParamF32 *qp,
+                                                 float *out_alpha, int32_t *out_knn,
+                                                 const uint32_t *perm)
+{
+    const int64_t qo = perm ? static_cast<int64_t>(perm[q]) : q;  // caller's query index
+    float v[KP];
+#pragma unroll
+    for (int r = 0; r < KP; ++r)
+        v[r] = r < k ? __ldcg(part_d2 + static_cast<int64_t>(r) * m + q) : kEpsF32;
+    if (out_knn) {
+        for (int r = 0; r < k; ++r)
+            out_knn[qo * k + r] = __ldcg(part_idx + static_cast<int64_t>(r) * m + q);
+    }
+    const float d1 = v[0];
+#pragma unroll
+    for (int r = 0; r < KP; ++r)
+        v[r] = __fsqrt_rn(__fsub_rn(v[r], kEpsF32));
+#pragma unroll
+    for (int stride = 1; stride < KP; stride *= 2) {
+#pragma unroll
+        for (int i = 0; i + stride < KP; i += 2 * stride)
+            v[i] = __fadd_rn(v[i], v[i + stride]);
+    }
+    double alpha;
+    qp[q] = select_power(v[0], d1, k, r_exp, am, &alpha);
     if (out_alpha)
         out_alpha[qo] = static_cast<float>(alpha);
 }

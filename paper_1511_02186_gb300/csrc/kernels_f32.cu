@@ -56,16 +56,25 @@ __device__ __forceinline__ int power_class(const QParamF32 &p, int pow_a, int po
                                                 : kClassG;
 }
 
-__global__ void __launch_bounds__(256)
+// KP > 0: one split, k <= KP.
+template <int KP>
+__global__ void __launch_bounds__(kSelectThreads)
 f32_select_kernel(int64_t m, int S, int k, double r_exp, AlphaMap am,
                   const float *__restrict__ part_d2, const int32_t *__restrict__ part_idx,
                   QParamF32 *__restrict__ qp, float *__restrict__ out_alpha,
                   int32_t *__restrict__ out_knn, const uint32_t *__restrict__ perm,
                   const float *__restrict__ qx, const float *__restrict__ qy, ClassOrder co)
 {
+    grid_trigger();
+    grid_wait();
     const int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (q < m)
-        select_query(q, m, S, k, r_exp, am, part_d2, part_idx, qp, out_alpha, out_knn, perm);
+    if (q < m) {
+        if constexpr (KP > 0)
+            select_query_one<KP>(q, m, k, r_exp, am, part_d2, part_idx, qp, out_alpha, out_knn,
+                                 perm);
+        else
+            select_query(q, m, S, k, r_exp, am, part_d2, part_idx, qp, out_alpha, out_knn, perm);
+    }
     if (!co.cnt)
         return;
     // Each query to the next place of its class (a warp's queries stay together).
@@ -100,6 +109,8 @@ f32_knn_warp_kernel(DatasetDev ds, int64_t m, const float *__restrict__ qx,
                     const float *__restrict__ qy, int k, float *__restrict__ part_d2,
                     int32_t *__restrict__ part_idx, uint32_t *cls_cnt)
 {
+    grid_trigger();
+    grid_wait();
     zero_classes(cls_cnt);
     constexpr int W = kThreads / 32;
     __shared__ __align__(16) float bd[W][kWarpBuffer];
@@ -149,6 +160,8 @@ f32_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const float *__restric
     const int s = blockIdx.y;
     const int64_t p_begin = static_cast<int64_t>(s) * pp.split_len;
     const int64_t p_end = min(p_begin + pp.split_len, ds.n_pad);
+    grid_trigger();
+    grid_wait();
     const int64_t qbase = static_cast<int64_t>(blockIdx.x) * pp.q_per_block;
     weights_unit<Q, TW, PG>(ds, unit_queries(qx, qy, qp, m, qbase, pp.q_per_block), p_begin,
                             p_end, s, part_sum, err, txy, tz, ts);
@@ -175,6 +188,8 @@ f32_weights_class_kernel(DatasetDev ds, int64_t m, PassPlan pp, ClassOrder co,
     __shared__ __align__(128) float4 txy[2][512];
     __shared__ __align__(128) float2 tz[2][512];
     __shared__ __align__(8) uint64_t bar[2];
+    grid_trigger();
+    grid_wait();
     constexpr int kB = 2 * kThreads;
     const int order[kClasses] = {kClassG, kClassA, kClassB};
     int64_t u = blockIdx.x, col = 0;
@@ -234,6 +249,8 @@ __global__ void __launch_bounds__(256)
 f32_finalize_kernel(int64_t m, int S, const float *__restrict__ part_sum,
                     float *__restrict__ out, const uint32_t *__restrict__ perm, ClassOrder co)
 {
+    grid_trigger();
+    grid_wait();
     constexpr int C = 256 / R;
     const int col = threadIdx.x % C, r = threadIdx.x / C;
     const int64_t q = static_cast<int64_t>(blockIdx.x) * C + col;
@@ -394,12 +411,13 @@ cudaError_t launch_f32_select(const Plan &pl, int k, double r_exp, const AlphaMa
                               cudaStream_t st, const float *qx, const float *qy,
                               const uint32_t *perm)
 {
-    const int64_t blocks = (pl.m + 255) / 256;
-    f32_select_kernel<<<static_cast<unsigned>(blocks), 256, 0, st>>>(
-        pl.m, pl.knn.splits, k, r_exp, am, static_cast<const float *>(sc.part_d2),
+    const int64_t blocks = (pl.m + kSelectThreads - 1) / kSelectThreads;
+    auto fn = pl.knn.splits > 1 ? f32_select_kernel<0>
+              : k <= 16         ? f32_select_kernel<16>
+                                : f32_select_kernel<32>;
+    return launch_chained(fn, dim3(static_cast<unsigned>(blocks)), kSelectThreads, 0, st, pl.m, pl.knn.splits, k, r_exp, am, static_cast<const float *>(sc.part_d2),
         pl.with_idx ? sc.part_idx : nullptr, static_cast<QParamF32 *>(sc.qparam), out_alpha,
         out_knn, perm, qx, qy, sc.cls);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_f32_knn_warp(const DatasetDev &ds, int64_t m, const float *qx,
@@ -411,9 +429,8 @@ cudaError_t launch_f32_knn_warp(const DatasetDev &ds, int64_t m, const float *qx
     const int64_t cap = static_cast<int64_t>(sm_count) * 16;
     const unsigned grid = static_cast<unsigned>(std::max<int64_t>(1, std::min(want, cap)));
     auto fn = sc.part_idx ? f32_knn_warp_kernel<true> : f32_knn_warp_kernel<false>;
-    fn<<<grid, kThreads, 0, st>>>(ds, m, qx, qy, k, static_cast<float *>(sc.part_d2),
-                                  sc.part_idx, sc.cls.cnt);
-    return cudaGetLastError();
+    return launch_chained(fn, dim3(grid), kThreads, 0, st, ds, m, qx, qy, k,
+                          static_cast<float *>(sc.part_d2), sc.part_idx, sc.cls.cnt);
 }
 
 cudaError_t launch_f32_knn_cull(const DatasetDev &ds, const Plan &pl, const float *sqx,
@@ -448,16 +465,14 @@ cudaError_t launch_f32_weights(const DatasetDev &ds, const Plan &pl, const float
 {
     if (sc.cls.cnt) {
         const dim3 grid(pl.w.qblocks + kClasses - 1, pl.w.splits);
-        f32_weights_class_kernel<<<grid, kThreads, 0, st>>>(
-            ds, pl.m, pl.w, sc.cls, static_cast<float *>(sc.part_sum), err);
-        return cudaGetLastError();
+        return launch_chained(f32_weights_class_kernel, grid, kThreads, 0, st, ds, pl.m, pl.w,
+                              sc.cls, static_cast<float *>(sc.part_sum), err);
     }
     dim3 grid(pl.w.qblocks, pl.w.splits);
     const WeightsKernel fn = weights_kernel_for(pl.qw, pl.tw, pl.pg);
-    fn<<<grid, kThreads, 0, st>>>(ds, pl.m, pl.w, qx, qy,
-                                  static_cast<const QParamF32 *>(sc.qparam),
-                                  static_cast<float *>(sc.part_sum), err);
-    return cudaGetLastError();
+    return launch_chained(fn, grid, kThreads, 0, st, ds, pl.m, pl.w, qx, qy,
+                          static_cast<const QParamF32 *>(sc.qparam),
+                          static_cast<float *>(sc.part_sum), err);
 }
 
 cudaError_t launch_f32_finalize(const Plan &pl, const Scratch &sc, float *out, cudaStream_t st,
@@ -467,9 +482,8 @@ cudaError_t launch_f32_finalize(const Plan &pl, const Scratch &sc, float *out, c
     const unsigned blocks = static_cast<unsigned>((pl.m * R + 255) / 256);
     auto fn = R == 32 ? f32_finalize_kernel<32>
                       : (R == 8 ? f32_finalize_kernel<8> : f32_finalize_kernel<1>);
-    fn<<<blocks, 256, 0, st>>>(pl.m, pl.w.splits, static_cast<const float *>(sc.part_sum), out,
-                               perm, sc.cls);
-    return cudaGetLastError();
+    return launch_chained(fn, dim3(blocks), 256, 0, st, pl.m, pl.w.splits,
+                          static_cast<const float *>(sc.part_sum), out, perm, sc.cls);
 }
 
 }  // namespace aidw

@@ -643,6 +643,7 @@ f64_knn_warp_kernel(DatasetDev ds, int64_t m, const double *__restrict__ qx,
                     int32_t *__restrict__ part_idx)
 {
     constexpr int W = kThreads / 32;
+    grid_wait();
     __shared__ __align__(16) unsigned long long bd[W][kWarpBuffer];
     __shared__ int32_t bi[W][kWarpBuffer];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -663,15 +664,12 @@ f64_knn_warp_kernel(DatasetDev ds, int64_t m, const double *__restrict__ qx,
     }
 }
 
-__global__ void __launch_bounds__(256)
-f64_select_kernel(int64_t m, int S, int k, double r_exp, AlphaMap am,
-                  const double *__restrict__ part_d2, const int32_t *__restrict__ part_idx,
-                  QParamF64 *__restrict__ qp, float *__restrict__ out_alpha,
-                  int32_t *__restrict__ out_knn, const uint32_t *__restrict__ perm)
+// The merge of S split lists of one query: the sum of the k smallest distances in ascending order
+// (Eq. 3) and the smallest squared distance; out_knn (nullable) takes the merged indices.
+__device__ __forceinline__ void merge_lists64(int64_t q, int64_t m, int S, int k,
+                                              const double *part_d2, const int32_t *part_idx,
+                                              int32_t *out_knn, double &r_sum, double &d1)
 {
-    const int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (q >= m)
-        return;
     int cur[kMaxSplits];
     double hd[kMaxSplits];
     int32_t hi[kMaxSplits];
@@ -681,7 +679,6 @@ f64_select_kernel(int64_t m, int S, int k, double r_exp, AlphaMap am,
         hd[s] = part_d2[o];
         hi[s] = part_idx ? part_idx[o] : 0;
     }
-    double r_sum = 0.0, d1 = 0.0;
     for (int r = 0; r < k; ++r) {
         int bs = 0;
         for (int s = 1; s < S; ++s)
@@ -689,9 +686,9 @@ f64_select_kernel(int64_t m, int S, int k, double r_exp, AlphaMap am,
                 bs = s;
         if (r == 0)
             d1 = hd[bs];
-        r_sum = __dadd_rn(r_sum, __dsqrt_rn(hd[bs]));  // Eq. 3, ascending order
+        r_sum = __dadd_rn(r_sum, __dsqrt_rn(hd[bs]));
         if (out_knn)
-            out_knn[(perm ? static_cast<int64_t>(perm[q]) : q) * k + r] = hi[bs];
+            out_knn[r] = hi[bs];
         if (++cur[bs] < k) {
             const int64_t o = (static_cast<int64_t>(bs) * k + cur[bs]) * m + q;
             hd[bs] = part_d2[o];
@@ -700,6 +697,39 @@ f64_select_kernel(int64_t m, int S, int k, double r_exp, AlphaMap am,
             hd[bs] = CUDART_INF;
             hi[bs] = INT32_MAX;
         }
+    }
+}
+
+// KP > 0: one split, k <= KP, its list in registers (every load and square root in flight at once).
+template <int KP>
+__global__ void __launch_bounds__(kSelectThreads)
+f64_select_kernel(int64_t m, int S, int k, double r_exp, AlphaMap am,
+                  const double *__restrict__ part_d2, const int32_t *__restrict__ part_idx,
+                  QParamF64 *__restrict__ qp, float *__restrict__ out_alpha,
+                  int32_t *__restrict__ out_knn, const uint32_t *__restrict__ perm)
+{
+    grid_wait();
+    const int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (q >= m)
+        return;
+    int32_t *knn = out_knn ? out_knn + (perm ? static_cast<int64_t>(perm[q]) : q) * k : nullptr;
+    double r_sum = 0.0, d1 = 0.0;
+    if constexpr (KP > 0) {
+        double v[KP];
+#pragma unroll
+        for (int r = 0; r < KP; ++r)
+            v[r] = r < k ? part_d2[static_cast<int64_t>(r) * m + q] : 0.0;
+        if (knn) {
+            for (int r = 0; r < k; ++r)
+                knn[r] = part_idx[static_cast<int64_t>(r) * m + q];
+        }
+        d1 = v[0];
+#pragma unroll
+        for (int r = 0; r < KP; ++r)
+            if (r < k)
+                r_sum = __dadd_rn(r_sum, __dsqrt_rn(v[r]));  // Eq. 3, ascending order
+    } else {
+        merge_lists64(q, m, S, k, part_d2, part_idx, knn, r_sum, d1);
     }
     const double r_obs = r_sum / k;
     const double R = r_obs / r_exp;           // Eq. 4
@@ -750,7 +780,9 @@ f64_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restri
 
     const int tid = threadIdx.x;
     const int s = blockIdx.y;
+    grid_trigger();
     f64math::load_tables(tabs);  // ordered before use by the barrier after the mbarrier set-up
+    grid_wait();
     const int64_t qbase = static_cast<int64_t>(blockIdx.x) * pp.q_per_block;
     const int64_t p_begin = static_cast<int64_t>(s) * pp.split_len;
     const int64_t p_end = min(p_begin + pp.split_len, ds.n_pad);
@@ -889,6 +921,8 @@ __global__ void __launch_bounds__(256)
 f64_finalize_kernel(int64_t m, int S, const double *__restrict__ part_sum,
                     double *__restrict__ out, const uint32_t *__restrict__ perm)
 {
+    grid_trigger();
+    grid_wait();
     constexpr int C = 256 / R;
     const int col = threadIdx.x % C, r = threadIdx.x / C;
     const int64_t q = static_cast<int64_t>(blockIdx.x) * C + col;
@@ -1019,12 +1053,13 @@ cudaError_t launch_f64_select(const Plan &pl, int k, double r_exp, const AlphaMa
                               const Scratch &sc, float *out_alpha, int32_t *out_knn,
                               cudaStream_t st, const uint32_t *perm)
 {
-    const int64_t blocks = (pl.m + 255) / 256;
-    f64_select_kernel<<<static_cast<unsigned>(blocks), 256, 0, st>>>(
-        pl.m, pl.knn.splits, k, r_exp, am, static_cast<const double *>(sc.part_d2),
+    const int64_t blocks = (pl.m + kSelectThreads - 1) / kSelectThreads;
+    auto fn = pl.knn.splits > 1 ? f64_select_kernel<0>
+              : k <= 16         ? f64_select_kernel<16>
+                                : f64_select_kernel<32>;
+    return launch_chained(fn, dim3(static_cast<unsigned>(blocks)), kSelectThreads, 0, st, pl.m, pl.knn.splits, k, r_exp, am, static_cast<const double *>(sc.part_d2),
         pl.with_idx ? sc.part_idx : nullptr, static_cast<QParamF64 *>(sc.qparam), out_alpha,
         out_knn, perm);
-    return cudaGetLastError();
 }
 
 template <int KP, bool IDX>
@@ -1072,10 +1107,9 @@ cudaError_t launch_f64_knn_warp(const DatasetDev &ds, const Plan &pl, const doub
     const int64_t want = (pl.m + W - 1) / W;
     const int64_t cap = static_cast<int64_t>(sm_count) * 16;
     const unsigned grid = static_cast<unsigned>(std::max<int64_t>(1, std::min(want, cap)));
-    f64_knn_warp_kernel<<<grid, kThreads, 0, st>>>(ds, pl.m, qx, qy, k,
+    return launch_chained(f64_knn_warp_kernel, dim3(grid), kThreads, 0, st, ds, pl.m, qx, qy, k,
                                                    static_cast<double *>(sc.part_d2),
                                                    pl.with_idx ? sc.part_idx : nullptr);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_f64_weights(const DatasetDev &ds, const Plan &pl, const double *qx,
@@ -1086,10 +1120,9 @@ cudaError_t launch_f64_weights(const DatasetDev &ds, const Plan &pl, const doubl
     const cudaError_t e = weights64_kernel_for(pl.pg, &fn);
     if (e != cudaSuccess)
         return e;
-    fn<<<grid, kThreadsW64, f64math::kTablesBytes, st>>>(
+    return launch_chained(fn, grid, kThreadsW64, f64math::kTablesBytes, st, 
         ds, pl.m, pl.w, qx, qy, static_cast<const QParamF64 *>(sc.qparam),
         static_cast<double *>(sc.part_sum), err);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_f64_finalize(const Plan &pl, const Scratch &sc, double *out,
@@ -1099,9 +1132,8 @@ cudaError_t launch_f64_finalize(const Plan &pl, const Scratch &sc, double *out,
     const unsigned blocks = static_cast<unsigned>((pl.m * R + 255) / 256);
     auto fn = R == 32 ? f64_finalize_kernel<32>
                       : (R == 8 ? f64_finalize_kernel<8> : f64_finalize_kernel<1>);
-    fn<<<blocks, 256, 0, st>>>(pl.m, pl.w.splits, static_cast<const double *>(sc.part_sum), out,
-                               perm);
-    return cudaGetLastError();
+    return launch_chained(fn, dim3(blocks), 256, 0, st, pl.m, pl.w.splits,
+                          static_cast<const double *>(sc.part_sum), out, perm);
 }
 
 }  // namespace aidw

@@ -46,7 +46,9 @@ f64x_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restr
 
     const int tid = threadIdx.x;
     const int s = blockIdx.y;
+    grid_trigger();
     dfm::load_tables(tabs);  // ordered before use by the barrier after the mbarrier set-up
+    grid_wait();
     const int64_t qbase = static_cast<int64_t>(blockIdx.x) * pp.q_per_block;
     const int64_t p_begin = static_cast<int64_t>(s) * pp.split_len;
     const int64_t p_end = min(p_begin + pp.split_len, ds.n_pad);
@@ -234,10 +236,9 @@ cudaError_t launch_f64x_weights(const DatasetDev &ds, const Plan &pl, const doub
                                 const double *qy, const Scratch &sc, int *err, cudaStream_t st)
 {
     dim3 grid(pl.w.qblocks, pl.w.splits);
-    weightsx_kernel_for(pl.pg)<<<grid, kThreads, 0, st>>>(
+    return launch_chained(weightsx_kernel_for(pl.pg), grid, kThreads, 0, st, 
         ds, pl.m, pl.w, qx, qy, static_cast<const QParamF64 *>(sc.qparam),
         static_cast<double *>(sc.part_sum), err);
-    return cudaGetLastError();
 }
 
 }  // namespace aidw
