@@ -20,14 +20,13 @@ namespace {
 
 constexpr int kChunkKnn = 16;
 constexpr int kChunkW = 32;
-// FP64 phase-2 queries per thread (8,192 x 1M with 256-thread CTAs: 104.6 ms with 2, 109.0 ms
-// with 4, 161.8 ms with 8)
-constexpr int kQW64 = 2;
+constexpr int kQW64 = 1;  // FP64 phase-2 queries per thread
 constexpr int kTileW64 = 256;  // FP64 phase-2 tile (points), beside 72 KB of tables
-// FP64 phase-2 CTA: 16 warps share one copy of the tables, one CTA per SM by registers (72 a
-// thread): the integer steps of log2 / exp2 are long dependent chains that need the warps
-// (8,192 x 1M: 101.7 ms; two CTAs of 256 threads per SM 104.6 ms, one of 768 threads 109.6 ms).
-constexpr int kThreadsW64 = 512;
+// FP64 phase-2 CTA: 32 warps share one copy of the tables, one CTA per SM: the integer steps of
+// log2 / exp2 are long dependent chains that need the warps. The whole call at 8,191 x 131,072
+// (ms): 1,024 threads with 1 query each 10.6, 512 with 2 11.8, 256 with 4 11.4, 640 and 768 with 2
+// 12.2 and 11.9.
+constexpr int kThreadsW64 = 1024;
 
 __device__ __forceinline__ double dist2_exact(double qx, double qy, double px, double py)
 {
@@ -847,8 +846,7 @@ f64_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restri
                 const int cg = c + i * kChunkW + pg * (kChunkW / PG);
                 if (PG > 1 && cg >= cend)
                     break;
-                // One point at a time (the Q queries' chains interleave): 109.1 ms on 8,192 x
-                // 1M against 124.5 ms unrolled by 4 and 109.6 ms by 2.
+                // One point at a time (unrolled by 2: 10.7 against 10.6 ms at 8,191 x 131,072).
 #pragma unroll 1
                 for (int u = 0; u < kChunkW / PG; ++u) {
                     const double2 p = txy[b][cg + u];
