@@ -337,7 +337,7 @@ static int weights_point_groups(int precision, int64_t m)
 static WeightsCost weights_cost(int precision)
 {
     return precision == AIDW_F32C ? WeightsCost{0.048, 150.0, 0.006, true}
-           : precision == AIDW_F64 ? WeightsCost{1.75, 6000.0, 0.05, false}
+           : precision == AIDW_F64 ? WeightsCost{1.5, 5000.0, 0.05, false}
                                    : WeightsCost{1.1, 500.0, 0.05, true};
 }
 
@@ -353,11 +353,15 @@ static WeightsCost weights_cost(int precision)
 static bool use_power_classes(int64_t n, int64_t m, float z_max)
 {
     return m >= 4096 && static_cast<double>(n) * static_cast<double>(m) >= 2e8 &&
-           static_cast<double>(n) * z_max <= 0x1p62;
+           power_classes_fit(n, z_max);
 }
 
-// The level as an integer power the class loops are built for, or 0.
-static int integer_level(double a)
+bool power_classes_fit(int64_t n, float z_max)
+{
+    return static_cast<double>(n) * z_max <= 0x1p62;
+}
+
+int integer_level(double a)
 {
     return a >= 1.0 && a <= 5.0 && a == std::floor(a) ? static_cast<int>(a) : 0;
 }

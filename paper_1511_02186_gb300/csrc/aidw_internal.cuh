@@ -56,6 +56,8 @@ inline int finalize_threads(int splits, int64_t m)
 }
 // Largest |log2 of d1^power| of a query in an integer power class.
 constexpr float kClassMaxLog2 = 64.0f;
+// Fewest queries of a batch item whose phase 2 runs by power classes.
+constexpr int64_t kBatchClassMinQueries = 4096;
 constexpr int kPointGroups = 4;  // phase 2 with point groups (Plan::pg)
 
 // Levels and bounds of Eq. 5 and Eq. 6, passed to kernels by value.
@@ -143,6 +145,10 @@ struct Scratch {
     ClassOrder cls;    // cnt null: no power classes
 };
 
+// Whether the unscaled sums of the integer power classes stay in range for a dataset, and a level
+// of Eq. 6 as an integer power the class loops are built for (0: none).
+bool power_classes_fit(int64_t n, float z_max);
+int integer_level(double a);
 size_t scratch_bytes(int precision, const Plan &pl, int k);
 void scratch_carve(void *base, int precision, const Plan &pl, int k, Scratch *s);
 

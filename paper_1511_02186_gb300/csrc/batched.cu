@@ -5,17 +5,18 @@
 // the batch), so an item's result is bit-identical whether it runs alone or in any mix:
 //   phase-1 list
 //     KNN     (item, query block)         pruned phase-1 scan of Z-ordered queries (nearest
-//                                         data tiles first) with the selection (Eq. 3-6)
-//                                         fused: the block's phase-2 parameters are ready
-//             (item, query block, split)  split scan for items too large to prune or with
-//                                         few queries
-//     SELECT  (item, query block)         merge of a split-scan block's lists + Eq. 3-6; waits
-//                                         for the block's KNN units (earlier in the list)
+//                                         data tiles first), or, for an item with few queries
+//                                         or too many data tiles, 16 queries scanned one per
+//                                         warp; with the selection (Eq. 3-6) fused: the
+//                                         block's phase-2 parameters are ready
 //   phase-2 list
 //     WEIGHTS (item, query block, split)  phase-2 scan of one data split; needs every query
 //                                         block of its item through selection
 //     FINAL   (item, query block)         split merge + Eq. 1 ratio; waits for the block's
 //                                         WEIGHTS units (earlier in the list)
+// An item with enough queries runs phase 2 by power classes, as aidw_interpolate does: its KNN
+// units sort the queries into those whose power is the integer alpha_5 and the others, and a
+// WEIGHTS or FINAL unit finds its block in the two from their final counts.
 // Before the persistent kernel, the queries of all items are put in Z-order item by item (one
 // radix sort of keys made of the item's index and the query's Morton cell in its dataset's
 // box) so that each KNN unit's block is compact; results go back to the caller's order.
@@ -38,15 +39,10 @@ namespace {
 
 using namespace f32dev;
 
-enum UnitType : int32_t { kUnitKnn = 0, kUnitSelect = 1, kUnitWeights = 2, kUnitFinal = 3 };
+enum UnitType : int32_t { kUnitKnn = 0, kUnitWeights = 1, kUnitFinal = 2 };
 
-// Queries per thread of the batch's split-scan phase-1 units (every list length).
-constexpr int kBatchSplitQ = 2;
-
-// Data-split length of the batched phase-1 plan (points) for datasets too large to prune; a
-// phase-1 split restarts the neighbour lists, so these splits are long. The phase-2 split
-// length is a tuning field (aidw_tune_config.split_points).
-constexpr int64_t kBatchKnnSplit = 262144;
+// Queries of a phase-1 unit that scans one query per warp.
+constexpr int kBatchWarpBlock = 16;
 
 struct BatchItemDev {
     DatasetDev ds;
@@ -63,10 +59,10 @@ struct BatchItemDev {
     const float *sqx, *sqy;  // the item's queries in Z-order
     const uint32_t *perm;    // Z-order position -> caller's query index
     int64_t qoff;            // offset of the item in the batch-wide query arrays
-    int32_t ntiles, ntiles_p2;
-    uint32_t *cnt_knn;   // [knn.qblocks] finished split-scan phase-1 units per query block
-    uint32_t *cnt_ready; // [1] query blocks through selection (pruned KNN or SELECT units)
-    uint32_t *cnt_w;     // [w.qblocks] finished phase-2 splits per query block
+    int32_t ntiles, ntiles_p2;  // ntiles_p2 0: one query per warp
+    ClassOrder co;       // two power classes in one region of m entries, or cnt null
+    uint32_t *cnt_ready; // [1] query blocks through selection
+    uint32_t *cnt_w;     // [weight blocks] finished phase-2 splits per block
 };
 
 struct WorkUnit {
@@ -113,6 +109,42 @@ __device__ __noinline__ bool batch_weights_unit(const BatchItemDev *itp, int qbl
                                 reinterpret_cast<float2(*)[TW]>(&g_tz[0][0]), ts);
 }
 
+// The class form (2 queries per thread, 512-point tiles, whatever the shape): block qblock of the
+// item's general class, then of class A. Which queries a block holds depends on the order in which
+// the KNN units counted them in, a query's own sums do not.
+struct ClassBlock {
+    int cls;      // -1: no such block
+    int64_t base, n, col0;
+    int dir;
+};
+
+__device__ __forceinline__ ClassBlock class_block(const BatchItemDev &it, int qblock)
+{
+    constexpr int64_t kB = 2 * kThreads;
+    const int64_t ng = __ldcg(it.co.cnt + kClassG), na = __ldcg(it.co.cnt + kClassA);
+    int64_t u = qblock;
+    if (u * kB < ng)
+        return {kClassG, it.m - 1 - u * kB, min(kB, ng - u * kB), u * kB, -1};
+    u -= (ng + kB - 1) / kB;
+    if (u * kB < na)
+        return {kClassA, u * kB, min(kB, na - u * kB), ng + u * kB, 1};
+    return {-1, 0, 0, 0, 1};
+}
+
+template <int POW>
+__device__ __noinline__ bool batch_class_unit(const BatchItemDev *itp, int qblock, int split,
+                                              int *err, uint32_t seq)
+{
+    const BatchItemDev &it = *itp;
+    const ClassBlock cb = class_block(it, qblock);
+    const int64_t p0 = static_cast<int64_t>(split) * it.w.split_len;
+    const int64_t p1 = min(p0 + it.w.split_len, it.ds.n_pad);
+    TileSeq ts{g_bar, seq};
+    const UnitQueries uq{it.co.qx, it.co.qy, it.co.qp, cb.base, cb.n, cb.col0, it.m, cb.dir};
+    return weights_unit<2, kTileF32W, 1, POW>(it.ds, uq, p0, p1, split, it.part_sum, err, g_txy,
+                                              g_tz, ts);
+}
+
 // Largest tile count whose pruned-scan tile order (8 bytes a tile) fits in g_tz.
 constexpr int kOrderInTz = static_cast<int>(sizeof(g_tz) / sizeof(unsigned long long));
 
@@ -155,6 +187,7 @@ f32_batch_kernel(const BatchItemDev *__restrict__ items, const WorkUnit *__restr
     unsigned long long *order =
         dyn_order_in_tz ? reinterpret_cast<unsigned long long *>(&g_tz[0][0]) : dyn_order;
     __shared__ CullShared cs;
+    __shared__ __align__(16) float s_buf[kThreads / 32][kWarpBuffer];
     // Phase-1 and phase-2 units take turns on the same coordinate tile buffers.
     static_assert(kTileF32Knn == kTileF32W, "shared tile buffers");
     float4(*ktile)[kTileF32Knn] = g_txy;
@@ -248,35 +281,32 @@ f32_batch_kernel(const BatchItemDev *__restrict__ items, const WorkUnit *__restr
         if (!ok) {
             // fall through to the error exit below
         } else if (wu.type == kUnitKnn && it.ntiles_p2 == 0) {
-            // Dataset too large for the shared-memory tile order: split scan.
-            const int64_t qbase = static_cast<int64_t>(wu.qblock) * it.knn.q_per_block;
-            const int64_t p0 = static_cast<int64_t>(wu.split) * it.knn.split_len;
-            const int64_t p1 = min(p0 + it.knn.split_len, it.ds.n_pad);
-#define AIDW_SPLIT_UNIT(KP)                                                                    \
-    ok = knn_unit<KP, kBatchSplitQ, false>(it.ds, it.m, qbase, p0, p1, it.sqx, it.sqy, it.k,     \
-                                           wu.split, it.part_d2, nullptr, err, ktile, ts, nullptr)
-            switch (it.kp) {
-            case 8:
-                AIDW_SPLIT_UNIT(8);
-                break;
-            case 12:
-                AIDW_SPLIT_UNIT(12);
-                break;
-            case 16:
-                AIDW_SPLIT_UNIT(16);
-                break;
-            default:
-                if constexpr (!LEAN)
-                    AIDW_SPLIT_UNIT(32);
-                break;
+            // One query per warp, then Eq. 3-6 with one query per thread.
+            constexpr int KP = LEAN ? 16 : AIDW_MAX_K;
+            const int64_t qbase = static_cast<int64_t>(wu.qblock) * kBatchWarpBlock;
+            const int64_t qend = min(qbase + kBatchWarpBlock, it.m);
+            const int lane = tid & 31, warp = tid >> 5;
+            for (int64_t q = qbase + warp; q < qend; q += kThreads / 32) {
+                const WarpEntry e = warp_knn<false>(it.ds, it.sqx[q], it.sqy[q], it.k, s_buf[warp],
+                                                    nullptr);
+                if (lane < it.k)
+                    it.part_d2[static_cast<int64_t>(lane) * it.m + q] = e.d;
             }
-#undef AIDW_SPLIT_UNIT
-            if (ok)
-                cta_publish(&it.cnt_knn[wu.qblock]);
+            __syncthreads();
+            const int64_t q = qbase + tid;
+            if (q < qend) {
+                double alpha;
+                const QParamF32 p = select_list<KP>(q, it.m, it.k, it.r_exp, it.am, it.part_d2,
+                                                    &alpha);
+                const FusedSelect fsel{it.r_exp, it.am, it.qparam, it.out_alpha, it.perm, it.co,
+                                       it.m};
+                fused_select_store(p, alpha, fsel, q, it.sqx[q], it.sqy[q]);
+            }
+            cta_publish(it.cnt_ready);
         } else if (wu.type == kUnitKnn) {
             // Pruned scan with the selection fused: the query block is complete afterwards.
             const int64_t qbase = static_cast<int64_t>(wu.qblock) * it.knn.q_per_block;
-            const FusedSelect fsel{it.r_exp, it.am, it.qparam, it.out_alpha, it.perm};
+            const FusedSelect fsel{it.r_exp, it.am, it.qparam, it.out_alpha, it.perm, it.co, it.m};
 #define AIDW_CULL_UNIT(KP, Q)                                                                  \
     ok = knn_cull_unit<KP, Q, false>(it.ds, it.m, qbase, it.ntiles, it.ntiles_p2, it.sqx, it.sqy, \
                                      it.k, it.part_d2, nullptr, err, ktile, ts, order, nullptr,  \
@@ -309,20 +339,38 @@ f32_batch_kernel(const BatchItemDev *__restrict__ items, const WorkUnit *__restr
 #undef AIDW_CULL_UNIT
             if (ok)
                 cta_publish(it.cnt_ready);
-        } else if (wu.type == kUnitSelect) {
-            ok = cta_wait_count(&it.cnt_knn[wu.qblock], it.knn.splits, &s_flag);
-            if (ok) {
-                const int64_t qbase = static_cast<int64_t>(wu.qblock) * it.knn.q_per_block;
-                const int64_t qend = min(qbase + it.knn.q_per_block, it.m);
-                for (int64_t q = qbase + tid; q < qend; q += kThreads)
-                    select_query(q, it.m, it.knn.splits, it.k, it.r_exp, it.am, it.part_d2,
-                                 nullptr, it.qparam, it.out_alpha, nullptr, it.perm);
-                cta_publish(it.cnt_ready);
-            }
         } else if (wu.type == kUnitWeights) {
             const int64_t p0 = static_cast<int64_t>(wu.split) * it.w.split_len;
             const int64_t p1 = min(p0 + it.w.split_len, it.ds.n_pad);
-            if (tw == 256) {
+            if (it.co.cnt) {
+                const int cls = class_block(it, wu.qblock).cls;
+                if (cls >= 0) {
+                    const int pow = cls == kClassA ? it.co.pow_a : 0;
+#define AIDW_CLASS_UNIT(POW) ok = batch_class_unit<POW>(&it, wu.qblock, wu.split, err, ts.seq)
+                    switch (pow) {
+                    case 1:
+                        AIDW_CLASS_UNIT(1);
+                        break;
+                    case 2:
+                        AIDW_CLASS_UNIT(2);
+                        break;
+                    case 3:
+                        AIDW_CLASS_UNIT(3);
+                        break;
+                    case 4:
+                        AIDW_CLASS_UNIT(4);
+                        break;
+                    case 5:
+                        AIDW_CLASS_UNIT(5);
+                        break;
+                    default:
+                        AIDW_CLASS_UNIT(0);
+                        break;
+                    }
+#undef AIDW_CLASS_UNIT
+                    ts.seq += static_cast<uint32_t>(weights_tiles<kTileF32W>(it.ds, p0, p1));
+                }
+            } else if (tw == 256) {
                 ok = batch_weights_unit<QW, 256>(&it, wu.qblock, wu.split, err, ts.seq);
                 ts.seq += static_cast<uint32_t>(weights_tiles<256>(it.ds, p0, p1));
             } else {
@@ -331,6 +379,11 @@ f32_batch_kernel(const BatchItemDev *__restrict__ items, const WorkUnit *__restr
             }
             if (ok)
                 cta_publish(&it.cnt_w[wu.qblock]);
+        } else if (it.co.cnt) {
+            const ClassBlock cb = class_block(it, wu.qblock);
+            for (int64_t i = tid; i < cb.n; i += kThreads)
+                it.out[__ldcg(it.co.id + cb.base + cb.dir * i)] =
+                    finalize_query(cb.col0 + i, it.m, it.w.splits, it.part_sum);
         } else {
             const int64_t qbase = static_cast<int64_t>(wu.qblock) * it.w.q_per_block;
             const int64_t qend = min(qbase + it.w.q_per_block, it.m);
@@ -432,17 +485,25 @@ int batch_grid(int sm_count, size_t dyn, int qw, bool lean, int ctas_per_sm, int
 
 }  // namespace
 
+// Whether phase-1 lists [k][m] fit the memory of the partial sums [S][4][m], which are written
+// only after the item's last list is read.
+bool lists_in_sums(int k, const PassPlan &pw)
+{
+    return k <= 4 * pw.splits;
+}
+
 // Phase-1 plan of a batch item: one pruned unit per query block when the dataset's tile order
-// fits in shared memory and the item has enough queries, else split scans. A pruned unit visits
-// the tiles near its block's queries; with few queries spread over the data that is most of
-// the tiles, scanned by one CTA (m = 256 against 800,000 points: 19 ms as one pruned unit, 5 ms
-// as split scans), so an item with fewer than kBatchCullMinQueries queries scans instead, its
-// data cut into enough splits for about kBatchKnnUnits units in all. Above that the pruned
-// units do several times less work than a scan of every pair, which a batch's throughput
-// needs (the 256-dataset batch: 80.5 ms with the pruned units from 1,024 queries on, 83.5 ms
-// from 4,096 on).
-constexpr int64_t kBatchCullMinQueries = 1024;
-constexpr int64_t kBatchKnnUnits = 128;
+// fits in shared memory and the item has enough queries, else units of kBatchWarpBlock queries
+// scanned one per warp. A pruned unit visits the tiles near its block's queries, on one CTA; with
+// queries sparse in the data that is a large part of the tiles (256 queries against 800,000
+// points: 19 ms as one pruned unit, 45 us one per warp), and the item's phase 2 waits for it.
+// Where the queries are dense the block shares the tiles it visits and needs fewer SM cycles.
+// Measured (64 uneven datasets in one launch / a burst of 24 served requests against up to 1M
+// points, ms): pruned from 1,024 queries on 10.39 / 31.9, from 8,192 on 10.36 / 25.0, from 32,768
+// on 10.75 / 21.8; from 8,192 on but one per warp from 131,072 points on 10.34 / 22.0.
+constexpr int64_t kBatchWarpMinPoints = 131072;
+constexpr int64_t kBatchWarpMaxQueries = 131072;
+constexpr int64_t kBatchCullMinQueries = 8192;
 
 // Phase-2 plan of a batch item: data splits of at most split_points points, and, for an item
 // with few queries, enough of them for about kBatchMinWeightUnits units of 256 queries, so
@@ -462,44 +523,57 @@ PassPlan batch_w_plan(int64_t m, int64_t n_pad, int qpb, int64_t split_points)
     return batch_pass(m, n_pad, qpb, std::min<int64_t>(split_points, target));
 }
 
-PassPlan batch_knn_plan(int64_t m, int64_t n_pad, int kp, int kq, bool *cull)
+PassPlan batch_knn_plan(int64_t m, int64_t n_pad, int k, int kq, const PassPlan &pw, bool *cull)
 {
-    *cull = n_pad / kTileF32Knn <= kMaxCullTiles && m >= kBatchCullMinQueries;
-    const int qk = kThreads * (*cull ? kq : kBatchSplitQ);
-    if (*cull)
-        return batch_pass(m, n_pad, qk, n_pad);
-    const int64_t qblocks = std::max<int64_t>(1, (m + qk - 1) / qk);
-    const int64_t splits = std::max<int64_t>(1, kBatchKnnUnits / qblocks);
-    const int64_t target = std::max<int64_t>(kPadPoints, (n_pad + splits - 1) / splits);
-    return batch_pass(m, n_pad, qk, std::min<int64_t>(target, kBatchKnnSplit));
+    *cull = n_pad / kTileF32Knn <= kMaxCullTiles &&
+            ((m >= kBatchCullMinQueries &&
+              (n_pad < kBatchWarpMinPoints || m > kBatchWarpMaxQueries)) ||
+             (m >= 1024 && !lists_in_sums(k, pw)));
+    return batch_pass(m, n_pad, *cull ? kThreads * kq : kBatchWarpBlock, n_pad);
 }
 
-// Phase-1 scratch of an item: split lists [S][k][m] for split-scan items; pruned items select
-// inside their KNN units and keep no lists.
-size_t batch_lists_bytes(const PassPlan &pk, bool cull, int k, int64_t m)
+// Whether an item runs phase 2 by power classes, and the integer power of its class A (0: no).
+int batch_class_power(int64_t m, const DatasetDev &ds, const aidw_params &p)
 {
-    return cull ? 0
-                : align256(pk.splits * static_cast<size_t>(k) * static_cast<size_t>(m) *
-                           sizeof(float));
+    if (m < kBatchClassMinQueries || !power_classes_fit(ds.n, ds.z_max))
+        return 0;
+    const int a = integer_level(p.alpha[4]);
+    return a ? a : integer_level(p.alpha[0]);
+}
+
+// Phase-1 scratch of an item of its own: the lists [k][m] of one-query-per-warp units where they
+// do not fit the partial sums' memory; pruned units select from their registers.
+size_t batch_lists_bytes(bool cull, int k, const PassPlan &pw, int64_t m)
+{
+    return cull || lists_in_sums(k, pw)
+               ? 0
+               : align256(static_cast<size_t>(k) * static_cast<size_t>(m) * sizeof(float));
 }
 
 size_t batch_item_bytes(int64_t n_pad, int64_t m, int k, const aidw_tune_config &cfg)
 {
     bool cull;
     const int kp = kp_for(k, cfg.knn_list);
-    const PassPlan pk = batch_knn_plan(m, n_pad, kp, cull_queries_per_thread(kp,
-                                       cfg.knn_queries_per_thread), &cull);
     const PassPlan pw = batch_w_plan(m, n_pad, kThreads * cfg.queries_per_thread,
                                      cfg.split_points);
+    const PassPlan pk = batch_knn_plan(m, n_pad, k, cull_queries_per_thread(kp,
+                                       cfg.knn_queries_per_thread), pw, &cull);
     const size_t mm = static_cast<size_t>(m);
-    return batch_lists_bytes(pk, cull, k, m) + align256(mm * sizeof(QParamF32)) +
+    return batch_lists_bytes(cull, k, pw, m) + align256(mm * sizeof(QParamF32)) +
            align256(pw.splits * 4 * mm * sizeof(float)) +
-           sizeof(uint32_t) * (pk.qblocks + 1 + pw.qblocks) + sizeof(BatchItemDev) +
-           sizeof(WorkUnit) * (pk.qblocks * (pk.splits + 1) + pw.qblocks * (pw.splits + 1)) +
+           sizeof(uint32_t) * (kClasses + 1 + pw.qblocks + 1) + sizeof(BatchItemDev) +
+           sizeof(WorkUnit) * (pk.qblocks + (pw.qblocks + 1) * (pw.splits + 1)) +
            mm * (6 * sizeof(uint32_t)) + radix_scratch_bytes(m);
 }
 
 // Validates the items and builds the device tables of a batch in library memory.
+// Blocks of queries an item's phase 2 may have: one more than q_per_block gives when its two
+// power classes each end in a partly filled one.
+static int weight_blocks(const BatchItemDev &d)
+{
+    return d.w.qblocks + (d.co.pow_a ? 1 : 0);
+}
+
 int batch_build(aidw_ctx *ctx, const aidw_batch_item *items, int32_t count, cudaStream_t st,
                 BatchState *bs, const aidw_tune_config &cfg, int reserve_ctas_per_sm)
 {
@@ -545,10 +619,12 @@ int batch_build(aidw_ctx *ctx, const aidw_batch_item *items, int32_t count, cuda
         d.r_exp = r_exp;
         d.am = alpha_map(b.params);
         bool cull;
-        d.knn = batch_knn_plan(b.m, dev.n_pad, d.kp, d.kq, &cull);
+        d.co.pow_a = batch_class_power(b.m, dev, b.params);
+        d.w = batch_w_plan(b.m, dev.n_pad,
+                           kThreads * (d.co.pow_a ? 2 : cfg.queries_per_thread), cfg.split_points);
+        d.knn = batch_knn_plan(b.m, dev.n_pad, d.k, d.kq, d.w, &cull);
         if (b.m > 0 && (d.kp > 16 || (cull && d.kq != 2)))
             lean = false;
-        d.w = batch_w_plan(b.m, dev.n_pad, kThreads * cfg.queries_per_thread, cfg.split_points);
         d.ntiles = static_cast<int32_t>(dev.n_pad / kTileF32Knn);
         int p2 = 1;
         while (p2 < d.ntiles)
@@ -561,14 +637,13 @@ int batch_build(aidw_ctx *ctx, const aidw_batch_item *items, int32_t count, cuda
         max_m = std::max<int64_t>(max_m, b.m);
         const size_t m = static_cast<size_t>(b.m);
         scratch_off[i] = scratch_total;
-        scratch_total += batch_lists_bytes(d.knn, cull, d.k, b.m) +
+        scratch_total += batch_lists_bytes(cull, d.k, d.w, b.m) +
                          align256(m * sizeof(QParamF32)) +
                          align256(d.w.splits * 4 * m * sizeof(float));
         cnt_off[i] = cnt_total;
-        cnt_total += sizeof(uint32_t) * (d.knn.qblocks + 1 + d.w.qblocks);
+        cnt_total += sizeof(uint32_t) * (kClasses + 1 + weight_blocks(d));
     }
-    // Two work lists, items in decreasing size in both: phase 1 (the KNN units of an item, and
-    // for a split-scan item the SELECT unit of each query block after them) and phase 2 (all
+    // Two work lists, items in decreasing size in both: phase 1 (KNN units) and phase 2 (all
     // WEIGHTS units, then all FINAL units: a FINAL unit waits for its block's WEIGHTS units,
     // which are all taken before it).
     std::vector<int32_t> order(count);
@@ -580,19 +655,15 @@ int batch_build(aidw_ctx *ctx, const aidw_batch_item *items, int32_t count, cuda
     std::vector<WorkUnit> u;
     for (int32_t i : order) {
         for (int qb = 0; qb < h[i].knn.qblocks; ++qb)
-            for (int sp = 0; sp < h[i].knn.splits; ++sp)
-                u.push_back({i, qb, sp, kUnitKnn});
-        if (h[i].ntiles_p2 == 0)
-            for (int qb = 0; qb < h[i].knn.qblocks; ++qb)
-                u.push_back({i, qb, 0, kUnitSelect});
+            u.push_back({i, qb, 0, kUnitKnn});
     }
     const size_t n1 = u.size();
     for (int32_t i : order)
-        for (int qb = 0; qb < h[i].w.qblocks; ++qb)
+        for (int qb = 0; qb < weight_blocks(h[i]); ++qb)
             for (int sp = 0; sp < h[i].w.splits; ++sp)
                 u.push_back({i, qb, sp, kUnitWeights});
     for (int32_t i : order)
-        for (int qb = 0; qb < h[i].w.qblocks; ++qb)
+        for (int qb = 0; qb < weight_blocks(h[i]); ++qb)
             u.push_back({i, qb, 0, kUnitFinal});
 
     const size_t tq = static_cast<size_t>(std::max<int64_t>(total_q, 1));
@@ -624,18 +695,27 @@ int batch_build(aidw_ctx *ctx, const aidw_batch_item *items, int32_t count, cuda
         const size_t m = static_cast<size_t>(d.m);
         char *p = scratch + scratch_off[i];
         d.part_d2 = reinterpret_cast<float *>(p);
-        p += batch_lists_bytes(d.knn, d.ntiles_p2 != 0, d.k, d.m);
+        p += batch_lists_bytes(d.ntiles_p2 != 0, d.k, d.w, d.m);
         d.qparam = reinterpret_cast<QParamF32 *>(p);
         p += align256(m * sizeof(QParamF32));
         d.part_sum = reinterpret_cast<float *>(p);
+        if (lists_in_sums(d.k, d.w))
+            d.part_d2 = d.part_sum;
         d.sqx = bs->sqx + d.qoff;
         d.sqy = bs->sqy + d.qoff;
         d.perm = bs->perm + d.qoff;
         uint32_t *c = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(bs->d_counters) +
                                                    cnt_off[i]);
-        d.cnt_knn = c;
-        d.cnt_ready = c + d.knn.qblocks;
-        d.cnt_w = c + d.knn.qblocks + 1;
+        if (d.co.pow_a) {
+            // The ordering's keys, values and item numbers are free once the queries are gathered.
+            d.co.cnt = c;
+            d.co.qx = reinterpret_cast<float *>(bs->vals + d.qoff);
+            d.co.qy = reinterpret_cast<float *>(bs->item_of + d.qoff);
+            d.co.id = bs->keys + d.qoff;
+            d.co.qp = d.qparam;
+        }
+        d.cnt_ready = c + kClasses;
+        d.cnt_w = c + kClasses + 1;
     }
     for (size_t j = n1; j < u.size(); ++j) {
         WorkUnit &w = u[j];

@@ -331,26 +331,72 @@ __device__ __forceinline__ QParamF32 select_params(const float *d, int k, double
     return select_power(v[0], d[0], k, r_exp, am, alpha_out);
 }
 
-// Selection fused into a pruned phase-1 unit (one unit holds every list of its queries, so
-// no merge is needed): Eq. 3-6 straight from the register lists, the phase-2 parameters to
-// qparam[q] and alpha to out_alpha[perm[q]] (nullable); the lists themselves are not stored.
+// A query's power class. Integer powers take the class loop where 2^c = d1^power (and with it
+// every unscaled weight d^-power) stays within 2^+-kClassMaxLog2.
+__device__ __forceinline__ int power_class(const QParamF32 &p, int pow_a, int pow_b)
+{
+    if (!(fabsf(p.c) <= kClassMaxLog2))
+        return kClassG;  // also NaN, and a query on a data point
+    const float twice = -2.0f * p.neg_s;
+    return twice == static_cast<float>(pow_a)   ? kClassA
+           : twice == static_cast<float>(pow_b) ? kClassB
+                                                : kClassG;
+}
+
+// The next place of class cls, counted in cnt: the threads here together take consecutive ones.
+__device__ __forceinline__ uint32_t class_place(uint32_t *cnt, int cls)
+{
+    const unsigned same = __match_any_sync(__activemask(), cls);
+    const int lane = threadIdx.x & 31, leader = __ffs(same) - 1;
+    uint32_t at = 0;
+    if (lane == leader)
+        at = atomicAdd(&cnt[cls], static_cast<uint32_t>(__popc(same)));
+    return __shfl_sync(same, at, leader) + __popc(same & ((1u << lane) - 1u));
+}
+
+// Selection fused into a phase-1 unit of a batch: Eq. 3-6 of a block's queries, alpha to
+// out_alpha[perm[q]] (nullable) and the phase-2 parameters to qparam[q], or, with two power classes
+// (co.cnt), the query and its parameters to the next place of its class: class A upwards from the
+// start of the item's m entries, the general class downwards from their end.
 struct FusedSelect {
     double r_exp;
     AlphaMap am;
     QParamF32 *qparam;
     float *out_alpha;
     const uint32_t *perm;  // Z-order position -> caller's query index
+    ClassOrder co;
+    int64_t m;
 };
+
+__device__ __forceinline__ void fused_select_store(const QParamF32 &p, double alpha,
+                                                   const FusedSelect &fs, int64_t q, float x,
+                                                   float y)
+{
+    const uint32_t qo = fs.perm[q];
+    if (fs.out_alpha)
+        fs.out_alpha[qo] = static_cast<float>(alpha);
+    if (!fs.co.cnt) {
+        fs.qparam[q] = p;
+        return;
+    }
+    const int cls = power_class(p, fs.co.pow_a, 0);
+    const int64_t at = class_place(fs.co.cnt, cls);
+    const int64_t o = cls == kClassA ? at : fs.m - 1 - at;
+    fs.co.qx[o] = x;
+    fs.co.qy[o] = y;
+    fs.co.qp[o] = p;
+    fs.co.id[o] = qo;
+}
 
 // One query of a fused selection (kept out of line: it runs once per query, and inlined into
 // the scan it would lengthen the scan's register life ranges).
 static __device__ __noinline__ void fused_select_query(const float *d, int k,
-                                                       const FusedSelect *fs, int64_t q)
+                                                       const FusedSelect *fs, int64_t q, float x,
+                                                       float y)
 {
     double alpha;
-    fs->qparam[q] = select_params(d, k, fs->r_exp, fs->am, &alpha);
-    if (fs->out_alpha)
-        fs->out_alpha[fs->perm[q]] = static_cast<float>(alpha);
+    const QParamF32 p = select_params(d, k, fs->r_exp, fs->am, &alpha);
+    fused_select_store(p, alpha, *fs, q, x, y);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -715,7 +761,7 @@ __device__ __forceinline__ bool knn_cull_unit(const DatasetDev &ds, int64_t m, i
             const int64_t q = wbase + j * 32;
             if (q >= m)
                 continue;
-            fused_select_query(d[j], k, fsel, q);
+            fused_select_query(d[j], k, fsel, q, sqx[q], sqy[q]);
         }
         return true;
     }
@@ -786,25 +832,18 @@ __device__ __forceinline__ void select_query(int64_t q, int64_t m, int S, int k,
         out_alpha[qo] = static_cast<float>(alpha);
 }
 
-// select_query for one split's list of k <= KP entries: the list in registers, every load and
-// square root in flight at once (the merge above keeps its lists in local memory and loads entry
-// by entry). Entries beyond k add 0 to the same pairwise sum, which changes no bit.
+// Eq. 3-6 from one split's list of k <= KP entries: the list in registers, every load and square
+// root in flight at once (the merge above keeps its lists in local memory and loads entry by
+// entry). Entries beyond k add 0 to the same pairwise sum, which changes no bit.
 template <int KP>
-__device__ __forceinline__ void select_query_one(int64_t q, int64_t m, int k, double r_exp,
+__device__ __forceinline__ QParamF32 select_list(int64_t q, int64_t m, int k, double r_exp,
                                                  const AlphaMap &am, const float *part_d2,
-                                                 const int32_t *part_idx, QParamF32 *qp,
-                                                 float *out_alpha, int32_t *out_knn,
-                                                 const uint32_t *perm)
+                                                 double *alpha)
 {
-    const int64_t qo = perm ? static_cast<int64_t>(perm[q]) : q;  // caller's query index
     float v[KP];
 #pragma unroll
     for (int r = 0; r < KP; ++r)
         v[r] = r < k ? __ldcg(part_d2 + static_cast<int64_t>(r) * m + q) : kEpsF32;
-    if (out_knn) {
-        for (int r = 0; r < k; ++r)
-            out_knn[qo * k + r] = __ldcg(part_idx + static_cast<int64_t>(r) * m + q);
-    }
     const float d1 = v[0];
 #pragma unroll
     for (int r = 0; r < KP; ++r)
@@ -815,8 +854,24 @@ __device__ __forceinline__ void select_query_one(int64_t q, int64_t m, int k, do
         for (int i = 0; i + stride < KP; i += 2 * stride)
             v[i] = __fadd_rn(v[i], v[i + stride]);
     }
+    return select_power(v[0], d1, k, r_exp, am, alpha);
+}
+
+// select_query for one split.
+template <int KP>
+__device__ __forceinline__ void select_query_one(int64_t q, int64_t m, int k, double r_exp,
+                                                 const AlphaMap &am, const float *part_d2,
+                                                 const int32_t *part_idx, QParamF32 *qp,
+                                                 float *out_alpha, int32_t *out_knn,
+                                                 const uint32_t *perm)
+{
+    const int64_t qo = perm ? static_cast<int64_t>(perm[q]) : q;  // caller's query index
+    if (out_knn) {
+        for (int r = 0; r < k; ++r)
+            out_knn[qo * k + r] = __ldcg(part_idx + static_cast<int64_t>(r) * m + q);
+    }
     double alpha;
-    qp[q] = select_power(v[0], d1, k, r_exp, am, &alpha);
+    qp[q] = select_list<KP>(q, m, k, r_exp, am, part_d2, &alpha);
     if (out_alpha)
         out_alpha[qo] = static_cast<float>(alpha);
 }
@@ -855,19 +910,21 @@ __device__ __forceinline__ int weights_tiles(const DatasetDev &ds, int64_t p_beg
     return e > p_begin ? static_cast<int>((e - p_begin + TW - 1) / TW) : 0;
 }
 
-// The queries of a phase-2 unit, consecutive in the order phase 2 runs in: query i (below n) at
-// (x, y) with parameters p; its partial sums go to column col(i) of m.
+// The queries of a phase-2 unit, consecutive in the order phase 2 runs in (upwards from base, or
+// downwards with dir -1): query i (below n) at (x, y) with parameters p; its partial sums go to
+// column col(i) of m. Loads come from L2: in a batch other SMs have written them.
 struct UnitQueries {
     const float *qx, *qy;
     const QParamF32 *qp;
     int64_t base, n, col0, m;
+    int dir = 1;
 
     __device__ __forceinline__ void load(int64_t i, float &x, float &y, float2 &p) const
     {
-        const int64_t q = base + min(i, n - 1);
+        const int64_t q = base + dir * min(i, n - 1);
         p = __ldcg(reinterpret_cast<const float2 *>(qp + q));
-        x = qx[q];
-        y = qy[q];
+        x = __ldcg(qx + q);
+        y = __ldcg(qy + q);
     }
     __device__ __forceinline__ int64_t col(int64_t i) const
     {

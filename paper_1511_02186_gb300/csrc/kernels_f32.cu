@@ -44,18 +44,6 @@ f32_knn_kernel(DatasetDev ds, int64_t m, PassPlan pp, const float *__restrict__ 
                          p_end, qx, qy, k, s, part_d2, part_idx, err, tile, ts, idx_smem);
 }
 
-// A query's power class. Integer powers take the class loop where 2^c = d1^power (and with it
-// every unscaled weight d^-power) stays within 2^+-kClassMaxLog2.
-__device__ __forceinline__ int power_class(const QParamF32 &p, int pow_a, int pow_b)
-{
-    if (!(fabsf(p.c) <= kClassMaxLog2))
-        return kClassG;  // also NaN, and a query on a data point
-    const float twice = -2.0f * p.neg_s;
-    return twice == static_cast<float>(pow_a)   ? kClassA
-           : twice == static_cast<float>(pow_b) ? kClassB
-                                                : kClassG;
-}
-
 // KP > 0: one split, k <= KP.
 template <int KP>
 __global__ void __launch_bounds__(kSelectThreads)
@@ -78,21 +66,10 @@ f32_select_kernel(int64_t m, int S, int k, double r_exp, AlphaMap am,
     if (!co.cnt)
         return;
     // Each query to the next place of its class (a warp's queries stay together).
-    const int lane = threadIdx.x & 31;
-    QParamF32 p{0.0f, 0.0f};
-    int cls = kClasses;
     if (q < m) {
-        p = qp[q];
-        cls = power_class(p, co.pow_a, co.pow_b);
-    }
-    const unsigned same = __match_any_sync(0xffffffffu, cls);
-    const int leader = __ffs(same) - 1;
-    uint32_t at = 0;
-    if (lane == leader && cls < kClasses)
-        at = atomicAdd(&co.cnt[cls], static_cast<uint32_t>(__popc(same)));
-    at = __shfl_sync(0xffffffffu, at, leader) + __popc(same & ((1u << lane) - 1u));
-    if (q < m) {
-        const int64_t o = static_cast<int64_t>(cls) * m + at;
+        const QParamF32 p = qp[q];
+        const int cls = power_class(p, co.pow_a, co.pow_b);
+        const int64_t o = static_cast<int64_t>(cls) * m + class_place(co.cnt, cls);
         co.qx[o] = qx[q];
         co.qy[o] = qy[q];
         co.qp[o] = p;
