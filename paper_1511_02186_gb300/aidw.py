@@ -264,15 +264,26 @@ class TuneCache:
 
 # ---- array marshalling -------------------------------------------------------------------
 
+_TORCH_DTYPES = {}  # array code -> torch dtype, filled when the first tensor comes in
+
+
 def _is_torch(a) -> bool:
     return type(a).__module__.startswith("torch")
+
+
+def _torch_dtype(dtype):
+    t = _TORCH_DTYPES.get(dtype)
+    if t is None:
+        import torch
+        _TORCH_DTYPES.update(f4=torch.float32, f8=torch.float64, i4=torch.int32)
+        t = _TORCH_DTYPES[dtype]
+    return t
 
 
 def _prep(a, dtype):
     """Returns (keepalive, pointer) for a 1-D contiguous array of `dtype` ('f4','f8','i4')."""
     if _is_torch(a):
-        import torch
-        tdt = {"f4": torch.float32, "f8": torch.float64, "i4": torch.int32}[dtype]
+        tdt = _torch_dtype(dtype)
         if a.dtype != tdt or not a.is_contiguous():
             raise TypeError(f"expected a contiguous {tdt} tensor, got {a.dtype}")
         return a, a.data_ptr()
@@ -292,11 +303,13 @@ def _prep_out(a, dtype):
 
 
 def _out_like(q, shape, dtype):
+    """(array, keepalive, pointer) of a new output beside the queries `q`."""
     if _is_torch(q):
         import torch
-        tdt = {"f4": torch.float32, "f8": torch.float64, "i4": torch.int32}[dtype]
-        return torch.empty(shape, dtype=tdt, device=q.device)
-    return np.empty(shape, dtype=dtype)
+        a = torch.empty(shape, dtype=_torch_dtype(dtype), device=q.device)
+        return a, a, a.data_ptr()
+    a = np.empty(shape, dtype=dtype)
+    return a, a, a.ctypes.data
 
 
 def _stream_of(a, stream):
@@ -405,15 +418,20 @@ class Context:
         kqx, pqx = _prep(qx, fdt)
         kqy, pqy = _prep(qy, fdt)
         m = int(kqx.shape[0])
+        # (array, keepalive, pointer) of each output: a new one, the caller's, or none.
         if out is None:
-            out = _out_like(qx, (m,), fdt)
-        if want_alpha and out_alpha is None:
-            out_alpha = _out_like(qx, (m,), "f4")
-        if want_knn and out_knn is None:
-            out_knn = _out_like(qx, (m, p.k), "i4")
-        ko, po = _prep(out, fdt)
-        ka, pa = (None, None) if out_alpha is None else _prep(out_alpha, "f4")
-        kn, pn = (None, None) if out_knn is None else _prep(out_knn, "i4")
+            out, ko, po = _out_like(qx, (m,), fdt)
+        else:
+            ko, po = _prep(out, fdt)
+        ka = pa = kn = pn = None
+        if out_alpha is not None:
+            ka, pa = _prep(out_alpha, "f4")
+        elif want_alpha:
+            out_alpha, ka, pa = _out_like(qx, (m,), "f4")
+        if out_knn is not None:
+            kn, pn = _prep(out_knn, "i4")
+        elif want_knn:
+            out_knn, kn, pn = _out_like(qx, (m, p.k), "i4")
         st = _stream_of(qx, stream)
         if splits is None:
             rc = self.lib.aidw_interpolate(self.ptr, ds.handle, pqx, pqy, m, ctypes.byref(p),
@@ -439,9 +457,9 @@ class Context:
         kqy, pqy = _prep(qy, fdt)
         m = int(kqx.shape[0])
         if out is None:
-            out = _out_like(qx, (m,), fdt)
+            out = _out_like(qx, (m,), fdt)[0]
         if want_alpha and out_alpha is None:
-            out_alpha = _out_like(qx, (m,), "f4")
+            out_alpha = _out_like(qx, (m,), "f4")[0]
         po = _prep_out(out, fdt)
         pa = None if out_alpha is None else _prep_out(out_alpha, "f4")
         _check(self.lib.aidw_interpolate_paper(self.ptr, ds.handle, pqx, pqy, m,
@@ -457,7 +475,7 @@ class Context:
         kqy, pqy = _prep(qy, fdt)
         m = int(kqx.shape[0])
         if out is None:
-            out = _out_like(qx, (m,), fdt)
+            out = _out_like(qx, (m,), fdt)[0]
         ko, po = _prep(out, fdt)
         _check(self.lib.aidw_idw(self.ptr, ds.handle, pqx, pqy, m, float(alpha), int(precision),
                                  po, _stream_of(qx, stream)), "aidw_idw")
@@ -508,7 +526,7 @@ class Context:
         kqy, pqy = _prep(qy, "f4")
         m = int(kqx.shape[0])
         if out is None:
-            out = _out_like(qx, (m,), "f4")
+            out = _out_like(qx, (m,), "f4")[0]
         po = _prep_out(out, "f4")
         c, ms = TuneConfig(), ctypes.c_double()
         _check(self.lib.aidw_autotune_interpolate(self.ptr, ds.handle, pqx, pqy, m,

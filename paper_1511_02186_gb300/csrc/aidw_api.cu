@@ -98,6 +98,7 @@ using namespace aidw;
 struct DatasetRec {
     DatasetDev dev;
     void *block = nullptr;
+    bool pooled = false;  // block comes from the context's pool
     size_t bytes = 0;
     double area = 0.0;
     double r_exp = 0.0;
@@ -112,6 +113,8 @@ struct aidw_ctx {
     int *d_err = nullptr;
     unsigned long long *d_bad = nullptr;
     cudaMemPool_t pool = nullptr;
+    void *pinned = nullptr;  // [kPinnedBytes] results of small host-array calls, and the error word
+    std::mutex pinned_mu;    // taken without waiting: a second call at once goes without
     std::mutex mu;
     std::unordered_map<int64_t, DatasetRec> datasets;
     int64_t next_ds = 1;
@@ -167,6 +170,33 @@ void ctx_free(aidw_ctx *ctx, void *p, size_t bytes, cudaStream_t st)
     cudaFreeAsync(p, st);
     std::lock_guard<std::mutex> g(ctx->mu);
     ctx->in_use -= bytes;
+}
+
+// Blocks of a dataset and of its construction: from the context's pool up to kPoolDatasetBytes
+// (cudaMalloc and cudaFree take about 95 us together and wait for the device), else by cudaMalloc.
+// What the pool keeps beyond kPoolKeepBytes is given back when a dataset is destroyed.
+constexpr size_t kPoolDatasetBytes = size_t(64) << 20;
+constexpr size_t kPoolKeepBytes = size_t(1) << 30;
+
+static cudaError_t dataset_alloc(aidw_ctx *ctx, size_t bytes, void **p, bool *pooled)
+{
+    *pooled = bytes <= kPoolDatasetBytes;
+    return *pooled ? cudaMallocFromPoolAsync(p, bytes, ctx->pool, 0) : cudaMalloc(p, bytes);
+}
+
+static void dataset_free(aidw_ctx *ctx, void *p, bool pooled)
+{
+    if (!pooled) {
+        cudaFree(p);
+        return;
+    }
+    cudaFreeAsync(p, 0);
+    uint64_t reserved = 0, used = 0;
+    if (cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrReservedMemCurrent, &reserved) ==
+            cudaSuccess &&
+        cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess &&
+        reserved - used > kPoolKeepBytes)
+        cudaMemPoolTrimTo(ctx->pool, used + kPoolKeepBytes);
 }
 
 size_t ctx_budget_left(aidw_ctx *ctx)
@@ -780,6 +810,11 @@ int enqueue_warp(aidw_ctx *ctx, const DatasetDev &ds, double r_exp, const Plan &
     return AIDW_OK;
 }
 
+// Host results of up to kPinnedBytes go through the context's pinned buffer: a device-to-host copy
+// into pageable memory waits for the stream by itself, and so does the error word's (17 us for
+// the two against 8 us for both through pinned memory and one wait).
+constexpr size_t kPinnedBytes = size_t(256) << 10;
+
 // Reads and clears the on-device error word (synchronous).
 int consume_device_error(aidw_ctx *ctx, cudaStream_t st)
 {
@@ -929,6 +964,30 @@ int interpolate_impl(aidw_ctx *ctx, aidw_dataset dsid, const void *qx, const voi
                 : enqueue_interpolation(ctx, ds, r_exp, pl, *p, dqx, dqy, sc, dout, dalpha, dknn,
                                         st, ctx->profiling);
     if (rc == AIDW_OK && host_any) {
+        std::unique_lock<std::mutex> pin(ctx->pinned_mu, std::defer_lock);
+        if (b_o + b_a + b_n + sizeof(int) <= kPinnedBytes && ctx->pinned && pin.try_lock()) {
+            // The staged results lie together in the block; the error word follows them.
+            const size_t staged = b_o + b_a + b_n;
+            char *h = static_cast<char *>(ctx->pinned);
+            int *herr = reinterpret_cast<int *>(h + staged);
+            ok = true;
+            if (staged)
+                ok &= cudaMemcpyAsync(h, stage - staged, staged, cudaMemcpyDeviceToHost, st) ==
+                      cudaSuccess;
+            ok &= cudaMemcpyAsync(herr, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, st) ==
+                  cudaSuccess;
+            ctx_free(ctx, blk, total, st);
+            ok &= cudaStreamSynchronize(st) == cudaSuccess;
+            if (!ok)
+                return AIDW_ERR_CUDA;
+            if (ko == 0)
+                std::memcpy(out, h, m * es);
+            if (b_a)
+                std::memcpy(out_alpha, h + b_o, m * sizeof(float));
+            if (b_n)
+                std::memcpy(out_knn, h + b_o + b_a, m * p->k * sizeof(int32_t));
+            return *herr ? consume_device_error(ctx, st) : AIDW_OK;
+        }
         ok = true;
         if (ko == 0)
             ok &= cudaMemcpyAsync(out, dout, m * es, cudaMemcpyDeviceToHost, st) == cudaSuccess;
@@ -1021,6 +1080,7 @@ int aidw_init(aidw_ctx **out, int device, size_t hbm_budget_bytes)
     ok = ok && cudaMemset(ctx->d_err, 0, sizeof(int)) == cudaSuccess;
     for (int i = 0; ok && i < 5; ++i)
         ok = cudaEventCreate(&ctx->ev[i]) == cudaSuccess;
+    ok = ok && cudaMallocHost(&ctx->pinned, kPinnedBytes) == cudaSuccess;
     // Places aidw_interpolate_noalloc's fixed scratch array on the device now, at set-up, so
     // that its calls never load a module (and its 16 MiB) in the middle of a request.
     ok = ok && noalloc_prepare(device) == AIDW_OK;
@@ -1042,8 +1102,10 @@ int aidw_shutdown(aidw_ctx *ctx)
     ctx->serving = nullptr;
     cudaDeviceSynchronize();
     for (auto &kv : ctx->datasets)
-        cudaFree(kv.second.block);
+        dataset_free(ctx, kv.second.block, kv.second.pooled);
     ctx->datasets.clear();
+    if (ctx->pinned)
+        cudaFreeHost(ctx->pinned);
     if (ctx->d_err)
         cudaFree(ctx->d_err);
     if (ctx->d_bad)
@@ -1105,7 +1167,8 @@ int aidw_create_dataset(aidw_ctx *ctx, const void *x, const void *y, const void 
         ctx->in_use -= bytes;
     };
     void *blk = nullptr;
-    if (cudaMalloc(&blk, bytes) != cudaSuccess) {
+    bool blk_pooled = false;
+    if (dataset_alloc(ctx, bytes, &blk, &blk_pooled) != cudaSuccess) {
         cudaGetLastError();
         unreserve();
         return AIDW_ERR_OOM;
@@ -1118,9 +1181,10 @@ int aidw_create_dataset(aidw_ctx *ctx, const void *x, const void *y, const void 
                              align256(np * sizeof(float)) + 2 * align256(np * sizeof(uint32_t)) +
                              align256(radix_scratch_bytes(n_pad)) + 256;
     void *tmp = nullptr;
-    if (cudaMalloc(&tmp, tmp_bytes) != cudaSuccess) {
+    bool tmp_pooled = false;
+    if (dataset_alloc(ctx, tmp_bytes, &tmp, &tmp_pooled) != cudaSuccess) {
         cudaGetLastError();
-        cudaFree(blk);
+        dataset_free(ctx, blk, blk_pooled);
         unreserve();
         return AIDW_ERR_OOM;
     }
@@ -1185,34 +1249,31 @@ int aidw_create_dataset(aidw_ctx *ctx, const void *x, const void *y, const void 
         convert_dataset_kernel<float><<<blocks, threads>>>(
             static_cast<const float *>(sx), static_cast<const float *>(sy),
             static_cast<const float *>(sz), n, n_pad, xy32, z32, xy64, z64, ctx->d_bad);
+    // Z-order the FP32 copy and box every tile. Non-finite inputs go through like any others; the
+    // count of them is looked at once, at the end.
     unsigned long long seen[2] = {0, 0};  // non-finite inputs, largest |z|
-    if (cudaGetLastError() != cudaSuccess ||
-        cudaMemcpy(seen, ctx->d_bad, sizeof(seen), cudaMemcpyDeviceToHost) != cudaSuccess)
-        rc = AIDW_ERR_CUDA;
-    else if (seen[0])
-        rc = AIDW_ERR_INVALID_ARG;
-    // Z-order the FP32 copy and box every tile.
-    if (rc == AIDW_OK) {
-        bool ok = bbox_of(xy32, n, box_scratch, box, 0) == cudaSuccess;
-        ok = ok && morton_keys(nullptr, nullptr, xy32, n, n_pad, box, keys, perm, 0) ==
-                       cudaSuccess;
-        ok = ok && radix_sort_pairs(keys, perm, n_pad, sort_tmp, 0) == cudaSuccess;
-        if (ok) {
-            gather_dataset_kernel<<<blocks, threads>>>(xy32, z32, perm, n, n_pad, nxy2, zz, orig);
-            ok = cudaGetLastError() == cudaSuccess;
-        }
-        ok = ok && tile_boxes(nxy2, ntiles, tbox, 0) == cudaSuccess;
-        ok = ok && sub_tile_boxes(nxy2, nsub, sbox, 0) == cudaSuccess;
-        ok = ok && super_tile_boxes(tbox, ntiles, nsuper, upbox, 0) == cudaSuccess;
-        ok = ok && cudaDeviceSynchronize() == cudaSuccess;
-        if (!ok) {
-            cudaGetLastError();
-            rc = AIDW_ERR_CUDA;
-        }
+    bool ok = cudaGetLastError() == cudaSuccess;
+    ok = ok && bbox_of(xy32, n, box_scratch, box, 0) == cudaSuccess;
+    ok = ok && morton_keys(nullptr, nullptr, xy32, n, n_pad, box, keys, perm, 0) == cudaSuccess;
+    ok = ok && radix_sort_pairs(keys, perm, n_pad, sort_tmp, 0) == cudaSuccess;
+    if (ok) {
+        gather_dataset_kernel<<<blocks, threads>>>(xy32, z32, perm, n, n_pad, nxy2, zz, orig);
+        ok = cudaGetLastError() == cudaSuccess;
     }
-    cudaFree(tmp);
+    ok = ok && tile_boxes(nxy2, ntiles, tbox, 0) == cudaSuccess;
+    ok = ok && sub_tile_boxes(nxy2, nsub, sbox, 0) == cudaSuccess;
+    ok = ok && super_tile_boxes(tbox, ntiles, nsuper, upbox, 0) == cudaSuccess;
+    ok = ok && cudaMemcpy(seen, ctx->d_bad, sizeof(seen), cudaMemcpyDeviceToHost) == cudaSuccess;
+    ok = ok && cudaDeviceSynchronize() == cudaSuccess;
+    if (!ok) {
+        cudaGetLastError();
+        rc = AIDW_ERR_CUDA;
+    } else if (seen[0]) {
+        rc = AIDW_ERR_INVALID_ARG;
+    }
+    dataset_free(ctx, tmp, tmp_pooled);
     if (rc) {
-        cudaFree(blk);
+        dataset_free(ctx, blk, blk_pooled);
         unreserve();
         return rc;
     }
@@ -1231,6 +1292,7 @@ int aidw_create_dataset(aidw_ctx *ctx, const void *x, const void *y, const void 
     const uint32_t z_bits = static_cast<uint32_t>(seen[1]);
     std::memcpy(&rec.dev.z_max, &z_bits, sizeof(z_bits));
     rec.block = blk;
+    rec.pooled = blk_pooled;
     rec.bytes = bytes;
     rec.area = area;
     rec.r_exp = 1.0 / (2.0 * std::sqrt(static_cast<double>(n) / area));  // Eq. 2
@@ -1256,7 +1318,7 @@ int aidw_destroy_dataset(aidw_ctx *ctx, aidw_dataset ds)
     }
     cudaSetDevice(ctx->device);
     cudaDeviceSynchronize();
-    cudaFree(rec.block);
+    dataset_free(ctx, rec.block, rec.pooled);
     std::lock_guard<std::mutex> g(ctx->mu);
     ctx->in_use -= rec.bytes;
     return AIDW_OK;
