@@ -28,6 +28,7 @@
 #include <cstdint>
 
 #include "aidw_internal.cuh"
+#include "sq_dist.cuh"
 
 namespace aidw {
 namespace dfm {
@@ -91,24 +92,23 @@ __device__ __forceinline__ float small_int_to_float(int v)
     return __fsub_rn(__int_as_float(0x4B400000 + v), 12582912.0f);
 }
 
-// log2 of a positive normal (or +inf) double x as e + (lh + ll) + (sh + sl): e the exponent,
-// lh + ll = log2 F_j, sh + sl = log2(1 + r) with |sh| < 2^-7.4.
+// log2 of a normalised value as e + (lh + ll) + (sh + sl): e the exponent, lh + ll = log2 F_j,
+// sh + sl = log2(1 + r) with |sh| < 2^-7.4.
 struct LogParts {
     int e;
     float lh, ll, sh, sl;
 };
 
-__device__ __forceinline__ LogParts log2_parts(double x, const Tables &t)
+__device__ __forceinline__ LogParts log2_parts(const NormU64 &x, const Tables &t)
 {
-    const uint32_t hi = static_cast<uint32_t>(__double2hiint(x));
-    const uint32_t lo = static_cast<uint32_t>(__double2loint(x));
+    const uint32_t hi = static_cast<uint32_t>(x.m >> 32);
     LogParts p;
-    p.e = static_cast<int>(hi >> 20) - 1023;
-    const int j = static_cast<int>((hi >> 12) & 255u);
-    // m - F_j = (A 2^22 + C) 2^-52 with A the next 22 mantissa bits and C the last 22; each
-    // becomes a float exactly as (1 + bits 2^-22) - 1, scaled.
-    const uint32_t a = (__funnelshift_l(lo, hi, 11) & 0x7FFFFEu) | 0x3F800000u;
-    const uint32_t c = ((lo << 1) & 0x7FFFFEu) | 0x3F800000u;
+    p.e = x.e;
+    const int j = static_cast<int>((hi >> 23) & 255u);
+    // m - F_j = (A 2^22 + C) 2^-52 with A the next 22 bits and C the 22 below (the last 11 of
+    // 63 are left out); each becomes a float exactly as (1 + bits 2^-22) - 1, scaled.
+    const uint32_t a = (hi & 0x7FFFFEu) | 0x3F800000u;
+    const uint32_t c = (static_cast<uint32_t>(x.m >> 10) & 0x7FFFFEu) | 0x3F800000u;
     const float th = __fmaf_rn(__uint_as_float(a), 0x1p-8f, -0x1p-8f);
     const float tl = __fmaf_rn(__uint_as_float(c), 0x1p-30f, -0x1p-30f);
     const float4 g = t.lg[j];
@@ -153,7 +153,7 @@ struct RefLog {
 
 __device__ __forceinline__ RefLog ref_log(double d1sq, const Tables &t)
 {
-    const LogParts p = log2_parts(d1sq, t);
+    const LogParts p = log2_parts(norm_of(d1sq), t);
     RefLog r;
     r.e1 = p.e;
     frac_log(p, r.f1h, r.f1l);
@@ -162,15 +162,15 @@ __device__ __forceinline__ RefLog ref_log(double d1sq, const Tables &t)
 
 // log2(d^2 / d1^2) as (vh, vl): the mantissa logarithms are formed by the same operations as
 // the reference's, so d^2 == d1^2 gives exactly 0 (the nearest point's weight is exactly 1).
-__device__ __forceinline__ void log2_ratio(double d2, const RefLog &ref, const Tables &t,
+__device__ __forceinline__ void log2_ratio(const NormU64 &d2, const RefLog &ref, const Tables &t,
                                            float &vh, float &vl)
 {
     const LogParts p = log2_parts(d2, t);
     float fh, fl, s, e1, e2;
     frac_log(p, fh, fl);
     two_sum(fh, -ref.f1h, s, e2);  // |s| < 1
-    // d^2 = +inf (a padding point): a ratio beyond every weight's reach.
-    const float a = p.e == 1024 ? 1e38f : small_int_to_float(p.e - ref.e1);
+    // d^2 beyond a double (a padding point): a ratio beyond every weight's reach.
+    const float a = p.e > 1023 ? 1e38f : small_int_to_float(p.e - ref.e1);
     fast_two_sum(a, s, vh, e1);    // a is an integer
     vl = __fadd_rn(__fadd_rn(e1, e2), __fsub_rn(fl, ref.f1l));
 }

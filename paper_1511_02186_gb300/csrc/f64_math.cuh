@@ -32,6 +32,7 @@
 #include <math_constants.h>
 
 #include "aidw_internal.cuh"
+#include "sq_dist.cuh"
 
 namespace aidw {
 namespace f64math {
@@ -106,24 +107,20 @@ __device__ __forceinline__ double fx52_to_double(long long a)
     return m == 0 ? 0.0 : __longlong_as_double(static_cast<long long>(b | s));
 }
 
-// log2(x) at 2^52 (+inf and NaN as about 1,024) from the table entries of j = log2_index(x): q_j's
-// coefficient magnitudes and log2 F_j, all at 2^62. Horner in magnitudes: q(u) = A1 - u (A2 - u (A3 - u A4)), every
-// bracket positive.
-__device__ __forceinline__ long long log2_fixed(double x, unsigned long long a4,
-                                                unsigned long long a3, unsigned long long a2,
-                                                unsigned long long a1, unsigned long long log2f)
+// log2 of 2^e (F_j + u) at 2^52 from the table entries of j: q_j's coefficient magnitudes and
+// log2 F_j, all at 2^62, and u at 2^73 (below 2^63). Horner in magnitudes: q(u) = A1 - u (A2 - u
+// (A3 - u A4)), every bracket positive.
+__device__ __forceinline__ long long log2_fixed(int e, unsigned long long u,
+                                                unsigned long long a4, unsigned long long a3,
+                                                unsigned long long a2, unsigned long long a1,
+                                                unsigned long long log2f)
 {
-    const long long b = __double_as_longlong(x);
-    // u: the mantissa bits below the index, exactly, at 2^73 (u 2^73 < 2^63).
-    const unsigned long long u =
-        static_cast<unsigned long long>(b & ((1ll << (52 - kLogBits)) - 1)) << 21;
     unsigned long long p = a3 - fx_mul32(a4, u);  // its error is scaled by u^3 below
     p = a2 - fx_mul32(p, u);                       // ... by u^2
     p = a1 - fx_mul(p, u);
     const unsigned long long f = log2f + fx_mul(p, u);  // log2 F + u q(u) in [0, 1), at 2^62
-    const int eb = static_cast<int>(b >> 52);
     // e + f at 2^52 (|e| <= 1074: below 2^63), f rounded to 2^-53.
-    return static_cast<long long>(eb - 1023) * (1ll << 52) +
+    return static_cast<long long>(e) * (1ll << 52) +
            static_cast<long long>((f + (1ull << 9)) >> 10);
 }
 
@@ -132,17 +129,27 @@ __device__ __forceinline__ bool inf_or_nan(double x)
     return (static_cast<uint32_t>(__double2hiint(x)) & 0x7FF00000u) == 0x7FF00000u;
 }
 
-// log2(x) at 2^52, x > 0 finite.
-__device__ __forceinline__ long long log2_52(double x, const Tables &t)
+__device__ __forceinline__ long long log2_52(int e, int j, unsigned long long u, const Tables &t)
 {
-    const int j = log2_index(x);
     const ulonglong2 a = t.la[j], c = t.lb[j];
-    return log2_fixed(x, a.x, a.y, c.x, c.y, t.lc[j]);
+    return log2_fixed(e, u, a.x, a.y, c.x, c.y, t.lc[j]);
+}
+
+// log2 of a normalised value at 2^52.
+__device__ __forceinline__ long long log2_52(const NormU64 &v, const Tables &t)
+{
+    return log2_52(v.e, static_cast<int>(v.m >> (63 - kLogBits)) & (kLogN - 1),
+                   (v.m & ((1ull << (63 - kLogBits)) - 1)) << kLogBits, t);
 }
 
 __device__ __forceinline__ double log2_t(double x, const Tables &t)
 {
-    return inf_or_nan(x) ? CUDART_INF : fx52_to_double(log2_52(x, t));  // NaN as +inf
+    const long long b = __double_as_longlong(x);
+    // u: the mantissa bits below the index, exactly, at 2^73 (u 2^73 < 2^63).
+    const unsigned long long u =
+        static_cast<unsigned long long>(b & ((1ll << (52 - kLogBits)) - 1)) << 21;
+    const long long v = log2_52(static_cast<int>(b >> 52) - 1023, log2_index(x), u, t);
+    return inf_or_nan(x) ? CUDART_INF : fx52_to_double(v);  // NaN as +inf
 }
 
 // 2^(k/1024 + r) for |k| < 2^21 and r at 2^73, |r| <= 2^62: T_j 2^r at 2^62 with j = k mod 1,024,
@@ -208,24 +215,28 @@ __device__ __forceinline__ FixedPower fixed_power(double kappa, double d1sq, con
         es = -1;
     }
     p.sh = 62 - es;
-    p.l1 = log2_52(d1sq, t);
+    p.l1 = log2_52(norm_of(d1sq), t);
+    if (inf_or_nan(d1sq)) {  // no finite distance: every weight 0, the ratio 0 / 0
+        p.S = 1ull << 63;
+        p.sh = 0;
+        p.l1 = -(1ll << 62);
+    }
     return p;
 }
 
 // (d^2 / d1^2)^(-s) as a double and in 96-bit fixed point: y = s (log2 d^2 - log2 d1^2) at 2^53 as
-// the shifted 128-bit product, exactly 0 at the nearest distance, and 2^-y. 0 from y = 1,021 on
-// and for an infinite (a padding point's) or NaN d^2. Between the logarithm and the exponential
-// nothing is rounded to a double, packed or unpacked, and the FP64 pipe does one operation per
-// pair less than with y = fma(log2 d^2, -s, c).
-__device__ __forceinline__ double power_weight(double d2, const FixedPower &fp, const Tables &t,
-                                               unsigned __int128 *w96)
+// the shifted 128-bit product, and 2^-y. 0 from y = 1,021 on and where d^2 is beyond a double
+// (a padding point, a non-finite query). From the differences of the coordinates to the weight
+// nothing is rounded to a double, packed or unpacked.
+__device__ __forceinline__ double power_weight(const NormU64 &d2, const FixedPower &fp,
+                                               const Tables &t, unsigned __int128 *w96)
 {
     const long long d = log2_52(d2, t) - fp.l1;
     const bool neg = d < 0;  // by rounding only
     const unsigned long long m = static_cast<unsigned long long>(neg ? -d : d);
     const unsigned long long hi = __umul64hi(m, fp.S), lo = m * fp.S;
     const unsigned long long y = (lo >> fp.sh) | ((hi << 1) << (63 - fp.sh));
-    if ((hi >> fp.sh) != 0 || y >= (1021ull << 53) || inf_or_nan(d2)) {
+    if ((hi >> fp.sh) != 0 || y >= (1021ull << 53) || d2.e > 1023) {
         *w96 = 0;
         return 0.0;
     }

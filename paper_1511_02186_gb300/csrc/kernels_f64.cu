@@ -35,13 +35,6 @@ __device__ __forceinline__ double dist2_exact(double qx, double qy, double px, d
     return __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
 }
 
-__device__ __forceinline__ double dist2_eps(double qx, double qy, double px, double py)
-{
-    const double dx = __dsub_rn(qx, px);
-    const double dy = __dsub_rn(qy, py);
-    return __fma_rn(dx, dx, __fma_rn(dy, dy, kEpsF64));
-}
-
 template <int KP>
 __device__ __forceinline__ void list_insert(double (&L)[KP], double v)
 {
@@ -846,14 +839,20 @@ f64_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restri
                 const int cg = c + i * kChunkW + pg * (kChunkW / PG);
                 if (PG > 1 && cg >= cend)
                     break;
-                // One point at a time (unrolled by 2: 10.7 against 10.6 ms at 8,191 x 131,072).
-#pragma unroll 1
+                // One point in four takes its squared distance on the integer pipe: the FP64 pipe
+                // (5 operations a pair) is busy 87 % of the time and the ALU (121) 64 %. 8,191 x
+                // 131,072, whole call (ms): none 10.53, one in four 10.24, one in two 10.46, all
+                // 11.14; none unrolled by 2 10.7.
+#pragma unroll 4
                 for (int u = 0; u < kChunkW / PG; ++u) {
                     const double2 p = txy[b][cg + u];
                     const double pz = tz[b][cg + u];
 #pragma unroll
                     for (int j = 0; j < Q; ++j) {
-                        const double d2 = dist2_eps(qxr[j], qyr[j], p.x, p.y);
+                        const double dx = __dsub_rn(qxr[j], p.x), dy = __dsub_rn(qyr[j], p.y);
+                        const NormU64 d2 =
+                            (u & 3) == 3 ? sum_of_squares(dx, dy)
+                                         : norm_of(__fma_rn(dx, dx, __fma_rn(dy, dy, kEpsF64)));
                         unsigned __int128 w96;
                         const double w = f64math::power_weight(d2, fp[j], tabs, &w96);
                         aw[j] += w96;

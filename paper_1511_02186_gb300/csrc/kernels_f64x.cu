@@ -1,10 +1,10 @@
-// AIDW_F64X phase 2 for sm_103a: Eq. 1 over all data points with FP64 inputs and output, the
-// squared distance formed in FP64 exactly as the FP64 path forms it, and the rest of each pair's
-// work (log2, the adaptive power, exp2, both weighted sums) in double-float arithmetic on the
-// FP32 pipes (df_math.cuh). GB300 runs FP64 at 1/64 of its FP32 rate, so the four FP64
-// operations of the distance bound this scan and the hundred-odd FP32 operations per pair run
-// beside them. Phase 1, the selection of alpha (Eq. 2-6) and the final division stay the FP64
-// path's kernels.
+// AIDW_F64X phase 2 for sm_103a: Eq. 1 over all data points with FP64 inputs and output. The
+// differences of the coordinates are formed in FP64, their sum of squares on the integer pipe
+// (sq_dist.cuh), and the rest of each pair's work (log2, the adaptive power, exp2, both weighted
+// sums) in double-float arithmetic on the FP32 pipes (df_math.cuh). GB300 runs FP64 at 1/64 of
+// its FP32 rate: the two subtractions take half the time of a pair's 197 instructions, which now
+// bound the scan (78 % of the issue slots). Phase 1, the selection of alpha (Eq. 2-6) and the
+// final division stay the FP64 path's kernels.
 #include <math_constants.h>
 
 #include "aidw_internal.cuh"
@@ -15,13 +15,6 @@ namespace {
 
 constexpr int kQX = 2;       // queries per thread
 constexpr int kChunkX = 16;  // points summed per double-float merge
-
-__device__ __forceinline__ double dist2_eps_x(double qx, double qy, double px, double py)
-{
-    const double dx = __dsub_rn(qx, px);
-    const double dy = __dsub_rn(qy, py);
-    return __fma_rn(dx, dx, __fma_rn(dy, dy, kEpsF64));
-}
 
 __device__ __forceinline__ void drain_x(uint64_t *bar, int t, int ntiles)
 {
@@ -129,7 +122,8 @@ f64x_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restr
                     const float2 pz = tzf[cg + u];
 #pragma unroll
                     for (int j = 0; j < Q; ++j) {
-                        const double d2 = dist2_eps_x(qxr[j], qyr[j], p.x, p.y);
+                        const NormU64 d2 = sum_of_squares(__dsub_rn(qxr[j], p.x),
+                                                          __dsub_rn(qyr[j], p.y));
                         float vh, vl, yh, yl, wh, wl, e, zh, zl;
                         dfm::log2_ratio(d2, ref[j], tabs, vh, vl);
                         dfm::mul(kh[j], kl[j], vh, vl, yh, yl);  // -y = kappa log2(d^2 / d1^2)
@@ -205,7 +199,7 @@ __global__ void df_weight_probe_kernel(const double *__restrict__ d2,
         const float kh = __double2float_rn(kappa[i]);
         const float kl = __double2float_rn(kappa[i] - static_cast<double>(kh));
         float vh, vl, yh, yl, wh, wl;
-        dfm::log2_ratio(d2[i], ref, tabs, vh, vl);
+        dfm::log2_ratio(norm_of(d2[i]), ref, tabs, vh, vl);
         dfm::mul(kh, kl, vh, vl, yh, yl);
         dfm::exp2_df(-yh, -yl, tabs, wh, wl);
         v[i] = static_cast<double>(vh) + static_cast<double>(vl);

@@ -50,3 +50,19 @@ def test_a_budget_below_the_planned_partial_sums_takes_fewer_splits():
         z = c.interpolate(ds, qx, qy, params_of(wl, aidw.F32C))[0]
         assert rel_err(z.cpu().numpy().astype(np.float64), ref).max() <= TOL_F32
         ds.destroy()
+
+
+@pytest.mark.parametrize("precision", [aidw.F64, aidw.F64X])
+@pytest.mark.parametrize("side", [1e-30, 1e-9, 1e9, 1e30])
+def test_fp64_scales(ctx, precision, side):
+    """The squared distances formed on the integer pipe, from far below to far above 1, with
+    queries on data points and on one axis with them."""
+    wl = workloads.small_case(9, 3001, 257, k=10, pattern="uniform", side=side)
+    wl.qx[:20], wl.qy[:20] = wl.x[:20], wl.y[:20]
+    wl.qx[20:40] = wl.x[20:40]
+    ref, _ = oracle_for(wl, precision)
+    ds = ctx.create_dataset(wl.x, wl.y, wl.z, wl.area)
+    qx, qy = to_device(wl, precision)
+    z = ctx.interpolate(ds, qx, qy, params_of(wl, precision))[0].cpu().numpy()
+    assert rel_err(z, ref).max() <= TOL_F64
+    ds.destroy()
