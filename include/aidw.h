@@ -156,7 +156,7 @@ int aidw_idw(aidw_ctx *ctx, aidw_dataset ds, const void *qx, const void *qy, int
  *   p            as for aidw_interpolate; p->precision must be AIDW_F32C
  * Phase 1 takes aidw_interpolate's route when its scratch fits the array: up to 32,768 queries
  * one warp per query (about m * (4k + 24) bytes), above that the pruned scan over queries put
- * in Z-order (about m * (4k + 49) bytes, m up to about 189,000 at k = 10); otherwise it scans
+ * along a Hilbert curve (about m * (4k + 49) bytes, m up to about 189,000 at k = 10); otherwise it scans
  * every (query, data point) pair in data splits, which for many queries costs far more (at
  * 131,072 queries x 1M points about 61 ms against 3.4 ms for the pruned scan; phase 2 is the
  * same either way). Limit: the split scan

@@ -65,7 +65,7 @@ __global__ void convert_dataset_kernel(const T *__restrict__ x, const T *__restr
         atomicMax(reinterpret_cast<unsigned *>(bad + 1), zb);
 }
 
-// Writes the Z-ordered FP32 layout: stored position i holds caller point perm[i] (padding
+// Writes the curve-ordered FP32 layout: stored position i holds caller point perm[i] (padding
 // positions, perm[i] >= n, hold +inf points with value 0).
 __global__ void gather_dataset_kernel(const float2 *__restrict__ xy32,
                                       const float *__restrict__ z32,
@@ -658,15 +658,15 @@ bool use_culled_knn(int precision, const DatasetDev &ds, int64_t m, bool with_id
 // queries get denser. Measured phase 1 in FP32 (us; pruned scan with the query ordering / warp
 // per query):
 //   queries              16,384       65,536      131,072     262,144      1,048,576
-//   1M uniform        3,276 / 102  1,976 / 303  1,544 / 580  1,415 / 1,124  1,902 / 4,345
-//   262,147 clustered 1,784 / 88   1,259 / 290  1,250 / 554  1,088 / 1,051  1,175 / 3,986
-//   65,536 clustered    660 / 68     498 / 212    474 / 409    558 / 777      609 / 3,011
-//   16,384 uniform      290 / 60     288 / 196    270 / 368    305 / 708      519 / 2,721
-// so the crossing lies near 3,500 n^(1/3) queries, and a call of many more queries than points
-// orders them. The FP64 pruned scan is slower than the warp scan at every count measured
-// (65,536 clustered, 262,144 queries: 8,184 / 1,375; 1M uniform, 16,384: 43,274 / 170).
+//   1M uniform        1,992 / 46     922 / 148    711 / 283    795 / 545  1,306 / 2,123
+//   262,147 clustered 1,347 / 47   1,348 / 152  1,219 / 281  1,418 / 537  1,145 / 2,084
+//   65,536 clustered    620 / 49     544 / 147    459 / 279    510 / 541    519 / 2,080
+//   16,384 uniform      237 / 39     210 / 126    210 / 244    241 / 475    446 / 1,852
+// so the crossing lies near 5,000 n^(1/3) queries from 65,536 points on; a call of many more
+// queries than points orders them. The FP64 pruned scan is slower than the warp scan at every
+// count measured (65,536 clustered, 262,144 queries: 7,758 / 940; 1M uniform, 16,384: 26,234 / 82).
 constexpr int64_t kWarpKnnMaxQueries = 32768;
-constexpr double kWarpKnnPerCbrt = 3500.0;
+constexpr double kWarpKnnPerCbrt = 5000.0;
 constexpr double kWarpKnnPerPoint = 1.9;
 
 bool use_warp_knn(int precision, const DatasetDev &ds, int64_t m)
@@ -694,7 +694,7 @@ size_t culled_extra_bytes(int64_t m, int precision)
            align256(radix_scratch_bytes(m));
 }
 
-// Interpolation with Z-ordered queries and the pruned phase-1 scan: Morton keys of the queries
+// Interpolation with curve-ordered queries and the pruned phase-1 scan: Hilbert keys of the queries
 // over the dataset's box, stable radix sort, gather, phase 1 (pruned), selection and
 // finalisation writing back to the caller's order; phase 2 runs on the ordered queries.
 int enqueue_culled(aidw_ctx *ctx, const DatasetDev &ds, double r_exp, const Plan &pl,
@@ -721,7 +721,7 @@ int enqueue_culled(aidw_ctx *ctx, const DatasetDev &ds, double r_exp, const Plan
     if (f64) {
         const double *x = static_cast<const double *>(qx), *y = static_cast<const double *>(qy);
         double *sx = static_cast<double *>(sqx), *sy = static_cast<double *>(sqy);
-        ok = morton_keys_f64(x, y, m, ds.box, keys, perm, st) == cudaSuccess;
+        ok = curve_keys_f64(x, y, m, ds.box, keys, perm, st) == cudaSuccess;
         ok = ok && radix_sort_pairs(keys, perm, m, sort_tmp, st) == cudaSuccess;
         ok = ok && gather_queries_f64(x, y, perm, m, sx, sy, st) == cudaSuccess;
         ok = ok && launch_f64_knn_cull(ds, pl, sx, sy, p.k, sc, ctx->d_err, st) == cudaSuccess;
@@ -736,7 +736,7 @@ int enqueue_culled(aidw_ctx *ctx, const DatasetDev &ds, double r_exp, const Plan
     } else {
         const float *x = static_cast<const float *>(qx), *y = static_cast<const float *>(qy);
         float *sx = static_cast<float *>(sqx), *sy = static_cast<float *>(sqy);
-        ok = morton_keys(x, y, nullptr, m, m, ds.box, keys, perm, st) == cudaSuccess;
+        ok = curve_keys(x, y, nullptr, m, m, ds.box, keys, perm, st) == cudaSuccess;
         ok = ok && radix_sort_pairs(keys, perm, m, sort_tmp, st) == cudaSuccess;
         ok = ok && gather_queries(x, y, perm, m, sx, sy, st) == cudaSuccess;
         ok = ok && launch_f32_knn_cull(ds, pl, sx, sy, p.k, sc, ctx->d_err, st) == cudaSuccess;
@@ -756,7 +756,7 @@ int enqueue_culled(aidw_ctx *ctx, const DatasetDev &ds, double r_exp, const Plan
         ctx->last = aidw_kernel_times{};
         ctx->last.splits = pl.knn.splits;
         ctx->last.query_blocks = pl.knn.qblocks;
-        ctx->last.launches = 4 + 14;  // + Morton keys, 12 radix-sort passes, gather
+        ctx->last.launches = 4 + 14;  // + Hilbert keys, 12 radix-sort passes, gather
         ctx->last.weight_splits = pl.w.splits;
         ctx->last_valid = true;
     }
@@ -1249,12 +1249,12 @@ int aidw_create_dataset(aidw_ctx *ctx, const void *x, const void *y, const void 
         convert_dataset_kernel<float><<<blocks, threads>>>(
             static_cast<const float *>(sx), static_cast<const float *>(sy),
             static_cast<const float *>(sz), n, n_pad, xy32, z32, xy64, z64, ctx->d_bad);
-    // Z-order the FP32 copy and box every tile. Non-finite inputs go through like any others; the
+    // Order the FP32 copy along the curve and box every tile. Non-finite inputs go through like any others; the
     // count of them is looked at once, at the end.
     unsigned long long seen[2] = {0, 0};  // non-finite inputs, largest |z|
     bool ok = cudaGetLastError() == cudaSuccess;
     ok = ok && bbox_of(xy32, n, box_scratch, box, 0) == cudaSuccess;
-    ok = ok && morton_keys(nullptr, nullptr, xy32, n, n_pad, box, keys, perm, 0) == cudaSuccess;
+    ok = ok && curve_keys(nullptr, nullptr, xy32, n, n_pad, box, keys, perm, 0) == cudaSuccess;
     ok = ok && radix_sort_pairs(keys, perm, n_pad, sort_tmp, 0) == cudaSuccess;
     if (ok) {
         gather_dataset_kernel<<<blocks, threads>>>(xy32, z32, perm, n, n_pad, nxy2, zz, orig);

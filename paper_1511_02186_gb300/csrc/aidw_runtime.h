@@ -66,7 +66,7 @@ int enqueue_interpolation(aidw_ctx *ctx, const DatasetDev &ds, double r_exp, con
                           const aidw_params &p, const void *qx, const void *qy,
                           const Scratch &sc, void *out, float *out_alpha, int32_t *out_knn,
                           cudaStream_t st, bool profile);
-// The pruned phase 1 (Z-ordered queries, nearest tiles first): whether a call takes it, the
+// The pruned phase 1 (curve-ordered queries, nearest tiles first): whether a call takes it, the
 // plan change it needs (one query block per CTA, no data splits), the scratch it needs beyond
 // scratch_bytes (query ordering), and the enqueue.
 bool use_culled_knn(int precision, const DatasetDev &ds, int64_t m, bool with_idx,
@@ -105,7 +105,7 @@ struct BatchState {
     bool order_in_tz = false;  // pruned units keep their tile order in the phase-2 z buffers
     int grid = 0;
     cudaGraphExec_t graph = nullptr;
-    // Batch-wide query ordering (Z-order within each item).
+    // Batch-wide query ordering (curve order within each item).
     int32_t count = 0;
     int64_t total_q = 0, max_m = 0;
     size_t dyn_smem = 0;

@@ -4,7 +4,7 @@
 // Every item is cut into units that depend only on the item itself (never on what else is in
 // the batch), so an item's result is bit-identical whether it runs alone or in any mix:
 //   phase-1 list
-//     KNN     (item, query block)         pruned phase-1 scan of Z-ordered queries (nearest
+//     KNN     (item, query block)         pruned phase-1 scan of curve-ordered queries (nearest
 //                                         data tiles first), or, for an item with few queries
 //                                         or too many data tiles, 16 queries scanned one per
 //                                         warp; with the selection (Eq. 3-6) fused: the
@@ -17,8 +17,8 @@
 // An item with enough queries runs phase 2 by power classes, as aidw_interpolate does: its KNN
 // units sort the queries into those whose power is the integer alpha_5 and the others, and a
 // WEIGHTS or FINAL unit finds its block in the two from their final counts.
-// Before the persistent kernel, the queries of all items are put in Z-order item by item (one
-// radix sort of keys made of the item's index and the query's Morton cell in its dataset's
+// Before the persistent kernel, the queries of all items are put in curve order item by item (one
+// radix sort of keys made of the item's index and the query's Hilbert key over its dataset's
 // box) so that each KNN unit's block is compact; results go back to the caller's order.
 // Both lists hold the items in decreasing size; CTAs take units from them through two atomic
 // counters, preferring a phase-2 unit whose inputs are complete and taking phase-1 units
@@ -56,8 +56,8 @@ struct BatchItemDev {
     float *part_d2;
     QParamF32 *qparam;
     float *part_sum;
-    const float *sqx, *sqy;  // the item's queries in Z-order
-    const uint32_t *perm;    // Z-order position -> caller's query index
+    const float *sqx, *sqy;  // the item's queries in curve order
+    const uint32_t *perm;    // curve order position -> caller's query index
     int64_t qoff;            // offset of the item in the batch-wide query arrays
     int32_t ntiles, ntiles_p2;  // ntiles_p2 0: one query per warp
     ClassOrder co;       // two power classes in one region of m entries, or cnt null
@@ -399,9 +399,9 @@ f32_batch_kernel(const BatchItemDev *__restrict__ items, const WorkUnit *__restr
 }
 
 // Batch-wide query ordering, step 1: one 32-bit key per query, the item's index in the high
-// item_bits bits and the top bits of the query's Morton key over its item's dataset box below
+// item_bits bits and the top bits of the query's Hilbert key over its item's dataset box below
 // (2^(32 - item_bits) cells: at least 256 x 256 per item), so that one radix sort groups the
-// items and puts each item's queries in Z-order; values are batch-wide positions, and the item
+// items and puts each item's queries in curve order; values are batch-wide positions, and the item
 // of every position is recorded.
 __global__ void batch_keys_kernel(const BatchItemDev *__restrict__ items, int item_bits,
                                   uint32_t *keys, uint32_t *vals, uint32_t *item_of)
@@ -412,7 +412,7 @@ __global__ void batch_keys_kernel(const BatchItemDev *__restrict__ items, int it
     for (int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; q < it.m;
          q += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         const int64_t g = it.qoff + q;
-        keys[g] = hi | (morton_of(it.qx[q], it.qy[q], box) >> item_bits);
+        keys[g] = hi | (hilbert_of(it.qx[q], it.qy[q], box) >> item_bits);
         vals[g] = static_cast<uint32_t>(g);
         item_of[g] = blockIdx.y;
     }
@@ -499,9 +499,10 @@ bool lists_in_sums(int k, const PassPlan &pw)
 // points: 19 ms as one pruned unit, 45 us one per warp), and the item's phase 2 waits for it.
 // Where the queries are dense the block shares the tiles it visits and needs fewer SM cycles.
 // Measured (64 uneven datasets in one launch / a burst of 24 served requests against up to 1M
-// points, ms): pruned from 1,024 queries on 10.39 / 31.9, from 8,192 on 10.36 / 25.0, from 32,768
-// on 10.75 / 21.8; from 8,192 on but one per warp from 131,072 points on 10.34 / 22.0.
-constexpr int64_t kBatchWarpMinPoints = 131072;
+// points, ms): pruned from 8,192 queries on unless the dataset has 65,536 points or more 10.08 /
+// 21.5, 131,072 10.13 / 21.7, 262,144 10.26 / 21.7; pruned from 16,384 queries on 10.21 / 21.6, from
+// 32,768 on 10.33 / 21.3, never 10.59 / 21.6.
+constexpr int64_t kBatchWarpMinPoints = 65536;
 constexpr int64_t kBatchWarpMaxQueries = 131072;
 constexpr int64_t kBatchCullMinQueries = 8192;
 
@@ -769,7 +770,7 @@ int batch_enqueue(aidw_ctx *ctx, const BatchState &bs, cudaStream_t st)
     const BatchItemDev *items = static_cast<const BatchItemDev *>(bs.d_items);
     const int64_t tq = bs.total_q;
     const unsigned gx = static_cast<unsigned>(std::min<int64_t>((bs.max_m + 255) / 256, 64));
-    // Bits for the item index (even, so that the Morton part keeps whole cells), at most 16.
+    // Bits for the item index (even, so that the curve part keeps whole cells), at most 16.
     int item_bits = 0;
     while ((int64_t(1) << item_bits) < bs.count)
         ++item_bits;

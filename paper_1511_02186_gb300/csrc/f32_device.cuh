@@ -277,7 +277,7 @@ __device__ __forceinline__ bool knn_unit(const DatasetDev &ds, int64_t m, int64_
 }
 
 // ---------------------------------------------------------------------------------------------
-// Phase 1 over Z-ordered queries, one CTA per query block and no data splits. The CTA takes the
+// Phase 1 over curve-ordered queries, one CTA per query block and no data splits. The CTA takes the
 // bounding box of its queries, computes for every data tile a lower bound of the squared
 // distance between the two boxes, sorts the tiles by it and, among equal bounds, by the distance
 // between the box centres (bitonic sort in shared memory), and visits them in that order. After
@@ -363,7 +363,7 @@ struct FusedSelect {
     AlphaMap am;
     QParamF32 *qparam;
     float *out_alpha;
-    const uint32_t *perm;  // Z-order position -> caller's query index
+    const uint32_t *perm;  // curve order position -> caller's query index
     ClassOrder co;
     int64_t m;
 };
@@ -547,7 +547,7 @@ struct CullShared {
     int issued;
 };
 
-// Phase-1 unit over one block of Z-ordered queries (qbase..), all data tiles, pruned as above.
+// Phase-1 unit over one block of curve-ordered queries (qbase..), all data tiles, pruned as above.
 // `order` holds ntiles_p2 (a power of two >= ntiles) 64-bit keys in shared memory. Returns false
 // if a tile wait timed out (the error word is then set).
 template <int KP, int Q, bool IDX>
@@ -571,7 +571,7 @@ __device__ __forceinline__ bool knn_cull_unit(const DatasetDev &ds, int64_t m, i
     float2 qxp[H], qyp[H], nthr[H];
     float L[Q][KP];
     float bx0 = CUDART_INF_F, by0 = CUDART_INF_F, bx1 = -CUDART_INF_F, by1 = -CUDART_INF_F;
-    // Each warp takes 32 Q consecutive Z-ordered queries, so its queries have a compact box.
+    // Each warp takes 32 Q consecutive curve-ordered queries, so its queries have a compact box.
     const int64_t wbase = qbase + static_cast<int64_t>(warp) * 32 * Q + lane;
 #pragma unroll
     for (int j = 0; j < Q; ++j) {

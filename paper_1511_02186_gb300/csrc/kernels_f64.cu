@@ -217,14 +217,14 @@ f64_knn_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restrict__
 }
 
 // ---------------------------------------------------------------------------------------------
-// Phase 1 over Z-ordered FP64 queries, pruned as the FP32 path's (one CTA per query block, data
+// Phase 1 over curve-ordered FP64 queries, pruned as the FP32 path's (one CTA per query block, data
 // tiles visited in order of a lower bound of the box-to-box distance, nearest centre first among
 // equal bounds, the block stopping at the first tile beyond its queries' largest k-th distance,
 // each warp skipping tiles beyond its own). Without the kNN output it keeps distances only (the
 // k nearest distances, and so r_obs, do not depend on which of two tied points is kept); with
 // it, it keeps the k smallest pairs (distance, caller index), i.e. ties to the lower index as
 // the caller-order scan with strict "<" has them. A tile's points are gathered from
-// the caller-order FP64 copy through the Z-order map. The tile boxes hold the FP32 coordinates;
+// the caller-order FP64 copy through the order map. The tile boxes hold the FP32 coordinates;
 // widened by 2^-23 of their largest magnitude they contain the FP64 points (FP32 rounding moves a
 // coordinate by at most 2^-24 of it), and the bound is shrunk by 2^-50 to cover its own rounding
 // and that of the exact distance, so no skipped point could have entered a list. Inside a
@@ -469,7 +469,7 @@ f64_knn_cull_kernel(DatasetDev ds, int64_t m, int qpb, int ntiles, int ntiles_p2
 
 // ---------------------------------------------------------------------------------------------
 // FP64 phase 1 with one warp per query (the FP32 form is in f32_device.cuh). warp_walk runs on
-// the FP32 copy of the points (sequential in Z-order, unlike the FP64 copy it maps to) with the
+// the FP32 copy of the points (sequential in curve order, unlike the FP64 copy it maps to) with the
 // query rounded to float, and a point whose FP32 distance is within thr goes into the buffer by
 // its stored position. Only when the buffer is cut are the new candidates read from the FP64 copy
 // and their exact distances formed, as in the other FP64 scans, two a lane at a time. The

@@ -16,7 +16,7 @@
 // the middle of a request.
 //
 // The call takes the same phase-1 route as aidw_interpolate when its scratch fits: up to
-// 32,768 queries one warp per query; above, the pruned scan over Z-ordered queries (the query
+// 32,768 queries one warp per query; above, the pruned scan over curve-ordered queries (the query
 // ordering needs about 24 more bytes per query); otherwise, or when that does not fit, the split
 // scan with as few splits as the area requires.
 #include <mutex>

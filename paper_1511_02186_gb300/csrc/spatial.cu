@@ -1,7 +1,7 @@
-// Spatial ordering helpers: Morton (Z-order) keys, a stable LSD radix sort of (key, value)
+// Spatial ordering helpers: Hilbert-curve keys, a stable LSD radix sort of (key, value)
 // pairs, gathers, bounding boxes.
 //
-// Data points are stored in Z-order so that each 512-point tile covers a compact region with a
+// Data points are stored along a Hilbert curve so that each 512-point tile covers a compact region with a
 // tight bounding box, and every call orders its queries the same way so that each query block
 // is compact too. The phase-1 scan can then visit data tiles nearest-first and skip every tile
 // whose box is provably farther than all of the block's current k-th neighbours. The order
@@ -63,7 +63,7 @@ __global__ void bbox_finish_kernel(const uint32_t *ord4, float4 *box)
 
 // Keys for points (x, y) given as separate float arrays or interleaved pairs; padding slots
 // [n, n_total) get the largest key so they sort last.
-__global__ void morton_keys_kernel(const float *__restrict__ x, const float *__restrict__ y,
+__global__ void curve_keys_kernel(const float *__restrict__ x, const float *__restrict__ y,
                                    const float2 *__restrict__ xy, int64_t n, int64_t n_total,
                                    const float4 *__restrict__ box, uint32_t *keys,
                                    uint32_t *vals)
@@ -75,7 +75,7 @@ __global__ void morton_keys_kernel(const float *__restrict__ x, const float *__r
         if (i < n) {
             const float px = xy ? xy[i].x : x[i];
             const float py = xy ? xy[i].y : y[i];
-            key = morton_of(px, py, b);
+            key = hilbert_of(px, py, b);
         }
         keys[i] = key;
         vals[i] = static_cast<uint32_t>(i);
@@ -285,8 +285,8 @@ __global__ void super_box_kernel(const float4 *__restrict__ tbox, int64_t ntiles
         boxes[s] = b;
 }
 
-// Morton keys of FP64 query coordinates (rounded to FP32 for the key: the key only orders).
-__global__ void morton_keys_f64_kernel(const double *__restrict__ x,
+// Hilbert keys of FP64 query coordinates (rounded to FP32 for the key: the key only orders).
+__global__ void curve_keys_f64_kernel(const double *__restrict__ x,
                                        const double *__restrict__ y, int64_t n,
                                        const float4 *__restrict__ box, uint32_t *keys,
                                        uint32_t *vals)
@@ -294,7 +294,7 @@ __global__ void morton_keys_f64_kernel(const double *__restrict__ x,
     const float4 b = *box;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        keys[i] = morton_of(static_cast<float>(x[i]), static_cast<float>(y[i]), b);
+        keys[i] = hilbert_of(static_cast<float>(x[i]), static_cast<float>(y[i]), b);
         vals[i] = static_cast<uint32_t>(i);
     }
 }
@@ -376,11 +376,11 @@ cudaError_t bbox_of(const float2 *xy, int64_t n, uint32_t *scratch4, float4 *box
     return cudaGetLastError();
 }
 
-cudaError_t morton_keys(const float *x, const float *y, const float2 *xy, int64_t n,
+cudaError_t curve_keys(const float *x, const float *y, const float2 *xy, int64_t n,
                         int64_t n_total, const float4 *box, uint32_t *keys, uint32_t *vals,
                         cudaStream_t st)
 {
-    morton_keys_kernel<<<grid_for(n_total, 256, 4096), 256, 0, st>>>(x, y, xy, n, n_total, box,
+    curve_keys_kernel<<<grid_for(n_total, 256, 4096), 256, 0, st>>>(x, y, xy, n, n_total, box,
                                                                      keys, vals);
     return cudaGetLastError();
 }
@@ -416,10 +416,10 @@ cudaError_t gather_queries(const float *qx, const float *qy, const uint32_t *per
     return cudaGetLastError();
 }
 
-cudaError_t morton_keys_f64(const double *x, const double *y, int64_t n, const float4 *box,
+cudaError_t curve_keys_f64(const double *x, const double *y, int64_t n, const float4 *box,
                             uint32_t *keys, uint32_t *vals, cudaStream_t st)
 {
-    morton_keys_f64_kernel<<<grid_for(n, 256, 4096), 256, 0, st>>>(x, y, n, box, keys, vals);
+    curve_keys_f64_kernel<<<grid_for(n, 256, 4096), 256, 0, st>>>(x, y, n, box, keys, vals);
     return cudaGetLastError();
 }
 

@@ -1,7 +1,7 @@
 // The one-warp-per-query phase-1 scans (FP32 in f32_device.cuh, FP64 in kernels_f64.cu): the walk
 // over the dataset's box hierarchy and the warp's candidate buffer.
 //
-// The dataset's Z-ordered points are grouped three ways, each with a bounding box: 32-tile
+// The dataset's curve-ordered points are grouped three ways, each with a bounding box: 32-tile
 // super-tiles (16,384 points), 512-point tiles and 64-point sub-tiles. A warp first descends to
 // the sub-tile nearest its query (smallest bound, then nearest centre), takes the k-th of its 64
 // distances as an upper bound T of the query's k-th distance, and then visits every other
@@ -13,9 +13,10 @@
 // The scan is latency bound when a call has few queries (one chain of dependent loads per
 // level) and issue bound when it has many. Before, a list was kept sorted across the lanes with
 // every arriving candidate, every next box was picked by a 64-bit minimum across the lanes, and
-// FP64 formed and compared every distance on the FP64 pipe. Phase 1 before / now, us: FP32
-// 1,024 x 1,024 62 / 15, 257 x 300,007 209 / 32, 8,192 x 1M 304 / 57, 32,768 x 1M 860 / 170; FP64
-// 1,024 x 1,024 51 / 25, 8,191 x 131,072 393 / 92, 16,384 x 262,144 797 / 152.
+// FP64 formed and compared every distance on the FP64 pipe. Phase 1 before / now, us (the points
+// along a Hilbert curve since): FP32 1,024 x 1,024 62 / 11, 257 x 300,007 209 / 15, 8,192 x 1M
+// 304 / 27, 32,768 x 1M 860 / 78; FP64 1,024 x 1,024 51 / 18, 8,191 x 131,072 393 / 49, 16,384 x
+// 262,144 797 / 80.
 #pragma once
 
 #include <math_constants.h>
