@@ -34,14 +34,19 @@ UNIT = "pair-evals/s"
 N_DATA = 1 << 20
 M_QUERY = 1 << 20
 L2_FLUSH_BYTES = 256 << 20
-# Algorithmic work per pair-evaluation. Phase 2 (Eq. 1 over all n points) needs, per pair,
-# 2 sub, 1 mul, 1 fma (squared distance), 1 fma (power scale), 1 add, 1 fma (the two sums) and
-# one MUFU lg2 plus one MUFU ex2. Phase 1 is exact but pruned (nearest-first tiles with
-# bounding-box bounds), so it has no per-pair minimum; a step's n * m pair-evaluations are bound
-# by phase 2.
-FP32_OPS_P2, MUFU_OPS_P2 = 7, 2
-FP64_OPS_P2 = 6  # FP64 instructions per pair in the FP64 phase-2 kernel
-FP64X_OPS_P2 = 4  # FP64 instructions per pair in the AIDW_F64X phase-2 kernel (the distance)
+# Algorithmic work per pair-evaluation. Phase 2 (Eq. 1 over all n points) needs, per pair, 2 sub,
+# 1 mul, 1 fma (squared distance), the weight, and 1 add, 1 fma (the two sums). The weight is 1 fma
+# (power scale) with one MUFU lg2 and one ex2, or, for a query whose power is an integer from 1 to
+# 5, one MUFU rsq (rcp for 2) and up to three products; at power 5 the kernel gives 20 of every 32
+# points the rsq form. An SM issues 128 lane-operations a clock, MUFU ones included. Phase 1 is
+# exact but pruned (nearest-first boxes), so it has no per-pair minimum; a step's n * m
+# pair-evaluations are bound by phase 2.
+P2_GENERAL = {"lg2_ex2": (1.0, 9)}  # form: (share of the pairs, issue slots per pair)
+P2_POWER5 = {"rsq": (20 / 32, 10), "lg2_ex2": (12 / 32, 9)}
+P2_POWER2 = {"rsq": (1.0, 7)}
+FP64_OPS_P2 = 4.5  # FP64 instructions per pair in the FP64 phase-2 kernel
+FP64_FLOOR_OPS_P2 = 2  # the two coordinate differences alone
+FP64X_SLOTS_P2 = 197  # instructions per pair in the AIDW_F64X phase-2 kernel (ncu)
 FP64_PIPE_PER_CLK_SM = 2.0  # GB300 FP64 pipe: 1.25 TFLOP/s nominal = 2 DFMA per clk per SM
 LANES_PER_SM = 128  # FP32 lanes and issue slots (4 schedulers x 32) per SM per clock
 
@@ -688,7 +693,6 @@ def run_gpu(args):
     ks = statistics.mean(t.select_ms for t in ktimes)
     kf = statistics.mean(t.finalize_ms for t in ktimes)
     rates = ctx.pipe_rates()
-    shape = ctx.tune_config()
     sm = rates.sm_count
     sm_mhz_peak = 2070.0
     try:
@@ -698,16 +702,16 @@ def run_gpu(args):
         pass
     clk_hz = sm_mhz_peak * 1e6
 
-    def peak_pairs(fp32_ops, mufu_ops):
-        # mufu_ops is one lg2 plus one ex2 per pair when nonzero.
-        mufu_clk = (1.0 / rates.ex2_per_clk_sm + 1.0 / rates.lg2_per_clk_sm) if mufu_ops else 0.0
-        per_pair_clk = max(fp32_ops / LANES_PER_SM, mufu_clk,
-                           (fp32_ops + mufu_ops) / LANES_PER_SM)
+    def peak_pairs(forms):
+        mufu = {"lg2_ex2": 1.0 / rates.ex2_per_clk_sm + 1.0 / rates.lg2_per_clk_sm,
+                "rsq": 1.0 / rates.lg2_per_clk_sm}  # rsq and rcp run at lg2's rate
+        per_pair_clk = max(sum(share * slots for share, slots in forms.values()) / LANES_PER_SM,
+                           sum(share * mufu[f] for f, (share, _) in forms.items()))
         return sm * clk_hz / per_pair_clk
 
-    dominant = "weights"
+    dominant = "weights_class"
     achieved = pairs / (kw / 1e3)
-    peak = peak_pairs(FP32_OPS_P2, MUFU_OPS_P2)
+    peak = peak_pairs(P2_POWER5)
     step_peak = peak
     kernel_sum_s = (kn + kw + ks + kf) / 1e3
 
@@ -742,14 +746,15 @@ def run_gpu(args):
     ctx.set_profiling(False)
     fp64_rate = q64 * wl.n / (e0.elapsed_time(e1) / 1e3)
     # FP64 phase 2 against the FP64 pipe: FP64 instructions per pair of the kernel as written
-    # (distance 4, power scale 1, the weighted sum 1; log2, exp2 and the sum of the weights run
-    # in fixed point on the integer pipe) at 2 per clock per SM, GB300's nominal FP64 rate
-    # (1.25 TFLOP/s) and the pipe's peak that ncu reports.
+    # (differences 2, their squares 2 for three points in four, the weighted sum 1; log2, the
+    # power, exp2, the sum of the weights and the other squares run in fixed point on the integer
+    # pipe) at 2 per clock per SM, GB300's nominal FP64 rate (1.25 TFLOP/s) and the pipe's peak that
+    # ncu reports.
     fp64_w_achieved = q64 * wl.n / (kt64.weights_ms / 1e3)
     fp64_w_peak = sm * clk_hz * FP64_PIPE_PER_CLK_SM / FP64_OPS_P2
 
     # AIDW_F64X (FP64 phase 1 and alpha, double-float phase 2) on a larger query sample, timed
-    # the same way; its phase 2 is bound by the four FP64 instructions of each pair's distance.
+    # the same way; its phase 2 is bound by the instructions an SM issues.
     q64x = 131072
     idx_x = torch.as_tensor(np.random.default_rng(10).choice(wl.m, q64x, replace=False))
     qx64x = torch.as_tensor(wl.qx, dtype=torch.float64, device=dev)[idx_x.to(dev)].contiguous()
@@ -765,7 +770,8 @@ def run_gpu(args):
     ctx.set_profiling(False)
     fp64x_rate = q64x * wl.n / (e0.elapsed_time(e1) / 1e3)
     fp64x_w_achieved = q64x * wl.n / (kt64x.weights_ms / 1e3)
-    fp64x_w_peak = sm * clk_hz * FP64_PIPE_PER_CLK_SM / FP64X_OPS_P2
+    fp64x_w_peak = sm * clk_hz * LANES_PER_SM / FP64X_SLOTS_P2
+    fp64_floor_peak = sm * clk_hz * FP64_PIPE_PER_CLK_SM / FP64_FLOOR_OPS_P2
 
     # End to end through the public API with host buffers: dataset upload (FP64 host arrays),
     # query upload from pinned memory, interpolation, result download.
@@ -789,7 +795,7 @@ def run_gpu(args):
     batched = bench_batched(ctx, max(2, args.steps), args.warmup, dev, stream, peak=peak)
     stress = bench_precision_stress(ctx, dev, stream)
     designs = bench_paper_designs(ctx, dev, stream)
-    idw = bench_standard_idw(ctx, ds, wl, dev, stream, peak)
+    idw = bench_standard_idw(ctx, ds, wl, dev, stream, peak_pairs(P2_POWER2))
     served = None
     if world == 1 or rank == 0:
         sctx = aidw.Context(local)
@@ -829,19 +835,19 @@ def run_gpu(args):
             "plan": {"knn_splits": ktimes[0].splits, "w_splits": ktimes[0].weight_splits,
                      "query_blocks": ktimes[0].query_blocks},
             "roofline": {"bound": "alu",
-                         "kernel": (f"f32_{dominant}_kernel<{shape.queries_per_thread}, "
-                                    f"{shape.tile_points}>"),
+                         "kernel": f"f32_{dominant}_kernel",
                          "achieved": achieved, "peak": peak, "unit": UNIT,
                          "frac": achieved / peak,
-                         "traffic": (measured_traffic(
-                             f"f32_weights_kernel<{shape.queries_per_thread}, "
-                             f"{shape.tile_points}>") if wl.n == N_DATA and wl.m == M_QUERY
-                             else None),
+                         "traffic": (measured_traffic(f"f32_{dominant}_kernel")
+                                     if wl.n == N_DATA and wl.m == M_QUERY else None),
                          "traffic_unit": "bytes per launch (ncu, committed capture)",
                          "peak_basis": (f"{sm} SMs x {sm_mhz_peak:.0f} MHz (max SM clock) / "
-                                        "max(7 FP32 ops / 128 lanes, 1/ex2 + 1/lg2 measured MUFU "
-                                        "rates per clk per SM, 9 instructions / 128 issue slots)"
-                                        " per pair-evaluation of phase 2"),
+                                        "max(9.6 instructions / 128 issue slots, measured MUFU "
+                                        "rates) per pair-evaluation of phase 2 at power 5, which "
+                                        "99 % of this workload's queries have: 20 of 32 pairs "
+                                        "as 6 FP32 ops, rsq and 3 products, 12 as 7 FP32 ops, "
+                                        "lg2 and ex2"),
+                         "peak_any_power": peak_pairs(P2_GENERAL),
                          "step_achieved": pairs / kernel_sum_s, "step_peak": step_peak,
                          "step_frac": (pairs / kernel_sum_s) / step_peak,
                          "step_note": "whole step (all kernels incl. query ordering and the "
@@ -866,31 +872,28 @@ def run_gpu(args):
                                                       "1.25 TFLOP/s; ncu's FP64 pipe peak) / "
                                                       f"{FP64_OPS_P2} FP64 instructions per "
                                                       "pair"),
-                                       "floor_peak": fp64x_w_peak,
-                                       "frac_of_floor": fp64_w_achieved / fp64x_w_peak,
-                                       "floor_basis": (f"the same FP64 pipe at {FP64X_OPS_P2} "
-                                                       "FP64 instructions per pair, the fewest "
-                                                       "a pair needs at the FP64 bar as the "
-                                                       "FP64X design shows (the squared "
-                                                       "distance in FP64, the rest in "
-                                                       "double-float on the FP32 pipes)")}},
+                                       "floor_peak": fp64_floor_peak,
+                                       "frac_of_floor": fp64_w_achieved / fp64_floor_peak,
+                                       "floor_basis": ("the same FP64 pipe at "
+                                                       f"{FP64_FLOOR_OPS_P2} FP64 instructions "
+                                                       "per pair, the fewest a pair needs at "
+                                                       "the FP64 bar as the FP64X design shows "
+                                                       "(the coordinate differences)")}},
             "fp64x_path": {"value": fp64x_rate, "unit": UNIT,
                            "sample": f"{q64x} seeded queries x all {wl.n} data points",
                            "kernel_ms": {"knn_incl_query_ordering": kt64x.knn_ms,
                                          "select": kt64x.select_ms,
                                          "weights": kt64x.weights_ms,
                                          "finalize": kt64x.finalize_ms},
-                           "roofline": {"bound": "fp64", "kernel": "f64x_weights_kernel",
+                           "roofline": {"bound": "alu", "kernel": "f64x_weights_kernel",
                                         "achieved": fp64x_w_achieved, "peak": fp64x_w_peak,
                                         "unit": UNIT, "frac": fp64x_w_achieved / fp64x_w_peak,
                                         "peak_basis": (f"{sm} SMs x {sm_mhz_peak:.0f} MHz x "
-                                                       f"{FP64_PIPE_PER_CLK_SM:g} FP64 "
-                                                       "instructions per clk per SM / "
-                                                       f"{FP64X_OPS_P2} FP64 instructions "
-                                                       "per pair (the squared distance; "
-                                                       "log2, the power, exp2 and the sums "
-                                                       "run in double-float on the FP32 "
-                                                       "pipes)")}},
+                                                       f"{LANES_PER_SM} issue slots per clk per "
+                                                       f"SM / {FP64X_SLOTS_P2} instructions per "
+                                                       "pair (differences in FP64, squares on "
+                                                       "the integer pipe, the rest in "
+                                                       "double-float)")}},
             "e2e": {"value": e2e_val, "unit": UNIT, "h2d_bytes_per_step": h2d,
                     "d2h_bytes_per_step": d2h,
                     "includes": "dataset upload + conversion, query upload, both phases, "

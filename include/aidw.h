@@ -49,15 +49,16 @@ extern "C" {
 /* AIDW_F32C: distances, kNN selection and weights in FP32; the two weighted sums in FP32 with
  * Kahan-compensated merges; alpha mapping (Eq. 2, 4, 5, 6) and the final ratio in FP64.
  * Queries and the output are float arrays.
- * AIDW_F64: every step at double precision or finer: distances, kNN selection, alpha, the
- * power scale, the weighted sum of z and the final ratio in FP64; log2, exp2 and the sum of the
- * weights in 62-bit fixed point on the integer pipe (within about an ulp of the FP64 result).
+ * AIDW_F64: every step at double precision or finer: coordinate differences, kNN selection,
+ * alpha, the weighted sum of z and the final ratio in FP64; in phase 2 log2, the power, exp2, the
+ * sum of the weights and part of the squared distances in 59- to 62-bit fixed point on the integer
+ * pipe.
  * Queries and the output are double arrays.
  * AIDW_F64X (the library's addition; the paper has FP32 and FP64 only): FP64 arrays and the
- * FP64 path's phase 1, neighbour lists and alpha; in phase 2 each pair's squared distance is
- * formed in FP64 and the rest of its work (log2, the power of Eq. 1, both weighted sums) runs
- * in double-float arithmetic (pairs of floats, about 48 bits) on the FP32 pipes, which on
- * GB300 run at 64 times the FP64 rate. Results agree with the FP64 path to about 1e-13
+ * FP64 path's phase 1, neighbour lists and alpha; in phase 2 each pair's coordinate differences
+ * are formed in FP64, their sum of squares in 64-bit integers, and the rest of its work (log2, the
+ * power of Eq. 1, both weighted sums) runs in double-float arithmetic (pairs of floats, about 48
+ * bits) on the FP32 pipes, which on GB300 run at 64 times the FP64 rate. Results agree with the FP64 path to about 1e-13
  * relative to max(|Z|, sum w|z| / sum w); weights below 2^-126 of the nearest point's are
  * dropped. */
 #define AIDW_F32C 0
@@ -154,12 +155,13 @@ int aidw_idw(aidw_ctx *ctx, aidw_dataset ds, const void *qx, const void *qy, int
  * (or runs with CUDA_MODULE_LOADING=EAGER).
  *   qx, qy, out  DEVICE arrays of m floats on the context's device (host arrays are rejected)
  *   p            as for aidw_interpolate; p->precision must be AIDW_F32C
- * Phase 1 takes aidw_interpolate's route when its scratch fits the array: up to 32,768 queries
- * one warp per query (about m * (4k + 24) bytes), above that the pruned scan over queries put
- * along a Hilbert curve (about m * (4k + 49) bytes, m up to about 189,000 at k = 10); otherwise it scans
- * every (query, data point) pair in data splits, which for many queries costs far more (at
- * 131,072 queries x 1M points about 61 ms against 3.4 ms for the pruned scan; phase 2 is the
- * same either way). Limit: the split scan
+ * Phase 1 takes aidw_interpolate's route when its scratch fits the array: one warp per query up to
+ * 32,768 queries, and beyond with at most 1.9 queries per point and 5,000 n^(1/3) queries (about
+ * m * (4k + 24) bytes), else the pruned scan over queries put along a Hilbert curve (about
+ * m * (4k + 49) bytes, m up to about 189,000 at k = 10); otherwise it scans every (query, data
+ * point) pair in data splits, which for many queries costs far more. Phase 2 runs in the queries'
+ * own order (aidw_interpolate sorts large calls by power first, which takes more scratch), so
+ * results agree with aidw_interpolate's within the FP32 tolerance. Limit: the split scan
  * needs about m * (4k + 24) bytes within 16 MiB (m <= 262,144 for k = 10, about 110,000 for
  * k = 32); larger calls return AIDW_ERR_INVALID_ARG. All calls share the one array and it keeps
  * the last call's contents (every element a call reads, it has written first): calls whose

@@ -15,10 +15,11 @@
 // this file's module, and with it the array, on the device, so it belongs at set-up and not in
 // the middle of a request.
 //
-// The call takes the same phase-1 route as aidw_interpolate when its scratch fits: up to
-// 32,768 queries one warp per query; above, the pruned scan over curve-ordered queries (the query
+// The call takes the same phase-1 route as aidw_interpolate when its scratch fits: one warp per
+// query up to that scan's limit; above, the pruned scan over curve-ordered queries (the query
 // ordering needs about 24 more bytes per query); otherwise, or when that does not fit, the split
-// scan with as few splits as the area requires.
+// scan with as few splits as the area requires. Phase 2 by power classes is not taken: its order
+// and its copies of the queries need 60 more bytes per query.
 #include <mutex>
 
 #include "aidw_internal.cuh"
