@@ -111,7 +111,6 @@ struct aidw_ctx {
     size_t in_use = 0;
     int64_t fail_after = -1;
     int *d_err = nullptr;
-    unsigned long long *d_bad = nullptr;
     cudaMemPool_t pool = nullptr;
     void *pinned = nullptr;  // [kPinnedBytes] results of small host-array calls, and the error word
     std::mutex pinned_mu;    // taken without waiting: a second call at once goes without
@@ -311,9 +310,9 @@ struct WeightsCost {
 };
 
 // The split count with the least estimated time among those that give every SM about 1, 2, ...
-// 48 CTAs (at least up to 8 splits): an SM's share of the CTAs (rounded up) times their cost, over the rate a few
-// co-resident CTAs reach, plus a part of one CTA for the uneven end and the cost of the partial
-// sums. Measured (FP32, us with the finalisation; the split count the estimate takes, and
+// 48 CTAs (at least up to 8 splits): an SM's share of the CTAs (rounded up) times their cost, over
+// the rate a few co-resident CTAs reach, plus a part of one CTA for the uneven end and the cost of
+// the partial sums. Measured (FP32, us with the finalisation; the split count the estimate takes, and
 // 2,048-point granules with at most 64 splits before): 1,024 x 1,024: 14 against 29; 257 x
 // 300,007: 57 against 143; 8,192 x 1M: 2,800 against 2,959 (37 splits of 1,216 slots).
 static PassPlan plan_weights(int64_t m, int64_t n_sum, int qpb, int sm_count,
@@ -726,7 +725,8 @@ int enqueue_culled(aidw_ctx *ctx, const DatasetDev &ds, double r_exp, const Plan
         ok = ok && gather_queries_f64(x, y, perm, m, sx, sy, st) == cudaSuccess;
         ok = ok && launch_f64_knn_cull(ds, pl, sx, sy, p.k, sc, ctx->d_err, st) == cudaSuccess;
         marks.at(1);
-        ok = ok && launch_f64_select(pl, p.k, r_exp, am, sc, out_alpha, out_knn, st, perm) == cudaSuccess;
+        ok = ok && launch_f64_select(pl, p.k, r_exp, am, sc, out_alpha, out_knn, st, perm) ==
+                       cudaSuccess;
         marks.at(2);
         ok = ok && (xp ? launch_f64x_weights(ds, pl, sx, sy, sc, ctx->d_err, st)
                        : launch_f64_weights(ds, pl, sx, sy, sc, ctx->d_err, st)) == cudaSuccess;
@@ -1076,7 +1076,6 @@ int aidw_init(aidw_ctx **out, int device, size_t hbm_budget_bytes)
         cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &thr);
     }
     ok = ok && cudaMalloc(&ctx->d_err, sizeof(int)) == cudaSuccess;
-    ok = ok && cudaMalloc(&ctx->d_bad, 2 * sizeof(unsigned long long)) == cudaSuccess;
     ok = ok && cudaMemset(ctx->d_err, 0, sizeof(int)) == cudaSuccess;
     for (int i = 0; ok && i < 5; ++i)
         ok = cudaEventCreate(&ctx->ev[i]) == cudaSuccess;
@@ -1108,8 +1107,6 @@ int aidw_shutdown(aidw_ctx *ctx)
         cudaFreeHost(ctx->pinned);
     if (ctx->d_err)
         cudaFree(ctx->d_err);
-    if (ctx->d_bad)
-        cudaFree(ctx->d_bad);
     for (int i = 0; i < 5; ++i)
         if (ctx->ev[i])
             cudaEventDestroy(ctx->ev[i]);
@@ -1174,12 +1171,13 @@ int aidw_create_dataset(aidw_ctx *ctx, const void *x, const void *y, const void 
         return AIDW_ERR_OOM;
     }
     // Temporary block: host-array staging (if any), unsorted FP32 copies, sort keys and values,
-    // radix-sort scratch, bounding-box scratch.
+    // radix-sort scratch, bounding-box scratch, the call's own input check words (several threads
+    // may create datasets at once).
     const size_t one = align256(static_cast<size_t>(n) * es);
     const bool stage_host = kx == 0 || ky == 0 || kz == 0;
     const size_t tmp_bytes = (stage_host ? 3 * one : 0) + align256(np * sizeof(float2)) +
                              align256(np * sizeof(float)) + 2 * align256(np * sizeof(uint32_t)) +
-                             align256(radix_scratch_bytes(n_pad)) + 256;
+                             align256(radix_scratch_bytes(n_pad)) + 2 * 256;
     void *tmp = nullptr;
     bool tmp_pooled = false;
     if (dataset_alloc(ctx, tmp_bytes, &tmp, &tmp_pooled) != cudaSuccess) {
@@ -1216,6 +1214,8 @@ int aidw_create_dataset(aidw_ctx *ctx, const void *x, const void *y, const void 
     void *sort_tmp = t;
     t += align256(radix_scratch_bytes(n_pad));
     uint32_t *box_scratch = reinterpret_cast<uint32_t *>(t);
+    t += 256;
+    auto *check = reinterpret_cast<unsigned long long *>(t);
 
     char *b = static_cast<char *>(blk);
     float4 *nxy2 = reinterpret_cast<float4 *>(b);
@@ -1237,20 +1237,20 @@ int aidw_create_dataset(aidw_ctx *ctx, const void *x, const void *y, const void 
     float4 *box = reinterpret_cast<float4 *>(b);
 
     int rc = AIDW_OK;
-    cudaMemset(ctx->d_bad, 0, 2 * sizeof(unsigned long long));
+    cudaMemset(check, 0, 2 * sizeof(unsigned long long));
     const int threads = 256;
     const int blocks = static_cast<int>(std::min<int64_t>((n_pad + threads - 1) / threads,
                                                           ctx->sm_count * 8));
     if (dtype == AIDW_DTYPE_F64)
         convert_dataset_kernel<double><<<blocks, threads>>>(
             static_cast<const double *>(sx), static_cast<const double *>(sy),
-            static_cast<const double *>(sz), n, n_pad, xy32, z32, xy64, z64, ctx->d_bad);
+            static_cast<const double *>(sz), n, n_pad, xy32, z32, xy64, z64, check);
     else
         convert_dataset_kernel<float><<<blocks, threads>>>(
             static_cast<const float *>(sx), static_cast<const float *>(sy),
-            static_cast<const float *>(sz), n, n_pad, xy32, z32, xy64, z64, ctx->d_bad);
-    // Order the FP32 copy along the curve and box every tile. Non-finite inputs go through like any others; the
-    // count of them is looked at once, at the end.
+            static_cast<const float *>(sz), n, n_pad, xy32, z32, xy64, z64, check);
+    // Order the FP32 copy along the curve and box every tile. Non-finite inputs go through like any
+    // others; the count of them is looked at once, at the end.
     unsigned long long seen[2] = {0, 0};  // non-finite inputs, largest |z|
     bool ok = cudaGetLastError() == cudaSuccess;
     ok = ok && bbox_of(xy32, n, box_scratch, box, 0) == cudaSuccess;
@@ -1263,7 +1263,7 @@ int aidw_create_dataset(aidw_ctx *ctx, const void *x, const void *y, const void 
     ok = ok && tile_boxes(nxy2, ntiles, tbox, 0) == cudaSuccess;
     ok = ok && sub_tile_boxes(nxy2, nsub, sbox, 0) == cudaSuccess;
     ok = ok && super_tile_boxes(tbox, ntiles, nsuper, upbox, 0) == cudaSuccess;
-    ok = ok && cudaMemcpy(seen, ctx->d_bad, sizeof(seen), cudaMemcpyDeviceToHost) == cudaSuccess;
+    ok = ok && cudaMemcpy(seen, check, sizeof(seen), cudaMemcpyDeviceToHost) == cudaSuccess;
     ok = ok && cudaDeviceSynchronize() == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
