@@ -68,9 +68,10 @@ struct AlphaMap {
 
 // FP32 copies are stored negated and duplicated, (-x, -x, -y, -y) and (z, z), so that one
 // shared-memory load yields the register pairs that packed FP32x2 instructions operate on for
-// two queries at once (q + (-x) is exactly q - x). They are kept in curve order (along a Hilbert curve of
-// the points), with orig[] mapping a stored position back to the caller's index and one
-// bounding box per 512-point tile. The FP64 copies keep the caller's order.
+// two queries at once (q + (-x) is exactly q - x). They are kept in curve order (along a Hilbert
+// curve of the points), with orig[] mapping a stored position back to the caller's index and one
+// bounding box per 512-point tile. Points packed instead of queries (12 bytes a point, three loads
+// for four of them) measured the same: 18.53 against 18.54 ms at 262,144 x 262,144. The FP64 copies keep the caller's order.
 struct DatasetDev {
     const float4 *nxy2;     // [n_pad] (-x, -x, -y, -y), curve order
     const float2 *zz;       // [n_pad] (z, z), curve order

@@ -159,16 +159,15 @@ __device__ __forceinline__ bool p2_ready(const WorkUnit &wu)
 // What a CTA does next (decided by thread 0, shared through shared memory).
 enum NextKind : int32_t { kExit = 0, kRunP1 = 1, kRunP2 = 2, kWaitP2 = 3 };
 
-// The persistent batch kernel. Units come from two lists: phase 1 (KNN units, with the
-// selection fused into pruned ones, and SELECT units after the split-scan KNN units of their
-// query block) and phase 2 (WEIGHTS units, then FINAL units), both in decreasing item size,
+// The persistent batch kernel. Units come from two lists: phase 1 (KNN units of the pruned scan or
+// of 16 queries at a warp each, with the selection fused in) and phase 2 (WEIGHTS units, then FINAL units), both in decreasing item size,
 // each with its own counter. A CTA takes the next phase-2 unit when its inputs are complete
 // and a phase-1 unit otherwise; a phase-2 unit taken before its inputs are complete is held
 // while the CTA runs phase-1 units, and waited for (bounded) once none are left. With
 // p1_every > 0, every p1_every-th CTA takes phase-1 units first, so phase 1 runs ahead of
 // phase 2 on part of the SMs while the rest run phase 2. A unit only ever waits for units
-// that running CTAs have already taken (phase-1 units never wait for phase 2, a SELECT unit
-// only for earlier phase-1 units, a FINAL unit for WEIGHTS units, all earlier in their list),
+// that running CTAs have already taken (phase-1 units never wait, a WEIGHTS unit
+// for phase-1 units, a FINAL unit for WEIGHTS units earlier in its list),
 // so every wait ends; each is still bounded and raises the error word if it runs out. Which
 // CTA runs a unit never changes its arithmetic.
 // QW: phase-2 queries per thread; tw: phase-2 tile points (256 or 512). LEAN: the variant for

@@ -241,7 +241,8 @@ __device__ __forceinline__ double power_weight(const NormU64 &d2, const FixedPow
         return 0.0;
     }
     const int k = static_cast<int>((y + (1ull << 42)) >> 43);  // round(1024 y)
-    const long long r = static_cast<long long>((y - (static_cast<unsigned long long>(k) << 43)) << 20);
+    const unsigned long long k43 = static_cast<unsigned long long>(k) << 43;
+    const long long r = static_cast<long long>((y - k43) << 20);
     int kk;
     const unsigned long long v = exp2_fixed(neg ? k : -k, neg ? r : -r, t, kk);
     return exp2_round<true>(v, kk, w96);

@@ -392,9 +392,11 @@ cudaError_t launch_f32_select(const Plan &pl, int k, double r_exp, const AlphaMa
     auto fn = pl.knn.splits > 1 ? f32_select_kernel<0>
               : k <= 16         ? f32_select_kernel<16>
                                 : f32_select_kernel<32>;
-    return launch_chained(fn, dim3(static_cast<unsigned>(blocks)), kSelectThreads, 0, st, pl.m, pl.knn.splits, k, r_exp, am, static_cast<const float *>(sc.part_d2),
-        pl.with_idx ? sc.part_idx : nullptr, static_cast<QParamF32 *>(sc.qparam), out_alpha,
-        out_knn, perm, qx, qy, sc.cls);
+    return launch_chained(fn, dim3(static_cast<unsigned>(blocks)), kSelectThreads, 0, st,
+                          pl.m, pl.knn.splits, k, r_exp, am,
+                          static_cast<const float *>(sc.part_d2),
+                          pl.with_idx ? sc.part_idx : nullptr,
+                          static_cast<QParamF32 *>(sc.qparam), out_alpha, out_knn, perm, qx, qy, sc.cls);
 }
 
 cudaError_t launch_f32_knn_warp(const DatasetDev &ds, int64_t m, const float *qx,

@@ -1054,9 +1054,11 @@ cudaError_t launch_f64_select(const Plan &pl, int k, double r_exp, const AlphaMa
     auto fn = pl.knn.splits > 1 ? f64_select_kernel<0>
               : k <= 16         ? f64_select_kernel<16>
                                 : f64_select_kernel<32>;
-    return launch_chained(fn, dim3(static_cast<unsigned>(blocks)), kSelectThreads, 0, st, pl.m, pl.knn.splits, k, r_exp, am, static_cast<const double *>(sc.part_d2),
-        pl.with_idx ? sc.part_idx : nullptr, static_cast<QParamF64 *>(sc.qparam), out_alpha,
-        out_knn, perm);
+    return launch_chained(fn, dim3(static_cast<unsigned>(blocks)), kSelectThreads, 0, st,
+                          pl.m, pl.knn.splits, k, r_exp, am,
+                          static_cast<const double *>(sc.part_d2),
+                          pl.with_idx ? sc.part_idx : nullptr,
+                          static_cast<QParamF64 *>(sc.qparam), out_alpha, out_knn, perm);
 }
 
 template <int KP, bool IDX>

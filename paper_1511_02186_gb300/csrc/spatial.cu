@@ -1,9 +1,9 @@
 // Spatial ordering helpers: Hilbert-curve keys, a stable LSD radix sort of (key, value)
 // pairs, gathers, bounding boxes.
 //
-// Data points are stored along a Hilbert curve so that each 512-point tile covers a compact region with a
-// tight bounding box, and every call orders its queries the same way so that each query block
-// is compact too. The phase-1 scan can then visit data tiles nearest-first and skip every tile
+// Data points are stored along a Hilbert curve so that each 512-point tile covers a compact region
+// with a tight bounding box, and a call that scans by query blocks orders its queries the same way
+// so that each block is compact too. The phase-1 scan can then visit data tiles nearest-first and skip every tile
 // whose box is provably farther than all of the block's current k-th neighbours. The order
 // changes which tiles are read, never the result: the neighbour lists are exact.
 #include <math_constants.h>

@@ -3,9 +3,9 @@
 // GB300 runs FP64 arithmetic at 2 operations per clock per SM, so that the two operations of
 // dx^2 + dy^2 cost a clock; the integer steps here are about 45 of an SM's 128 issue slots a
 // clock. 16,384 x 262,144 with FP64X: 31.9 -> 27.1 ms (2 FP64 operations a pair instead of 4; now
-// 78 % of the issue slots). The differences dx and dy stay FP64 subtractions. Their significands are squared to the
-// high word of the 128-bit product, aligned, added and normalised: the sum is exact to about
-// 2^-59 relative, where the FP64 form rounds it to 2^-52.
+// 78 % of the issue slots). The differences dx and dy stay FP64 subtractions. Their significands
+// are squared to the high word of the 128-bit product, aligned, added and normalised: the sum is
+// exact to about 2^-59 relative, where the FP64 form rounds it to 2^-52.
 #pragma once
 
 #include <cstdint>
