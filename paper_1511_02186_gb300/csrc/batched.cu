@@ -111,7 +111,9 @@ __device__ __noinline__ bool batch_weights_unit(const BatchItemDev *itp, int qbl
 
 // The class form (2 queries per thread, 512-point tiles, whatever the shape): block qblock of the
 // item's general class, then of class A. Which queries a block holds depends on the order in which
-// the KNN units counted them in, a query's own sums do not.
+// the KNN units counted them in, a query's own sums do not. Out of line like the general form
+// (inlined: 64 items of 1,024 to 65,536 queries 10.65 against 10.11 ms, a burst of 24 served
+// requests 22.9 against 21.5).
 struct ClassBlock {
     int cls;      // -1: no such block
     int64_t base, n, col0;
