@@ -308,7 +308,10 @@ __device__ __forceinline__ QParamF32 select_power(float sum, float d1, int k, do
         o.neg_s = -kCoincScaleF32;
         o.c = kCoincScaleF32 * L1;
     } else {
-        const float sh = static_cast<float>(0.5 * alpha);
+        // Kept within [2^-100, 2^100], as the FP64 path keeps it: a power that rounds to 0 would give
+        // a padding point (log2 = inf) a weight of NaN, and one that overflows every point.
+        const float sh = static_cast<float>(
+            fmax(fmin(0.5 * alpha, static_cast<double>(kCoincScaleF32)), 0x1p-100));
         o.neg_s = -sh;
         o.c = sh * L1;
     }
