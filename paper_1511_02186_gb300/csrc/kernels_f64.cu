@@ -729,11 +729,12 @@ f64_select_kernel(int64_t m, int S, int k, double r_exp, AlphaMap am,
     const double alpha = alpha_eq6(mu, am);   // Eq. 6
     if (out_alpha)
         out_alpha[perm ? perm[q] : q] = static_cast<float>(alpha);
-    // kappa kept within [2^-100, 2^100] (beyond, the weights are those of the bounds to far below
-    // the tolerance: all equal, or only the nearest points').
+    // kappa kept within [2^-100, 2^40]: below, all weights are equal; above, any point 2^-29 farther
+    // than the nearest has weight 0, and a larger scale would only magnify the rounding between the
+    // nearest point's distance here and in phase 2 (at 2^62 to a weight of 0 for every point). A
+    // coincidence has no such rounding.
     QParamF64 o;
-    o.kappa = d1 == 0.0 ? kCoincScaleDf
-                        : fmax(fmin(0.5 * alpha, kCoincScaleDf), 1.0 / kCoincScaleDf);
+    o.kappa = d1 == 0.0 ? kCoincScaleDf : fmax(fmin(0.5 * alpha, 0x1p40), 1.0 / kCoincScaleDf);
     o.d1sq = __dadd_rn(d1, kEpsF64);
     qp[q] = o;
 }

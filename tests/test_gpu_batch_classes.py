@@ -68,7 +68,7 @@ def test_levels(ctx, levels):
                 for i, m in enumerate(SIZES)])
 
 
-@pytest.mark.parametrize("precision", [aidw.F32C])
+@pytest.mark.parametrize("precision", [aidw.F32C, aidw.F64, aidw.F64X])
 @pytest.mark.parametrize("level", [1e-50, 1e-300, 1e40, 1e300])
 @pytest.mark.parametrize("m", [301, 7001])
 def test_powers_beyond_fp32(ctx, precision, level, m):
