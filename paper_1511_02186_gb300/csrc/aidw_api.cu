@@ -24,7 +24,8 @@ inline size_t align256(size_t b)
 
 // Converts caller arrays (float or double) into unsorted FP32 staging arrays and the padded
 // FP64 layout, counts non-finite inputs (bad[0]) and takes the largest |z| (the low word of
-// bad[1], a float's bits). FP64 padding points are +inf with value 0.
+// bad[1], a float's bits) and the smallest other than 0 (the high word, the bits' complement, or 0
+// where there is none). FP64 padding points are +inf with value 0.
 template <typename T>
 __global__ void convert_dataset_kernel(const T *__restrict__ x, const T *__restrict__ y,
                                        const T *__restrict__ z, int64_t n, int64_t n_pad,
@@ -34,6 +35,7 @@ __global__ void convert_dataset_kernel(const T *__restrict__ x, const T *__restr
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     unsigned long long nb = 0;
     float zm = 0.0f;
+    unsigned zn = 0;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n_pad;
          i += stride) {
         double a, b, c;
@@ -50,6 +52,8 @@ __global__ void convert_dataset_kernel(const T *__restrict__ x, const T *__restr
             xy32[i] = make_float2(fa, fb);
             z32[i] = fc;
             zm = fmaxf(zm, fabsf(fc));
+            if (fc != 0.0f)
+                zn = max(zn, ~__float_as_uint(fabsf(fc)));
         } else {
             a = b = CUDART_INF;
             c = 0.0;
@@ -61,8 +65,18 @@ __global__ void convert_dataset_kernel(const T *__restrict__ x, const T *__restr
         atomicAdd(bad, nb);
     // Non-negative floats order like their bits.
     const unsigned zb = __reduce_max_sync(0xffffffffu, __float_as_uint(zm));
-    if ((threadIdx.x & 31) == 0)
-        atomicMax(reinterpret_cast<unsigned *>(bad + 1), zb);
+    const unsigned znb = __reduce_max_sync(0xffffffffu, zn);
+    __shared__ unsigned most[2];
+    if (threadIdx.x < 2)
+        most[threadIdx.x] = 0;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(&most[0], zb);
+        atomicMax(&most[1], znb);
+    }
+    __syncthreads();
+    if (threadIdx.x < 2)
+        atomicMax(reinterpret_cast<unsigned *>(bad + 1) + threadIdx.x, most[threadIdx.x]);
 }
 
 // Writes the curve-ordered FP32 layout: stored position i holds caller point perm[i] (padding
@@ -390,6 +404,20 @@ bool power_classes_fit(int64_t n, float z_max)
     return static_cast<double>(n) * z_max <= 0x1p62;
 }
 
+// The class loops sum unscaled products: adding one errs by up to 2^-150 where the sum is subnormal,
+// which is 2^(c - 150) on the scale where the nearest point's weight is 1, and n times that in all.
+// With c <= 84 - log2 n + log2 z_min it is below 2^-66 z_min, so below FP32 rounding even where
+// every value near the query is 0 and the first other one has a weight of 2^-40 (the general loop's
+// products underflow only below a weight of 2^-126 / |z|).
+float class_c_max(const DatasetDev &ds)
+{
+    if (!(ds.z_min < INFINITY))
+        return kClassMaxLog2;
+    const double c = 84.0 - std::log2(static_cast<double>(ds.n)) +
+                     std::log2(static_cast<double>(ds.z_min));
+    return static_cast<float>(std::min<double>(kClassMaxLog2, c));
+}
+
 int integer_level(double a)
 {
     return a >= 1.0 && a <= 5.0 && a == std::floor(a) ? static_cast<int>(a) : 0;
@@ -402,7 +430,7 @@ static int kp_bucket(int kp)
 
 Plan make_plan(aidw_ctx *ctx, int precision, int64_t n, int64_t n_pad, int64_t m, int k,
                bool with_idx, int force_knn_splits, int force_w_splits,
-               const aidw_tune_config *cfg, const aidw_params *classes, float z_max)
+               const aidw_tune_config *cfg, const aidw_params *classes, const DatasetDev *ds)
 {
     const aidw_tune_config &tc = cfg ? *cfg : ctx->tune;
     const bool f64 = f64_arrays(precision);
@@ -418,7 +446,8 @@ Plan make_plan(aidw_ctx *ctx, int precision, int64_t n, int64_t n_pad, int64_t m
     if (!ks)
         ks = f64 ? f64_knn_slots_per_sm(k, with_idx) : f32_knn_slots_per_sm(pl.kp, with_idx);
     pl.pg = weights_point_groups(precision, m);
-    if (classes && precision == AIDW_F32C && use_power_classes(n, m, z_max)) {
+    if (classes && precision == AIDW_F32C && use_power_classes(n, m, ds->z_max)) {
+        pl.c_max = class_c_max(*ds);
         pl.pow_a = integer_level(classes->alpha[4]);
         pl.pow_b = integer_level(classes->alpha[0]);
         if (pl.pow_a || pl.pow_b) {
@@ -508,6 +537,7 @@ void scratch_carve(void *base, int precision, const Plan &pl, int k, Scratch *s)
         s->cls.qp = reinterpret_cast<QParamF32 *>(p);
         s->cls.pow_a = pl.pow_a;
         s->cls.pow_b = pl.pow_b;
+        s->cls.c_max = pl.c_max;
     }
 }
 
@@ -894,7 +924,7 @@ int interpolate_impl(aidw_ctx *ctx, aidw_dataset dsid, const void *qx, const voi
     for (int w_splits = force_w_splits;;) {
         pl = make_plan(ctx, p->precision, ds.n, ds.n_pad, m, p->k, out_knn != nullptr,
                        force_knn_splits > 0 ? force_knn_splits : 0, w_splits, cfg,
-                       classes ? p : nullptr, ds.z_max);
+                       classes ? p : nullptr, &ds);
         cull = force_cull || (!warp && force_knn_splits == 0 &&
                               use_culled_knn(p->precision, ds, m, out_knn != nullptr, pl));
         if (cull)
@@ -1251,7 +1281,7 @@ int aidw_create_dataset(aidw_ctx *ctx, const void *x, const void *y, const void 
             static_cast<const float *>(sz), n, n_pad, xy32, z32, xy64, z64, check);
     // Order the FP32 copy along the curve and box every tile. Non-finite inputs go through like any
     // others; the count of them is looked at once, at the end.
-    unsigned long long seen[2] = {0, 0};  // non-finite inputs, largest |z|
+    unsigned long long seen[2] = {0, 0};  // non-finite inputs, largest and smallest |z|
     bool ok = cudaGetLastError() == cudaSuccess;
     ok = ok && bbox_of(xy32, n, box_scratch, box, 0) == cudaSuccess;
     ok = ok && curve_keys(nullptr, nullptr, xy32, n, n_pad, box, keys, perm, 0) == cudaSuccess;
@@ -1291,6 +1321,8 @@ int aidw_create_dataset(aidw_ctx *ctx, const void *x, const void *y, const void 
     rec.dev.n_pad = n_pad;
     const uint32_t z_bits = static_cast<uint32_t>(seen[1]);
     std::memcpy(&rec.dev.z_max, &z_bits, sizeof(z_bits));
+    const uint32_t zn = static_cast<uint32_t>(seen[1] >> 32), zn_bits = zn ? ~zn : 0x7f800000u;
+    std::memcpy(&rec.dev.z_min, &zn_bits, sizeof(zn_bits));
     rec.block = blk;
     rec.pooled = blk_pooled;
     rec.bytes = bytes;

@@ -54,7 +54,8 @@ inline int finalize_threads(int splits, int64_t m)
 {
     return splits >= 64 && m <= 2048 ? 32 : (splits >= 16 ? 8 : 1);
 }
-// Largest |log2 of d1^power| of a query in an integer power class.
+// Largest |log2 of d1^power| of a query in an integer power class (class_c_max: less where values
+// are small).
 constexpr float kClassMaxLog2 = 64.0f;
 // Fewest queries of a batch item whose phase 2 runs by power classes.
 constexpr int64_t kBatchClassMinQueries = 4096;
@@ -85,6 +86,7 @@ struct DatasetDev {
     int64_t n;
     int64_t n_pad;
     float z_max;            // largest |z| of the FP32 copy
+    float z_min;            // smallest |z| of it other than 0 (+inf: all are 0)
 };
 
 // How one scan pass is cut into work: query blocks (one CTA each) times data-range splits,
@@ -109,6 +111,7 @@ struct Plan {
     int pg;        // phase 2: point groups per CTA (1: every thread sees every point)
     int pow_a;     // FP32 phase 2 by power classes: the integer powers of the two saturated levels
     int pow_b;     // of Eq. 6 (0: none); both 0: phase 2 runs in the queries' own order
+    float c_max;   // ClassOrder::c_max
 };
 
 // Per-query parameters of phase 2 produced by the selection kernel.
@@ -134,6 +137,7 @@ struct ClassOrder {
     QParamF32 *qp;  // [kClasses][m]
     uint32_t *id;   // [kClasses][m] caller's query index
     int pow_a, pow_b;
+    float c_max;    // largest log2 of d1^power in class A or B
 };
 
 // Scratch buffers of one interpolation (device memory owned by the library or by the
@@ -149,6 +153,8 @@ struct Scratch {
 // Whether the unscaled sums of the integer power classes stay in range for a dataset, and a level
 // of Eq. 6 as an integer power the class loops are built for (0: none).
 bool power_classes_fit(int64_t n, float z_max);
+// Largest log2 of d1^power for which a dataset's products d^-power z stay clear of underflow.
+float class_c_max(const DatasetDev &ds);
 int integer_level(double a);
 size_t scratch_bytes(int precision, const Plan &pl, int k);
 void scratch_carve(void *base, int precision, const Plan &pl, int k, Scratch *s);

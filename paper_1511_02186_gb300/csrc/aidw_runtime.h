@@ -50,11 +50,11 @@ int pointer_kind(const void *p, int device);
 int validate_params(const aidw_params *p, int64_t n);
 AlphaMap alpha_map(const aidw_params &p);
 // Shape from `cfg`, or from the context's shape when cfg is null. With `classes` (the call's
-// parameters) FP32 phase 2 may run by power classes; z_max is the dataset's largest |z|.
+// parameters and its dataset) FP32 phase 2 may run by power classes.
 Plan make_plan(aidw_ctx *ctx, int precision, int64_t n, int64_t n_pad, int64_t m, int k,
                bool with_idx, int force_knn_splits, int force_w_splits,
                const aidw_tune_config *cfg = nullptr, const aidw_params *classes = nullptr,
-               float z_max = 0.0f);
+               const DatasetDev *ds = nullptr);
 aidw_tune_config ctx_tune(aidw_ctx *ctx);
 void ctx_set_tune(aidw_ctx *ctx, const aidw_tune_config &c);
 int interpolate_impl(aidw_ctx *ctx, int64_t dsid, const void *qx, const void *qy, int64_t m,

@@ -711,6 +711,7 @@ int batch_build(aidw_ctx *ctx, const aidw_batch_item *items, int32_t count, cuda
         if (d.co.pow_a) {
             // The ordering's keys, values and item numbers are free once the queries are gathered.
             d.co.cnt = c;
+            d.co.c_max = class_c_max(d.ds);
             d.co.qx = reinterpret_cast<float *>(bs->vals + d.qoff);
             d.co.qy = reinterpret_cast<float *>(bs->item_of + d.qoff);
             d.co.id = bs->keys + d.qoff;

@@ -334,16 +334,16 @@ __device__ __forceinline__ QParamF32 select_params(const float *d, int k, double
     return select_power(v[0], d[0], k, r_exp, am, alpha_out);
 }
 
-// A query's power class. Integer powers take the class loop where 2^c = d1^power (and with it
-// every unscaled weight d^-power) stays within 2^+-kClassMaxLog2.
-__device__ __forceinline__ int power_class(const QParamF32 &p, int pow_a, int pow_b)
+// A query's power class. Integer powers take the class loop where c = log2 d1^power, and with it
+// every unscaled weight d^-power, stays within [-kClassMaxLog2, co.c_max]. A pow_b of 0 is none.
+__device__ __forceinline__ int power_class(const QParamF32 &p, const ClassOrder &co, int pow_b)
 {
-    if (!(fabsf(p.c) <= kClassMaxLog2))
+    if (!(p.c >= -kClassMaxLog2 && p.c <= co.c_max))
         return kClassG;  // also NaN, and a query on a data point
     const float twice = -2.0f * p.neg_s;
-    return twice == static_cast<float>(pow_a)   ? kClassA
-           : twice == static_cast<float>(pow_b) ? kClassB
-                                                : kClassG;
+    return twice == static_cast<float>(co.pow_a)             ? kClassA
+           : pow_b > 0 && twice == static_cast<float>(pow_b) ? kClassB
+                                                             : kClassG;
 }
 
 // The next place of class cls, counted in cnt: the threads here together take consecutive ones.
@@ -382,7 +382,7 @@ __device__ __forceinline__ void fused_select_store(const QParamF32 &p, double al
         fs.qparam[q] = p;
         return;
     }
-    const int cls = power_class(p, fs.co.pow_a, 0);
+    const int cls = power_class(p, fs.co, 0);
     const int64_t at = class_place(fs.co.cnt, cls);
     const int64_t o = cls == kClassA ? at : fs.m - 1 - at;
     fs.co.qx[o] = x;

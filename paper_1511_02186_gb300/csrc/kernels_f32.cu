@@ -68,7 +68,7 @@ f32_select_kernel(int64_t m, int S, int k, double r_exp, AlphaMap am,
     // Each query to the next place of its class (a warp's queries stay together).
     if (q < m) {
         const QParamF32 p = qp[q];
-        const int cls = power_class(p, co.pow_a, co.pow_b);
+        const int cls = power_class(p, co, co.pow_b);
         const int64_t o = static_cast<int64_t>(cls) * m + class_place(co.cnt, cls);
         co.qx[o] = qx[q];
         co.qy[o] = qy[q];
