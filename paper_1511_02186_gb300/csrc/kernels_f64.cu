@@ -27,6 +27,7 @@ constexpr int kTileW64 = 256;  // FP64 phase-2 tile (points), beside 72 KB of ta
 // (ms): 1,024 threads with 1 query each 10.6, 512 with 2 11.8, 256 with 4 11.4, 640 and 768 with 2
 // 12.2 and 11.9.
 constexpr int kThreadsW64 = 1024;
+constexpr int kTinySquare = -900;
 
 __device__ __forceinline__ double dist2_exact(double qx, double qy, double px, double py)
 {
@@ -735,7 +736,7 @@ f64_select_kernel(int64_t m, int S, int k, double r_exp, AlphaMap am,
     // coincidence has no such rounding.
     QParamF64 o;
     o.kappa = d1 == 0.0 ? kCoincScaleDf : fmax(fmin(0.5 * alpha, 0x1p40), 1.0 / kCoincScaleDf);
-    o.d1sq = __dadd_rn(d1, kEpsF64);
+    o.d1sq = fmax(d1, kEpsF64);
     qp[q] = o;
 }
 
@@ -755,7 +756,7 @@ __device__ __forceinline__ void fixed_to_doubles(unsigned __int128 v, double &hi
     lo = __ll2double_rn(dA) * 0x1p-32 + __ull2double_rn(B) * 0x1p-96;
 }
 
-// One CTA of 512 threads per SM (12 KB of 256-point tiles plus 72 KB of tables).
+// One CTA of 1,024 threads per SM (12 KB of 256-point tiles plus 72 KB of tables).
 // With PG point groups the CTA serves Q kThreadsW64 / PG queries: each group sums its own part of
 // every chunk and the groups' sums are merged at the end (a call with few queries fills its CTAs
 // that way). Only the chunks up to the last real point are summed.
@@ -851,9 +852,13 @@ f64_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restri
 #pragma unroll
                     for (int j = 0; j < Q; ++j) {
                         const double dx = __dsub_rn(qxr[j], p.x), dy = __dsub_rn(qyr[j], p.y);
-                        const NormU64 d2 =
-                            (u & 3) == 3 ? sum_of_squares(dx, dy)
-                                         : norm_of(__fma_rn(dx, dx, __fma_rn(dy, dy, kEpsF64)));
+                        // Both forms are max(dx^2 + dy^2, kEpsF64) where a query may meet them:
+                        // the FP64 one adds kEpsF64, which is absorbed above 2^kTinySquare.
+                        NormU64 d2;
+                        if ((u & 3) != 3)
+                            d2 = norm_of(__fma_rn(dx, dx, __fma_rn(dy, dy, kEpsF64)));
+                        if ((u & 3) == 3 || d2.e < kTinySquare)
+                            d2 = sum_of_squares(dx, dy);
                         unsigned __int128 w96;
                         const double w = f64math::power_weight(d2, fp[j], tabs, &w96);
                         aw[j] += w96;
