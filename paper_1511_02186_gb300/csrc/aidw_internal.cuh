@@ -262,6 +262,10 @@ cudaError_t run_pipe_probe(int sm_count, aidw_pipe_rates *out);
 // may start once every block of the kernel before it has started (grid_trigger), and waits
 // (grid_wait) for that kernel to finish before it touches anything but the dataset and constant
 // tables: launch latency, block start-up and table loads overlap the tail of the kernel before.
+// What an earlier kernel of the chain or of the stream writes (the caller's queries among it) is
+// read with __ldcg or through a pointer without __restrict__: a plain load of a const __restrict__
+// array may become a read-only load, which wants the array unchanged from the kernel's start on,
+// and that may now come before the array is written.
 // A kernel without grid_trigger releases the next one when its blocks end: the FP64 phase 1 and
 // selection, which the next kernel's large blocks would crowd (FP64 1,024 x 1,024: 74 us without
 // chaining, 63 us chained, 80 us with triggers there too; FP32 1,024 x 1,024: 37 and 33 us).

@@ -801,7 +801,7 @@ __device__ __forceinline__ void select_query(int64_t q, int64_t m, int S, int k,
                                              float *out_alpha, int32_t *out_knn,
                                              const uint32_t *perm = nullptr)
 {
-    const int64_t qo = perm ? static_cast<int64_t>(perm[q]) : q;  // caller's query index
+    const int64_t qo = perm ? static_cast<int64_t>(__ldcg(perm + q)) : q;  // caller's query index
     int cur[kMaxSplits];
     float hd[kMaxSplits];
     int32_t hi[kMaxSplits];
@@ -868,7 +868,7 @@ __device__ __forceinline__ void select_query_one(int64_t q, int64_t m, int k, do
                                                  float *out_alpha, int32_t *out_knn,
                                                  const uint32_t *perm)
 {
-    const int64_t qo = perm ? static_cast<int64_t>(perm[q]) : q;  // caller's query index
+    const int64_t qo = perm ? static_cast<int64_t>(__ldcg(perm + q)) : q;  // caller's query index
     if (out_knn) {
         for (int r = 0; r < k; ++r)
             out_knn[qo * k + r] = __ldcg(part_idx + static_cast<int64_t>(r) * m + q);

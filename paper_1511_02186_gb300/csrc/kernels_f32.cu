@@ -70,10 +70,10 @@ f32_select_kernel(int64_t m, int S, int k, double r_exp, AlphaMap am,
         const QParamF32 p = qp[q];
         const int cls = power_class(p, co, co.pow_b);
         const int64_t o = static_cast<int64_t>(cls) * m + class_place(co.cnt, cls);
-        co.qx[o] = qx[q];
-        co.qy[o] = qy[q];
+        co.qx[o] = __ldcg(qx + q);
+        co.qy[o] = __ldcg(qy + q);
         co.qp[o] = p;
-        co.id[o] = perm ? perm[q] : static_cast<uint32_t>(q);
+        co.id[o] = perm ? __ldcg(perm + q) : static_cast<uint32_t>(q);
     }
 }
 
@@ -82,9 +82,9 @@ f32_select_kernel(int64_t m, int S, int k, double r_exp, AlphaMap am,
 // lists [k][m], for the selection kernel, which amortises its FP64 work over a thread per query.
 template <bool IDX>
 __global__ void __launch_bounds__(kThreads)
-f32_knn_warp_kernel(DatasetDev ds, int64_t m, const float *__restrict__ qx,
-                    const float *__restrict__ qy, int k, float *__restrict__ part_d2,
-                    int32_t *__restrict__ part_idx, uint32_t *cls_cnt)
+f32_knn_warp_kernel(DatasetDev ds, int64_t m, const float *qx, const float *qy, int k,
+                    float *__restrict__ part_d2, int32_t *__restrict__ part_idx,
+                    uint32_t *cls_cnt)
 {
     grid_trigger();
     grid_wait();
@@ -248,13 +248,13 @@ f32_finalize_kernel(int64_t m, int S, const float *__restrict__ part_sum,
     }
     if (q >= m)
         return;
-    int64_t o = perm ? static_cast<int64_t>(perm[q]) : q;
+    int64_t o = perm ? static_cast<int64_t>(__ldcg(perm + q)) : q;
     if (co.cnt) {
         // Column q of the class order: the general class, class A, class B.
-        const int64_t ng = co.cnt[kClassG], na = co.cnt[kClassA];
-        o = co.id[q < ng        ? kClassG * m + q
-                  : q < ng + na ? kClassA * m + (q - ng)
-                                : kClassB * m + (q - ng - na)];
+        const int64_t ng = __ldcg(co.cnt + kClassG), na = __ldcg(co.cnt + kClassA);
+        o = __ldcg(co.id + (q < ng        ? kClassG * m + q
+                            : q < ng + na ? kClassA * m + (q - ng)
+                                          : kClassB * m + (q - ng - na)));
     }
     out[o] = static_cast<float>(WZ / W);
 }

@@ -631,8 +631,8 @@ struct WarpNearest64 {
 // One warp per query (grid-stride over the queries, caller order); writes one split's lists
 // [k][m] (distances, and caller indices when part_idx is not null) for f64_select_kernel.
 __global__ void __launch_bounds__(kThreads)
-f64_knn_warp_kernel(DatasetDev ds, int64_t m, const double *__restrict__ qx,
-                    const double *__restrict__ qy, int k, double *__restrict__ part_d2,
+f64_knn_warp_kernel(DatasetDev ds, int64_t m, const double *qx,
+                    const double *qy, int k, double *__restrict__ part_d2,
                     int32_t *__restrict__ part_idx)
 {
     constexpr int W = kThreads / 32;
@@ -697,15 +697,16 @@ __device__ __forceinline__ void merge_lists64(int64_t q, int64_t m, int S, int k
 template <int KP>
 __global__ void __launch_bounds__(kSelectThreads)
 f64_select_kernel(int64_t m, int S, int k, double r_exp, AlphaMap am,
-                  const double *__restrict__ part_d2, const int32_t *__restrict__ part_idx,
-                  QParamF64 *__restrict__ qp, float *__restrict__ out_alpha,
-                  int32_t *__restrict__ out_knn, const uint32_t *__restrict__ perm)
+                  const double *part_d2, const int32_t *part_idx, QParamF64 *__restrict__ qp,
+                  float *__restrict__ out_alpha, int32_t *__restrict__ out_knn,
+                  const uint32_t *perm)
 {
     grid_wait();
     const int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (q >= m)
         return;
-    int32_t *knn = out_knn ? out_knn + (perm ? static_cast<int64_t>(perm[q]) : q) * k : nullptr;
+    const int64_t qo = perm ? static_cast<int64_t>(perm[q]) : q;  // caller's query index
+    int32_t *knn = out_knn ? out_knn + qo * k : nullptr;
     double r_sum = 0.0, d1 = 0.0;
     if constexpr (KP > 0) {
         double v[KP];
@@ -713,8 +714,14 @@ f64_select_kernel(int64_t m, int S, int k, double r_exp, AlphaMap am,
         for (int r = 0; r < KP; ++r)
             v[r] = r < k ? part_d2[static_cast<int64_t>(r) * m + q] : 0.0;
         if (knn) {
-            for (int r = 0; r < k; ++r)
-                knn[r] = part_idx[static_cast<int64_t>(r) * m + q];
+            int32_t id[KP];  // every load before the first store
+#pragma unroll
+            for (int r = 0; r < KP; ++r)
+                id[r] = r < k ? part_idx[static_cast<int64_t>(r) * m + q] : 0;
+#pragma unroll
+            for (int r = 0; r < KP; ++r)
+                if (r < k)
+                    knn[r] = id[r];
         }
         d1 = v[0];
 #pragma unroll
@@ -729,7 +736,7 @@ f64_select_kernel(int64_t m, int S, int k, double r_exp, AlphaMap am,
     const double mu = membership_eq5(R, am);  // Eq. 5
     const double alpha = alpha_eq6(mu, am);   // Eq. 6
     if (out_alpha)
-        out_alpha[perm ? perm[q] : q] = static_cast<float>(alpha);
+        out_alpha[qo] = static_cast<float>(alpha);
     // kappa kept within [2^-100, 2^40]: below, all weights are equal; above, any point 2^-29 farther
     // than the nearest has weight 0, and a larger scale would only magnify the rounding between the
     // nearest point's distance here and in phase 2 (at 2^62 to a weight of 0 for every point). A
@@ -762,8 +769,8 @@ __device__ __forceinline__ void fixed_to_doubles(unsigned __int128 v, double &hi
 // that way). Only the chunks up to the last real point are summed.
 template <int Q, int PG>
 __global__ void __launch_bounds__(kThreadsW64, 1)
-f64_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restrict__ qx,
-                   const double *__restrict__ qy, const QParamF64 *__restrict__ qp,
+f64_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *qx,
+                   const double *qy, const QParamF64 *qp,
                    double *__restrict__ part_sum, int *__restrict__ err)
 {
     __shared__ __align__(128) double2 txy[2][kTileW64];
@@ -921,8 +928,8 @@ f64_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restri
 // R threads per query, as f32_finalize_kernel's.
 template <int R>
 __global__ void __launch_bounds__(256)
-f64_finalize_kernel(int64_t m, int S, const double *__restrict__ part_sum,
-                    double *__restrict__ out, const uint32_t *__restrict__ perm)
+f64_finalize_kernel(int64_t m, int S, const double *part_sum, double *__restrict__ out,
+                    const uint32_t *perm)
 {
     grid_trigger();
     grid_wait();

@@ -27,8 +27,8 @@ __device__ __forceinline__ void drain_x(uint64_t *bar, int t, int ntiles)
 // FP64 finalisation adds up.
 template <int Q, int PG>
 __global__ void __launch_bounds__(kThreads)
-f64x_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *__restrict__ qx,
-                    const double *__restrict__ qy, const QParamF64 *__restrict__ qp,
+f64x_weights_kernel(DatasetDev ds, int64_t m, PassPlan pp, const double *qx,
+                    const double *qy, const QParamF64 *qp,
                     double *__restrict__ part_sum, int *__restrict__ err)
 {
     __shared__ __align__(128) double2 txy[2][kTileF64W];
