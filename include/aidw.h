@@ -108,7 +108,8 @@ int aidw_shutdown(aidw_ctx *ctx);
  * dtype is AIDW_DTYPE_F32 or AIDW_DTYPE_F64 for all three arrays.
  * Errors: INVALID_ARG if n < 1, n > 2^31 - 2048, area is not finite and > 0, or any x, y, z
  * is NaN or infinite (checked on the device after the copy); OOM if the memory or the budget
- * runs out. This call is synchronous. */
+ * runs out. This call is synchronous; with device arrays it first waits for the device, so that
+ * work already enqueued on any stream that writes them is done. */
 int aidw_create_dataset(aidw_ctx *ctx, const void *x, const void *y, const void *z, int64_t n,
                         double area, int32_t dtype, aidw_dataset *out);
 

@@ -1165,6 +1165,9 @@ int aidw_create_dataset(aidw_ctx *ctx, const void *x, const void *y, const void 
     const int kz = pointer_kind(z, ctx->device);
     if (kx < 0 || ky < 0 || kz < 0)
         return AIDW_ERR_INVALID_ARG;
+    // Device arrays may still be written on a stream that the legacy one does not wait for.
+    if ((kx == 1 || ky == 1 || kz == 1) && cudaDeviceSynchronize() != cudaSuccess)
+        return AIDW_ERR_CUDA;
     const size_t es = dtype == AIDW_DTYPE_F64 ? sizeof(double) : sizeof(float);
     const int64_t n_pad = (n + kPadPoints - 1) / kPadPoints * kPadPoints;
     const size_t np = static_cast<size_t>(n_pad);
