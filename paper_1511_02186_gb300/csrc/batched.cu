@@ -552,12 +552,12 @@ size_t batch_lists_bytes(bool cull, int k, const PassPlan &pw, int64_t m)
                : align256(static_cast<size_t>(k) * static_cast<size_t>(m) * sizeof(float));
 }
 
-size_t batch_item_bytes(int64_t n_pad, int64_t m, int k, const aidw_tune_config &cfg)
+// Device bytes of an item with qpt queries per thread in phase 2.
+static size_t item_bytes(int64_t n_pad, int64_t m, int k, const aidw_tune_config &cfg, int qpt)
 {
     bool cull;
     const int kp = kp_for(k, cfg.knn_list);
-    const PassPlan pw = batch_w_plan(m, n_pad, kThreads * cfg.queries_per_thread,
-                                     cfg.split_points);
+    const PassPlan pw = batch_w_plan(m, n_pad, kThreads * qpt, cfg.split_points);
     const PassPlan pk = batch_knn_plan(m, n_pad, k, cull_queries_per_thread(kp,
                                        cfg.knn_queries_per_thread), pw, &cull);
     const size_t mm = static_cast<size_t>(m);
@@ -566,6 +566,14 @@ size_t batch_item_bytes(int64_t n_pad, int64_t m, int k, const aidw_tune_config 
            sizeof(uint32_t) * (kClasses + 1 + pw.qblocks + 1) + sizeof(BatchItemDev) +
            sizeof(WorkUnit) * (pk.qblocks + (pw.qblocks + 1) * (pw.splits + 1)) +
            mm * (6 * sizeof(uint32_t)) + radix_scratch_bytes(m);
+}
+
+// Device bytes an item of any dataset and levels takes: one large enough for the power classes may
+// run by them, with 2 queries per thread whatever the shape, and so with more work units.
+size_t batch_item_bytes(int64_t n_pad, int64_t m, int k, const aidw_tune_config &cfg)
+{
+    const size_t b = item_bytes(n_pad, m, k, cfg, cfg.queries_per_thread);
+    return m < kBatchClassMinQueries ? b : std::max(b, item_bytes(n_pad, m, k, cfg, 2));
 }
 
 // Validates the items and builds the device tables of a batch in library memory.
