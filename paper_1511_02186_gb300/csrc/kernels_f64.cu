@@ -569,7 +569,29 @@ __device__ __noinline__ WarpEntry64 warp_cut64(unsigned long long *bd, int32_t *
     return {kInfBits, INT32_MAX};
 }
 
-// The FP64 visitor of warp_walk.
+// Of the candidates c (one stored position pos a lane), those that precede the pair (td, ti).
+__device__ __noinline__ unsigned warp_precede64(unsigned c, int32_t pos, unsigned long long td,
+                                                int32_t ti, const int32_t *orig,
+                                                const double2 *xy64, double qx, double qy)
+{
+    bool precedes = false;
+    if ((c >> (threadIdx.x & 31)) & 1u) {
+        const int32_t o = orig[pos];
+        if (o >= 0) {
+            const double2 p = xy64[o];
+            const unsigned long long d = static_cast<unsigned long long>(
+                __double_as_longlong(dist2_exact(qx, qy, p.x, p.y)));
+            precedes = d < td || (d == td && o < ti);
+        }
+    }
+    return __ballot_sync(kFullMask, precedes);
+}
+
+// The FP64 visitor of warp_walk. Candidates wait in the buffer for the next cut; once it has
+// overflowed for a query, which a poor first bound or many points at nearly one distance bring
+// about, they are compared exactly with the k-th pair of the last cut first. Otherwise every point
+// of such a distance enters and the buffer is cut every 32 points: 2,048 queries against 262,144
+// points at one location took 70.5 ms, now 15.2 (and 1,024 x 1,024 58.9 us, now 56.0).
 struct WarpNearest64 {
     const int32_t *orig;
     const double2 *xy64;
@@ -581,6 +603,9 @@ struct WarpNearest64 {
     float thr;   // +inf at first
     int sorted;  // entries cut so far
     int cnt;
+    unsigned long long td;  // the k-th pair of the last cut, (+inf, INT32_MAX) if fewer are known
+    int32_t ti;
+    bool crowded;
 
     __device__ __forceinline__ bool usable(float, float4 box) const
     {
@@ -591,8 +616,9 @@ struct WarpNearest64 {
         const WarpEntry64 e = warp_cut64(bd, bi, sorted, cnt, k, orig, xy64, qxd, qyd);
         cnt = min(cnt, k);
         sorted = cnt;
-        const double T = __longlong_as_double(
-            static_cast<long long>(__shfl_sync(kFullMask, e.d, k - 1)));
+        td = __shfl_sync(kFullMask, e.d, k - 1);
+        ti = __shfl_sync(kFullMask, e.i, k - 1);
+        const double T = __longlong_as_double(static_cast<long long>(td));
         const float mag = __fadd_ru(fabsf(qx), fabsf(qy));
         const float r = __fsqrt_ru(__double2float_ru(T));
         const float rt = __fadd_ru(__fmul_ru(r, 1.0f + 0x1p-20f), __fmul_ru(mag, 0x1p-21f));
@@ -611,8 +637,11 @@ struct WarpNearest64 {
             return;
         if (cnt + __popc(c) > kWarpBuffer) {
             cut();
+            crowded = true;
             c = __ballot_sync(kFullMask, !(df > thr));
         }
+        if (crowded)
+            c = warp_precede64(c, pos, td, ti, orig, xy64, qxd, qyd);
         const int lane = threadIdx.x & 31;
         if ((c >> lane) & 1u)
             bi[cnt + __popc(c & ((1u << lane) - 1u))] = pos;
@@ -644,7 +673,7 @@ f64_knn_warp_kernel(DatasetDev ds, int64_t m, const double *qx,
     for (int64_t q = static_cast<int64_t>(blockIdx.x) * W + w; q < m; q += nwarps) {
         const double x = qx[q], y = qy[q];
         WarpNearest64 v{ds.orig, ds.xy64, x, y, static_cast<float>(x), static_cast<float>(y), k,
-                        bd[w], bi[w], CUDART_INF_F, 0, 0};
+                        bd[w], bi[w], CUDART_INF_F, 0, 0, kInfBits, INT32_MAX, false};
         if (!isnan(x) && !isnan(y))  // a NaN query has no neighbours
             warp_walk(ds, v);
         const WarpEntry64 e = v.cut();

@@ -42,7 +42,8 @@ def test_results(precision, k):
         assert all(len(set(row)) == k for row in kn.tolist())
 
 
-@pytest.mark.parametrize("precision,m,most", [(aidw.F32C, 8192, 20.0)])
+@pytest.mark.parametrize("precision,m,most", [(aidw.F32C, 8192, 20.0), (aidw.F64, 2048, 6.0),
+                                              (aidw.F64X, 2048, 8.0)])
 @pytest.mark.parametrize("locations", [1, 3])
 def test_time(precision, m, most, locations):
     import torch
