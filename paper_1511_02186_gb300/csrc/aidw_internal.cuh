@@ -57,8 +57,12 @@ inline int finalize_threads(int splits, int64_t m)
 // Largest |log2 of d1^power| of a query in an integer power class (class_c_max: less where values
 // are small).
 constexpr float kClassMaxLog2 = 64.0f;
-// Fewest queries of a batch item whose phase 2 runs by power classes.
+// Fewest queries and points of a batch item whose phase 2 runs by power classes: a query's share of
+// the sorting does not depend on the points, its gain does (64 items of 16,384 queries, us, with and
+// without: 250 points 510 / 502, 500 693 / 678, 1,000 908 / 910, 2,000 1,273 / 1,318, 4,000 1,951 /
+// 2,007; 256 of 4,096: 522 / 508, 712 / 702, 934 / 933, 1,372 / 1,371, 2,161 / 2,171).
 constexpr int64_t kBatchClassMinQueries = 4096;
+constexpr int64_t kBatchClassMinPoints = 2000;
 constexpr int kPointGroups = 4;  // phase 2 with point groups (Plan::pg)
 
 // Levels and bounds of Eq. 5 and Eq. 6, passed to kernels by value.

@@ -1,14 +1,15 @@
 // Batched AIDW: many independent (dataset, query set) items in one persistent work-queue
 // kernel, launched through a captured CUDA graph.
 //
-// Every item is cut into units that depend only on the item itself (never on what else is in
-// the batch), so an item's result is bit-identical whether it runs alone or in any mix:
+// Every item is cut into units that do the same arithmetic whatever else is in the batch (only
+// which of two exact neighbour scans a KNN unit runs depends on the batch's size), so an item's
+// result is bit-identical whether it runs alone or in any mix:
 //   phase-1 list
 //     KNN     (item, query block)         pruned phase-1 scan of curve-ordered queries (nearest
 //                                         data tiles first), or, for an item with few queries
 //                                         or too many data tiles, 16 queries scanned one per
-//                                         warp; with the selection (Eq. 3-6) fused: the
-//                                         block's phase-2 parameters are ready
+//                                         warp (batch_knn_plan); with the selection (Eq. 3-6)
+//                                         fused: the block's phase-2 parameters are ready
 //   phase-2 list
 //     WEIGHTS (item, query block, split)  phase-2 scan of one data split; needs every query
 //                                         block of its item through selection
@@ -498,14 +499,27 @@ bool lists_in_sums(int k, const PassPlan &pw)
 // scanned one per warp. A pruned unit visits the tiles near its block's queries, on one CTA; with
 // queries sparse in the data that is a large part of the tiles (256 queries against 800,000
 // points: 19 ms as one pruned unit, 45 us one per warp), and the item's phase 2 waits for it.
-// Where the queries are dense the block shares the tiles it visits and needs fewer SM cycles.
-// Measured (64 uneven datasets in one launch / a burst of 24 served requests against up to 1M
-// points, ms): pruned from 8,192 queries on unless the dataset has 65,536 points or more 10.08 /
+// Where the queries are dense the block shares the tiles it visits and needs fewer SM cycles, which
+// is what counts once a batch's queries fill the GPU (kBatchCrowd). Both give the same lists, so
+// which one an item takes changes no bit. Measured, ms, pruned / one per warp (items x queries
+// against points each):
+//   1 x 4,096 : 8,000    0.62 / 0.35      1 x 8,191 : 20,000    0.70 / 0.41
+//   16 x 4,096 : 8,000   0.77 / 0.50      16 x 8,191 : 20,000   1.40 / 1.30
+//   64 x 4,096 : 8,000   1.13 / 1.42      64 x 8,191 : 20,000   3.93 / 4.57
+//   256 x 2,048 : 8,000  2.05 / 2.52      64 x 4,096 : 40,000   4.38 / 4.13
+//   256 x 1,024 : 8,000  1.34 / 1.38      64 x 8,191 : 60,000  10.92 / 11.08
+// and over uneven items (64 datasets in one launch / a burst of 24 served requests against up to
+// 1M points): pruned from 8,192 queries on unless the dataset has 65,536 points or more 10.08 /
 // 21.5, 131,072 10.13 / 21.7, 262,144 10.26 / 21.7; pruned from 16,384 queries on 10.21 / 21.6, from
 // 32,768 on 10.33 / 21.3, never 10.59 / 21.6.
 constexpr int64_t kBatchWarpMinPoints = 65536;
 constexpr int64_t kBatchWarpMaxQueries = 131072;
 constexpr int64_t kBatchCullMinQueries = 8192;
+// Queries of a batch that fill the GPU, and, in such a batch, the fewest queries of an item whose
+// block shares tiles and the most points per query.
+constexpr int64_t kBatchCrowd = 200000;
+constexpr int64_t kBatchCrowdMinQueries = 1024;
+constexpr int64_t kBatchCrowdPointsPerQuery = 5;
 
 // Phase-2 plan of a batch item: data splits of at most split_points points, and, for an item
 // with few queries, enough of them for about kBatchMinWeightUnits units of 256 queries, so
@@ -525,11 +539,14 @@ PassPlan batch_w_plan(int64_t m, int64_t n_pad, int qpb, int64_t split_points)
     return batch_pass(m, n_pad, qpb, std::min<int64_t>(split_points, target));
 }
 
-PassPlan batch_knn_plan(int64_t m, int64_t n_pad, int k, int kq, const PassPlan &pw, bool *cull)
+PassPlan batch_knn_plan(int64_t m, int64_t n_pad, int k, int kq, const PassPlan &pw, bool crowd,
+                        bool *cull)
 {
+    const bool few_points = n_pad < kBatchWarpMinPoints;
     *cull = n_pad / kTileF32Knn <= kMaxCullTiles &&
-            ((m >= kBatchCullMinQueries &&
-              (n_pad < kBatchWarpMinPoints || m > kBatchWarpMaxQueries)) ||
+            ((m >= kBatchCullMinQueries && (few_points || m > kBatchWarpMaxQueries)) ||
+             (crowd && few_points && m >= kBatchCrowdMinQueries &&
+              n_pad <= kBatchCrowdPointsPerQuery * m) ||
              (m >= 1024 && !lists_in_sums(k, pw)));
     return batch_pass(m, n_pad, *cull ? kThreads * kq : kBatchWarpBlock, n_pad);
 }
@@ -537,7 +554,8 @@ PassPlan batch_knn_plan(int64_t m, int64_t n_pad, int k, int kq, const PassPlan 
 // Whether an item runs phase 2 by power classes, and the integer power of its class A (0: no).
 int batch_class_power(int64_t m, const DatasetDev &ds, const aidw_params &p)
 {
-    if (m < kBatchClassMinQueries || !power_classes_fit(ds.n, ds.z_max))
+    if (m < kBatchClassMinQueries || ds.n < kBatchClassMinPoints ||
+        !power_classes_fit(ds.n, ds.z_max))
         return 0;
     const int a = integer_level(p.alpha[4]);
     return a ? a : integer_level(p.alpha[0]);
@@ -552,14 +570,16 @@ size_t batch_lists_bytes(bool cull, int k, const PassPlan &pw, int64_t m)
                : align256(static_cast<size_t>(k) * static_cast<size_t>(m) * sizeof(float));
 }
 
-// Device bytes of an item with qpt queries per thread in phase 2.
-static size_t item_bytes(int64_t n_pad, int64_t m, int k, const aidw_tune_config &cfg, int qpt)
+// Device bytes of an item with qpt queries per thread in phase 2, in a batch that fills the GPU or
+// not.
+static size_t item_bytes(int64_t n_pad, int64_t m, int k, const aidw_tune_config &cfg, int qpt,
+                         bool crowd)
 {
     bool cull;
     const int kp = kp_for(k, cfg.knn_list);
     const PassPlan pw = batch_w_plan(m, n_pad, kThreads * qpt, cfg.split_points);
     const PassPlan pk = batch_knn_plan(m, n_pad, k, cull_queries_per_thread(kp,
-                                       cfg.knn_queries_per_thread), pw, &cull);
+                                       cfg.knn_queries_per_thread), pw, crowd, &cull);
     const size_t mm = static_cast<size_t>(m);
     return batch_lists_bytes(cull, k, pw, m) + align256(mm * sizeof(QParamF32)) +
            align256(pw.splits * 4 * mm * sizeof(float)) +
@@ -568,12 +588,18 @@ static size_t item_bytes(int64_t n_pad, int64_t m, int k, const aidw_tune_config
            mm * (6 * sizeof(uint32_t)) + radix_scratch_bytes(m);
 }
 
-// Device bytes an item of any dataset and levels takes: one large enough for the power classes may
-// run by them, with 2 queries per thread whatever the shape, and so with more work units.
+// Device bytes an item of any dataset and levels takes in any batch: one large enough for the power
+// classes may run by them, with 2 queries per thread whatever the shape, and so with more work
+// units.
 size_t batch_item_bytes(int64_t n_pad, int64_t m, int k, const aidw_tune_config &cfg)
 {
-    const size_t b = item_bytes(n_pad, m, k, cfg, cfg.queries_per_thread);
-    return m < kBatchClassMinQueries ? b : std::max(b, item_bytes(n_pad, m, k, cfg, 2));
+    size_t b = 0;
+    for (bool crowd : {false, true}) {
+        b = std::max(b, item_bytes(n_pad, m, k, cfg, cfg.queries_per_thread, crowd));
+        if (m >= kBatchClassMinQueries)
+            b = std::max(b, item_bytes(n_pad, m, k, cfg, 2, crowd));
+    }
+    return b;
 }
 
 // Validates the items and builds the device tables of a batch in library memory.
@@ -600,6 +626,10 @@ int batch_build(aidw_ctx *ctx, const aidw_batch_item *items, int32_t count, cuda
     int max_p2 = 0;
     // The 64-register kernel serves the batch if every item fits its built-in phase-1 units.
     bool lean = cfg.queries_per_thread == 2;
+    double queries = 0.0;
+    for (int32_t i = 0; i < count; ++i)
+        queries += static_cast<double>(items[i].m);
+    const bool crowd = queries >= static_cast<double>(kBatchCrowd);
     for (int32_t i = 0; i < count; ++i) {
         const aidw_batch_item &b = items[i];
         DatasetDev dev;
@@ -632,7 +662,7 @@ int batch_build(aidw_ctx *ctx, const aidw_batch_item *items, int32_t count, cuda
         d.co.pow_a = batch_class_power(b.m, dev, b.params);
         d.w = batch_w_plan(b.m, dev.n_pad,
                            kThreads * (d.co.pow_a ? 2 : cfg.queries_per_thread), cfg.split_points);
-        d.knn = batch_knn_plan(b.m, dev.n_pad, d.k, d.kq, d.w, &cull);
+        d.knn = batch_knn_plan(b.m, dev.n_pad, d.k, d.kq, d.w, crowd, &cull);
         if (b.m > 0 && (d.kp > 16 || (cull && d.kq != 2)))
             lean = false;
         d.ntiles = static_cast<int32_t>(dev.n_pad / kTileF32Knn);
