@@ -446,39 +446,6 @@ __device__ __forceinline__ double alpha_eq6(double mu, const AlphaMap &am)
     return am.level[seg] * (1.0 - t) + am.level[seg + 1] * t;
 }
 
-// Position on the Hilbert curve of order 16 of the cell (x, y), 0 <= x, y < 65,536: from the top
-// bit down, the quadrant (two bits of the position) and the rest turned into the quadrant's frame.
-__device__ __forceinline__ uint32_t hilbert_index(uint32_t x, uint32_t y)
-{
-    uint32_t d = 0;
-#pragma unroll
-    for (int b = 15; b >= 0; --b) {
-        const uint32_t rx = (x >> b) & 1u, ry = (y >> b) & 1u;
-        d = (d << 2) | ((3u * rx) ^ ry);
-        const uint32_t flip = (rx & ~ry & 1u) ? 0xffffu : 0u;
-        const uint32_t u = x ^ flip, v = y ^ flip;
-        x = ry ? u : v;
-        y = ry ? v : u;
-    }
-    return d;
-}
-
-// Hilbert key of (x, y) on a 65,536 x 65,536 grid over `box` (xmin, ymin, xmax, ymax); points
-// outside the box, or NaN, clamp to its edges. A run of points along the curve never jumps, so
-// its bounding box is compact (a run of the Z-order curve may straddle two far quadrants).
-// Against Z-order a query's walk visits 3 sub-tiles instead of 11 (1M uniform points, k = 10), and
-// phase 1 takes, us, before / now: 257 x 300,007 30 / 15, 8,192 x 1M 57 / 27, 153,984 x 262,147
-// clustered 720 / 356, 1M x 1M (pruned scan with the ordering) 1,890 / 1,293; FP64 8,191 x 131,072
-// 92 / 49.
-__device__ __forceinline__ uint32_t hilbert_of(float x, float y, float4 box)
-{
-    const float sx = box.z > box.x ? 65535.0f / (box.z - box.x) : 0.0f;
-    const float sy = box.w > box.y ? 65535.0f / (box.w - box.y) : 0.0f;
-    const float fx = fminf(fmaxf((x - box.x) * sx, 0.0f), 65535.0f);
-    const float fy = fminf(fmaxf((y - box.y) * sy, 0.0f), 65535.0f);
-    return hilbert_index(static_cast<uint32_t>(fx), static_cast<uint32_t>(fy));
-}
-
 // Kahan step: adds v to the running sum h whose compensation (excess added so far) is c.
 template <typename T>
 __device__ __forceinline__ void kahan_add(T &h, T &c, T v)

@@ -33,6 +33,7 @@
 
 #include "aidw_runtime.h"
 #include "f32_device.cuh"
+#include "hilbert.cuh"
 
 namespace aidw {
 
@@ -409,12 +410,17 @@ __global__ void batch_keys_kernel(const BatchItemDev *__restrict__ items, int it
                                   uint32_t *keys, uint32_t *vals, uint32_t *item_of)
 {
     const BatchItemDev &it = items[blockIdx.y];
+    if (static_cast<int64_t>(blockIdx.x) * blockDim.x >= it.m)
+        return;
+    __shared__ __align__(4) uint16_t hilbert[1024];
+    load_hilbert_table(hilbert);
+    __syncthreads();
     const float4 box = *it.ds.box;
     const uint32_t hi = item_bits > 0 ? (blockIdx.y << (32 - item_bits)) : 0u;
     for (int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; q < it.m;
          q += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         const int64_t g = it.qoff + q;
-        keys[g] = hi | (hilbert_of(it.qx[q], it.qy[q], box) >> item_bits);
+        keys[g] = hi | (hilbert_of(it.qx[q], it.qy[q], box, hilbert) >> item_bits);
         vals[g] = static_cast<uint32_t>(g);
         item_of[g] = blockIdx.y;
     }

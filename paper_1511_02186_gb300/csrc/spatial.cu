@@ -11,6 +11,7 @@
 #include <cstdint>
 
 #include "aidw_internal.cuh"
+#include "hilbert.cuh"
 
 namespace aidw {
 namespace {
@@ -68,6 +69,9 @@ __global__ void curve_keys_kernel(const float *__restrict__ x, const float *__re
                                    const float4 *__restrict__ box, uint32_t *keys,
                                    uint32_t *vals)
 {
+    __shared__ __align__(4) uint16_t hilbert[1024];
+    load_hilbert_table(hilbert);
+    __syncthreads();
     const float4 b = *box;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n_total;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
@@ -75,7 +79,7 @@ __global__ void curve_keys_kernel(const float *__restrict__ x, const float *__re
         if (i < n) {
             const float px = xy ? xy[i].x : x[i];
             const float py = xy ? xy[i].y : y[i];
-            key = hilbert_of(px, py, b);
+            key = hilbert_of(px, py, b, hilbert);
         }
         keys[i] = key;
         vals[i] = static_cast<uint32_t>(i);
@@ -291,10 +295,13 @@ __global__ void curve_keys_f64_kernel(const double *__restrict__ x,
                                        const float4 *__restrict__ box, uint32_t *keys,
                                        uint32_t *vals)
 {
+    __shared__ __align__(4) uint16_t hilbert[1024];
+    load_hilbert_table(hilbert);
+    __syncthreads();
     const float4 b = *box;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        keys[i] = hilbert_of(static_cast<float>(x[i]), static_cast<float>(y[i]), b);
+        keys[i] = hilbert_of(static_cast<float>(x[i]), static_cast<float>(y[i]), b, hilbert);
         vals[i] = static_cast<uint32_t>(i);
     }
 }
