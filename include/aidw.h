@@ -92,7 +92,9 @@ void aidw_params_default(aidw_params *p);
 
 /* ---- context -------------------------------------------------------------------------- */
 /* Creates a context on CUDA device `device`. hbm_budget_bytes caps the device memory the
- * context holds at once (datasets + per-call scratch); 0 means "whatever the device has".
+ * context holds at once (datasets + per-call scratch); 0 means "whatever the device has". The
+ * context keeps up to 1 GiB of the memory of destroyed datasets (of up to 64 MiB each) for its
+ * next calls, and no more than the budget leaves beside what it holds.
  * It also places aidw_interpolate_noalloc's 16 MiB scratch array on the device (once per
  * device and process; not charged to the budget).
  * Returns AIDW_ERR_UNSUPPORTED if the device is not compute capability 10.3. */
@@ -108,8 +110,9 @@ int aidw_shutdown(aidw_ctx *ctx);
  * dtype is AIDW_DTYPE_F32 or AIDW_DTYPE_F64 for all three arrays.
  * Errors: INVALID_ARG if n < 1, n > 2^31 - 2048, area is not finite and > 0, or any x, y, z
  * is NaN or infinite (checked on the device after the copy); OOM if the memory or the budget
- * runs out. This call is synchronous; with device arrays it first waits for the device, so that
- * work already enqueued on any stream that writes them is done. */
+ * runs out (idle memory the context keeps is given back first). This call is synchronous; with
+ * device arrays it first waits for the device, so that work already enqueued on any stream that
+ * writes them is done. */
 int aidw_create_dataset(aidw_ctx *ctx, const void *x, const void *y, const void *z, int64_t n,
                         double area, int32_t dtype, aidw_dataset *out);
 

@@ -187,29 +187,51 @@ void ctx_free(aidw_ctx *ctx, void *p, size_t bytes, cudaStream_t st)
 
 // Blocks of a dataset and of its construction: from the context's pool up to kPoolDatasetBytes
 // (cudaMalloc and cudaFree take about 95 us together and wait for the device), else by cudaMalloc.
-// What the pool keeps beyond kPoolKeepBytes is given back when a dataset is destroyed.
+// What the pool keeps idle beyond kPoolKeepBytes, or beyond what the budget leaves, is given back
+// when a dataset is created by cudaMalloc or destroyed, and all of it where memory has run out.
 constexpr size_t kPoolDatasetBytes = size_t(64) << 20;
 constexpr size_t kPoolKeepBytes = size_t(1) << 30;
+
+static void pool_trim(aidw_ctx *ctx, size_t keep)
+{
+    if (ctx->budget) {
+        std::lock_guard<std::mutex> g(ctx->mu);
+        keep = std::min(keep, ctx->budget - std::min(ctx->budget, ctx->in_use));
+    }
+    uint64_t reserved = 0, used = 0;
+    if (cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrReservedMemCurrent, &reserved) ==
+            cudaSuccess &&
+        reserved > keep && cudaStreamSynchronize(0) == cudaSuccess &&
+        cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess &&
+        reserved - used > keep)
+        cudaMemPoolTrimTo(ctx->pool, used + keep);
+}
 
 static cudaError_t dataset_alloc(aidw_ctx *ctx, size_t bytes, void **p, bool *pooled)
 {
     *pooled = bytes <= kPoolDatasetBytes;
-    return *pooled ? cudaMallocFromPoolAsync(p, bytes, ctx->pool, 0) : cudaMalloc(p, bytes);
+    const auto alloc = [&] {
+        return *pooled ? cudaMallocFromPoolAsync(p, bytes, ctx->pool, 0) : cudaMalloc(p, bytes);
+    };
+    if (!*pooled)
+        pool_trim(ctx, kPoolKeepBytes);
+    cudaError_t e = alloc();
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        cudaDeviceSynchronize();
+        pool_trim(ctx, 0);
+        e = alloc();
+    }
+    return e;
 }
 
-static void dataset_free(aidw_ctx *ctx, void *p, bool pooled)
+// Frees a block whose use has ended (the caller has synchronised).
+static void dataset_free(void *p, bool pooled)
 {
-    if (!pooled) {
+    if (pooled)
+        cudaFreeAsync(p, 0);
+    else
         cudaFree(p);
-        return;
-    }
-    cudaFreeAsync(p, 0);
-    uint64_t reserved = 0, used = 0;
-    if (cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrReservedMemCurrent, &reserved) ==
-            cudaSuccess &&
-        cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess &&
-        reserved - used > kPoolKeepBytes)
-        cudaMemPoolTrimTo(ctx->pool, used + kPoolKeepBytes);
 }
 
 size_t ctx_budget_left(aidw_ctx *ctx)
@@ -1131,7 +1153,7 @@ int aidw_shutdown(aidw_ctx *ctx)
     ctx->serving = nullptr;
     cudaDeviceSynchronize();
     for (auto &kv : ctx->datasets)
-        dataset_free(ctx, kv.second.block, kv.second.pooled);
+        dataset_free(kv.second.block, kv.second.pooled);
     ctx->datasets.clear();
     if (ctx->pinned)
         cudaFreeHost(ctx->pinned);
@@ -1215,7 +1237,7 @@ int aidw_create_dataset(aidw_ctx *ctx, const void *x, const void *y, const void 
     bool tmp_pooled = false;
     if (dataset_alloc(ctx, tmp_bytes, &tmp, &tmp_pooled) != cudaSuccess) {
         cudaGetLastError();
-        dataset_free(ctx, blk, blk_pooled);
+        dataset_free(blk, blk_pooled);
         unreserve();
         return AIDW_ERR_OOM;
     }
@@ -1304,12 +1326,15 @@ int aidw_create_dataset(aidw_ctx *ctx, const void *x, const void *y, const void 
     } else if (seen[0]) {
         rc = AIDW_ERR_INVALID_ARG;
     }
-    dataset_free(ctx, tmp, tmp_pooled);
+    dataset_free(tmp, tmp_pooled);
     if (rc) {
-        dataset_free(ctx, blk, blk_pooled);
+        dataset_free(blk, blk_pooled);
         unreserve();
-        return rc;
     }
+    if (ctx->budget)
+        pool_trim(ctx, kPoolKeepBytes);
+    if (rc)
+        return rc;
     DatasetRec rec;
     rec.dev.nxy2 = nxy2;
     rec.dev.zz = zz;
@@ -1353,9 +1378,13 @@ int aidw_destroy_dataset(aidw_ctx *ctx, aidw_dataset ds)
     }
     cudaSetDevice(ctx->device);
     cudaDeviceSynchronize();
-    dataset_free(ctx, rec.block, rec.pooled);
-    std::lock_guard<std::mutex> g(ctx->mu);
-    ctx->in_use -= rec.bytes;
+    dataset_free(rec.block, rec.pooled);
+    {
+        std::lock_guard<std::mutex> g(ctx->mu);
+        ctx->in_use -= rec.bytes;
+    }
+    if (rec.pooled)
+        pool_trim(ctx, kPoolKeepBytes);
     return AIDW_OK;
 }
 
