@@ -191,12 +191,14 @@ void ctx_free(aidw_ctx *ctx, void *p, size_t bytes, cudaStream_t st)
 // when a dataset is created by cudaMalloc or destroyed, and all of it where memory has run out.
 constexpr size_t kPoolDatasetBytes = size_t(64) << 20;
 constexpr size_t kPoolKeepBytes = size_t(1) << 30;
+constexpr size_t kPoolGranule = size_t(32) << 20;  // the pool trims in steps of this at most
 
 static void pool_trim(aidw_ctx *ctx, size_t keep)
 {
     if (ctx->budget) {
         std::lock_guard<std::mutex> g(ctx->mu);
-        keep = std::min(keep, ctx->budget - std::min(ctx->budget, ctx->in_use));
+        const size_t left = ctx->budget - std::min(ctx->budget, ctx->in_use);
+        keep = std::min(keep, left - std::min(left, kPoolGranule));
     }
     uint64_t reserved = 0, used = 0;
     if (cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrReservedMemCurrent, &reserved) ==
