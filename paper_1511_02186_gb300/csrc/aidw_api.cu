@@ -731,6 +731,22 @@ bool use_warp_knn(int precision, const DatasetDev &ds, int64_t m)
     return m <= kWarpKnnMaxQueries || static_cast<double>(m) <= most;
 }
 
+bool same_call_kernels(aidw_ctx *ctx, const DatasetDev &ds, int64_t m, const aidw_params &p,
+                       const aidw_tune_config &a, const aidw_tune_config &b)
+{
+    const Plan pa = make_plan(ctx, p.precision, ds.n, ds.n_pad, m, p.k, false, 0, 0, &a, &p, &ds);
+    const Plan pb = make_plan(ctx, p.precision, ds.n, ds.n_pad, m, p.k, false, 0, 0, &b, &p, &ds);
+    // Phase 2 with point groups has one shape of its own.
+    if (pa.w.qblocks != pb.w.qblocks || pa.w.splits != pb.w.splits ||
+        (pa.pg == 1 && (pa.qw != pb.qw || pa.tw != pb.tw)))
+        return false;
+    if (use_warp_knn(p.precision, ds, m))
+        return true;  // the per-query scan has no lists
+    const bool cull = use_culled_knn(p.precision, ds, m, false, pa);
+    return cull == use_culled_knn(p.precision, ds, m, false, pb) && pa.kp == pb.kp &&
+           (!cull || pa.kq == pb.kq);
+}
+
 void plan_culled_knn(Plan *pl, int64_t n_pad)
 {
     pl->knn.splits = 1;

@@ -55,6 +55,9 @@ Plan make_plan(aidw_ctx *ctx, int precision, int64_t n, int64_t n_pad, int64_t m
                bool with_idx, int force_knn_splits, int force_w_splits,
                const aidw_tune_config *cfg = nullptr, const aidw_params *classes = nullptr,
                const DatasetDev *ds = nullptr);
+// Whether an FP32 call (planned route, no kNN output) runs the same kernels under two shapes.
+bool same_call_kernels(aidw_ctx *ctx, const DatasetDev &ds, int64_t m, const aidw_params &p,
+                       const aidw_tune_config &a, const aidw_tune_config &b);
 aidw_tune_config ctx_tune(aidw_ctx *ctx);
 void ctx_set_tune(aidw_ctx *ctx, const aidw_tune_config &c);
 int interpolate_impl(aidw_ctx *ctx, int64_t dsid, const void *qx, const void *qy, int64_t m,

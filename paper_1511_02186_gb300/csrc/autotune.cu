@@ -387,16 +387,9 @@ int aidw_autotune_interpolate(aidw_ctx *ctx, aidw_dataset ds, const void *qx, co
             *t = best_run;
             return r;
         };
-        const int k = p->k;
         auto skip = [&](const aidw_tune_config &c, const aidw_tune_config &b) {
             // The same kernels as the shape already timed: nothing to time.
-            const int kc = f32_list_length(k, c.knn_list), kb = f32_list_length(k, b.knn_list);
-            return kc == kb &&
-                   cull_queries_per_thread(kc, c.knn_queries_per_thread) ==
-                       cull_queries_per_thread(kb, b.knn_queries_per_thread) &&
-                   c.queries_per_thread == b.queries_per_thread &&
-                   c.tile_points == b.tile_points && c.split_points == b.split_points &&
-                   c.ctas_per_sm == b.ctas_per_sm;
+            return same_call_kernels(ctx, dev, m, *p, c, b);
         };
         const std::vector<Field> fields = {
             {&aidw_tune_config::queries_per_thread, {2, 4, 8}},
