@@ -270,9 +270,12 @@ cudaError_t run_pipe_probe(int sm_count, aidw_pipe_rates *out);
 // read with __ldcg or through a pointer without __restrict__: a plain load of a const __restrict__
 // array may become a read-only load, which wants the array unchanged from the kernel's start on,
 // and that may now come before the array is written.
-// A kernel without grid_trigger releases the next one when its blocks end: the FP64 phase 1 and
-// selection, which the next kernel's large blocks would crowd (FP64 1,024 x 1,024: 74 us without
-// chaining, 63 us chained, 80 us with triggers there too; FP32 1,024 x 1,024: 37 and 33 us).
+// A kernel without grid_trigger releases the next one when its blocks end: the FP64 phase 1, and the
+// selections, which the phase-2 blocks behind them would crowd and then lie unevenly on the SMs
+// (us, FP64 1,024 x 1,024: without chaining 74, chained 63, with triggers there too 80; FP32 with /
+// without the selection's trigger: 1,024 x 1,024 33 / 31, 5,000 x 4,000 84 / 64, 5,000 x 30,000 150 /
+// 120, 32,000 x 4,000 202 / 156, 34,231 x 4,373 over ordered queries 303 / 261, and before
+// chaining 300).
 #if defined(__CUDACC__)
 
 template <typename... P, typename... A>

@@ -53,7 +53,6 @@ f32_select_kernel(int64_t m, int S, int k, double r_exp, AlphaMap am,
                   int32_t *__restrict__ out_knn, const uint32_t *__restrict__ perm,
                   const float *__restrict__ qx, const float *__restrict__ qy, ClassOrder co)
 {
-    grid_trigger();
     grid_wait();
     const int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (q < m) {
