@@ -62,7 +62,7 @@ constexpr float kClassMaxLog2 = 64.0f;
 // without: 250 points 510 / 502, 500 693 / 678, 1,000 908 / 910, 2,000 1,273 / 1,318, 4,000 1,951 /
 // 2,007; 256 of 4,096: 522 / 508, 712 / 702, 934 / 933, 1,372 / 1,371, 2,161 / 2,171).
 constexpr int64_t kBatchClassMinQueries = 4096;
-constexpr int64_t kBatchClassMinPoints = 2000;
+constexpr int64_t kBatchClassMinPoints = 1000;
 constexpr int kPointGroups = 4;  // phase 2 with point groups (Plan::pg)
 
 // Levels and bounds of Eq. 5 and Eq. 6, passed to kernels by value.

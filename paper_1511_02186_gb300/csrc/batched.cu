@@ -302,14 +302,15 @@ f32_batch_kernel(const BatchItemDev *__restrict__ items, const WorkUnit *__restr
                 const QParamF32 p = select_list<KP>(q, it.m, it.k, it.r_exp, it.am, it.part_d2,
                                                     &alpha);
                 const FusedSelect fsel{it.r_exp, it.am, it.qparam, it.out_alpha, it.perm, it.co,
-                                       it.m};
-                fused_select_store(p, alpha, fsel, q, it.sqx[q], it.sqy[q]);
+                                       it.m, it.sqx, it.sqy};
+                fused_select_store(p, alpha, fsel, q);
             }
             cta_publish(it.cnt_ready);
         } else if (wu.type == kUnitKnn) {
             // Pruned scan with the selection fused: the query block is complete afterwards.
             const int64_t qbase = static_cast<int64_t>(wu.qblock) * it.knn.q_per_block;
-            const FusedSelect fsel{it.r_exp, it.am, it.qparam, it.out_alpha, it.perm, it.co, it.m};
+            const FusedSelect fsel{it.r_exp, it.am, it.qparam, it.out_alpha, it.perm, it.co,
+                                   it.m, it.sqx, it.sqy};
 #define AIDW_CULL_UNIT(KP, Q)                                                                  \
     ok = knn_cull_unit<KP, Q, false>(it.ds, it.m, qbase, it.ntiles, it.ntiles_p2, it.sqx, it.sqy, \
                                      it.k, it.part_d2, nullptr, err, ktile, ts, order, nullptr,  \
@@ -521,9 +522,10 @@ bool lists_in_sums(int k, const PassPlan &pw)
 constexpr int64_t kBatchWarpMinPoints = 65536;
 constexpr int64_t kBatchWarpMaxQueries = 131072;
 constexpr int64_t kBatchCullMinQueries = 8192;
-// Queries of a batch that fill the GPU, and, in such a batch, the fewest queries of an item whose
-// block shares tiles and the most points per query.
-constexpr int64_t kBatchCrowd = 200000;
+// Queries of a batch that fill the GPU (64 items of 2,048 queries against 8,000 points: pruned 0.87,
+// one per warp 0.82 ms; 89 of 756 to 4,536 against 7,153, 188,000 queries: 1.00 / 1.10), and, in such
+// a batch, the fewest queries of an item whose block shares tiles and the most points per query.
+constexpr int64_t kBatchCrowd = 150000;
 constexpr int64_t kBatchCrowdMinQueries = 1024;
 constexpr int64_t kBatchCrowdPointsPerQuery = 5;
 

@@ -369,11 +369,11 @@ struct FusedSelect {
     const uint32_t *perm;  // curve order position -> caller's query index
     ClassOrder co;
     int64_t m;
+    const float *sqx, *sqy;  // the queries in curve order
 };
 
 __device__ __forceinline__ void fused_select_store(const QParamF32 &p, double alpha,
-                                                   const FusedSelect &fs, int64_t q, float x,
-                                                   float y)
+                                                   const FusedSelect &fs, int64_t q)
 {
     const uint32_t qo = fs.perm[q];
     if (fs.out_alpha)
@@ -385,8 +385,8 @@ __device__ __forceinline__ void fused_select_store(const QParamF32 &p, double al
     const int cls = power_class(p, fs.co, 0);
     const int64_t at = class_place(fs.co.cnt, cls);
     const int64_t o = cls == kClassA ? at : fs.m - 1 - at;
-    fs.co.qx[o] = x;
-    fs.co.qy[o] = y;
+    fs.co.qx[o] = fs.sqx[q];
+    fs.co.qy[o] = fs.sqy[q];
     fs.co.qp[o] = p;
     fs.co.id[o] = qo;
 }
@@ -394,12 +394,11 @@ __device__ __forceinline__ void fused_select_store(const QParamF32 &p, double al
 // One query of a fused selection (kept out of line: it runs once per query, and inlined into
 // the scan it would lengthen the scan's register life ranges).
 static __device__ __noinline__ void fused_select_query(const float *d, int k,
-                                                       const FusedSelect *fs, int64_t q, float x,
-                                                       float y)
+                                                       const FusedSelect *fs, int64_t q)
 {
     double alpha;
     const QParamF32 p = select_params(d, k, fs->r_exp, fs->am, &alpha);
-    fused_select_store(p, alpha, *fs, q, x, y);
+    fused_select_store(p, alpha, *fs, q);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -767,7 +766,7 @@ __device__ __forceinline__ bool knn_cull_unit(const DatasetDev &ds, int64_t m, i
             const int64_t q = wbase + j * 32;
             if (q >= m)
                 continue;
-            fused_select_query(d[j], k, fsel, q, sqx[q], sqy[q]);
+            fused_select_query(d[j], k, fsel, q);
         }
         return true;
     }
