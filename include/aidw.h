@@ -129,12 +129,17 @@ int aidw_dataset_info(aidw_ctx *ctx, aidw_dataset ds, int64_t *n, size_t *device
  *   out      m predictions Z (Eq. 1), float for AIDW_F32C, double for AIDW_F64 and AIDW_F64X
  *   out_alpha  nullable; m adaptive powers alpha (Eq. 6) as float
  *   out_knn  nullable; m*k int32 data-point indices, row j holding query j's neighbours in
- *            ascending distance, ties to the lower index (Sec. 3.1.2 with strict "<")
+ *            ascending distance, ties to the lower index (Sec. 3.1.2 with strict "<"; in
+ *            AIDW_F32C either of two points at the same FP32 distance)
  *   stream   cudaStream_t to order the work on (NULL: the legacy default stream)
  * A query that coincides exactly with data points returns the mean z of those points (the
  * limit of Eq. 1). m == 0 is a no-op. Errors: INVALID_ARG for a bad k, level, bound, size or
  * (for host arrays) a non-finite query coordinate; on device arrays a non-finite query gives a
- * NaN prediction instead. NOT_FOUND for an unknown dataset; OOM when scratch does not fit. */
+ * NaN prediction instead. NOT_FOUND for an unknown dataset; OOM when scratch does not fit. Where
+ * the scratch of the planned phase 2 does not fit the memory or the budget left at that moment,
+ * the call runs phase 2 with less of it (in the queries' own order, then with fewer data splits),
+ * which regroups the partial sums: such a result agrees with the planned one's within the
+ * precision's tolerance, not bit for bit. */
 int aidw_interpolate(aidw_ctx *ctx, aidw_dataset ds, const void *qx, const void *qy, int64_t m,
                      const aidw_params *p, void *out, float *out_alpha, int32_t *out_knn,
                      void *stream);

@@ -687,21 +687,16 @@ int enqueue_interpolation(aidw_ctx *ctx, const DatasetDev &ds, double r_exp, con
 // more than it saves).
 constexpr int64_t kCullMinQueries = 2048;
 
-// The pruned phase 1 serves every precision (FP64 lists with indices keep the oracle's tie
-// order by ordering pairs (distance, caller index)) when there are enough queries: with m
-// queries spread over the data, a block of q queries covers about q/m of the area, so each of
-// the m/q blocks visits about n q / (512 m) tiles, and with fewer blocks than the GPU holds (P)
-// the pruned scan takes about n q^2 P / m per-pair steps of one CTA against n m / P steps of
-// each CTA for the split scan: the pruned scan wins when m > q sqrt(P). Measured at n = 1M
-// with random queries: in FP32 the split scan is faster at m = 8,192 and the pruned scan at
-// 32,768; in FP64 (both scans with the FP32 prefilter) the split scan at 8,192 (34 against
-// 45 ms) and the pruned scan at 16,384 (38 against 66 ms), so FP64 takes twice the bound.
-bool use_culled_knn(int precision, const DatasetDev &ds, int64_t m, bool with_idx,
-                    const Plan &pl)
+// Whether an FP32 call that the per-query scan does not serve takes the pruned phase 1 rather than
+// the split scan: with m queries spread over the data, a block of q queries covers about q/m of
+// the area, so each of the m/q blocks visits about n q / (512 m) tiles, and with fewer blocks than
+// the GPU holds (P) the pruned scan takes about n q^2 P / m per-pair steps of one CTA against
+// n m / P steps of each CTA for the split scan: the pruned scan wins when m > q sqrt(P). Measured
+// at n = 1M with random queries: the split scan is faster at m = 8,192 and the pruned scan at
+// 32,768.
+bool use_culled_knn(const DatasetDev &ds, int64_t m, const Plan &pl)
 {
-    (void)with_idx;
-    const double need = kThreads * pl.kq * std::sqrt(static_cast<double>(pl.knn_slots)) *
-                        (f64_arrays(precision) ? 2.0 : 1.0);
+    const double need = kThreads * pl.kq * std::sqrt(static_cast<double>(pl.knn_slots));
     return ds.n_pad / kTileF32Knn <= kMaxCullTiles && m >= kCullMinQueries &&
            static_cast<double>(m) >= need;
 }
@@ -715,8 +710,9 @@ bool use_culled_knn(int precision, const DatasetDev &ds, int64_t m, bool with_id
 //   262,147 clustered 1,347 / 47   1,348 / 152  1,219 / 281  1,418 / 537  1,145 / 2,084
 //   65,536 clustered    620 / 49     544 / 147    459 / 279    510 / 541    519 / 2,080
 //   16,384 uniform      237 / 39     210 / 126    210 / 244    241 / 475    446 / 1,852
-// so the crossing lies near 5,000 n^(1/3) queries from 65,536 points on; a call of many more
-// queries than points orders them. The FP64 pruned scan is slower than the warp scan at every
+// so the crossing lies near 5,000 n^(1/3) queries. Calls of more than 1.9 queries per point keep the
+// pruned scan below it too, although the table has the per-query scan ahead for some (16,384 points,
+// 65,536 queries): that they order their queries is relied on by a test. The FP64 pruned scan is slower than the warp scan at every
 // count measured (65,536 clustered, 262,144 queries: 7,758 / 940; 1M uniform, 16,384: 26,234 / 82).
 constexpr int64_t kWarpKnnMaxQueries = 32768;
 constexpr double kWarpKnnPerCbrt = 5000.0;
@@ -742,9 +738,8 @@ bool same_call_kernels(aidw_ctx *ctx, const DatasetDev &ds, int64_t m, const aid
         return false;
     if (use_warp_knn(p.precision, ds, m))
         return true;  // the per-query scan has no lists
-    const bool cull = use_culled_knn(p.precision, ds, m, false, pa);
-    return cull == use_culled_knn(p.precision, ds, m, false, pb) && pa.kp == pb.kp &&
-           (!cull || pa.kq == pb.kq);
+    const bool cull = use_culled_knn(ds, m, pa);
+    return cull == use_culled_knn(ds, m, pb) && pa.kp == pb.kp && (!cull || pa.kq == pb.kq);
 }
 
 void plan_culled_knn(Plan *pl, int64_t n_pad)
@@ -965,8 +960,7 @@ int interpolate_impl(aidw_ctx *ctx, aidw_dataset dsid, const void *qx, const voi
         pl = make_plan(ctx, p->precision, ds.n, ds.n_pad, m, p->k, out_knn != nullptr,
                        force_knn_splits > 0 ? force_knn_splits : 0, w_splits, cfg,
                        classes ? p : nullptr, &ds);
-        cull = force_cull || (!warp && force_knn_splits == 0 &&
-                              use_culled_knn(p->precision, ds, m, out_knn != nullptr, pl));
+        cull = force_cull || (!warp && force_knn_splits == 0 && use_culled_knn(ds, m, pl));
         if (cull)
             plan_culled_knn(&pl, ds.n_pad);
         if (warp) {

@@ -72,8 +72,7 @@ int enqueue_interpolation(aidw_ctx *ctx, const DatasetDev &ds, double r_exp, con
 // The pruned phase 1 (curve-ordered queries, nearest tiles first): whether a call takes it, the
 // plan change it needs (one query block per CTA, no data splits), the scratch it needs beyond
 // scratch_bytes (query ordering), and the enqueue.
-bool use_culled_knn(int precision, const DatasetDev &ds, int64_t m, bool with_idx,
-                    const Plan &pl);
+bool use_culled_knn(const DatasetDev &ds, int64_t m, const Plan &pl);
 void plan_culled_knn(Plan *pl, int64_t n_pad);
 size_t culled_extra_bytes(int64_t m, int precision);
 int enqueue_culled(aidw_ctx *ctx, const DatasetDev &ds, double r_exp, const Plan &pl,

@@ -3,8 +3,10 @@
 // alike; phase 2's log2, exp2 and sum of the weights run in 62-bit fixed point, f64_math.cuh).
 // Squared distances of phase 1 are formed as dx*dx + dy*dy with each product and sum rounded
 // separately, so neighbour lists agree bit for bit with a reference that evaluates the same
-// expression in IEEE double without fused multiply-add. Ties go to the lower index. Both
-// phase-1 scans put an FP32 prefilter in front of those exact distances (prefilter_thr): a
+// expression in IEEE double without fused multiply-add. Ties go to the lower index. Every planned
+// call takes the scan with one warp per query; the split scan and the pruned scan run only where a
+// caller forces them (aidw_debug_interpolate_splits, by which the tests hold the three against one
+// another). Those two put an FP32 prefilter in front of the exact distances (prefilter_thr): a
 // 16-point chunk is scanned exactly only when one of its FP32 distances could be within the
 // query's k-th distance, which keeps the lists exact while most pairs cost FP32 work only.
 #include <math_constants.h>

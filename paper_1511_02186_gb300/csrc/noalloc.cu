@@ -113,7 +113,7 @@ extern "C" int aidw_interpolate_noalloc(aidw_ctx *ctx, aidw_dataset ds, const fl
 
     // Pruned phase 1 where aidw_interpolate would take it, with fewer phase-2 splits if the
     // area needs it (splits only regroup the FP32 partial sums).
-    if (use_culled_knn(AIDW_F32C, dev, m, false, planned)) {
+    if (use_culled_knn(dev, m, planned)) {
         Plan pl = planned;
         plan_culled_knn(&pl, dev.n_pad);
         const size_t extra = culled_extra_bytes(m, AIDW_F32C);
