@@ -79,19 +79,36 @@ __global__ void convert_dataset_kernel(const T *__restrict__ x, const T *__restr
         atomicMax(reinterpret_cast<unsigned *>(bad + 1) + threadIdx.x, most[threadIdx.x]);
 }
 
+// The exponent t of the power of two that the values of the FP32 copy are multiplied by: the largest
+// from 0 to 100 with n max|z| 2^t below 2^62 (n <= 2^log_n). The unscaled products of the power
+// classes, d^-power z, then stay far from underflow, and the scale changes no bit of a result.
+__host__ __device__ inline int value_exponent(uint32_t z_max_bits, int log_n)
+{
+    const int e = static_cast<int>(z_max_bits >> 23) - 126;  // max|z| < 2^e
+    const int t = 62 - log_n - e;
+    return z_max_bits == 0 || t < 0 ? 0 : (t > 100 ? 100 : t);
+}
+
+__host__ __device__ inline uint32_t pow2_bits(int e)
+{
+    return static_cast<uint32_t>(127 + e) << 23;
+}
+
 // Writes the curve-ordered FP32 layout: stored position i holds caller point perm[i] (padding
-// positions, perm[i] >= n, hold +inf points with value 0).
+// positions, perm[i] >= n, hold +inf points with value 0); z_max is the largest |z|'s bits.
 __global__ void gather_dataset_kernel(const float2 *__restrict__ xy32,
                                       const float *__restrict__ z32,
                                       const uint32_t *__restrict__ perm, int64_t n,
-                                      int64_t n_pad, float4 *nxy2, float2 *zz, int32_t *orig)
+                                      int64_t n_pad, const uint32_t *z_max, int log_n,
+                                      float4 *nxy2, float2 *zz, int32_t *orig)
 {
+    const float scale = __uint_as_float(pow2_bits(value_exponent(*z_max, log_n)));
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n_pad;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         const uint32_t p = perm[i];
         if (p < n) {
             const float2 q = xy32[p];
-            const float v = z32[p];
+            const float v = z32[p] * scale;
             nxy2[i] = make_float4(-q.x, -q.x, -q.y, -q.y);
             zz[i] = make_float2(v, v);
             orig[i] = static_cast<int32_t>(p);
@@ -429,7 +446,8 @@ bool power_classes_fit(int64_t n, float z_max)
 }
 
 // The class loops sum unscaled products: adding one errs by up to 2^-150 where the sum is subnormal,
-// which is 2^(c - 150) on the scale where the nearest point's weight is 1, and n times that in all.
+// which is 2^(c - 150) on the scale where the nearest point's weight is 1, and n times that in all
+// (values as stored, n max|z| near 2^62 unless they are larger by themselves).
 // With c <= 84 - log2 n + log2 z_min it is below 2^-66 z_min, so below FP32 rounding even where
 // every value near the query is 0 and the first other one has a weight of 2^-40 (the general loop's
 // products underflow only below a weight of 2^-126 / |z|).
@@ -668,7 +686,7 @@ int enqueue_interpolation(aidw_ctx *ctx, const DatasetDev &ds, double r_exp, con
         return AIDW_ERR_CUDA;
     marks.at(3);
     e = f64 ? launch_f64_finalize(pl, sc, static_cast<double *>(out), st)
-            : launch_f32_finalize(pl, sc, static_cast<float *>(out), st);
+            : launch_f32_finalize(ds, pl, sc, static_cast<float *>(out), st);
     if (e != cudaSuccess)
         return AIDW_ERR_CUDA;
     marks.at(4);
@@ -811,7 +829,7 @@ int enqueue_culled(aidw_ctx *ctx, const DatasetDev &ds, double r_exp, const Plan
         marks.at(2);
         ok = ok && launch_f32_weights(ds, pl, sx, sy, sc, ctx->d_err, st) == cudaSuccess;
         marks.at(3);
-        ok = ok && launch_f32_finalize(pl, sc, static_cast<float *>(out), st, perm) ==
+        ok = ok && launch_f32_finalize(ds, pl, sc, static_cast<float *>(out), st, perm) ==
                        cudaSuccess;
     }
     if (!ok)
@@ -847,7 +865,7 @@ int enqueue_warp(aidw_ctx *ctx, const DatasetDev &ds, double r_exp, const Plan &
         marks.at(2);
         ok = ok && launch_f32_weights(ds, pl, fx, fy, sc, ctx->d_err, st) == cudaSuccess;
         marks.at(3);
-        ok = ok && launch_f32_finalize(pl, sc, static_cast<float *>(out), st) == cudaSuccess;
+        ok = ok && launch_f32_finalize(ds, pl, sc, static_cast<float *>(out), st) == cudaSuccess;
     } else {
         const bool x = p.precision == AIDW_F64X;
         const double *dx = static_cast<const double *>(qx), *dy = static_cast<const double *>(qy);
@@ -1319,12 +1337,17 @@ int aidw_create_dataset(aidw_ctx *ctx, const void *x, const void *y, const void 
     // Order the FP32 copy along the curve and box every tile. Non-finite inputs go through like any
     // others; the count of them is looked at once, at the end.
     unsigned long long seen[2] = {0, 0};  // non-finite inputs, largest and smallest |z|
+    int log_n = 0;
+    while ((int64_t(1) << log_n) < n)
+        ++log_n;
     bool ok = cudaGetLastError() == cudaSuccess;
     ok = ok && bbox_of(xy32, n, box_scratch, box, 0) == cudaSuccess;
     ok = ok && curve_keys(nullptr, nullptr, xy32, n, n_pad, box, keys, perm, 0) == cudaSuccess;
     ok = ok && radix_sort_pairs(keys, perm, n_pad, sort_tmp, 0) == cudaSuccess;
     if (ok) {
-        gather_dataset_kernel<<<blocks, threads>>>(xy32, z32, perm, n, n_pad, nxy2, zz, orig);
+        gather_dataset_kernel<<<blocks, threads>>>(xy32, z32, perm, n, n_pad,
+                                                   reinterpret_cast<uint32_t *>(check + 1),
+                                                   log_n, nxy2, zz, orig);
         ok = cudaGetLastError() == cudaSuccess;
     }
     ok = ok && tile_boxes(nxy2, ntiles, tbox, 0) == cudaSuccess;
@@ -1359,10 +1382,17 @@ int aidw_create_dataset(aidw_ctx *ctx, const void *x, const void *y, const void 
     rec.dev.z64 = z64;
     rec.dev.n = n;
     rec.dev.n_pad = n_pad;
+    const auto from_bits = [](uint32_t b) {
+        float f;
+        std::memcpy(&f, &b, sizeof(f));
+        return f;
+    };
     const uint32_t z_bits = static_cast<uint32_t>(seen[1]);
-    std::memcpy(&rec.dev.z_max, &z_bits, sizeof(z_bits));
-    const uint32_t zn = static_cast<uint32_t>(seen[1] >> 32), zn_bits = zn ? ~zn : 0x7f800000u;
-    std::memcpy(&rec.dev.z_min, &zn_bits, sizeof(zn_bits));
+    const uint32_t zn = static_cast<uint32_t>(seen[1] >> 32);
+    const int z_exp = value_exponent(z_bits, log_n);
+    rec.dev.z_max = from_bits(z_bits) * from_bits(pow2_bits(z_exp));
+    rec.dev.z_min = zn ? from_bits(~zn) * from_bits(pow2_bits(z_exp)) : INFINITY;
+    rec.dev.z_unscale = from_bits(pow2_bits(-z_exp));
     rec.block = blk;
     rec.pooled = blk_pooled;
     rec.bytes = bytes;

@@ -79,7 +79,7 @@ struct AlphaMap {
 // for four of them) measured the same: 18.53 against 18.54 ms at 262,144 x 262,144. The FP64 copies keep the caller's order.
 struct DatasetDev {
     const float4 *nxy2;     // [n_pad] (-x, -x, -y, -y), curve order
-    const float2 *zz;       // [n_pad] (z, z), curve order
+    const float2 *zz;       // [n_pad] (z, z) / z_unscale, curve order
     const int32_t *orig;    // [n_pad] caller's index of each stored point, -1 for padding
     const float4 *tile_box; // [n_pad / kTileF32Knn] (xmin, ymin, xmax, ymax) of finite points
     const float4 *sub_box;  // [n_pad / kSubTile] the same per 64-point sub-tile
@@ -89,8 +89,9 @@ struct DatasetDev {
     const double *z64;      // [n_pad] caller's order
     int64_t n;
     int64_t n_pad;
-    float z_max;            // largest |z| of the FP32 copy
+    float z_max;            // largest |z| of the FP32 copy, as stored
     float z_min;            // smallest |z| of it other than 0 (+inf: all are 0)
+    float z_unscale;        // power of two that takes a stored value back to the caller's
 };
 
 // How one scan pass is cut into work: query blocks (one CTA each) times data-range splits,
@@ -173,7 +174,7 @@ cudaError_t launch_f32_select(const Plan &pl, int k, double r_exp, const AlphaMa
                               const uint32_t *perm = nullptr);
 cudaError_t launch_f32_weights(const DatasetDev &ds, const Plan &pl, const float *qx,
                                const float *qy, const Scratch &sc, int *err, cudaStream_t st);
-cudaError_t launch_f32_finalize(const Plan &pl, const Scratch &sc, float *out,
+cudaError_t launch_f32_finalize(const DatasetDev &ds, const Plan &pl, const Scratch &sc, float *out,
                                 cudaStream_t st, const uint32_t *perm = nullptr);
 // Phase 1 with one warp per query, in the caller's order (queries that lie far apart compared
 // with the data points): one split's lists in sc.part_d2 (and sc.part_idx when non-null).

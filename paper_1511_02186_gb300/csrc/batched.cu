@@ -387,12 +387,13 @@ f32_batch_kernel(const BatchItemDev *__restrict__ items, const WorkUnit *__restr
             const ClassBlock cb = class_block(it, wu.qblock);
             for (int64_t i = tid; i < cb.n; i += kThreads)
                 it.out[__ldcg(it.co.id + cb.base + cb.dir * i)] =
-                    finalize_query(cb.col0 + i, it.m, it.w.splits, it.part_sum);
+                    finalize_query(cb.col0 + i, it.m, it.w.splits, it.part_sum, it.ds.z_unscale);
         } else {
             const int64_t qbase = static_cast<int64_t>(wu.qblock) * it.w.q_per_block;
             const int64_t qend = min(qbase + it.w.q_per_block, it.m);
             for (int64_t q = qbase + tid; q < qend; q += kThreads)
-                it.out[it.perm[q]] = finalize_query(q, it.m, it.w.splits, it.part_sum);
+                it.out[it.perm[q]] =
+                    finalize_query(q, it.m, it.w.splits, it.part_sum, it.ds.z_unscale);
         }
         if (!ok) {
             if (tid == 0)

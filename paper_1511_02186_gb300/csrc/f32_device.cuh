@@ -1156,11 +1156,11 @@ __device__ __forceinline__ void merge_splits(int64_t q, int64_t m, int s0, int s
 
 // Eq. 1 for one query: merge the S splits' compensated sums in FP64 and divide.
 __device__ __forceinline__ float finalize_query(int64_t q, int64_t m, int S,
-                                                const float *part_sum)
+                                                const float *part_sum, float z_unscale)
 {
     double W = 0.0, WZ = 0.0;
     merge_splits(q, m, 0, 1, S, part_sum, W, WZ);
-    return static_cast<float>(WZ / W);
+    return static_cast<float>(WZ / W * z_unscale);
 }
 
 // Shared-memory barrier set-up common to every kernel that streams tiles.

@@ -223,7 +223,8 @@ f32_weights_class_kernel(DatasetDev ds, int64_t m, PassPlan pp, ClassOrder co,
 template <int R>
 __global__ void __launch_bounds__(256)
 f32_finalize_kernel(int64_t m, int S, const float *__restrict__ part_sum,
-                    float *__restrict__ out, const uint32_t *__restrict__ perm, ClassOrder co)
+                    float *__restrict__ out, const uint32_t *__restrict__ perm, ClassOrder co,
+                    float z_unscale)
 {
     grid_trigger();
     grid_wait();
@@ -255,7 +256,7 @@ f32_finalize_kernel(int64_t m, int S, const float *__restrict__ part_sum,
                             : q < ng + na ? kClassA * m + (q - ng)
                                           : kClassB * m + (q - ng - na)));
     }
-    out[o] = static_cast<float>(WZ / W);
+    out[o] = static_cast<float>(WZ / W * z_unscale);
 }
 
 template <int KP, int Q, bool IDX>
@@ -453,15 +454,16 @@ cudaError_t launch_f32_weights(const DatasetDev &ds, const Plan &pl, const float
                           static_cast<float *>(sc.part_sum), err);
 }
 
-cudaError_t launch_f32_finalize(const Plan &pl, const Scratch &sc, float *out, cudaStream_t st,
-                                const uint32_t *perm)
+cudaError_t launch_f32_finalize(const DatasetDev &ds, const Plan &pl, const Scratch &sc,
+                                float *out, cudaStream_t st, const uint32_t *perm)
 {
     const int R = finalize_threads(pl.w.splits, pl.m);
     const unsigned blocks = static_cast<unsigned>((pl.m * R + 255) / 256);
     auto fn = R == 32 ? f32_finalize_kernel<32>
                       : (R == 8 ? f32_finalize_kernel<8> : f32_finalize_kernel<1>);
     return launch_chained(fn, dim3(blocks), 256, 0, st, pl.m, pl.w.splits,
-                          static_cast<const float *>(sc.part_sum), out, perm, sc.cls);
+                          static_cast<const float *>(sc.part_sum), out, perm, sc.cls,
+                          ds.z_unscale);
 }
 
 }  // namespace aidw

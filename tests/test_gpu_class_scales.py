@@ -51,3 +51,22 @@ def test_points_on_a_line_far_from_the_origin(ctx, levels, span):
     wl.y[:] *= span
     wl.qy[:] *= span
     check(ctx, wl)
+
+
+@pytest.mark.parametrize("side", [10.0, 1e3, 1e5])
+@pytest.mark.parametrize("values", ["zeros", "tiny", "huge", "wide", "mostly zero"])
+def test_value_ranges(ctx, side, values):
+    """The FP32 copy holds the values times a power of two: none at all, the ends of FP32's range,
+    values over 30 orders of magnitude in one dataset, and nearly all 0."""
+    wl = workloads.small_case(43, N, M, k=10, pattern="uniform", side=side)
+    rng = np.random.default_rng(5)
+    wl.z[:] = {"zeros": np.zeros(N), "tiny": rng.uniform(1, 2, N) * 2e-37,
+               "huge": rng.uniform(-1, 1, N) * 1e33, "wide": 10.0 ** rng.uniform(-30, 0, N),
+               "mostly zero": (rng.uniform(0, 1, N) < 1e-3) * rng.uniform(1, 2, N)}[values]
+    if values == "zeros":
+        ds = ctx.create_dataset(wl.x, wl.y, wl.z, wl.area)
+        qx, qy = to_device(wl, aidw.F32C)
+        assert (ctx.interpolate(ds, qx, qy, params_of(wl, aidw.F32C))[0] == 0.0).all()
+        ds.destroy()
+    else:
+        check(ctx, wl)
