@@ -447,10 +447,10 @@ bool power_classes_fit(int64_t n, float z_max)
 
 // The class loops sum unscaled products: adding one errs by up to 2^-150 where the sum is subnormal,
 // which is 2^(c - 150) on the scale where the nearest point's weight is 1, and n times that in all
-// (values as stored, n max|z| near 2^62 unless they are larger by themselves).
-// With c <= 84 - log2 n + log2 z_min it is below 2^-66 z_min, so below FP32 rounding even where
-// every value near the query is 0 and the first other one has a weight of 2^-40 (the general loop's
-// products underflow only below a weight of 2^-126 / |z|).
+// (values as stored, n max|z| near 2^62 unless they are larger by themselves). With c <= 84 - log2 n +
+// log2 z_min it is below 2^-66 z_min, so below FP32 rounding even where every value near the query
+// is 0 and the first other one has a weight of 2^-40 (the general loop's products underflow only
+// below a weight of 2^-126 / |z|).
 float class_c_max(const DatasetDev &ds)
 {
     if (!(ds.z_min < INFINITY))
@@ -730,8 +730,9 @@ bool use_culled_knn(const DatasetDev &ds, int64_t m, const Plan &pl)
 //   16,384 uniform      237 / 39     210 / 126    210 / 244    241 / 475    446 / 1,852
 // so the crossing lies near 5,000 n^(1/3) queries. Calls of more than 1.9 queries per point keep the
 // pruned scan below it too, although the table has the per-query scan ahead for some (16,384 points,
-// 65,536 queries): that they order their queries is relied on by a test. The FP64 pruned scan is slower than the warp scan at every
-// count measured (65,536 clustered, 262,144 queries: 7,758 / 940; 1M uniform, 16,384: 26,234 / 82).
+// 65,536 queries): a test relies on such a call ordering its queries. The FP64 pruned scan is slower
+// than the warp scan at every count measured (65,536 clustered, 262,144 queries: 7,758 / 940; 1M
+// uniform, 16,384: 26,234 / 82).
 constexpr int64_t kWarpKnnMaxQueries = 32768;
 constexpr double kWarpKnnPerCbrt = 5000.0;
 constexpr double kWarpKnnPerPoint = 1.9;
