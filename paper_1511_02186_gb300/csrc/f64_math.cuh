@@ -142,6 +142,8 @@ __device__ __forceinline__ long long log2_52(const NormU64 &v, const Tables &t)
                    (v.m & ((1ull << (63 - kLogBits)) - 1)) << kLogBits, t);
 }
 
+// log2 and (below) exp2 with doubles on both sides, as aidw_debug_f64_log2_exp2 evaluates them. The
+// scan takes the same steps from log2_52 on through power_weight, without a double in between.
 __device__ __forceinline__ double log2_t(double x, const Tables &t)
 {
     const long long b = __double_as_longlong(x);

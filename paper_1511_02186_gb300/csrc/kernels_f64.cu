@@ -779,7 +779,7 @@ f64_select_kernel(int64_t m, int S, int k, double r_exp, AlphaMap am,
 }
 
 // The sum of the weights of one query is kept as an unsigned fixed-point integer with 96
-// fraction bits, accumulated exactly on the integer pipe from the weights exp2_t gives in that
+// fraction bits, accumulated exactly on the integer pipe from the weights power_weight gives in that
 // form (weights are at most 1 + a few ulps, the nearest point's being 1, so the sum of any
 // n < 2^31 of them fits; each weight is truncated below 2^-96, at most n 2^-96 in all against a
 // sum of at least 1).
